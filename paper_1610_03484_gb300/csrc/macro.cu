@@ -23,23 +23,40 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "node_graph.h"
 
 struct rve_macro_s {
     rve_ctx ctx = nullptr;
     int64_t nv = 0, nt = 0;
-    rve::DevBuf tets, geo, mask, hold, diag, x, b, r, z, p, q, acc, gp, W, flags;
-    std::vector<double> vol_h, grad_h;    // host copies of the geometry
+    rve::DevBuf tets, geo, mask, hold, x, b, r, p, q, acc, gp, W, flags;
     std::vector<int32_t> tets_h;
-    std::vector<uint8_t> mask_h;
     double KT[6] = {}, Dc[6] = {};          // symmetric (xx, yy, zz, xy, yz, zx)
     double rho_cp = 0;
     bool have_transport = false, have_face = false, have_state = false;
-    double diag_dt = -1;                    // dt [s] the diagonal was formed for
-    // macro mechanics: held DOFs and their values, traction load, Jacobi
-    // diagonal, displacement, per-tet mean stiffness [nt][36], Gauss-point
-    // stiffness staged from the host [nt*4][36] and stresses [nt*4][6]
-    rve::DevBuf mfix, mval, mload, mdiag, mu, cm, cgp, msig;
+    // assembled operators on the node graph, sliced by 32 rows (see "assembled
+    // operators" below); built on the first solve
+    int64_t n_slices = 0, n_ell = 0;
+    rve::DevBuf g_base, g_col, g_len, g_eptr, g_inc;
+    bool have_graph = false;
+    rve::DevBuf t_mass, t_stiff, t_mat, t_dinv;
+    bool have_stiff = false;
+    double mat_dt = -1;                     // dt [s] that t_mat and t_dinv were formed for
+    // macro mechanics: held DOFs and their values, traction load, inverse Jacobi
+    // diagonal, displacement, per-tet mean stiffness [nt][36], the assembled
+    // stiffness, Gauss-point stiffness staged from the host [nt*4][36] and stresses
+    // [nt*4][6]
+    rve::DevBuf mfix, mval, mload, mdinv, mu, cm, mmat, cgp, msig;
     bool have_mech_bc = false, have_mech_load = false, have_mech_u = false, have_mech_sig = false;
+    // instantiated PCG loops (0 transport, 1 mechanics), reused while the captured
+    // launch parameters stay the same
+    struct Loop {
+        cudaGraphExec_t exec = nullptr;
+        std::vector<unsigned char> key;
+    } loop[2];
+    ~rve_macro_s() {
+        for (auto& l : loop)
+            if (l.exec) cudaGraphExecDestroy(l.exec);
+    }
 };
 
 namespace rve {
@@ -47,165 +64,294 @@ namespace {
 
 constexpr double kKelvin = 273.15;
 
+struct TransportTensors {
+    double KT[6], Dc[6];
+};
+
 __device__ __forceinline__ double sym3(const double* k, int i, int j) {
     if (i == j) return k[i];
     const int s = i + j;   // (0,1) -> 3, (1,2) -> 4, (0,2) -> 5
     return k[s == 1 ? 3 : (s == 3 ? 4 : 5)];
 }
 
-struct MacroParams {
-    double KT[6], Dc[6];
-    double capT, capC;   // capacity / dt of each field (0: stiffness only)
-    int stiff;           // 0: capacity part only
-};
+// --------------------------------------------------- assembled operators
+// Both macro problems are solved with assembled matrices.  On linear tetrahedra a
+// node couples to about 15 nodes, so a row of the elastic matrix costs 15 x 9 FMAs
+// per node, 24 per tetrahedron, where the element-by-element product takes about 117
+// and 12 atomic additions; the transport pair needs 30 per node against 120 per
+// tetrahedron.  FP64 runs at two FMAs per clock and SM here, which is what bounds
+// both forms: on 480k tetrahedra (200 x 40 x 10 cells) one product element by element
+// takes 109 us for either problem; assembled 39 us (mechanics) and 13 us (transport),
+// cold cache.
+//
+// Storage: rows in slices of 32 nodes (sliced ELL); slice s holds ELL rows
+// base[s] .. base[s + 1], ELL row k of a slice the k-th coupled node of its 32 rows,
+// one per lane, so that every load of a warp is contiguous.  Short rows are padded
+// with their own node and zero values.
 
-// y += (C/dt + K) x over both fields, one element per thread, FP64 atomics.
-__global__ void k_macro_apply(int64_t nt, const int32_t* __restrict__ tets, const double* __restrict__ geo,
-                              const double* __restrict__ x, double* __restrict__ y, MacroParams prm) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
-        int v[4];
+// y += C/dt x etc. need the consistent capacity and the stiffness of both fields per
+// entry: mass [ell][32], stiff [ell][32] (conductivity, diffusivity).
+// One thread per (ELL row of the slice, lane).
+__global__ void __launch_bounds__(256) k_transport_entries(int64_t nv, const int64_t* __restrict__ base,
+                                                           const int32_t* __restrict__ col,
+                                                           const int32_t* __restrict__ len,
+                                                           const int32_t* __restrict__ eptr,
+                                                           const int32_t* __restrict__ inc,
+                                                           const int32_t* __restrict__ tets,
+                                                           const double* __restrict__ geo, TransportTensors prm,
+                                                           double* __restrict__ mass, double2* __restrict__ stiff) {
+    const int lane = threadIdx.x & 31;
+    const int64_t s = blockIdx.x, i = s * 32 + lane, row0 = base[s], row1 = base[s + 1];
+    const int n_len = i < nv ? len[i] : 0;
+    for (int64_t row = row0 + (threadIdx.x >> 5); row < row1; row += blockDim.x >> 5) {
+        double m = 0.0, kt = 0.0, kc = 0.0;
+        if (row - row0 < n_len) {
+            const int c = col[row * 32 + lane];
+            for (int q = eptr[i]; q < eptr[i + 1]; ++q) {
+                const int e = inc[q] >> 2, a = inc[q] & 3;
+                for (int b = 0; b < 4; ++b) {
+                    if (tets[(int64_t)e * 4 + b] != c) continue;
+                    const double vol = geo[(int64_t)e * 13];
+                    const double* ga = geo + (int64_t)e * 13 + 1 + a * 3;
+                    const double* gb = geo + (int64_t)e * 13 + 1 + b * 3;
+                    m += (a == b ? 2.0 : 1.0) * vol / 20.0;
+                    double ft = 0.0, fc = 0.0;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = tets[e * 4 + a];
-        const double vol = geo[e * 13];
-        const double* g = geo + e * 13 + 1;   // grad lambda_a, [4][3]
-#pragma unroll
-        for (int f = 0; f < 2; ++f) {
-            double xa[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) xa[a] = x[(int64_t)v[a] * 2 + f];
-            const double* Kf = f == 0 ? prm.KT : prm.Dc;
-            const double cap = f == 0 ? prm.capT : prm.capC;
-            double gr[3] = {0, 0, 0};
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) gr[i] += g[a * 3 + i] * xa[a];
-            double fl[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-                fl[i] = sym3(Kf, i, 0) * gr[0] + sym3(Kf, i, 1) * gr[1] + sym3(Kf, i, 2) * gr[2];
-            const double sum = xa[0] + xa[1] + xa[2] + xa[3];
-            const double cm = cap * vol / 20.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                double ya = cm * (sum + xa[a]);
-                if (prm.stiff) ya += vol * (g[a * 3] * fl[0] + g[a * 3 + 1] * fl[1] + g[a * 3 + 2] * fl[2]);
-                atomicAdd(y + (int64_t)v[a] * 2 + f, ya);
+                    for (int j = 0; j < 3; ++j) {
+                        ft += ga[j] * (sym3(prm.KT, j, 0) * gb[0] + sym3(prm.KT, j, 1) * gb[1] + sym3(prm.KT, j, 2) * gb[2]);
+                        fc += ga[j] * (sym3(prm.Dc, j, 0) * gb[0] + sym3(prm.Dc, j, 1) * gb[1] + sym3(prm.Dc, j, 2) * gb[2]);
+                    }
+                    kt += vol * ft;
+                    kc += vol * fc;
+                }
             }
         }
+        mass[row * 32 + lane] = m;
+        stiff[row * 32 + lane] = make_double2(kt, kc);
     }
 }
 
-// block sum of two values per thread, added atomically to out[0..1]
-__device__ __forceinline__ void block_add2(double a0, double a1, double* out) {
-    __shared__ double s0[256], s1[256];
-    s0[threadIdx.x] = a0;
-    s1[threadIdx.x] = a1;
+// mat = cap mass + stiff for the two fields' capacities per time step, and the
+// inverse diagonal; one warp per slice
+__global__ void __launch_bounds__(256) k_transport_matrix(int64_t nv, int64_t n_slices,
+                                                          const int64_t* __restrict__ base,
+                                                          const int32_t* __restrict__ col,
+                                                          const int32_t* __restrict__ len,
+                                                          const double* __restrict__ mass,
+                                                          const double2* __restrict__ stiff, double capT, double capC,
+                                                          double2* __restrict__ mat, double2* __restrict__ dinv) {
+    const int lane = threadIdx.x & 31;
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, i = s * 32 + lane;
+    if (s >= n_slices) return;
+    const int64_t row0 = base[s], row1 = base[s + 1];
+    const int n_len = i < nv ? len[i] : 0;
+    for (int64_t row = row0; row < row1; ++row) {
+        const double m = mass[row * 32 + lane];
+        const double2 k = stiff[row * 32 + lane];
+        const double2 v = make_double2(fma(capT, m, k.x), fma(capC, m, k.y));
+        mat[row * 32 + lane] = v;
+        if (row - row0 < n_len && col[row * 32 + lane] == i) dinv[i] = make_double2(1.0 / v.x, 1.0 / v.y);
+    }
+}
+
+// b = C/dt x
+__global__ void __launch_bounds__(256) k_transport_rhs(int64_t nv, int64_t n_slices, const int64_t* __restrict__ base,
+                                                       const int32_t* __restrict__ col,
+                                                       const double* __restrict__ mass, double capT, double capC,
+                                                       const double2* __restrict__ x, double2* __restrict__ b) {
+    const int lane = threadIdx.x & 31;
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, i = s * 32 + lane;
+    if (s >= n_slices) return;
+    double at = 0.0, ac = 0.0;
+#pragma unroll 4
+    for (int64_t row = base[s]; row < base[s + 1]; ++row) {
+        const double m = mass[row * 32 + lane];
+        const double2 v = x[col[row * 32 + lane]];
+        at = fma(m, v.x, at);
+        ac = fma(m, v.y, ac);
+    }
+    if (i < nv) b[i] = make_double2(capT * at, capC * ac);
+}
+
+// Scalars of the PCG loop (doubles in device memory).  Two fields each:
+//   [0] (r, z) of this iteration, [2] (p, q), [4] (r, z) of the previous one,
+//   [6] the reference max((b, M^-1 b), (r0, M^-1 r0)), [8] 1 while the field iterates,
+//   [10] the same for the next iteration, [12] iterations, [14] (b, M^-1 b);
+//   [16] iterations of the loop, [17] their limit, [18] the squared tolerance.
+// An iteration is three kernels: the product (which also moves (r, z) and the
+// active flags on), the x/r update and the p update (which also runs the loop
+// control).  Every scalar is written by one thread in a kernel whose other blocks do
+// not read it.
+constexpr int PCG_SCALARS = 20;
+
+// moves the scalars on to the next iteration; one thread per field of one block
+__device__ __forceinline__ void pcg_roll(double* acc, int f) {
+    acc[4 + f] = acc[f];
+    acc[f] = 0.0;
+    acc[8 + f] = acc[10 + f];
+}
+
+// block sums of up to two values per thread, added atomically to out[0..nf-1]
+template <int NF>
+__device__ __forceinline__ void block_add(const double (&a)[NF], double* out) {
+    __shared__ double part[NF][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        double v = a[f];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) part[f][warp] = v;
+    }
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s0[threadIdx.x] += s0[threadIdx.x + w];
-            s1[threadIdx.x] += s1[threadIdx.x + w];
-        }
-        __syncthreads();
+    if (threadIdx.x < NF) {
+        double v = 0.0;
+        for (int w = 0; w < nw; ++w) v += part[threadIdx.x][w];
+        atomicAdd(out + threadIdx.x, v);
     }
-    if (threadIdx.x == 0) {
-        atomicAdd(out, s0[0]);
-        atomicAdd(out + 1, s1[0]);
-    }
+    __syncthreads();
 }
 
-// r = b - y on free rows (0 on held rows), z = r / diag, acc[0..1] += (r, z)
-// and acc[14..15] += (b, M^-1 b) over the free rows (the reference norm)
-// (Vector kernels: nf interleaved fields per row group, field of row i is
-// i % nf; the held mask is indexed by i / mdiv: 2 for the per-node mask of the
-// transport pair, 1 for the per-DOF mask of the mechanics.)
-__global__ void __launch_bounds__(256) k_macro_residual(int64_t n, int nf, int mdiv, const double* __restrict__ b,
+// q = A x for the transport pair and (x, q) per field into acc[2..3]; one warp per
+// slice, one lane per node.  acc null: the product alone.
+__global__ void __launch_bounds__(256) k_transport_product(int64_t nv, int64_t n_slices,
+                                                           const int64_t* __restrict__ base,
+                                                           const int32_t* __restrict__ col,
+                                                           const double2* __restrict__ mat,
+                                                           const double2* __restrict__ x, double2* __restrict__ y,
+                                                           double* __restrict__ acc) {
+    if (acc && blockIdx.x == 0 && threadIdx.x < 2) pcg_roll(acc, threadIdx.x);
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    double dot[2] = {0.0, 0.0};
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < n_slices; s += nw) {
+        const int64_t i = s * 32 + lane, row1 = base[s + 1];
+        double at = 0.0, ac = 0.0;
+#pragma unroll 4
+        for (int64_t row = base[s]; row < row1; ++row) {
+            const double2 m = mat[row * 32 + lane];
+            const double2 v = x[col[row * 32 + lane]];
+            at = fma(m.x, v.x, at);
+            ac = fma(m.y, v.y, ac);
+        }
+        if (i < nv) {
+            const double2 v = x[i];
+            y[i] = make_double2(at, ac);
+            dot[0] = fma(v.x, at, dot[0]);
+            dot[1] = fma(v.y, ac, dot[1]);
+        }
+    }
+    if (acc) block_add<2>(dot, acc + 2);
+}
+
+// Vector kernels: nf interleaved fields of n entries in all, the field of entry i is
+// i % nf; the held mask is indexed by i / mdiv (2 for the per-node mask of the
+// transport pair, 1 for the per-DOF mask of the mechanics).
+
+// r = b - y on free rows (0 on held rows), p = M^-1 r, acc[0] += (r, p) and
+// acc[14] += (b, M^-1 b) over the free rows (the reference norm)
+template <int NF>
+__global__ void __launch_bounds__(256) k_macro_residual(int64_t n, int mdiv, const double* __restrict__ b,
                                                         const double* __restrict__ y,
                                                         const uint8_t* __restrict__ mask,
-                                                        const double* __restrict__ diag, double* __restrict__ r,
-                                                        double* __restrict__ z, double* __restrict__ acc) {
-    double a[2] = {0, 0}, bb[2] = {0, 0};
+                                                        const double* __restrict__ dinv, double* __restrict__ r,
+                                                        double* __restrict__ p, double* __restrict__ acc) {
+    double a[NF] = {}, bb[NF] = {};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = nf == 2 ? (int)(i & 1) : 0;
         const bool held = mask[i / mdiv] != 0;
-        const double ri = held ? 0.0 : b[i] - y[i];
-        const double zi = ri / diag[i];
+        const double bi = b[i], di = dinv[i];
+        const double ri = held ? 0.0 : bi - y[i];
+        const double zi = ri * di;
         r[i] = ri;
-        z[i] = zi;
-        a[f] += ri * zi;
-        if (!held) bb[f] += b[i] * b[i] / diag[i];
+        p[i] = zi;
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            if (NF == 1 || (int)(i & 1) == f) {
+                a[f] += ri * zi;
+                if (!held) bb[f] += bi * (bi * di);
+            }
     }
-    block_add2(a[0], a[1], acc);
-    block_add2(bb[0], bb[1], acc + 14);
+    block_add<NF>(a, acc);
+    block_add<NF>(bb, acc + 14);
 }
 
-// acc[2..3] += (p, q) per field
-__global__ void __launch_bounds__(256) k_macro_dot(int64_t n, int nf, const double* __restrict__ p,
-                                                   const double* __restrict__ q, double* __restrict__ acc) {
-    double a[2] = {0, 0};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[nf == 2 ? (int)(i & 1) : 0] += p[i] * q[i];
-    block_add2(a[0], a[1], acc + 2);
-}
-
-// Per-field scalars, one thread.  acc: [0..1] (r,z) new, [2..3] (p,q),
-// [4..5] (r,z) of the previous iteration, [6..7] the reference max((b, M^-1 b), (r0, M^-1 r0)),
-// [8..9] alpha, [10..11] beta, [12..13] active flags (as doubles).
-__global__ void k_macro_alpha(double* acc) {
-    for (int f = 0; f < 2; ++f) {
-        const double pq = acc[2 + f];
-        const bool ok = acc[12 + f] != 0.0 && pq > 0.0;
-        acc[8 + f] = ok ? acc[4 + f] / pq : 0.0;
-        acc[2 + f] = 0.0;
-        acc[f] = 0.0;                       // for the (r, z) of this iteration
-    }
-}
-__global__ void k_macro_beta(double* acc, double tol2) {
-    for (int f = 0; f < 2; ++f) {
-        const double rz = acc[f];
-        if (acc[12 + f] != 0.0) {
-            acc[10 + f] = acc[4 + f] > 0.0 ? rz / acc[4 + f] : 0.0;
-            acc[4 + f] = rz;
-            if (!(rz > tol2 * acc[6 + f])) acc[12 + f] = 0.0;   // converged (or not finite)
-        }
+// Convergence is relative to the larger of the right-hand side and the initial
+// residual (which carries the held values): a field already at rest
+// (rounding-level residual) takes no iteration.  One thread per field.
+__global__ void k_macro_start(double* acc, int nf, double tol2, int max_iter) {
+    const int f = threadIdx.x;
+    const double rz = f < nf ? acc[f] : 0.0, bb = f < nf ? acc[14 + f] : 0.0;
+    acc[6 + f] = fmax(bb, rz);
+    acc[10 + f] = rz > tol2 * acc[6 + f] ? 1.0 : 0.0;
+    acc[2 + f] = 0.0;
+    acc[12 + f] = 0.0;
+    if (f == 0) {
+        acc[16] = 0.0;
+        acc[17] = (double)max_iter;
+        acc[18] = tol2;
     }
 }
 
-// x += alpha p, r -= alpha q (held rows stay 0), z = r / diag, acc[0..1] += (r, z)
-__global__ void __launch_bounds__(256) k_macro_update(int64_t n, int nf, int mdiv, const uint8_t* __restrict__ mask,
-                                                     const double* __restrict__ diag, double* __restrict__ x,
-                                                     double* __restrict__ r, double* __restrict__ z,
-                                                     const double* __restrict__ p, const double* __restrict__ q,
-                                                     double* __restrict__ acc) {
-    const double al[2] = {acc[8], acc[9]};
-    double a[2] = {0, 0};
+// x += alpha p, r -= alpha q (held rows stay 0), acc[0] += (r, M^-1 r)
+template <int NF>
+__global__ void __launch_bounds__(256) k_macro_update(int64_t n, int mdiv, const uint8_t* __restrict__ mask,
+                                                     const double* __restrict__ dinv, double* __restrict__ x,
+                                                     double* __restrict__ r, const double* __restrict__ p,
+                                                     const double* __restrict__ q, double* __restrict__ acc) {
+    __shared__ double alpha[NF];
+    if (threadIdx.x < NF) {
+        const double pq = acc[2 + threadIdx.x];
+        const bool ok = acc[8 + threadIdx.x] != 0.0 && pq > 0.0;
+        alpha[threadIdx.x] = ok ? acc[4 + threadIdx.x] / pq : 0.0;
+    }
+    __syncthreads();
+    double a[NF] = {};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = nf == 2 ? (int)(i & 1) : 0;
+        const int f = NF == 2 ? (int)(i & 1) : 0;
+        const double al = alpha[f];
         double ri = r[i];
-        if (al[f] != 0.0) {
-            x[i] += al[f] * p[i];
-            ri = mask[i / mdiv] ? 0.0 : ri - al[f] * q[i];
+        if (al != 0.0) {
+            x[i] = fma(al, p[i], x[i]);
+            ri = mask[i / mdiv] ? 0.0 : fma(-al, q[i], ri);
             r[i] = ri;
         }
-        const double zi = ri / diag[i];
-        z[i] = zi;
-        a[f] += ri * zi;
+        const double v = ri * (ri * dinv[i]);
+#pragma unroll
+        for (int g = 0; g < NF; ++g)
+            if (NF == 1 || f == g) a[g] += v;
     }
-    block_add2(a[0], a[1], acc);
+    block_add<NF>(a, acc);
 }
 
-// p = z + beta p for active fields; q = 0
-__global__ void __launch_bounds__(256) k_macro_pupdate(int64_t n, int nf, const double* __restrict__ z,
-                                                      double* __restrict__ p, double* __restrict__ q,
-                                                      const double* __restrict__ acc, int first) {
+// p = M^-1 r + beta p for fields still iterating; loop control
+template <int NF>
+__global__ void __launch_bounds__(256) k_macro_pupdate(int64_t n, const double* __restrict__ dinv,
+                                                      const double* __restrict__ r, double* __restrict__ p,
+                                                      double* __restrict__ acc, cudaGraphConditionalHandle h) {
+    __shared__ double beta[NF];
+    __shared__ int on[NF];
+    if (threadIdx.x < NF) {
+        const int f = threadIdx.x;
+        const double rz = acc[f], old = acc[4 + f];
+        // converged (or not finite): the field stops
+        on[f] = acc[8 + f] != 0.0 && rz > acc[18] * acc[6 + f];
+        beta[f] = old > 0.0 ? rz / old : 0.0;
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        bool any = false;
+        for (int f = 0; f < NF; ++f) {
+            acc[12 + f] += acc[8 + f];
+            acc[10 + f] = on[f] ? 1.0 : 0.0;
+            acc[2 + f] = 0.0;
+            any = any || on[f];
+        }
+        const double it = acc[16] + 1.0;
+        acc[16] = it;
+        cudaGraphSetConditional(h, any && it < acc[17] ? 1u : 0u);
+    }
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = nf == 2 ? (int)(i & 1) : 0;
-        if (first)
-            p[i] = z[i];
-        else if (acc[12 + f] != 0.0)
-            p[i] = z[i] + acc[10 + f] * p[i];
-        q[i] = 0.0;
+        const int f = NF == 2 ? (int)(i & 1) : 0;
+        if (on[f]) p[i] = fma(beta[f], p[i], r[i] * dinv[i]);
     }
 }
 
@@ -317,78 +463,107 @@ __device__ __forceinline__ void mech_bt(double gx, double gy, double gz, const d
     f[2] = gz * sg[2] + gy * sg[4] + gx * sg[5];
 }
 
-// Per tetrahedron: cm = mean over its Gauss points of the symmetric part of C_g,
-// and the Jacobi diagonal |T| b^T cm b of each of its 12 DOFs (b the DOF's
-// column of B), added atomically into diag.
-__global__ void k_mech_material(int64_t nt, const int32_t* __restrict__ tets, const double* __restrict__ geo,
-                                const double* __restrict__ Cgp, double* __restrict__ cm,
-                                double* __restrict__ diag) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
-        double C[36];
+// Per tetrahedron: cm = mean over its Gauss points of the symmetric part of C_g
+__global__ void k_mech_material(int64_t nt, const double* __restrict__ Cgp, double* __restrict__ cm) {
+    const int64_t n = nt * 36;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = i / 36;
+        const int J = (int)(i % 36) / 6, K = (int)(i % 36) % 6;
+        const double* Cq = Cgp + e * 4 * 36;
+        double c = 0.0;
 #pragma unroll
-        for (int k = 0; k < 36; ++k) C[k] = 0.0;
-        for (int q = 0; q < 4; ++q) {
-            const double* Cq = Cgp + (e * 4 + q) * 36;
-#pragma unroll
-            for (int J = 0; J < 6; ++J)
-#pragma unroll
-                for (int K = 0; K < 6; ++K) C[J * 6 + K] += 0.125 * (Cq[J * 6 + K] + Cq[K * 6 + J]);
-        }
-#pragma unroll
-        for (int k = 0; k < 36; ++k) cm[e * 36 + k] = C[k];
-        const double vol = geo[e * 13];
-        const double* g = geo + e * 13 + 1;
-        for (int a = 0; a < 4; ++a) {
-            const double gx = g[a * 3], gy = g[a * 3 + 1], gz = g[a * 3 + 2];
-            const int v = tets[e * 4 + a];
-            for (int i = 0; i < 3; ++i) {
-                double b[6] = {0, 0, 0, 0, 0, 0};
-                if (i == 0) { b[0] = gx; b[3] = gy; b[5] = gz; }
-                if (i == 1) { b[1] = gy; b[3] = gx; b[4] = gz; }
-                if (i == 2) { b[2] = gz; b[4] = gy; b[5] = gx; }
-                double d = 0.0;
-#pragma unroll
-                for (int J = 0; J < 6; ++J)
-#pragma unroll
-                    for (int K = 0; K < 6; ++K) d += b[J] * C[J * 6 + K] * b[K];
-                atomicAdd(diag + (int64_t)v * 3 + i, vol * d);
-            }
-        }
+        for (int q = 0; q < 4; ++q) c += 0.125 * (Cq[q * 36 + J * 6 + K] + Cq[q * 36 + K * 6 + J]);
+        cm[i] = c;
     }
 }
 
-// y += K x: per tetrahedron eps = B x_T, sigma = cm eps, y_a += |T| B_a^T sigma
-__global__ void k_mech_apply(int64_t nt, const int32_t* __restrict__ tets, const double* __restrict__ geo,
-                             const double* __restrict__ cm, const double* __restrict__ x, double* __restrict__ y) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
-        int v[4];
-        double ua[12];
+// The assembled stiffness: 3 x 3 blocks sum_T |T| B_a^T cm B_b of every entry, stored
+// val[(ell row * 9 + 3 r + c) * 32 + lane] (block row r), and the inverse Jacobi
+// diagonal.  One thread per (ELL row of the slice, lane).
+__global__ void __launch_bounds__(256) k_mech_entries(int64_t nv, const int64_t* __restrict__ base,
+                                                      const int32_t* __restrict__ col,
+                                                      const int32_t* __restrict__ len,
+                                                      const int32_t* __restrict__ eptr,
+                                                      const int32_t* __restrict__ inc,
+                                                      const int32_t* __restrict__ tets,
+                                                      const double* __restrict__ geo, const double* __restrict__ cm,
+                                                      double* __restrict__ val, double* __restrict__ dinv) {
+    const int lane = threadIdx.x & 31;
+    const int64_t s = blockIdx.x, i = s * 32 + lane, row0 = base[s], row1 = base[s + 1];
+    const int n_len = i < nv ? len[i] : 0;
+    for (int64_t row = row0 + (threadIdx.x >> 5); row < row1; row += blockDim.x >> 5) {
+        double A[9];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            v[a] = tets[e * 4 + a];
+        for (int k = 0; k < 9; ++k) A[k] = 0.0;
+        int c = -1;
+        if (row - row0 < n_len) {
+            c = col[row * 32 + lane];
+            for (int q = eptr[i]; q < eptr[i + 1]; ++q) {
+                const int e = inc[q] >> 2, a = inc[q] & 3;
+                for (int b = 0; b < 4; ++b) {
+                    if (tets[(int64_t)e * 4 + b] != c) continue;
+                    const double vol = geo[(int64_t)e * 13];
+                    const double* ga = geo + (int64_t)e * 13 + 1 + a * 3;
+                    const double* gb = geo + (int64_t)e * 13 + 1 + b * 3;
+                    const double* C = cm + (int64_t)e * 36;
+                    const double gx = vol * gb[0], gy = vol * gb[1], gz = vol * gb[2];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) ua[a * 3 + i] = x[(int64_t)v[a] * 3 + i];
+                    for (int d = 0; d < 3; ++d) {
+                        // |T| C times the strain of the unit displacement d of node b
+                        double sg[6], f[3];
+#pragma unroll
+                        for (int J = 0; J < 6; ++J)
+                            sg[J] = d == 0   ? C[J * 6] * gx + C[J * 6 + 3] * gy + C[J * 6 + 5] * gz
+                                    : d == 1 ? C[J * 6 + 1] * gy + C[J * 6 + 3] * gx + C[J * 6 + 4] * gz
+                                             : C[J * 6 + 2] * gz + C[J * 6 + 4] * gy + C[J * 6 + 5] * gx;
+                        mech_bt(ga[0], ga[1], ga[2], sg, f);
+#pragma unroll
+                        for (int r = 0; r < 3; ++r) A[3 * r + d] += f[r];
+                    }
+                }
+            }
         }
-        const double vol = geo[e * 13];
-        const double* g = geo + e * 13 + 1;
-        double eps[6], sg[6];
-        mech_strain(g, ua, eps);
-        const double* C = cm + e * 36;
 #pragma unroll
-        for (int J = 0; J < 6; ++J) {
-            double t = 0.0;
+        for (int k = 0; k < 9; ++k) val[(row * 9 + k) * 32 + lane] = A[k];
+        if (c == i)
 #pragma unroll
-            for (int K = 0; K < 6; ++K) t += C[J * 6 + K] * eps[K];
-            sg[J] = vol * t;
+            for (int r = 0; r < 3; ++r) dinv[i * 3 + r] = 1.0 / A[4 * r];
+    }
+}
+
+// y = K x and (x, y) into acc[2].  A warp takes one of the three displacement
+// components of a slice's 32 nodes (three warps share the slice's column indices and
+// gathered values in L1): three times the warps of one lane per node, which is what
+// covers the latency of the gathers.  Bound by the FP64 pipe.  acc null: the product
+// alone.
+constexpr int MECH_THREADS = 192;
+__global__ void __launch_bounds__(MECH_THREADS) k_mech_product(int64_t nv, int64_t n_slices,
+                                                               const int64_t* __restrict__ base,
+                                                               const int32_t* __restrict__ col,
+                                                               const double* __restrict__ val,
+                                                               const double* __restrict__ x, double* __restrict__ y,
+                                                               double* __restrict__ acc) {
+    if (acc && blockIdx.x == 0 && threadIdx.x == 0) pcg_roll(acc, 0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = warp % 3;
+    double dot[1] = {0.0};
+    for (int64_t s = (int64_t)blockIdx.x * (MECH_THREADS / 96) + warp / 3; s < n_slices;
+         s += (int64_t)gridDim.x * (MECH_THREADS / 96)) {
+        const int64_t i = s * 32 + lane, row1 = base[s + 1];
+        double a = 0.0;
+#pragma unroll 4
+        for (int64_t row = base[s]; row < row1; ++row) {
+            const int64_t c = 3 * (int64_t)col[row * 32 + lane];
+            const double* v = val + (row * 9 + 3 * r) * 32 + lane;
+            a = fma(v[0], x[c], a);
+            a = fma(v[32], x[c + 1], a);
+            a = fma(v[64], x[c + 2], a);
         }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            double f[3];
-            mech_bt(g[a * 3], g[a * 3 + 1], g[a * 3 + 2], sg, f);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) atomicAdd(y + (int64_t)v[a] * 3 + i, f[i]);
+        if (i < nv) {
+            y[i * 3 + r] = a;
+            dot[0] = fma(x[i * 3 + r], a, dot[0]);
         }
     }
+    if (acc) block_add<1>(dot, acc + 2);
 }
 
 // Consistent nodal forces of a uniform traction t on every tetrahedron face
@@ -482,92 +657,141 @@ void to_sym6(const double k[9], double out[6]) {
     out[5] = k[2];
 }
 
-// Jacobi diagonal of C/dt + K per node and field (host, FP64).
-int build_diag(rve_macro m, double dt_s) {
-    std::vector<double> d((size_t)m->nv * 2, 0.0);
-    double K6[2][6];
-    std::memcpy(K6[0], m->KT, sizeof(K6[0]));
-    std::memcpy(K6[1], m->Dc, sizeof(K6[1]));
-    const double cap[2] = {m->rho_cp / dt_s, 1.0 / dt_s};
-    for (int64_t e = 0; e < m->nt; ++e) {
-        const double vol = m->vol_h[e];
-        const double* g = &m->grad_h[(size_t)e * 12];
-        for (int a = 0; a < 4; ++a) {
-            const int v = m->tets_h[e * 4 + a];
-            for (int f = 0; f < 2; ++f) {
-                const double* k = K6[f];
-                const double gx = g[a * 3], gy = g[a * 3 + 1], gz = g[a * 3 + 2];
-                const double kgg = gx * (k[0] * gx + k[3] * gy + k[5] * gz) + gy * (k[3] * gx + k[1] * gy + k[4] * gz) +
-                                   gz * (k[5] * gx + k[4] * gy + k[2] * gz);
-                d[(size_t)v * 2 + f] += vol * kgg + cap[f] * vol / 10.0;
-            }
-        }
+// Node graph of the mesh in slices of 32 rows, on the device (once per mesh).
+int ensure_graph(rve_macro m) {
+    if (m->have_graph) return RVE_OK;
+    NodeGraph g;
+    if (!build_node_graph(m->tets_h.data(), m->nt, 4, nullptr, m->nv, g)) {
+        set_error("macro mesh too large for 32-bit matrix indices");
+        return RVE_ERR_INVALID_ARGUMENT;
     }
-    RVE_TRY(upload(m->diag, d.data(), d.size(), m->ctx->stream));
-    m->diag_dt = dt_s;
+    const int64_t ns = (m->nv + 31) / 32;
+    std::vector<int64_t> base(ns + 1, 0);
+    std::vector<int32_t> len(m->nv);
+    for (int64_t i = 0; i < m->nv; ++i) len[i] = g.ptr[i + 1] - g.ptr[i];
+    for (int64_t s = 0; s < ns; ++s) {
+        int32_t most = 0;
+        for (int64_t i = s * 32; i < std::min(m->nv, s * 32 + 32); ++i) most = std::max(most, len[i]);
+        base[s + 1] = base[s] + most;
+    }
+    std::vector<int32_t> col((size_t)base[ns] * 32);
+    for (int64_t s = 0; s < ns; ++s)
+        for (int lane = 0; lane < 32; ++lane) {
+            const int64_t i = std::min(s * 32 + lane, m->nv - 1);
+            for (int64_t k = 0; k < base[s + 1] - base[s]; ++k)
+                col[(base[s] + k) * 32 + lane] = k < len[i] ? g.col[g.ptr[i] + k] : (int32_t)i;
+        }
+    cudaStream_t s = m->ctx->stream;
+    RVE_TRY(upload(m->g_base, base.data(), base.size(), s));
+    RVE_TRY(upload(m->g_col, col.data(), col.size(), s));
+    RVE_TRY(upload(m->g_len, len.data(), len.size(), s));
+    RVE_TRY(upload(m->g_eptr, g.eptr.data(), g.eptr.size(), s));
+    RVE_TRY(upload(m->g_inc, g.inc.data(), g.inc.size(), s));
+    RVE_CUDA(cudaStreamSynchronize(s));
+    m->n_slices = ns;
+    m->n_ell = base[ns];
+    m->have_graph = true;
     return RVE_OK;
 }
 
-// Jacobi PCG on the macro mesh over nf (1 or 2) interleaved fields of n rows in
-// all.  On entry x holds the start (held rows at their values) and b the
-// right-hand side; apply(in, out) adds the operator times in to out.  A field
-// has converged when (r, M^-1 r) <= rtol^2 max((b, M^-1 b), (r0, M^-1 r0)) over
-// the free rows.  Returns the iterations and final relative residuals per field.
-template <class Apply>
-int macro_pcg(rve_macro mm, int64_t n, int nf, int mdiv, const uint8_t* mask, const double* diag, double* x,
-              const double* b, Apply apply, double rtol, int max_iter, int its[2], double rel[2], bool& conv) {
+// The transport matrix and inverse diagonal for one time step length.
+int ensure_transport_matrix(rve_macro m, double dt_s) {
+    RVE_TRY(ensure_graph(m));
+    cudaStream_t s = m->ctx->stream;
+    const int64_t *base = m->g_base.as<int64_t>();
+    const int32_t *col = m->g_col.as<int32_t>(), *len = m->g_len.as<int32_t>();
+    if (!m->have_stiff) {
+        RVE_TRY(m->t_mass.ensure((size_t)m->n_ell * 32 * 8));
+        RVE_TRY(m->t_stiff.ensure((size_t)m->n_ell * 32 * 16));
+        RVE_TRY(m->t_mat.ensure((size_t)m->n_ell * 32 * 16));
+        RVE_TRY(m->t_dinv.ensure((size_t)m->nv * 16));
+        RVE_CUDA(cudaMemsetAsync(m->t_dinv.p, 0, (size_t)m->nv * 16, s));   // nodes of no element: z = 0
+        TransportTensors prm;
+        std::memcpy(prm.KT, m->KT, sizeof(prm.KT));
+        std::memcpy(prm.Dc, m->Dc, sizeof(prm.Dc));
+        k_transport_entries<<<(unsigned)m->n_slices, 256, 0, s>>>(m->nv, base, col, len, m->g_eptr.as<int32_t>(),
+                                                                  m->g_inc.as<int32_t>(), m->tets.as<int32_t>(),
+                                                                  m->geo.as<double>(), prm, m->t_mass.as<double>(),
+                                                                  m->t_stiff.as<double2>());
+        RVE_CUDA(cudaGetLastError());
+        m->have_stiff = true;
+        m->mat_dt = -1;
+    }
+    if (m->mat_dt != dt_s) {
+        k_transport_matrix<<<(unsigned)((m->n_slices + 7) / 8), 256, 0, s>>>(
+            m->nv, m->n_slices, base, col, len, m->t_mass.as<double>(), m->t_stiff.as<double2>(), m->rho_cp / dt_s,
+            1.0 / dt_s, m->t_mat.as<double2>(), m->t_dinv.as<double2>());
+        RVE_CUDA(cudaGetLastError());
+        m->mat_dt = dt_s;
+    }
+    return RVE_OK;
+}
+
+// Jacobi PCG on the macro mesh over NF interleaved fields of n entries in all.  On
+// entry x holds the start (held rows at their values) and b the right-hand side;
+// product(stream, in, out, acc) forms out = A in and adds (in, out) to acc[2..].  A
+// field has converged when (r, M^-1 r) <= rtol^2 max((b, M^-1 b), (r0, M^-1 r0)) over
+// the free rows.  The iterations run as one CUDA graph with a conditional WHILE node
+// that ends on the device.  Returns the iterations and final relative residuals per
+// field.
+template <int NF, class Product>
+int macro_pcg(rve_macro mm, int64_t n, int mdiv, const uint8_t* mask, const double* dinv, double* x, const double* b,
+              const void* mat, Product product, double rtol, int max_iter, int its[2], double rel[2], bool& conv) {
     cudaStream_t s = mm->ctx->stream;
     double* r = mm->r.as<double>();
-    double* z = mm->z.as<double>();
     double* p = mm->p.as<double>();
     double* q = mm->q.as<double>();
     double* acc = mm->acc.as<double>();
     const unsigned gv = grid_for(n);
-    // r = b - A x, z = M^-1 r, (r, z)
-    RVE_CUDA(cudaMemsetAsync(q, 0, n * 8, s));
-    RVE_CUDA(cudaMemsetAsync(acc, 0, 16 * 8, s));
-    apply(x, q);
-    k_macro_residual<<<gv, 256, 0, s>>>(n, nf, mdiv, b, q, mask, diag, r, z, acc);
-    const double tol2 = rtol * rtol;
-    double h[16];
-    RVE_CUDA(cudaMemcpyAsync(h, acc, 16 * 8, cudaMemcpyDeviceToHost, s));
+    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+    product(s, x, q, nullptr);
+    k_macro_residual<NF><<<gv, 256, 0, s>>>(n, mdiv, b, q, mask, dinv, r, p, acc);
+    k_macro_start<<<1, 2, 0, s>>>(acc, NF, rtol * rtol, max_iter);
+    RVE_CUDA(cudaGetLastError());
+    const void* key[9] = {r, p, q, acc, x, mask, dinv, mat, mm->g_col.p};
+    const unsigned char* kb = reinterpret_cast<const unsigned char*>(key);
+    auto& loop = mm->loop[NF == 2 ? 0 : 1];
+    if (!loop.exec || loop.key.size() != sizeof(key) || std::memcmp(loop.key.data(), kb, sizeof(key)) != 0) {
+        if (loop.exec) {
+            cudaGraphExecDestroy(loop.exec);
+            loop.exec = nullptr;
+        }
+        cudaGraph_t graph = nullptr;
+        RVE_CUDA(cudaGraphCreate(&graph, 0));
+        struct GraphGuard {
+            cudaGraph_t g;
+            ~GraphGuard() { cudaGraphDestroy(g); }
+        } guard{graph};
+        cudaGraphConditionalHandle handle;
+        RVE_CUDA(cudaGraphConditionalHandleCreate(&handle, graph, 1, cudaGraphCondAssignDefault));
+        cudaGraphNodeParams np = {};
+        np.type = cudaGraphNodeTypeConditional;
+        np.conditional.handle = handle;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaGraphNode_t node;
+        RVE_CUDA(cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np));
+        cudaGraph_t body = np.conditional.phGraph_out[0];
+        cudaStream_t cap = mm->ctx->capture;
+        RVE_CUDA(cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+        product(cap, p, q, acc);
+        k_macro_update<NF><<<gv, 256, 0, cap>>>(n, mdiv, mask, dinv, x, r, p, q, acc);
+        k_macro_pupdate<NF><<<gv, 256, 0, cap>>>(n, dinv, r, p, acc, handle);
+        RVE_CUDA(cudaStreamEndCapture(cap, &body));
+        RVE_CUDA(cudaGraphInstantiate(&loop.exec, graph, 0));
+        loop.key.assign(kb, kb + sizeof(key));
+    }
+    RVE_CUDA(cudaGraphLaunch(loop.exec, s));
+    double h[PCG_SCALARS];
+    RVE_CUDA(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
     RVE_CUDA(cudaStreamSynchronize(s));
-    // convergence is relative to the larger of the right-hand side and the
-    // initial residual (which carries the held values): a field already at
-    // rest (rounding-level residual) needs no iteration
+    conv = true;
     for (int f = 0; f < 2; ++f) {
-        h[4 + f] = h[f];                                  // current (r, z)
-        h[6 + f] = std::max(h[14 + f], h[f]);             // reference
-        h[12 + f] = h[f] > tol2 * h[6 + f] ? 1.0 : 0.0;   // active
+        const bool used = f < NF;
+        its[f] = used ? (int)h[12 + f] : 0;
+        rel[f] = used && h[6 + f] > 0 ? std::sqrt(std::max(h[f], 0.0) / h[6 + f]) : 0.0;
+        if (used && h[10 + f] != 0.0) conv = false;
     }
-    h[0] = h[1] = h[2] = h[3] = 0.0;
-    RVE_CUDA(cudaMemcpyAsync(acc, h, 16 * 8, cudaMemcpyHostToDevice, s));
-    k_macro_pupdate<<<gv, 256, 0, s>>>(n, nf, z, p, q, acc, 1);
-    int it = 0;
-    its[0] = its[1] = 0;
-    bool active[2] = {h[12] != 0.0, h[13] != 0.0};
-    while ((active[0] || active[1]) && it < max_iter) {
-        const int chunk = std::min(8, max_iter - it);
-        for (int k = 0; k < chunk; ++k) {
-            apply(p, q);
-            k_macro_dot<<<gv, 256, 0, s>>>(n, nf, p, q, acc);
-            k_macro_alpha<<<1, 1, 0, s>>>(acc);
-            k_macro_update<<<gv, 256, 0, s>>>(n, nf, mdiv, mask, diag, x, r, z, p, q, acc);
-            k_macro_beta<<<1, 1, 0, s>>>(acc, tol2);
-            k_macro_pupdate<<<gv, 256, 0, s>>>(n, nf, z, p, q, acc, 0);
-        }
-        RVE_CUDA(cudaGetLastError());
-        it += chunk;
-        RVE_CUDA(cudaMemcpyAsync(h, acc, 16 * 8, cudaMemcpyDeviceToHost, s));
-        RVE_CUDA(cudaStreamSynchronize(s));
-        for (int f = 0; f < 2; ++f) {
-            if (active[f]) its[f] = it;
-            active[f] = h[12 + f] != 0.0;
-        }
-    }
-    conv = !(active[0] || active[1]);
-    rel[0] = h[6] > 0 ? std::sqrt(std::max(h[4], 0.0) / h[6]) : 0.0;
-    rel[1] = h[7] > 0 ? std::sqrt(std::max(h[5], 0.0) / h[7]) : 0.0;
     return RVE_OK;
 }
 
@@ -589,8 +813,6 @@ int rve_macro_create(rve_ctx c, const double* xyz, int64_t nv, const int32_t* te
     m->nv = nv;
     m->nt = nt;
     m->tets_h.assign(tets, tets + nt * 4);
-    m->vol_h.resize(nt);
-    m->grad_h.resize((size_t)nt * 12);
     std::vector<double> geo((size_t)nt * 13);
     for (int64_t e = 0; e < nt; ++e) {
         const double* X[4];
@@ -629,21 +851,17 @@ int rve_macro_create(rve_ctx c, const double* xyz, int64_t nv, const int32_t* te
         for (int r = 0; r < 3; ++r)
             for (int k = 0; k < 3; ++k) g[r + 1][k] = inv[k][r];
         for (int k = 0; k < 3; ++k) g[0][k] = -(g[1][k] + g[2][k] + g[3][k]);
-        m->vol_h[e] = det / 6.0;
         geo[(size_t)e * 13] = det / 6.0;
         for (int a = 0; a < 4; ++a)
-            for (int k = 0; k < 3; ++k) {
-                geo[(size_t)e * 13 + 1 + a * 3 + k] = g[a][k];
-                m->grad_h[(size_t)e * 12 + a * 3 + k] = g[a][k];
-            }
+            for (int k = 0; k < 3; ++k) geo[(size_t)e * 13 + 1 + a * 3 + k] = g[a][k];
     }
     cudaStream_t s = c->stream;
     int rc = upload(m->tets, tets, (size_t)nt * 4, s);
     if (rc == RVE_OK) rc = upload(m->geo, geo.data(), geo.size(), s);
     const size_t n2 = (size_t)nv * 2;
-    for (DevBuf* bfr : {&m->x, &m->b, &m->r, &m->z, &m->p, &m->q})
+    for (DevBuf* bfr : {&m->x, &m->b, &m->r, &m->p, &m->q})
         if (rc == RVE_OK) rc = bfr->ensure(n2 * 8);
-    if (rc == RVE_OK) rc = m->acc.ensure(16 * 8);
+    if (rc == RVE_OK) rc = m->acc.ensure(PCG_SCALARS * 8);
     if (rc == RVE_OK) rc = m->gp.ensure((size_t)nt * 4 * 4 * 8);
     if (rc == RVE_OK) rc = m->W.ensure((size_t)nt * 4 * 8);
     if (rc == RVE_OK) rc = m->flags.ensure(16);
@@ -680,7 +898,7 @@ int rve_macro_set_transport(rve_ctx c, rve_macro m, const double K_T[9], double 
     to_sym6(D_c, m->Dc);
     m->rho_cp = rho_cp;
     m->have_transport = true;
-    m->diag_dt = -1;
+    m->have_stiff = false;
     return RVE_OK;
 }
 
@@ -704,9 +922,7 @@ int rve_macro_set_held(rve_ctx c, rve_macro m, const uint8_t* node_mask, const d
         set_error("rve_macro_set_held: invalid argument");
         return RVE_ERR_INVALID_ARGUMENT;
     }
-    m->mask_h.assign(node_mask, node_mask + m->nv);
-    for (auto& v : m->mask_h) v = v ? 1 : 0;
-    RVE_TRY(upload(m->mask, m->mask_h.data(), m->mask_h.size(), c->stream));
+    RVE_TRY(upload(m->mask, node_mask, (size_t)m->nv, c->stream));
     RVE_TRY(upload(m->hold, values, (size_t)m->nv * 2, c->stream));
     RVE_CUDA(cudaStreamSynchronize(c->stream));
     m->have_face = true;
@@ -721,8 +937,7 @@ int rve_macro_reset(rve_ctx c, rve_macro m, double T0_C, double c0_wt) {
     }
     cudaStream_t s = c->stream;
     k_macro_fill<<<grid_for(m->nv), 256, 0, s>>>(m->nv, T0_C, c0_wt, m->x.as<double>());
-    std::vector<double> ones((size_t)m->nt * 4, 1.0);
-    RVE_TRY(upload(m->W, ones.data(), ones.size(), s));
+    launch_fill(m->nt * 4, 1.0, m->W.as<double>(), s);
     RVE_CUDA(cudaGetLastError());
     RVE_CUDA(cudaStreamSynchronize(s));
     m->have_state = true;
@@ -735,28 +950,24 @@ int rve_macro_reset(rve_ctx c, rve_macro m, double T0_C, double c0_wt) {
 static int transport_solve(rve_macro mm, double dt_s, double rtol, int max_iter, int its[2], double rel[2],
                            bool& conv) {
     cudaStream_t s = mm->ctx->stream;
-    if (mm->diag_dt != dt_s) RVE_TRY(build_diag(mm, dt_s));
-    const int64_t n = mm->nv * 2;
+    RVE_TRY(ensure_transport_matrix(mm, dt_s));
+    const int64_t n = mm->nv * 2, ns = mm->n_slices;
     double* x = mm->x.as<double>();
     double* b = mm->b.as<double>();
     const uint8_t* mask = mm->mask.as<uint8_t>();
-    const unsigned ge = grid_for(mm->nt);
-    MacroParams prm;
-    std::memcpy(prm.KT, mm->KT, sizeof(prm.KT));
-    std::memcpy(prm.Dc, mm->Dc, sizeof(prm.Dc));
-    prm.capT = mm->rho_cp / dt_s;
-    prm.capC = 1.0 / dt_s;
+    const int64_t* base = mm->g_base.as<int64_t>();
+    const int32_t* col = mm->g_col.as<int32_t>();
+    const double2* mat = mm->t_mat.as<double2>();
+    const unsigned gs = (unsigned)((ns + 7) / 8);
     // b = C/dt x^n; start from x^n with the held values in place
-    MacroParams mass = prm;
-    mass.stiff = 0;
-    prm.stiff = 1;
-    RVE_CUDA(cudaMemsetAsync(b, 0, n * 8, s));
-    k_macro_apply<<<ge, 256, 0, s>>>(mm->nt, mm->tets.as<int32_t>(), mm->geo.as<double>(), x, b, mass);
+    k_transport_rhs<<<gs, 256, 0, s>>>(mm->nv, ns, base, col, mm->t_mass.as<double>(), mm->rho_cp / dt_s, 1.0 / dt_s,
+                                       reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(b));
     k_macro_hold<<<grid_for(mm->nv), 256, 0, s>>>(mm->nv, mask, mm->hold.as<double>(), x);
-    auto apply = [&](const double* in, double* out) {
-        k_macro_apply<<<ge, 256, 0, s>>>(mm->nt, mm->tets.as<int32_t>(), mm->geo.as<double>(), in, out, prm);
+    auto product = [&](cudaStream_t st, const double* in, double* out, double* acc) {
+        k_transport_product<<<gs, 256, 0, st>>>(mm->nv, ns, base, col, mat, reinterpret_cast<const double2*>(in),
+                                                reinterpret_cast<double2*>(out), acc);
     };
-    return macro_pcg(mm, n, 2, 2, mask, mm->diag.as<double>(), x, b, apply, rtol, max_iter, its, rel, conv);
+    return macro_pcg<2>(mm, n, 2, mask, mm->t_dinv.as<double>(), x, b, mat, product, rtol, max_iter, its, rel, conv);
 }
 
 int rve_macro_step(rve_ctx c, rve_macro m, double dt_h, const rve_degradation* deg, double rtol, int max_iter,
@@ -1110,27 +1321,36 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
         RVE_TRY(upload(m->cgp, C_gp, (size_t)m->nt * 4 * 36, s));
         Cg = m->cgp.as<double>();
     }
-    for (DevBuf* bfr : {&m->b, &m->r, &m->z, &m->p, &m->q, &m->mdiag}) RVE_TRY(bfr->ensure((size_t)n * 8));
+    RVE_TRY(ensure_graph(m));
+    for (DevBuf* bfr : {&m->b, &m->r, &m->p, &m->q, &m->mdinv}) RVE_TRY(bfr->ensure((size_t)n * 8));
     RVE_TRY(m->cm.ensure((size_t)m->nt * 36 * 8));
+    RVE_TRY(m->mmat.ensure((size_t)m->n_ell * 9 * 32 * 8));
     RVE_TRY(m->msig.ensure((size_t)m->nt * 4 * 6 * 8));
-    RVE_CUDA(cudaMemsetAsync(m->mdiag.p, 0, n * 8, s));
-    const unsigned ge = grid_for(m->nt);
     const int32_t* tets = m->tets.as<int32_t>();
     const double* geo = m->geo.as<double>();
-    k_mech_material<<<ge, 256, 0, s>>>(m->nt, tets, geo, Cg, m->cm.as<double>(), m->mdiag.as<double>());
+    const int64_t* base = m->g_base.as<int64_t>();
+    const int32_t* col = m->g_col.as<int32_t>();
+    k_mech_material<<<(unsigned)std::min<int64_t>((m->nt * 36 + 255) / 256, (int64_t)sm_count() * 16), 256, 0, s>>>(
+        m->nt, Cg, m->cm.as<double>());
+    RVE_CUDA(cudaMemsetAsync(m->mdinv.p, 0, (size_t)n * 8, s));   // nodes of no element: z = 0
+    k_mech_entries<<<(unsigned)m->n_slices, 256, 0, s>>>(m->nv, base, col, m->g_len.as<int32_t>(),
+                                                         m->g_eptr.as<int32_t>(), m->g_inc.as<int32_t>(), tets, geo,
+                                                         m->cm.as<double>(), m->mmat.as<double>(),
+                                                         m->mdinv.as<double>());
     double* b = m->b.as<double>();
     double* u = m->mu.as<double>();
     RVE_CUDA(cudaMemcpyAsync(b, m->mload.p, n * 8, cudaMemcpyDeviceToDevice, s));
     k_mech_hold<<<grid_for(n), 256, 0, s>>>(n, m->mfix.as<uint8_t>(), m->mval.as<double>(), u);
-    const double* cm = m->cm.as<double>();
-    auto apply = [&](const double* in, double* out) {
-        k_mech_apply<<<ge, 256, 0, s>>>(m->nt, tets, geo, cm, in, out);
+    const double* mat = m->mmat.as<double>();
+    const unsigned gm = (unsigned)std::min<int64_t>((m->n_slices + 1) / 2, (int64_t)sm_count() * 10);
+    auto product = [&](cudaStream_t st, const double* in, double* out, double* acc) {
+        k_mech_product<<<gm, MECH_THREADS, 0, st>>>(m->nv, m->n_slices, base, col, mat, in, out, acc);
     };
     int its[2] = {0, 0};
     double rel[2] = {0, 0};
     bool conv = false;
-    RVE_TRY(macro_pcg(m, n, 1, 1, m->mfix.as<uint8_t>(), m->mdiag.as<double>(), u, b, apply, rtol, max_iter, its,
-                      rel, conv));
+    RVE_TRY(macro_pcg<1>(m, n, 1, m->mfix.as<uint8_t>(), m->mdinv.as<double>(), u, b, mat, product, rtol, max_iter,
+                         its, rel, conv));
     k_mech_stress<<<grid_for(m->nt * 4), 256, 0, s>>>(m->nt, tets, geo, Cg, u, m->msig.as<double>());
     RVE_CUDA(cudaGetLastError());
     RVE_CUDA(cudaStreamSynchronize(s));
