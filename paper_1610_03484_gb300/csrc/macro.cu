@@ -39,13 +39,14 @@ struct rve_macro_s {
     rve::DevBuf g_base, g_col, g_len, g_eptr, g_inc;
     bool have_graph = false;
     rve::DevBuf t_mass, t_stiff, t_mat, t_dinv;
+    rve::DevBuf c_r, c_z, c_z2, c_d, c_dinv;   // FP32 vectors of the elastic preconditioner
     bool have_stiff = false;
     double mat_dt = -1;                     // dt [s] that t_mat and t_dinv were formed for
     // macro mechanics: held DOFs and their values, traction load, inverse Jacobi
     // diagonal, displacement, per-tet mean stiffness [nt][36], the assembled
     // stiffness, Gauss-point stiffness staged from the host [nt*4][36] and stresses
     // [nt*4][6]
-    rve::DevBuf mfix, mval, mload, mdinv, mu, cm, mmat, cgp, msig;
+    rve::DevBuf mfix, mval, mload, mdinv, mu, cm, mmat, mmat32, cgp, msig;
     bool have_mech_bc = false, have_mech_load = false, have_mech_u = false, have_mech_sig = false;
     // instantiated PCG loops (0 transport, 1 mechanics), reused while the captured
     // launch parameters stay the same
@@ -177,17 +178,20 @@ __global__ void __launch_bounds__(256) k_transport_rhs(int64_t nv, int64_t n_sli
 //   [0] (r, z) of this iteration, [2] (p, q), [4] (r, z) of the previous one,
 //   [6] the reference max((b, M^-1 b), (r0, M^-1 r0)), [8] 1 while the field iterates,
 //   [10] the same for the next iteration, [12] iterations, [14] (b, M^-1 b);
-//   [16] iterations of the loop, [17] their limit, [18] the squared tolerance.
-// An iteration is three kernels: the product (which also moves (r, z) and the
-// active flags on), the x/r update and the p update (which also runs the loop
+//   [16] iterations of the loop, [17] their limit, [18] the squared tolerance,
+//   [20] (r, D^-1 r) of this iteration where M is not the Jacobi diagonal D (the stopping
+//   test's norm, also of [6] and [14]).
+// An iteration is the product (which also moves (r, z) and the active flags on), the x/r
+// update, the preconditioner's steps if any and the p update (which also runs the loop
 // control).  Every scalar is written by one thread in a kernel whose other blocks do
 // not read it.
-constexpr int PCG_SCALARS = 20;
+constexpr int PCG_SCALARS = 22;
 
 // moves the scalars on to the next iteration; one thread per field of one block
 __device__ __forceinline__ void pcg_roll(double* acc, int f) {
     acc[4 + f] = acc[f];
     acc[f] = 0.0;
+    acc[20 + f] = 0.0;
     acc[8 + f] = acc[10 + f];
 }
 
@@ -243,97 +247,75 @@ __global__ void __launch_bounds__(256) k_transport_product(int64_t nv, int64_t n
     if (acc) block_add<2>(dot, acc + 2);
 }
 
-// Vector kernels: nf interleaved fields of n entries in all, the field of entry i is
-// i % nf; the held mask is indexed by i / mdiv (2 for the per-node mask of the
-// transport pair, 1 for the per-DOF mask of the mechanics).
-
-// r = b - y on free rows (0 on held rows), p = M^-1 r, acc[0] += (r, p) and
-// acc[14] += (b, M^-1 b) over the free rows (the reference norm)
-template <int NF>
-__global__ void __launch_bounds__(256) k_macro_residual(int64_t n, int mdiv, const double* __restrict__ b,
-                                                        const double* __restrict__ y,
-                                                        const uint8_t* __restrict__ mask,
-                                                        const double* __restrict__ dinv, double* __restrict__ r,
-                                                        double* __restrict__ p, double* __restrict__ acc) {
-    double a[NF] = {}, bb[NF] = {};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const bool held = mask[i / mdiv] != 0;
-        const double bi = b[i], di = dinv[i];
-        const double ri = held ? 0.0 : bi - y[i];
-        const double zi = ri * di;
+// The transport pair's vector passes, Jacobi-preconditioned, a thread per node (both
+// fields, 16-byte loads).
+//
+// r = b - y on free nodes (0 on held ones), p = D^-1 r, acc[0] += (r, p) and
+// acc[14] += (b, D^-1 b) over the free nodes (the reference norm)
+__global__ void __launch_bounds__(256) k_transport_residual(int64_t nv, const double2* __restrict__ b,
+                                                            const double2* __restrict__ y,
+                                                            const uint8_t* __restrict__ mask,
+                                                            const double2* __restrict__ dinv, double2* __restrict__ r,
+                                                            double2* __restrict__ p, double* __restrict__ acc) {
+    double a[2] = {0.0, 0.0}, bb[2] = {0.0, 0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool held = mask[i] != 0;
+        const double2 bi = b[i], yi = y[i], di = dinv[i];
+        const double2 ri = held ? make_double2(0.0, 0.0) : make_double2(bi.x - yi.x, bi.y - yi.y);
+        const double2 zi = make_double2(ri.x * di.x, ri.y * di.y);
         r[i] = ri;
         p[i] = zi;
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-            if (NF == 1 || (int)(i & 1) == f) {
-                a[f] += ri * zi;
-                if (!held) bb[f] += bi * (bi * di);
-            }
+        a[0] = fma(ri.x, zi.x, a[0]);
+        a[1] = fma(ri.y, zi.y, a[1]);
+        if (!held) {
+            bb[0] = fma(bi.x, bi.x * di.x, bb[0]);
+            bb[1] = fma(bi.y, bi.y * di.y, bb[1]);
+        }
     }
-    block_add<NF>(a, acc);
-    block_add<NF>(bb, acc + 14);
+    block_add<2>(a, acc);
+    block_add<2>(bb, acc + 14);
 }
 
-// Convergence is relative to the larger of the right-hand side and the initial
-// residual (which carries the held values): a field already at rest
-// (rounding-level residual) takes no iteration.  One thread per field.
-__global__ void k_macro_start(double* acc, int nf, double tol2, int max_iter) {
-    const int f = threadIdx.x;
-    const double rz = f < nf ? acc[f] : 0.0, bb = f < nf ? acc[14 + f] : 0.0;
-    acc[6 + f] = fmax(bb, rz);
-    acc[10 + f] = rz > tol2 * acc[6 + f] ? 1.0 : 0.0;
-    acc[2 + f] = 0.0;
-    acc[12 + f] = 0.0;
-    if (f == 0) {
-        acc[16] = 0.0;
-        acc[17] = (double)max_iter;
-        acc[18] = tol2;
-    }
-}
-
-// x += alpha p, r -= alpha q (held rows stay 0), acc[0] += (r, M^-1 r)
-template <int NF>
-__global__ void __launch_bounds__(256) k_macro_update(int64_t n, int mdiv, const uint8_t* __restrict__ mask,
-                                                     const double* __restrict__ dinv, double* __restrict__ x,
-                                                     double* __restrict__ r, const double* __restrict__ p,
-                                                     const double* __restrict__ q, double* __restrict__ acc) {
-    __shared__ double alpha[NF];
-    if (threadIdx.x < NF) {
+// x += alpha p, r -= alpha q (held nodes stay 0), acc[0] += (r, D^-1 r)
+__global__ void __launch_bounds__(256) k_transport_update(int64_t nv, const uint8_t* __restrict__ mask,
+                                                          const double2* __restrict__ dinv, double2* __restrict__ x,
+                                                          double2* __restrict__ r, const double2* __restrict__ p,
+                                                          const double2* __restrict__ q, double* __restrict__ acc) {
+    __shared__ double alpha[2];
+    if (threadIdx.x < 2) {
         const double pq = acc[2 + threadIdx.x];
         const bool ok = acc[8 + threadIdx.x] != 0.0 && pq > 0.0;
         alpha[threadIdx.x] = ok ? acc[4 + threadIdx.x] / pq : 0.0;
     }
     __syncthreads();
-    double a[NF] = {};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = NF == 2 ? (int)(i & 1) : 0;
-        const double al = alpha[f];
-        double ri = r[i];
-        if (al != 0.0) {
-            x[i] = fma(al, p[i], x[i]);
-            ri = mask[i / mdiv] ? 0.0 : fma(-al, q[i], ri);
-            r[i] = ri;
-        }
-        const double v = ri * (ri * dinv[i]);
-#pragma unroll
-        for (int g = 0; g < NF; ++g)
-            if (NF == 1 || f == g) a[g] += v;
+    const double al = alpha[0], be = alpha[1];
+    double a[2] = {0.0, 0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
+        const double2 pi = p[i], qi = q[i], di = dinv[i];
+        double2 xi = x[i], ri = r[i];
+        const bool held = mask[i] != 0;
+        xi.x = fma(al, pi.x, xi.x);
+        xi.y = fma(be, pi.y, xi.y);
+        ri.x = held ? 0.0 : fma(-al, qi.x, ri.x);
+        ri.y = held ? 0.0 : fma(-be, qi.y, ri.y);
+        x[i] = xi;
+        r[i] = ri;
+        a[0] = fma(ri.x, ri.x * di.x, a[0]);
+        a[1] = fma(ri.y, ri.y * di.y, a[1]);
     }
-    block_add<NF>(a, acc);
+    block_add<2>(a, acc);
 }
 
-// p = M^-1 r + beta p for fields still iterating; loop control
+// Per-field tail of an iteration, NF fields: whether the field goes on (the norm at
+// acc[norm + f]), beta, and by one thread of the grid the flags and the loop control.
 template <int NF>
-__global__ void __launch_bounds__(256) k_macro_pupdate(int64_t n, const double* __restrict__ dinv,
-                                                      const double* __restrict__ r, double* __restrict__ p,
-                                                      double* __restrict__ acc, cudaGraphConditionalHandle h) {
-    __shared__ double beta[NF];
-    __shared__ int on[NF];
+__device__ __forceinline__ void pcg_tail(double* acc, int norm, cudaGraphConditionalHandle h, double (&beta)[NF],
+                                         int (&on)[NF]) {
     if (threadIdx.x < NF) {
         const int f = threadIdx.x;
         const double rz = acc[f], old = acc[4 + f];
         // converged (or not finite): the field stops
-        on[f] = acc[8 + f] != 0.0 && rz > acc[18] * acc[6 + f];
+        on[f] = acc[8 + f] != 0.0 && acc[norm + f] > acc[18] * acc[6 + f] && isfinite(rz);
         beta[f] = old > 0.0 ? rz / old : 0.0;
     }
     __syncthreads();
@@ -349,10 +331,197 @@ __global__ void __launch_bounds__(256) k_macro_pupdate(int64_t n, const double* 
         acc[16] = it;
         cudaGraphSetConditional(h, any && it < acc[17] ? 1u : 0u);
     }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = NF == 2 ? (int)(i & 1) : 0;
-        if (on[f]) p[i] = fma(beta[f], p[i], r[i] * dinv[i]);
+}
+
+// p = D^-1 r + beta p for fields still iterating; loop control
+__global__ void __launch_bounds__(256) k_transport_pupdate(int64_t nv, const double2* __restrict__ dinv,
+                                                           const double2* __restrict__ r, double2* __restrict__ p,
+                                                           double* __restrict__ acc, cudaGraphConditionalHandle h) {
+    __shared__ double beta[2];
+    __shared__ int on[2];
+    pcg_tail<2>(acc, 0, h, beta, on);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
+        const double2 di = dinv[i], ri = r[i];
+        double2 pi = p[i];
+        if (on[0]) pi.x = fma(beta[0], pi.x, ri.x * di.x);
+        if (on[1]) pi.y = fma(beta[1], pi.y, ri.y * di.y);
+        p[i] = pi;
     }
+}
+
+// Convergence is relative to the larger of the right-hand side and the initial residual
+// (which carries the held values): a field already at rest (rounding-level residual)
+// takes no iteration.  One thread per field; `norm` as in pcg_tail.
+__global__ void k_macro_start(double* acc, int nf, int norm, double tol2, int max_iter) {
+    const int f = threadIdx.x;
+    const double rj = f < nf ? acc[norm + f] : 0.0, bb = f < nf ? acc[14 + f] : 0.0;
+    acc[6 + f] = fmax(bb, rj);
+    acc[10 + f] = rj > tol2 * acc[6 + f] ? 1.0 : 0.0;
+    acc[2 + f] = 0.0;
+    acc[12 + f] = 0.0;
+    if (f == 0) {
+        acc[16] = 0.0;
+        acc[17] = (double)max_iter;
+        acc[18] = tol2;
+    }
+}
+
+// The mechanics' vector passes around the Chebyshev preconditioner (below).
+//
+// r = b - y on free rows (0 on held rows), acc[20] += (r, D^-1 r) and acc[14] += (b, D^-1 b)
+// over the free rows; the preconditioner's start r32 = r, z = w D^-1 r
+__global__ void __launch_bounds__(256) k_mech_residual(int64_t n, const double* __restrict__ b,
+                                                       const double* __restrict__ y, const uint8_t* __restrict__ mask,
+                                                       const double* __restrict__ dinv, double* __restrict__ r,
+                                                       float* __restrict__ r32, float* __restrict__ z,
+                                                       float* __restrict__ dinv32, float w, double* __restrict__ acc) {
+    double a[1] = {0.0}, bb[1] = {0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool held = mask[i] != 0;
+        const double bi = b[i], di = dinv[i];
+        const double ri = held ? 0.0 : bi - y[i];
+        const float df = held ? 0.f : (float)di;   // the polynomial leaves held rows alone
+        r[i] = ri;
+        r32[i] = (float)ri;
+        dinv32[i] = df;
+        z[i] = w * (df * (float)ri);
+        a[0] = fma(ri, ri * di, a[0]);
+        if (!held) bb[0] = fma(bi, bi * di, bb[0]);
+    }
+    block_add<1>(a, acc + 20);
+    block_add<1>(bb, acc + 14);
+}
+
+// p = z
+__global__ void __launch_bounds__(256) k_mech_first(int64_t n, const float* __restrict__ z, double* __restrict__ p) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        p[i] = z[i];
+}
+
+// x += alpha p, r -= alpha q (held rows stay 0), acc[20] += (r, D^-1 r); the
+// preconditioner's start
+__global__ void __launch_bounds__(256) k_mech_update(int64_t n, const uint8_t* __restrict__ mask,
+                                                     const double* __restrict__ dinv, double* __restrict__ x,
+                                                     double* __restrict__ r, const double* __restrict__ p,
+                                                     const double* __restrict__ q, float* __restrict__ r32,
+                                                     float* __restrict__ z, const float* __restrict__ dinv32, float w,
+                                                     double* __restrict__ acc) {
+    __shared__ double alpha;
+    if (threadIdx.x == 0) {
+        const double pq = acc[2];
+        alpha = acc[8] != 0.0 && pq > 0.0 ? acc[4] / pq : 0.0;
+    }
+    __syncthreads();
+    const double al = alpha;
+    double a[1] = {0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        x[i] = fma(al, p[i], x[i]);
+        const double ri = mask[i] ? 0.0 : fma(-al, q[i], r[i]);
+        const float rf = (float)ri;
+        r[i] = ri;
+        r32[i] = rf;
+        z[i] = w * (dinv32[i] * rf);
+        a[0] = fma(ri, ri * dinv[i], a[0]);
+    }
+    block_add<1>(a, acc + 20);
+}
+
+// p = z + beta p; loop control
+__global__ void __launch_bounds__(256) k_mech_pupdate(int64_t n, const float* __restrict__ z, double* __restrict__ p,
+                                                      double* __restrict__ acc, cudaGraphConditionalHandle h) {
+    __shared__ double beta[1];
+    __shared__ int on[1];
+    pcg_tail<1>(acc, 20, h, beta, on);
+    if (!on[0]) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        p[i] = fma(beta[0], p[i], (double)z[i]);
+}
+
+// The elastic solve's preconditioner: a Chebyshev polynomial in D^-1 K evaluated in FP32
+// with an FP32 copy of the matrix.  An FP32 product is bound by reading that copy, an
+// FP64 one by the FP64 pipe, so the polynomial's products cost less than the FP64
+// iterations they replace.  (Not for the transport pair: the equivalent time of a Gauss
+// point ahead of the moisture front is a ratio of quantities at the solver's tolerance,
+// which another preconditioner leaves elsewhere.)  One kernel per step: d = c1 d_in +
+// c2 D^-1 (r - K z), z_new = z + d; the last one adds (r64, z_new) into acc instead of
+// storing d.  A warp takes one displacement component of 32 nodes, as the FP64 product.
+struct MechCheb {
+    const float* z;
+    float* z_new;
+    const float* d_in;
+    float* d_out;
+    const float* r;
+    const float* dinv;
+    const double* r64;
+    float c1, c2;
+    double* acc;   // null: not the last step
+};
+
+__global__ void __launch_bounds__(192) k_mech_cheb(int64_t nv, int64_t n_slices, const int64_t* __restrict__ base,
+                                                   const int32_t* __restrict__ col, const float* __restrict__ val,
+                                                   MechCheb ch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = warp % 3;
+    const int64_t s = (int64_t)blockIdx.x * 2 + warp / 3, i = s * 32 + lane;
+    double dot[1] = {0.0};
+    if (s < n_slices) {
+        const int64_t row1 = base[s + 1];
+        float a = 0.f;
+#pragma unroll 4
+        for (int64_t row = base[s]; row < row1; ++row) {
+            const int64_t c = 3 * (int64_t)__ldg(col + row * 32 + lane);
+            const float* v = val + (row * 9 + 3 * r) * 32 + lane;
+            a = fmaf(__ldg(v), __ldg(ch.z + c), a);
+            a = fmaf(__ldg(v + 32), __ldg(ch.z + c + 1), a);
+            a = fmaf(__ldg(v + 64), __ldg(ch.z + c + 2), a);
+        }
+        if (i < nv) {
+            const int64_t k = i * 3 + r;
+            const float d = fmaf(ch.c1, ch.d_in[k], ch.c2 * (ch.dinv[k] * (ch.r[k] - a)));
+            const float zn = ch.z[k] + d;
+            ch.z_new[k] = zn;
+            if (ch.acc)
+                dot[0] = ch.r64[k] * (double)zn;
+            else
+                ch.d_out[k] = d;
+        }
+    }
+    if (ch.acc) block_add<1>(dot, ch.acc);
+}
+
+// Power iteration for the largest eigenvalue of D^-1 K over all rows (held rows can only
+// lower it): the step kernel with d_in = r = 0 and c2 = 1 gives d = -D^-1 K x, then
+// x = -d / 2; k_power_sums adds (x, K x) and (x, D x).
+__global__ void __launch_bounds__(256) k_power_start(int64_t n, const double* __restrict__ dinv, float* __restrict__ x,
+                                                     float* __restrict__ zero, float* __restrict__ dinv32) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t h = (uint32_t)i * 2654435761u + 12345u;
+        h ^= h >> 15;
+        h *= 2246822519u;
+        h ^= h >> 13;
+        x[i] = (float)(h & 0xffffu) * (1.f / 32768.f) - 1.f;
+        zero[i] = 0.f;
+        dinv32[i] = (float)dinv[i];
+    }
+}
+__global__ void __launch_bounds__(256) k_power_next(int64_t n, const float* __restrict__ d, float* __restrict__ x) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        x[i] = -0.5f * d[i];
+}
+__global__ void __launch_bounds__(256) k_power_sums(int64_t n, const float* __restrict__ x, const float* __restrict__ d,
+                                                    const float* __restrict__ dinv, double* __restrict__ out) {
+    double a[2] = {0.0, 0.0};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        if (dinv[i] > 0.f) {
+            const double w = 1.0 / (double)dinv[i];
+            a[0] += (double)x[i] * (double)(-d[i]) * w;
+            a[1] += (double)x[i] * (double)x[i] * w;
+        }
+    block_add<2>(a, out);
+}
+
+__global__ void k_narrow(int64_t n, const double* __restrict__ a, float* __restrict__ b) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        b[i] = (float)a[i];
 }
 
 // held rows take their prescribed values (hold[node * 2 + field])
@@ -727,31 +896,17 @@ int ensure_transport_matrix(rve_macro m, double dt_s) {
     return RVE_OK;
 }
 
-// Jacobi PCG on the macro mesh over NF interleaved fields of n entries in all.  On
-// entry x holds the start (held rows at their values) and b the right-hand side;
-// product(stream, in, out, acc) forms out = A in and adds (in, out) to acc[2..].  A
-// field has converged when (r, M^-1 r) <= rtol^2 max((b, M^-1 b), (r0, M^-1 r0)) over
-// the free rows.  The iterations run as one CUDA graph with a conditional WHILE node
-// that ends on the device.  Returns the iterations and final relative residuals per
-// field.
-template <int NF, class Product>
-int macro_pcg(rve_macro mm, int64_t n, int mdiv, const uint8_t* mask, const double* dinv, double* x, const double* b,
-              const void* mat, Product product, double rtol, int max_iter, int its[2], double rel[2], bool& conv) {
+// The PCG iterations of one problem (slot 0 transport, 1 mechanics) as a CUDA graph with
+// a conditional WHILE node that ends on the device: body(stream, handle) launches one
+// iteration.  The instantiated graph is kept while `key`, every captured pointer and
+// number, stays the same.  Then the iterations and final relative residuals per field.
+template <class Body>
+int macro_loop(rve_macro mm, int slot, const void* key, size_t key_bytes, int nf, int norm, Body body, int its[2],
+               double rel[2], bool& conv) {
     cudaStream_t s = mm->ctx->stream;
-    double* r = mm->r.as<double>();
-    double* p = mm->p.as<double>();
-    double* q = mm->q.as<double>();
-    double* acc = mm->acc.as<double>();
-    const unsigned gv = grid_for(n);
-    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
-    product(s, x, q, nullptr);
-    k_macro_residual<NF><<<gv, 256, 0, s>>>(n, mdiv, b, q, mask, dinv, r, p, acc);
-    k_macro_start<<<1, 2, 0, s>>>(acc, NF, rtol * rtol, max_iter);
-    RVE_CUDA(cudaGetLastError());
-    const void* key[9] = {r, p, q, acc, x, mask, dinv, mat, mm->g_col.p};
-    const unsigned char* kb = reinterpret_cast<const unsigned char*>(key);
-    auto& loop = mm->loop[NF == 2 ? 0 : 1];
-    if (!loop.exec || loop.key.size() != sizeof(key) || std::memcmp(loop.key.data(), kb, sizeof(key)) != 0) {
+    const unsigned char* kb = static_cast<const unsigned char*>(key);
+    auto& loop = mm->loop[slot];
+    if (!loop.exec || loop.key.size() != key_bytes || std::memcmp(loop.key.data(), kb, key_bytes) != 0) {
         if (loop.exec) {
             cudaGraphExecDestroy(loop.exec);
             loop.exec = nullptr;
@@ -771,28 +926,134 @@ int macro_pcg(rve_macro mm, int64_t n, int mdiv, const uint8_t* mask, const doub
         np.conditional.size = 1;
         cudaGraphNode_t node;
         RVE_CUDA(cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np));
-        cudaGraph_t body = np.conditional.phGraph_out[0];
+        cudaGraph_t inner = np.conditional.phGraph_out[0];
         cudaStream_t cap = mm->ctx->capture;
-        RVE_CUDA(cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        product(cap, p, q, acc);
-        k_macro_update<NF><<<gv, 256, 0, cap>>>(n, mdiv, mask, dinv, x, r, p, q, acc);
-        k_macro_pupdate<NF><<<gv, 256, 0, cap>>>(n, dinv, r, p, acc, handle);
-        RVE_CUDA(cudaStreamEndCapture(cap, &body));
+        RVE_CUDA(cudaStreamBeginCaptureToGraph(cap, inner, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+        body(cap, handle);
+        RVE_CUDA(cudaStreamEndCapture(cap, &inner));
         RVE_CUDA(cudaGraphInstantiate(&loop.exec, graph, 0));
-        loop.key.assign(kb, kb + sizeof(key));
+        loop.key.assign(kb, kb + key_bytes);
     }
     RVE_CUDA(cudaGraphLaunch(loop.exec, s));
     double h[PCG_SCALARS];
-    RVE_CUDA(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
+    RVE_CUDA(cudaMemcpyAsync(h, mm->acc.p, sizeof(h), cudaMemcpyDeviceToHost, s));
     RVE_CUDA(cudaStreamSynchronize(s));
     conv = true;
     for (int f = 0; f < 2; ++f) {
-        const bool used = f < NF;
-        its[f] = used ? (int)h[12 + f] : 0;
-        rel[f] = used && h[6 + f] > 0 ? std::sqrt(std::max(h[f], 0.0) / h[6 + f]) : 0.0;
-        if (used && h[10 + f] != 0.0) conv = false;
+        its[f] = f < nf ? (int)h[12 + f] : 0;
+        rel[f] = f < nf && h[6 + f] > 0 ? std::sqrt(std::max(h[norm + f], 0.0) / h[6 + f]) : 0.0;
+        if (f < nf && h[10 + f] != 0.0) conv = false;
     }
     return RVE_OK;
+}
+
+// Polynomial of the elastic solve's preconditioner: it covers [lambda / ratio, lambda]
+// of the spectrum with degree sqrt(ratio).  Measured on the 200 x 40 x 10 plate (solve
+// and results): degree 10, ratio 100 36.4 ms; 18, 300 31.4; 24, 600 28.8; 32, 1500 26.9.
+// The condition number grows with the square of the nodes along the longest side, at
+// most as the 2/3 power of their number for a cube.
+double mech_cheb_ratio(int64_t nv) { return std::min(1500.0, std::max(10.0, 0.75 * std::pow((double)nv, 2.0 / 3.0))); }
+
+// Bound of the spectrum of D^-1 K by power iteration with the preconditioner's step
+// kernel, rounded up to eighths (the quotient approaches the eigenvalue from below, and
+// the captured loop's coefficients then stay the same from solve to solve).
+template <class Step>
+int mech_spectrum(rve_macro m, int64_t n, Step step, double& lambda) {
+    cudaStream_t s = m->ctx->stream;
+    const unsigned g = grid_for(n);
+    float *x = m->c_z.as<float>(), *d = m->c_d.as<float>(), *zero = m->c_r.as<float>(), *dinv = m->c_dinv.as<float>();
+    double* acc = m->acc.as<double>();
+    RVE_CUDA(cudaMemsetAsync(acc, 0, 2 * 8, s));
+    k_power_start<<<g, 256, 0, s>>>(n, m->mdinv.as<double>(), x, zero, dinv);
+    const int steps = 30;
+    for (int k = 0; k <= steps; ++k) {
+        step(s, MechCheb{x, m->c_z2.as<float>(), zero, d, zero, dinv, nullptr, 0.f, 1.f, nullptr});
+        if (k < steps) k_power_next<<<g, 256, 0, s>>>(n, d, x);
+    }
+    k_power_sums<<<g, 256, 0, s>>>(n, x, d, dinv, acc);
+    double h[2];
+    RVE_CUDA(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
+    RVE_CUDA(cudaStreamSynchronize(s));
+    const double q = h[1] > 0.0 ? h[0] / h[1] : 0.0;
+    lambda = std::isfinite(q) && q > 0.0 ? std::ceil(8.0 * 1.1 * q) / 8.0 : 12.0;
+    return RVE_OK;
+}
+
+// FP64 PCG of the elastic problem with the polynomial preconditioner: converged when
+// (r, D^-1 r) <= rtol^2 max((f, D^-1 f), (r0, D^-1 r0)) over the free rows.
+// product(stream, in, out, acc) forms out = K in and adds (in, out) to acc[2].
+template <class Product, class Step>
+int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product product, Step step, double rtol,
+             int max_iter, int its[2], double rel[2], bool& conv) {
+    cudaStream_t s = mm->ctx->stream;
+    for (DevBuf* bfr : {&mm->c_r, &mm->c_z, &mm->c_z2, &mm->c_d, &mm->c_dinv}) RVE_TRY(bfr->ensure((size_t)n * 4));
+    double lambda = 0.0;
+    RVE_TRY(mech_spectrum(mm, n, step, lambda));
+    double *r = mm->r.as<double>(), *p = mm->p.as<double>(), *q = mm->q.as<double>(), *acc = mm->acc.as<double>();
+    float *r32 = mm->c_r.as<float>(), *zb[2] = {mm->c_z.as<float>(), mm->c_z2.as<float>()};
+    float *d = mm->c_d.as<float>(), *dinv32 = mm->c_dinv.as<float>();
+    const uint8_t* mask = mm->mfix.as<uint8_t>();
+    const double* dinv = mm->mdinv.as<double>();
+    const unsigned gv = grid_for(n);
+    const double ratio = mech_cheb_ratio(mm->nv);
+    const int degree = std::max(4, (int)std::lround(std::sqrt(ratio)));
+    const double hi = lambda, lo = hi / ratio, th = 0.5 * (hi + lo), de = 0.5 * (hi - lo);
+    const float w = (float)(1.0 / th);
+    // z = M^-1 r from z = w D^-1 r; returns the buffer that holds it
+    auto precondition = [&](cudaStream_t st) -> const float* {
+        double rho = de / th;
+        for (int k = 0; k + 1 < degree; ++k) {
+            const double rn = 1.0 / (2.0 * th / de - rho);
+            step(st, MechCheb{zb[k & 1], zb[(k & 1) ^ 1], k == 0 ? zb[0] : d, d, r32, dinv32, r, (float)(rn * rho),
+                              (float)(2.0 * rn / de), k + 2 == degree ? acc : nullptr});
+            rho = rn;
+        }
+        return zb[(degree - 1) & 1];
+    };
+    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+    product(s, x, q, nullptr);
+    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, r32, zb[0], dinv32, w, acc);
+    k_macro_start<<<1, 2, 0, s>>>(acc, 1, 20, rtol * rtol, max_iter);
+    k_mech_first<<<gv, 256, 0, s>>>(n, precondition(s), p);
+    RVE_CUDA(cudaGetLastError());
+    struct Key {
+        const void* ptr[14];
+        double lambda;
+    } key;
+    std::memset(&key, 0, sizeof(key));
+    const void* ptrs[14] = {r, p, q, acc, x, mask, dinv, mm->mmat.p, mm->g_col.p, r32, zb[0], zb[1], d, mm->mmat32.p};
+    std::memcpy(key.ptr, ptrs, sizeof(ptrs));
+    key.lambda = lambda;
+    return macro_loop(mm, 1, &key, sizeof(key), 1, 20, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+        product(cap, p, q, acc);
+        k_mech_update<<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
+        k_mech_pupdate<<<gv, 256, 0, cap>>>(n, precondition(cap), p, acc, h);
+    }, its, rel, conv);
+}
+
+// FP64 Jacobi PCG of the transport pair; per field converged when (r, D^-1 r) <=
+// rtol^2 max((b, D^-1 b), (r0, D^-1 r0)) over the free nodes.
+template <class Product>
+int transport_pcg(rve_macro mm, double2* x, const double2* b, Product product, double rtol, int max_iter, int its[2],
+                  double rel[2], bool& conv) {
+    cudaStream_t s = mm->ctx->stream;
+    double2 *r = mm->r.as<double2>(), *p = mm->p.as<double2>(), *q = mm->q.as<double2>();
+    double* acc = mm->acc.as<double>();
+    const uint8_t* mask = mm->mask.as<uint8_t>();
+    const double2* dinv = mm->t_dinv.as<double2>();
+    const int64_t nv = mm->nv;
+    const unsigned gv = grid_for(nv);
+    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+    product(s, x, q, nullptr);
+    k_transport_residual<<<gv, 256, 0, s>>>(nv, b, q, mask, dinv, r, p, acc);
+    k_macro_start<<<1, 2, 0, s>>>(acc, 2, 0, rtol * rtol, max_iter);
+    RVE_CUDA(cudaGetLastError());
+    const void* key[9] = {r, p, q, acc, x, mask, dinv, mm->t_mat.p, mm->g_col.p};
+    return macro_loop(mm, 0, key, sizeof(key), 2, 0, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+        product(cap, p, q, acc);
+        k_transport_update<<<gv, 256, 0, cap>>>(nv, mask, dinv, x, r, p, q, acc);
+        k_transport_pupdate<<<gv, 256, 0, cap>>>(nv, dinv, r, p, acc, h);
+    }, its, rel, conv);
 }
 
 }  // namespace
@@ -951,7 +1212,7 @@ static int transport_solve(rve_macro mm, double dt_s, double rtol, int max_iter,
                            bool& conv) {
     cudaStream_t s = mm->ctx->stream;
     RVE_TRY(ensure_transport_matrix(mm, dt_s));
-    const int64_t n = mm->nv * 2, ns = mm->n_slices;
+    const int64_t ns = mm->n_slices;
     double* x = mm->x.as<double>();
     double* b = mm->b.as<double>();
     const uint8_t* mask = mm->mask.as<uint8_t>();
@@ -963,11 +1224,11 @@ static int transport_solve(rve_macro mm, double dt_s, double rtol, int max_iter,
     k_transport_rhs<<<gs, 256, 0, s>>>(mm->nv, ns, base, col, mm->t_mass.as<double>(), mm->rho_cp / dt_s, 1.0 / dt_s,
                                        reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(b));
     k_macro_hold<<<grid_for(mm->nv), 256, 0, s>>>(mm->nv, mask, mm->hold.as<double>(), x);
-    auto product = [&](cudaStream_t st, const double* in, double* out, double* acc) {
-        k_transport_product<<<gs, 256, 0, st>>>(mm->nv, ns, base, col, mat, reinterpret_cast<const double2*>(in),
-                                                reinterpret_cast<double2*>(out), acc);
+    auto product = [&](cudaStream_t st, const double2* in, double2* out, double* acc) {
+        k_transport_product<<<gs, 256, 0, st>>>(mm->nv, ns, base, col, mat, in, out, acc);
     };
-    return macro_pcg<2>(mm, n, 2, mask, mm->t_dinv.as<double>(), x, b, mat, product, rtol, max_iter, its, rel, conv);
+    return transport_pcg(mm, reinterpret_cast<double2*>(x), reinterpret_cast<const double2*>(b), product, rtol,
+                         max_iter, its, rel, conv);
 }
 
 int rve_macro_step(rve_ctx c, rve_macro m, double dt_h, const rve_degradation* deg, double rtol, int max_iter,
@@ -1325,6 +1586,7 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
     for (DevBuf* bfr : {&m->b, &m->r, &m->p, &m->q, &m->mdinv}) RVE_TRY(bfr->ensure((size_t)n * 8));
     RVE_TRY(m->cm.ensure((size_t)m->nt * 36 * 8));
     RVE_TRY(m->mmat.ensure((size_t)m->n_ell * 9 * 32 * 8));
+    RVE_TRY(m->mmat32.ensure((size_t)m->n_ell * 9 * 32 * 4));
     RVE_TRY(m->msig.ensure((size_t)m->nt * 4 * 6 * 8));
     const int32_t* tets = m->tets.as<int32_t>();
     const double* geo = m->geo.as<double>();
@@ -1349,8 +1611,12 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
     int its[2] = {0, 0};
     double rel[2] = {0, 0};
     bool conv = false;
-    RVE_TRY(macro_pcg<1>(m, n, 1, m->mfix.as<uint8_t>(), m->mdinv.as<double>(), u, b, mat, product, rtol, max_iter,
-                         its, rel, conv));
+    const float* mat32 = m->mmat32.as<float>();
+    k_narrow<<<(unsigned)(sm_count() * 16), 256, 0, s>>>(m->n_ell * 288, mat, m->mmat32.as<float>());
+    auto step = [&](cudaStream_t st, const MechCheb& c) {
+        k_mech_cheb<<<(unsigned)((m->n_slices + 1) / 2), 192, 0, st>>>(m->nv, m->n_slices, base, col, mat32, c);
+    };
+    RVE_TRY(mech_pcg(m, n, u, b, product, step, rtol, max_iter, its, rel, conv));
     k_mech_stress<<<grid_for(m->nt * 4), 256, 0, s>>>(m->nt, tets, geo, Cg, u, m->msig.as<double>());
     RVE_CUDA(cudaGetLastError());
     RVE_CUDA(cudaStreamSynchronize(s));
