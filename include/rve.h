@@ -57,7 +57,7 @@ extern "C" {
 #define RVE_BC_PERIODIC  1   /* periodic fluctuation, anti-periodic traction */
 #define RVE_BC_NEUMANN   2   /* uniform traction t = sigma_bar n */
 
-#define RVE_PREC_FP64    0   /* FP64 operator, vectors and reductions */
+#define RVE_PREC_FP64    0   /* FP64 operator, vectors and reductions (preconditioner in FP32) */
 #define RVE_PREC_MIXED   1   /* FP32 operator and vectors, FP64 scalars, FP64 residual refinement */
 
 #define RVE_MODE_PCG     0   /* macro_update_gauss_points: plain batched PCG for every point */
@@ -100,8 +100,9 @@ typedef struct rve_options {
                                 mesh, else the matrix-free CUDA-core kernel; RVE_KERNEL_CUDA_CORE
                                 that kernel; RVE_KERNEL_TENSOR the tensor-core kernel (element
                                 matrices stored once per mesh and materials, 3 x TF32 products
-                                with FP32 accumulation).  Other cases always use the matrix-free
-                                kernel. */
+                                with FP32 accumulation).  Other cases always use a CUDA-core
+                                kernel: the assembled operator at p = 1 and in FP64 at p = 2, the
+                                matrix-free one elsewhere. */
     int     deterministic;   /* 1: bit-reproducible cell solves.  The scatter kernels (operator,
                                 true residual, right-hand side) run once per element colour (no
                                 two elements of a colour share a DOF; greedy colouring of the DOF
@@ -161,7 +162,7 @@ typedef struct rve_stats {
     double  op_ms;                /* summed device time of operator launches (profile mode) */
     int64_t op_launches;          /* operator launches counted in op_ms */
     double  op_bytes;             /* algorithmic bytes of those launches: x read + y written
-                                     (2 n_rows ncols sizeof(real)) + element data once */
+                                     (2 n_rows ncols sizeof(real)) + element data or matrix once */
     double  op_flops;             /* algorithmic flops of those launches (FMA = 2) */
     /* profile mode, the PCG vector kernels of the same iterations: */
     double  update_ms, update_bytes;     /* x, r read+written, p, q read (6 n_rows ncols s) */
@@ -503,7 +504,8 @@ int rve_macro_get(rve_ctx ctx, rve_macro m, double* T_nodal, double* c_nodal, do
 typedef struct rve_macro_mech_stats {
     int32_t iterations;         /* PCG iterations */
     int32_t converged;          /* 1 if rtol was reached */
-    double  rel_residual;       /* sqrt((r, M^-1 r) / max((f, M^-1 f), (r0, M^-1 r0))), free DOFs */
+    double  rel_residual;       /* sqrt((r, D^-1 r) / max((f, D^-1 f), (r0, D^-1 r0))), free DOFs,
+                                   D the Jacobi diagonal */
     double  seconds;
 } rve_macro_mech_stats;
 

@@ -15,6 +15,8 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "assembled.h"
+#include "node_graph.h"
 
 namespace rve {
 
@@ -127,6 +129,8 @@ int rebuild_map(rve_mesh m) {
         return rc;
     }
     const int ne = n_local(m->p);
+    m->a_graph_valid = false;
+    for (auto& row : m->a_valid) row[0] = row[1] = false;
     RVE_TRY(upload(m->d_edofs, m->map.edofs.data(), (size_t)m->nt * ne, s));
     RVE_TRY(build_colouring(m));
     RVE_TRY(upload(m->d_lverts, m->map.lverts.data(), (size_t)m->nt * 4, s));
@@ -275,6 +279,8 @@ int build_field_data(rve_mesh m) {
 int build_diagonals(rve_mesh m) {
     cudaStream_t s = m->ctx->stream;
     m->ke_valid = false;   // the element matrices follow the map and the materials
+    for (auto& row : m->a_valid) row[0] = row[1] = false;
+    m->a_lambda[0] = m->a_lambda[1] = 0.0;
     for (FieldDev* f : {&m->mech, &m->scal}) {
         const int64_t n = f->n_rows * 2 * f->nfield;
         RVE_TRY(f->diag64.ensure(sizeof(double) * n));
@@ -309,6 +315,128 @@ int ensure_element_matrices(rve_mesh m, cudaStream_t s) {
     m->ctx->launches++;
     m->ke_valid = true;
     return RVE_OK;
+}
+
+// Sparsity of the assembled operator.  Rows are stored along a Morton curve through the
+// nodes' neighbourhoods (the mean centroid of a node's elements), so that the rows of a
+// block gather nearby values of x, and inside windows of 1024 rows by length, so that
+// the lanes of a warp walk rows of like length.
+int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
+    if (m->a_graph_valid) return RVE_OK;
+    const int ne = n_local(m->p);
+    const int64_t N = m->map.N;
+    NodeGraph g;
+    if (!build_node_graph(m->map.edofs.data(), m->nt, ne, m->phase.data(), N, g)) {
+        set_error("mesh too large for 32-bit matrix indices");
+        return RVE_ERR_INVALID_ARGUMENT;
+    }
+    std::vector<float> cen((size_t)m->nt * 3);
+    float lo[3] = {HUGE_VALF, HUGE_VALF, HUGE_VALF}, hi[3] = {-HUGE_VALF, -HUGE_VALF, -HUGE_VALF};
+    for (int64_t e = 0; e < m->nt; ++e)
+        for (int a = 0; a < 3; ++a) {
+            double c = 0;
+            for (int v = 0; v < 4; ++v) c += 0.25 * m->xyz[3 * (int64_t)m->tets[4 * e + v] + a];
+            cen[e * 3 + a] = (float)c;
+            lo[a] = std::min(lo[a], (float)c);
+            hi[a] = std::max(hi[a], (float)c);
+        }
+    std::vector<std::pair<uint32_t, int32_t>> key(N);
+    for (int64_t i = 0; i < N; ++i) {
+        float c[3] = {0, 0, 0};
+        const int n = std::max(1, g.eptr[i + 1] - g.eptr[i]);
+        for (int32_t q = g.eptr[i]; q < g.eptr[i + 1]; ++q)
+            for (int a = 0; a < 3; ++a) c[a] += cen[(size_t)(g.inc[q] / ne) * 3 + a];
+        uint32_t k = 0;
+        for (int a = 0; a < 3; ++a) {
+            const float t = hi[a] > lo[a] ? (c[a] / n - lo[a]) / (hi[a] - lo[a]) : 0.f;
+            const uint32_t v = (uint32_t)std::min(1023.f, std::max(0.f, t * 1023.f));
+            for (int bit = 0; bit < 10; ++bit) k |= ((v >> bit) & 1u) << (3 * bit + a);
+        }
+        key[i] = {k, (int32_t)i};
+    }
+    std::sort(key.begin(), key.end());
+    std::vector<int32_t> order(N);
+    for (int64_t i = 0; i < N; ++i) order[i] = key[i].second;
+    for (int64_t w = 0; w < N; w += 1024)
+        std::stable_sort(order.begin() + w, order.begin() + std::min(N, w + 1024), [&](int32_t a, int32_t b) {
+            return g.ptr[a + 1] - g.ptr[a] > g.ptr[b + 1] - g.ptr[b];
+        });
+    std::vector<int32_t> ptr(N + 1, 0), split(N), col(g.col.size());
+    for (int64_t r = 0; r < N; ++r) {
+        const int32_t i = order[r], n = g.ptr[i + 1] - g.ptr[i];
+        std::copy(g.col.begin() + g.ptr[i], g.col.begin() + g.ptr[i + 1], col.begin() + ptr[r]);
+        split[r] = ptr[r] + (g.split[i] - g.ptr[i]);
+        ptr[r + 1] = ptr[r] + n;
+    }
+    RVE_TRY(upload(m->a_order, order.data(), order.size(), s));
+    RVE_TRY(upload(m->a_ptr, ptr.data(), ptr.size(), s));
+    RVE_TRY(upload(m->a_split, split.data(), split.size(), s));
+    RVE_TRY(upload(m->a_col, col.data(), col.size(), s));
+    RVE_TRY(upload(m->a_eptr, g.eptr.data(), g.eptr.size(), s));
+    RVE_TRY(upload(m->a_inc, g.inc.data(), g.inc.size(), s));
+    RVE_CUDA(cudaStreamSynchronize(s));
+    m->a_entries = (int64_t)col.size();
+    m->a_graph_valid = true;
+    return RVE_OK;
+}
+
+// Whether a solve uses the assembled operator.  FP64: orders 1 and 2, where it needs a
+// sixth and a half of the element form's FMAs (FP64-bound; 24x24x8, p = 2, 6 columns:
+// 231 -> 171 us a product).  FP32: order 1 only (16x16x6, 1536 columns: 206 -> 71 us); at
+// order 2 the matrix (48 B per entry, 30 entries a row) and the gathers of x through L1
+// cost more than recomputing from the element data (24x24x8, 6 columns: 37 us against
+// 16; 32x32x10, 48 columns: 273 against 127).  Not in the deterministic mode (whose sums
+// run colour by colour) and not in a checking build (which checks the element kernels'
+// indices).
+bool use_assembled(rve_mesh m, bool fp64) {
+    return m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built();
+}
+
+// Entries of one field (0 mechanics, 1 scalar), formed on first use after a change of the
+// map or the materials.
+int ensure_assembled(rve_mesh m, int fid, bool fp64, cudaStream_t s) {
+    if (m->a_graph_valid && m->a_valid[fid][fp64 ? 0 : 1]) return RVE_OK;
+    RVE_TRY(ensure_asm_graph(m, s));
+    const int ne = n_local(m->p);
+    // an FP64 solve's preconditioner takes the FP32 entries too where they are used
+    const bool want64 = fp64 && !m->a_valid[fid][0];
+    const bool want32 = (!fp64 || use_assembled(m, false)) && !m->a_valid[fid][1];
+    const int w64 = fid == 0 ? AsmEntry<double, 3>::WORDS : AsmEntry<double, 1>::WORDS;
+    const int w32 = fid == 0 ? AsmEntry<float, 3>::WORDS : AsmEntry<float, 1>::WORDS;
+    if (want64) RVE_TRY(m->a_ent[fid][0].ensure((size_t)m->a_entries * w64 * 8));
+    if (want32) RVE_TRY(m->a_ent[fid][1].ensure((size_t)m->a_entries * w32 * 4));
+    RVE_TRY(m->a_rtab.ensure((size_t)9 * ne * ne * 8));
+    AsmGraph g;
+    g.n = m->map.N;
+    g.entries = m->a_entries;
+    g.ne = ne;
+    g.order = m->a_order.as<int32_t>();
+    g.ptr = m->a_ptr.as<int32_t>();
+    g.split = m->a_split.as<int32_t>();
+    g.col = m->a_col.as<int32_t>();
+    g.eptr = m->a_eptr.as<int32_t>();
+    g.inc = m->a_inc.as<int32_t>();
+    launch_assemble(m->p, fid == 0 ? 3 : 1, g, m->d_edofs.as<int32_t>(), m->d_phase.as<uint8_t>(),
+                    m->d_geo64.as<double>(), (fid == 0 ? m->d_matm64 : m->d_mats64).as<double>(),
+                    m->a_rtab.as<double>(), want64 ? m->a_ent[fid][0].as<double>() : nullptr,
+                    want32 ? m->a_ent[fid][1].as<float>() : nullptr, s);
+    RVE_CUDA(cudaGetLastError());
+    m->ctx->launches++;
+    if (want64) m->a_valid[fid][0] = true;
+    if (want32) m->a_valid[fid][1] = true;
+    return RVE_OK;
+}
+
+template <typename T>
+AsmView<T> asm_view(rve_mesh m, int fid, const T* scale) {
+    AsmView<T> a;
+    a.n = m->map.N;
+    a.order = m->a_order.as<int32_t>();
+    a.ptr = m->a_ptr.as<int32_t>();
+    a.split = m->a_split.as<int32_t>();
+    a.ent = m->a_ent[fid][sizeof(T) == 4 ? 1 : 0].as<T>();
+    a.scale = scale;
+    return a;
 }
 
 // ------------------------------------------------------------- launch shape
@@ -360,12 +488,27 @@ struct WarmStart {
     const int32_t* kx_map = nullptr;   // [ncols][WARM_SOURCES]
 };
 
+// The preconditioner of the FP64 solves: a Chebyshev polynomial in D^-1 A, evaluated in
+// FP32.  An FP64 product runs at two FMAs per clock and SM, an FP32 one at 128, so a
+// polynomial of degree 17 (16 FP32 products) costs about what 1.5 FP64 iterations do and
+// takes the place of 12 of them (24x24x8, p = 2: 284 iterations in 89 ms before, 22 in 16
+// now).  The operator, the vectors, the inner products and the stopping test stay FP64,
+// so the solution is as accurate.  It covers [lambda / ratio, lambda] of the spectrum with
+// degree sqrt(ratio); the ratio follows the condition number, which grows with the square
+// of the nodes along a side.  Measured (ms a solve): 24x24x8, p = 2 (36 864 nodes, ratio
+// 277): degree 10, ratio 60 19.7; 14, 250 16.5; 18, 250 15.9; 6 x 6 x 4, p = 1 (144 nodes,
+// ratio 10): degree 6, ratio 15 1.60; 10, 60 1.90.
+double cheb_ratio(int64_t nodes) {
+    return std::min(300.0, std::max(10.0, 0.25 * std::pow((double)nodes, 2.0 / 3.0)));
+}
+
 struct Solver {
     rve_mesh m;
     FieldDev& f;
     int B, ncols;
     int64_t n_rows;
     int fid;   // 0 mechanics, 1 scalar fields
+    bool free_rows = false;   // leave the constraint rows out (traction_start)
     Launch L;
     cudaStream_t s;
     ColState cs64{};
@@ -403,7 +546,7 @@ struct Solver {
         r.scale = scale.as<T>();
         r.nfield = f.nfield;
         r.nc = f.nc;
-        r.m = f.m;
+        r.m = free_rows ? 0 : f.m;
         r.n_sup = f.n_sup;
         r.sup_row = f.sup_row.as<int64_t>();
         r.sup_coef = f.sup_coef.as<double>();
@@ -439,9 +582,9 @@ struct Solver {
         RVE_TRY(m->gsum.ensure((size_t)ncols * 12 * 8));
         RVE_TRY(m->msum.ensure((size_t)ncols * 12 * 8));
         // col state: rz, rz0, alpha, beta (4*ncols) + mu (12*ncols) + schur (144*ncols) + the fused
-        // iteration's pq and rz accumulators (2*ACC_SLOTS*ncols) doubles,
+        // iteration's pq, rz and rj accumulators (3*ACC_SLOTS*ncols) doubles,
         // then active, iters (ints) and flags
-        const size_t nd = (size_t)ncols * (4 + 12 + 144 + 2 * ACC_SLOTS);
+        const size_t nd = (size_t)ncols * (4 + 12 + 144 + 3 * ACC_SLOTS);
         RVE_TRY(m->colstate.ensure(nd * 8 + (size_t)ncols * 12 + 64));
         double* base = m->colstate.as<double>();
         cs64.rz = base;
@@ -452,6 +595,7 @@ struct Solver {
         cs64.schur = base + 16 * ncols;
         cs64.pq_acc = base + 160 * ncols;
         cs64.rz_acc = base + (160 + ACC_SLOTS) * ncols;
+        cs64.rj_acc = base + (160 + 2 * ACC_SLOTS) * ncols;
         int32_t* ib = reinterpret_cast<int32_t*>(base + nd);
         cs64.active = ib;
         cs64.iters = ib + ncols;
@@ -552,10 +696,19 @@ struct Solver {
             evs.push_back(e);
         }
         if (prof) RVE_CUDA(cudaEventRecord(evs[0], s));
-        RVE_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * n_rows * ncols, s));
-        launch_operator<double>(m->p, f.nc, true, ev<double>(m->scale64), x, y, nullptr, L);
-        launch_neg(n_rows * ncols, y, s);
-        *launches += 2;
+        if (use_assembled(m, true)) {
+            // b is the right-hand side less what the constraint forces carry, which the
+            // projection of the residual removes anyway
+            RVE_TRY(ensure_assembled(m, fid, true, s));
+            launch_asm_residual<double>(f.nc, asm_view<double>(m, fid, m->scale64.as<double>()), x,
+                                        m->b64.as<double>(), y, ncols, s);
+            *launches += 1;
+        } else {
+            RVE_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * n_rows * ncols, s));
+            launch_operator<double>(m->p, f.nc, true, ev<double>(m->scale64), x, y, nullptr, L);
+            launch_neg(n_rows * ncols, y, s);
+            *launches += 2;
+        }
         if (prof) {
             RVE_CUDA(cudaEventRecord(evs[1], s));
             RVE_CUDA(cudaEventSynchronize(evs[1]));
@@ -564,6 +717,49 @@ struct Solver {
             m->ctx->prof.res_ms += ms;
             m->ctx->prof.res_launches++;
         }
+        return RVE_OK;
+    }
+
+    // Upper bound of the spectrum of D^-1 A of this field for any positive phase scales, by
+    // power iteration on each phase alone (see assembled.h).
+    int ensure_lambda() {
+        if (m->a_lambda[fid] > 0.0) return RVE_OK;
+        const bool asm32 = use_assembled(m, false);
+        if (asm32) RVE_TRY(ensure_assembled(m, fid, false, s));
+        const size_t nv = (size_t)n_rows * 6;
+        RVE_TRY(m->x32.ensure(nv * 4));
+        RVE_TRY(m->r32.ensure(nv * 4));
+        RVE_TRY(m->dscale32.ensure(12 * 4));
+        RVE_TRY(m->gsum.ensure(12 * 8));
+        float sc[12];
+        power_scales(f.nc, sc);
+        RVE_TRY(upload(m->dscale32, sc, 12, s));
+        RVE_CUDA(cudaMemsetAsync(m->gsum.p, 0, 12 * 8, s));
+        float* xv = m->x32.as<float>();
+        float* yv = m->r32.as<float>();
+        const Launch L6 = make_launch(6, std::max<int64_t>(n_rows, m->nt), s);
+        const int steps = 30;
+        launch_power_start(n_rows, xv, s);
+        for (int k = 0; k <= steps; ++k) {
+            if (asm32) {
+                launch_asm_product<float>(f.nc, asm_view<float>(m, fid, m->dscale32.as<float>()), xv, yv, 6, nullptr,
+                                          nullptr, s);
+            } else {
+                RVE_CUDA(cudaMemsetAsync(yv, 0, nv * 4, s));
+                launch_operator<float>(m->p, f.nc, false, ev<float>(m->dscale32), xv, yv, nullptr, L6);
+            }
+            launch_power_next(f.nc, n_rows, f.diag64.as<double>(), xv, yv, k == steps ? m->gsum.as<double>() : nullptr,
+                              s);
+        }
+        *launches += 2 * steps + 3;
+        double h[12];
+        RVE_CUDA(cudaMemcpyAsync(h, m->gsum.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+        RVE_CUDA(cudaStreamSynchronize(s));
+        double lam = 0.0;
+        for (int c = 0; c < 6; ++c)
+            if (h[6 + c] > 0.0) lam = std::max(lam, h[c] / h[6 + c]);
+        // the quotient approaches the eigenvalue from below
+        m->a_lambda[fid] = std::isfinite(lam) && lam > 0.0 ? 1.15 * lam : 4.0;
         return RVE_OK;
     }
 
@@ -580,6 +776,9 @@ struct Solver {
         const bool use_tc =
             !det && sizeof(T) == 4 && operator_tc_supported(m->p, f.nc) && kern == RVE_KERNEL_TENSOR;
         if (use_tc) RVE_TRY(ensure_element_matrices(m, s));
+        const bool use_asm = !use_tc && use_assembled(m, sizeof(T) == 8);
+        if (use_asm) RVE_TRY(ensure_assembled(m, fid, sizeof(T) == 8, s));
+        const AsmView<T> av = use_asm ? asm_view<T>(m, fid, scale.as<T>()) : AsmView<T>();
         ColState cs = cs64;
         // the operator of the iteration runs one wave of resident blocks; its energy
         // partials (and the alpha reduction over them) have as many rows
@@ -590,25 +789,114 @@ struct Solver {
         // p-update): FP64 atomic accumulators replace the alpha and beta partial-row
         // reductions.  Not with constraint rows (their multipliers need the partial
         // rows), the tensor-core operator or the deterministic mode (atomic order).
-        const bool fused = !det && !use_tc && f.m == 0;
-        if (fused) {
-            Lop.energy_acc = cs.pq_acc;
-            RVE_CUDA(cudaMemsetAsync(cs.pq_acc, 0, sizeof(double) * 2 * ACC_SLOTS * ncols, s));   // pq_acc, rz_acc
+        const int m_rows = free_rows ? 0 : f.m;
+        const bool fused = !det && !use_tc && m_rows == 0;
+        if (fused || use_asm) {
+            if (fused) Lop.energy_acc = cs.pq_acc;
+            RVE_CUDA(cudaMemsetAsync(cs.pq_acc, 0, sizeof(double) * 3 * ACC_SLOTS * ncols, s));   // pq, rz and rj
         }
-        const int kernels_per_iter = fused ? 4 : 6;
+        // FP64 without constraint rows: polynomial preconditioner
+        const bool cheb = sizeof(T) == 8 && fused && !bounds_check_built();
+        const bool cheb_asm = cheb && use_assembled(m, false);
+        AsmView<float> av32;
+        ChebArgs cha;
+        float cheb_w = 0.f;
+        std::vector<std::pair<float, float>> cheb_c;
+        if (cheb) {
+            RVE_TRY(ensure_lambda());
+            const size_t nvv = (size_t)n_rows * ncols;
+            for (DevBuf* bfr : {&m->x32, &m->r32, &m->p32, &m->q32}) RVE_TRY(bfr->ensure(nvv * 4));
+            if (cheb_asm) av32 = asm_view<float>(m, fid, m->scale32.as<float>());
+            const double hi = m->a_lambda[fid], ratio = cheb_ratio(n_rows / f.nc), lo = hi / ratio, th = 0.5 * (hi + lo), de = 0.5 * (hi - lo);
+            cheb_w = (float)(1.0 / th);
+            double rho = de / th;
+            const int degree = std::max(4, (int)std::lround(std::sqrt(ratio)));
+            for (int k = 1; k < degree; ++k) {
+                const double rn = 1.0 / (2.0 * th / de - rho);
+                cheb_c.emplace_back((float)(rn * rho), (float)(2.0 * rn / de));
+                rho = rn;
+            }
+        }
+        const int kernels_per_iter = cheb ? 4 + (cheb_asm ? 1 : 2) * (int)cheb_c.size() : (fused ? 4 : 6);
         RVE_CUDA(cudaMemcpyAsync(const_cast<double*>(cs.tol), &tol, sizeof(double), cudaMemcpyHostToDevice, s));
         RowView<T> rvw = rv<T>(scale);
         ElemView<T> evw = ev<T>(scale);
+        if constexpr (sizeof(T) == 8) {
+            rvw.dinv_groups = f.nfield == 2 ? 2 : B;
+            RVE_TRY(m->dinv64.ensure((size_t)n_rows * rvw.dinv_groups * 8));
+            RVE_TRY(m->dinv32.ensure((size_t)n_rows * rvw.dinv_groups * 4));
+            launch_jacobi_inverse(rvw, rvw.dinv_groups, m->dinv64.as<double>(), m->dinv32.as<float>(), s);
+            rvw.dinv = m->dinv64.as<double>();
+            *launches += 1;
+            cha.dinv = m->dinv32.as<float>();
+            cha.groups = rvw.dinv_groups;
+        }
+        T* q_add = use_asm ? nullptr : q;   // the element operators add into q
         launch_schur<T>(rvw, cs, L);
         launch_update<T>(rvw, x, r, p, q, cs, m->rzp.as<double>(), false, L, m->cpart.as<double>());
-        launch_finalize_beta(f.m, m->rzp.as<double>(), m->cpart.as<double>(), cs, true, L);
+        launch_finalize_beta(m_rows, m->rzp.as<double>(), m->cpart.as<double>(), cs, true, L);
         if (tolc) {
             RVE_TRY(upload(m->coltol, tolc->data(), tolc->size(), s));
             launch_column_tol(ncols, m->coltol.as<double>(), cs, s);
             *launches += 1;
         }
+        const int nby32 = cheb && !cheb_asm ? operator_grid_y<float>(m->p, f.nc, L, m->nt) : 0;
+        if (cheb && !cheb_asm) RVE_CUDA(cudaMemsetAsync(m->q32.p, 0, (size_t)n_rows * ncols * 4, s));
+        // z = M^-1 r by the Chebyshev polynomial; returns the buffer that holds it
+        auto precondition = [&](const Launch& Lx, bool apply) -> const float* {
+            const float* z = m->x32.as<float>();
+            if constexpr (sizeof(T) == 8) {
+                float* zb[2] = {m->x32.as<float>(), m->p32.as<float>()};
+                float* d = m->q32.as<float>();
+                launch_cheb_update(rvw, cha.dinv, x, r, p, q, m->r32.as<float>(), zb[0], cheb_w, cs, apply, Lx);
+                const int n = (int)cheb_c.size();
+                if (!cheb_asm) {
+                    // element by element: z in place, the products in q32
+                    ElemView<float> ev32 = ev<float>(m->scale32);
+                    float* y = m->q32.as<float>();
+                    float* dd = zb[1];
+                    Launch Le = Lx;
+                    Le.energy_acc = nullptr;
+                    Le.nby_op = nby32;
+                    for (int k = 0; k < n; ++k) {
+                        launch_operator<float>(m->p, f.nc, false, ev32, zb[0], y, nullptr, Le, cs.active, cs.list,
+                                               cs.n_list);
+                        ChebArgs c2 = cha;
+                        c2.d_in = k == 0 ? zb[0] : dd;
+                        c2.d_out = dd;
+                        c2.c1 = cheb_c[k].first;
+                        c2.c2 = cheb_c[k].second;
+                        c2.r64 = r;
+                        launch_cheb_vector(n_rows, f.nfield, m->r32.as<float>(), c2, zb[0], y, cs.active,
+                                           k == n - 1 ? cs.rz_acc : nullptr, Lx);
+                    }
+                    return zb[0];
+                }
+                for (int k = 0; k < n; ++k) {
+                    ChebArgs c2 = cha;
+                    c2.d_in = k == 0 ? zb[0] : d;
+                    c2.d_out = d;
+                    c2.c1 = cheb_c[k].first;
+                    c2.c2 = cheb_c[k].second;
+                    c2.r64 = r;
+                    launch_cheb_step(f.nc, av32, zb[k & 1], m->r32.as<float>(), zb[(k & 1) ^ 1], c2, ncols, cs.active,
+                                     k == n - 1 ? cs.rz_acc : nullptr, Lx.stream);
+                }
+                z = zb[n & 1];
+            }
+            return z;
+        };
         launch_compact_active(cs.active, ncols, cs.list, cs.n_list, s);
-        launch_pupdate<T>(rvw, r, p, q, cs, true, L);
+        if (cheb) {
+            if constexpr (sizeof(T) == 8) {
+                const float* z = precondition(L, false);
+                launch_cheb_beta(cs, ncols, true, 0, nullptr, 0, false, s);
+                launch_cheb_direction(n_rows, z, p, q_add, cs, true, L);
+                *launches += kernels_per_iter;
+            }
+        } else {
+            launch_pupdate<T>(rvw, r, p, q_add, cs, true, L);
+        }
         *launches += 6;
         std::vector<int32_t> act(ncols);
         conv = false;
@@ -644,7 +932,9 @@ struct Solver {
             Lx.energy_acc = Lop.energy_acc;
             double* epart_it = fused ? nullptr : m->epart.as<double>();
             evr(0, Lx.stream);
-            if constexpr (sizeof(T) == 4) {
+            if (use_asm) {
+                launch_asm_product<T>(f.nc, av, p, q, ncols, cs.active, cs.pq_acc, Lx.stream);
+            } else if constexpr (sizeof(T) == 4) {
                 if (use_tc) {
                     const cudaError_t e = launch_operator_tc(
                         m->p, m->nt, m->d_edofs.as<int32_t>(), m->d_ke32.as<float>(), m->d_kepairs.as<uint16_t>(),
@@ -658,8 +948,22 @@ struct Solver {
                 launch_operator<T>(m->p, f.nc, false, evw, p, q, epart_it, Lx, cs.active, cs.list, cs.n_list);
             }
             evr(1, Lx.stream);
-            if (!fused) launch_finalize_alpha<T>(m->epart.as<double>(), cs, Lx);
+            if (!fused && use_asm)
+                launch_finalize_alpha<T>(cs.pq_acc, cs, Lx, cs.pq_acc);
+            else if (!fused)
+                launch_finalize_alpha<T>(m->epart.as<double>(), cs, Lx);
             evr(2, Lx.stream);
+            if (cheb) {
+                if constexpr (sizeof(T) == 8) {
+                    const float* z = precondition(Lx, true);
+                    evr(3, Lx.stream);
+                    launch_cheb_beta(cs, ncols, false, loop_handle, cs.flags + 1, max_iter, loop_ctl, Lx.stream);
+                    evr(4, Lx.stream);
+                    launch_cheb_direction(n_rows, z, p, q_add, cs, false, Lx);
+                    evr(5, Lx.stream);
+                }
+                return;
+            }
             if (fused)
                 launch_update_fused<T>(rvw, x, r, p, q, cs, Lx);
             else
@@ -668,7 +972,7 @@ struct Solver {
             if (fused) {
                 launch_beta_compact_continue(cs, ncols, loop_handle, cs.flags + 1, max_iter, loop_ctl, Lx.stream);
             } else {
-                launch_finalize_beta(f.m, m->rzp.as<double>(), m->cpart.as<double>(), cs, false, Lx);
+                launch_finalize_beta(m_rows, m->rzp.as<double>(), m->cpart.as<double>(), cs, false, Lx);
                 if (loop_ctl)
                     launch_compact_continue(cs.active, ncols, cs.list, cs.n_list, loop_handle, cs.flags + 1,
                                             max_iter, Lx.stream);
@@ -676,7 +980,7 @@ struct Solver {
                     launch_compact_active(cs.active, ncols, cs.list, cs.n_list, Lx.stream);
             }
             evr(4, Lx.stream);
-            launch_pupdate<T>(rvw, r, p, q, cs, false, Lx);
+            launch_pupdate<T>(rvw, r, p, q_add, cs, false, Lx);
             evr(5, Lx.stream);
         };
         if (!prof) {
@@ -690,7 +994,9 @@ struct Solver {
             struct Key {
                 int ncols, cpb, rows, nby, nby_op, p, nc, m, max_iter, tc, ncolour, fused;
                 int64_t n_rows, n_sup, nt, n_nodes;
-                const void* ptr[19];
+                const void* ptr[31];
+                double lambda;
+                int64_t cheb_n;
             } key;
             std::memset(&key, 0, sizeof(key));
             key.ncols = L.ncols;
@@ -706,13 +1012,19 @@ struct Solver {
             key.n_sup = rvw.n_sup;
             key.nt = evw.nt;
             key.n_nodes = evw.n_nodes;
-            key.tc = use_tc ? 1 : 0;
+            key.tc = use_tc ? 1 : (use_asm ? 2 : 0);
             key.ncolour = Lop.n_colour;
             key.fused = fused ? 1 : 0;
-            const void* ptrs[19] = {x, r, p, q, m->epart.p, m->rzp.p, m->cpart.p, cs.rz, rvw.scale, rvw.diag,
+            const void* ptrs[31] = {x, r, p, q, m->epart.p, m->rzp.p, m->cpart.p, cs.rz, rvw.scale, rvw.diag,
                                     rvw.mask, rvw.sup_row, rvw.sup_coef, rvw.sup_of_row, evw.edofs, evw.geo,
-                                    evw.mat, evw.phase, use_tc ? m->d_ke32.p : nullptr};
+                                    evw.mat, evw.phase, use_tc ? m->d_ke32.p : nullptr, av.ent, rvw.dinv,
+                                    av.order, av.ptr, av.split, cheb ? av32.ent : nullptr,
+                                    cheb ? m->r32.p : nullptr, cheb ? m->p32.p : nullptr, cheb ? m->q32.p : nullptr,
+                                    cheb ? m->x32.p : nullptr, cheb ? m->dinv32.p : nullptr,
+                                    cheb ? m->scale32.p : nullptr};
             std::memcpy(key.ptr, ptrs, sizeof(ptrs));
+            key.lambda = cheb ? m->a_lambda[fid] : 0.0;
+            key.cheb_n = (int)cheb_c.size();
             auto& gc = m->graph_cache[fid][sizeof(T) == 4 ? 1 : 0];
             const unsigned char* kb = reinterpret_cast<const unsigned char*>(&key);
             const bool hit = gc.exec && gc.key.size() == sizeof(key) && std::memcmp(gc.key.data(), kb, sizeof(key)) == 0;
@@ -784,13 +1096,17 @@ struct Solver {
                 const int ne = n_local(m->p), nmod = n_modes(m->p), nc = f.nc;
                 const double sz = sizeof(T);
                 const int na = n_act_run;
-                const double bytes = 2.0 * n_rows * na * sz +
-                                     (double)m->nt * (4.0 * ne + 10 * sz + (nc == 3 ? 21 : 6) * sz + 1);
+                // (the assembled operator: its entries once)
+                const double entries = (double)m->a_entries;
+                const double bytes =
+                    2.0 * n_rows * na * sz +
+                    (use_asm ? entries * ((nc == 3 ? 9 : 2) * sz + 4)
+                             : (double)m->nt * (4.0 * ne + 10 * sz + (nc == 3 ? 21 : 6) * sz + 1));
                 // FMAs per element and column: forward and backward contractions with the
                 // non-zero entries of the edge/face table, plus per-mode gradient, stress
                 // and back-mapping
                 const double fma = 2.0 * table_nonzeros(m->p) * nc + nmod * (18.0 * nc + (nc == 3 ? 36 : 9));
-                const double flops = 2.0 * fma * (double)m->nt * na;
+                const double flops = 2.0 * na * (use_asm ? entries * nc * nc : fma * (double)m->nt);
                 const double vb = (double)n_rows * na * sz;
                 auto el = [&](int a2, int b2) {
                     float ms = 0;
@@ -871,6 +1187,112 @@ struct Solver {
         return t;
     }
 
+    // Cold start of an FP64 uniform-traction solve.  The total field under the unit
+    // traction modes c_j (the strain or flux rows of the constraint) needs no constraint
+    // rows: K v_j = c_j is consistent and singular only by the rigid modes, so the
+    // polynomial-preconditioned PCG of the other boundary conditions solves it.  The
+    // fluctuation of load case i is then u_i = sum_j mu_ji v_j + a rigid mode - X_i with
+    // the coefficients from C u_i = 0, a 12 x 12 (4 x 4) system per RVE; its residual against
+    // b is a combination of constraint forces, which the projection removes, and of the
+    // v_j's residuals.  Leaves x, and r = b - K x projected with its norm in `rel`; the
+    // caller's constrained PCG takes on whatever is left above the tolerance.
+    int traction_start(double* x64, double* r64, double rtol, int max_iter, int& iters, double& rel,
+                       const std::vector<double>& bn) {
+        const int ni = f.nc == 3 ? 6 : 3, first = f.nc == 3 ? 6 : 1, mr = f.m;
+        const size_t nv = (size_t)n_rows * ncols;
+        RVE_CUDA(cudaMemsetAsync(x64, 0, nv * 8, s));
+        RVE_CUDA(cudaMemsetAsync(r64, 0, nv * 8, s));
+        launch_traction_loads(f.n_sup, mr, first, ni, f.sup_row.as<int64_t>(), f.sup_coef.as<double>(), ncols, r64, s);
+        *launches += 1;
+        bool conv = false;
+        free_rows = true;
+        const int rc = pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64, 0.3 * rtol,
+                                   max_iter, iters, conv);
+        free_rows = false;
+        RVE_TRY(rc);
+        // the constraint products of V per RVE, of the rigid modes and of the unit macro
+        // fields (both live on the vertex nodes)
+        const int nr = mr - ni;
+        DevBuf& cv_dev = m->cpart;   // 12 values per column and partial row: large enough
+        launch_rows_dot(f.n_sup, mr, f.sup_row.as<int64_t>(), f.sup_coef.as<double>(), x64, ncols,
+                        cv_dev.as<double>(), s);
+        *launches += 1;
+        std::vector<double> cv((size_t)mr * ncols), cx((size_t)mr * ni, 0.0), cr((size_t)mr * nr, 0.0);
+        RVE_CUDA(cudaMemcpyAsync(cv.data(), cv_dev.p, cv.size() * 8, cudaMemcpyDeviceToHost, s));
+        for (size_t q = 0; q < f.h_sup_row.size(); ++q) {
+            const int64_t node = f.h_sup_row[q] / f.nc;
+            const int c = (int)(f.h_sup_row[q] % f.nc);
+            const int32_t v = m->map.dof_vertex[node];
+            if (v < 0) continue;
+            const double* y = &m->xyz[3 * (int64_t)v];
+            const double* row = &f.h_sup_coef[q * mr];
+            double X[6] = {0, 0, 0, 0, 0, 0}, Rg[6] = {1, 0, 0, 0, 0, 0};
+            if (f.nc == 3) {
+                X[c] = y[c];
+                if (c == 0) X[3] = 0.5 * y[1], X[5] = 0.5 * y[2];
+                if (c == 1) X[3] = 0.5 * y[0], X[4] = 0.5 * y[2];
+                if (c == 2) X[4] = 0.5 * y[1], X[5] = 0.5 * y[0];
+                const double rot[3][3] = {{0, -y[2], y[1]}, {y[2], 0, -y[0]}, {-y[1], y[0], 0}};
+                for (int k = 0; k < 3; ++k) {
+                    Rg[k] = k == c ? 1.0 : 0.0;
+                    Rg[3 + k] = rot[k][c];
+                }
+            } else {
+                for (int k = 0; k < 3; ++k) X[k] = y[k];
+            }
+            for (int j = 0; j < mr; ++j) {
+                for (int k = 0; k < ni; ++k) cx[(size_t)j * ni + k] += row[j] * X[k];
+                for (int k = 0; k < nr; ++k) cr[(size_t)j * nr + k] += row[j] * Rg[k];
+            }
+        }
+        RVE_CUDA(cudaStreamSynchronize(s));
+        // per RVE: the multipliers mu [6][6] and the rigid modes' coefficients [6][6]
+        std::vector<double> mu((size_t)B * 72, 0.0);
+        bool ok = true;
+        for (int b = 0; b < B && ok; ++b)
+            for (int fld = 0; fld < (f.nc == 3 ? 1 : 2) && ok; ++fld) {
+                // Gauss-Jordan with partial pivoting on [C V, C R | C X]
+                double A[12][18];
+                for (int j = 0; j < mr; ++j) {
+                    for (int k = 0; k < ni; ++k) A[j][k] = cv[(size_t)j * ncols + 6 * b + 3 * fld + k];
+                    for (int k = 0; k < nr; ++k) A[j][ni + k] = cr[(size_t)j * nr + k];
+                    for (int k = 0; k < ni; ++k) A[j][mr + k] = cx[(size_t)j * ni + k];
+                }
+                for (int p = 0; p < mr && ok; ++p) {
+                    int best = p;
+                    for (int j = p + 1; j < mr; ++j)
+                        if (std::fabs(A[j][p]) > std::fabs(A[best][p])) best = j;
+                    ok = std::isfinite(A[best][p]) && A[best][p] != 0.0;
+                    if (!ok) break;
+                    for (int k = 0; k < mr + ni; ++k) std::swap(A[p][k], A[best][k]);
+                    const double d = 1.0 / A[p][p];
+                    for (int k = p; k < mr + ni; ++k) A[p][k] *= d;
+                    for (int j = 0; j < mr; ++j)
+                        if (j != p) {
+                            const double t = A[j][p];
+                            for (int k = p; k < mr + ni; ++k) A[j][k] -= t * A[p][k];
+                        }
+                }
+                for (int k = 0; k < ni && ok; ++k) {
+                    for (int j = 0; j < ni; ++j) mu[(size_t)b * 72 + (3 * fld + j) * 6 + 3 * fld + k] = A[j][mr + k];
+                    for (int j = 0; j < nr; ++j) mu[(size_t)b * 72 + 36 + j * 6 + 3 * fld + k] = A[ni + j][mr + k];
+                }
+            }
+        if (!ok) {   // no usable start: from zero
+            RVE_CUDA(cudaMemcpyAsync(r64, m->b64.p, nv * 8, cudaMemcpyDeviceToDevice, s));
+            RVE_CUDA(cudaMemsetAsync(x64, 0, nv * 8, s));
+            return RVE_OK;
+        }
+        RVE_TRY(upload(m->traction_mu, mu.data(), mu.size(), s));
+        RVE_TRY(upload(m->d_dof_vertex, m->map.dof_vertex.data(), m->map.dof_vertex.size(), s));
+        launch_traction_combine(n_rows, f.nc, B, m->traction_mu.as<double>(), m->d_dof_vertex.as<int32_t>(),
+                                m->d_xyz.as<double>(), x64, s);
+        *launches += 1;
+        RVE_TRY(residual64(x64, r64));
+        RVE_TRY(rel_residual(r64, bn, rel));
+        return RVE_OK;
+    }
+
     // warm: optional starting data from the previous batch (see WarmStart).
     int run(int precision, SolveOut& out, const WarmStart* warm = nullptr) {
         NvtxRange nvtx_("cell solve, field %d, p = %d, %d columns, %s", fid, m->p, ncols,
@@ -942,8 +1364,14 @@ struct Solver {
                     for (int c = 0; c < ncols; ++c)
                         for (int ph = 0; ph < 2; ++ph) sc32[2 * c + ph] = (float)-warm->degrade[ph];
                     RVE_TRY(upload(m->dscale32, sc32.data(), sc32.size(), s));
-                    RVE_CUDA(cudaMemsetAsync(y32, 0, nv * 4, s));
-                    launch_operator<float>(m->p, f.nc, false, ev<float>(m->dscale32), v32, y32, nullptr, L);
+                    if (use_assembled(m, false)) {
+                        RVE_TRY(ensure_assembled(m, fid, false, s));
+                        launch_asm_product<float>(f.nc, asm_view<float>(m, fid, m->dscale32.as<float>()), v32, y32,
+                                                  ncols, nullptr, nullptr, s);
+                    } else {
+                        RVE_CUDA(cudaMemsetAsync(y32, 0, nv * 4, s));
+                        launch_operator<float>(m->p, f.nc, false, ev<float>(m->dscale32), v32, y32, nullptr, L);
+                    }
                     launch_axpy_f2d((int64_t)nv, y32, r64, s);      // r0 -= K_deg v
                     *launches += 3;
                     bool any_alpha = false;
@@ -976,6 +1404,14 @@ struct Solver {
             RVE_TRY(zero_noise_columns());
             last_rel.assign(ncols, 1.0);
             for (int c : zero_cols) last_rel[c] = 0.0;
+            // a constrained FP64 solve starts from the unconstrained traction problems
+            if (!mixed && f.m > 0 && m->bc == RVE_BC_NEUMANN && o.deterministic == 0 && !bounds_check_built() &&
+                (int)zero_cols.size() < ncols) {
+                int its = 0;
+                RVE_TRY(traction_start(x64, r64, o.rtol, o.max_iter, its, rel, bn));
+                out.iterations = its;
+                if (!zero_cols.empty()) RVE_TRY(zero_noise_columns());
+            }
         }
         out.rel_res = rel;
         if (!mixed) {
@@ -985,7 +1421,7 @@ struct Solver {
                 const std::vector<double> tolc = column_tolerances(o.rtol);
                 RVE_TRY(pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64,
                                     o.rtol / rel, o.max_iter, its, conv, &tolc));
-                out.iterations = its;
+                out.iterations += its;
                 RVE_TRY(residual64(x64, r64));
                 RVE_TRY(zero_noise_columns());
                 RVE_TRY(rel_residual(r64, bn, out.rel_res));
@@ -1281,7 +1717,13 @@ static int warm_galerkin(rve_mesh m, int B, const double* w_host, bool mixed, cu
     } else {
         // FP64 operator with the scales -K_part
         RVE_TRY(upload(m->warm_phs, nsc.data(), nsc.size(), s));
-        launch_operator<double>(m->p, f.nc, false, sk.ev<double>(m->warm_phs), xs64, kx, nullptr, sk.L);
+        if (use_assembled(m, true)) {
+            RVE_TRY(ensure_assembled(m, 0, true, s));
+            launch_asm_product<double>(f.nc, asm_view<double>(m, 0, m->warm_phs.as<double>()), xs64, kx, k2, nullptr,
+                                       nullptr, s);
+        } else {
+            launch_operator<double>(m->p, f.nc, false, sk.ev<double>(m->warm_phs), xs64, kx, nullptr, sk.L);
+        }
     }
     const int splits = 16, nout = 2 * ns + 2;
     RVE_TRY(m->warm_gram.ensure((size_t)splits * 6 * ns * nout * 8));

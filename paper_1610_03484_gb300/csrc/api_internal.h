@@ -205,6 +205,15 @@ struct rve_mesh_s {
     // invalidated whenever the DOF map or the materials change) and their index tables
     rve::DevBuf d_ke32, d_kepairs, d_keptab;
     bool ke_valid = false;
+    // assembled operator (p = 1, 2; assembled.h): sparsity of the current DOF map and the
+    // entries per field (0 mechanics, 1 scalar) and precision (0 FP64, 1 FP32), formed
+    // by the first solve that needs them
+    rve::DevBuf a_order, a_ptr, a_split, a_col, a_eptr, a_inc, a_rtab, a_ent[2][2];
+    int64_t a_entries = 0;
+    bool a_graph_valid = false, a_valid[2][2] = {{false, false}, {false, false}};
+    rve::DevBuf dinv64, dinv32;   // inverse Jacobi diagonal of the FP64 solve in progress
+    double a_lambda[2] = {0, 0};  // per field: bound of the spectrum of D^-1 A (0: not formed)
+    rve::DevBuf d_dof_vertex, traction_mu;   // uniform traction: original vertex of each node, multipliers
     // element colouring of the current DOF map (no two elements of a colour share a
     // DOF): elements sorted by colour on the device, colour offsets on the host
     rve::DevBuf d_colour_elems;

@@ -1187,9 +1187,13 @@ struct ColJacobi {
     const T* d0;
     const T* d1;
     const uint8_t* mask;
+    const T* dinv;
+    int groups;
     T s0, s1;
     __device__ __forceinline__ ColJacobi(const RowView<T>& rv, int col) {
         const int f = (rv.nfield == 2 && (col % 6) >= 3) ? 1 : 0;
+        dinv = rv.dinv ? rv.dinv + (rv.nfield == 2 ? f : col / 6) : nullptr;
+        groups = rv.dinv_groups;
         d0 = rv.diag + (int64_t)(2 * f) * rv.n_rows;
         d1 = d0 + rv.n_rows;
         mask = rv.mask;
@@ -1197,14 +1201,15 @@ struct ColJacobi {
         s1 = rv.scale[2 * col + 1];
     }
     __device__ __forceinline__ T inv(int64_t row) const {
+        if (sizeof(T) == 8 && dinv) return __ldg(dinv + row * groups);
         if (mask && mask[row / NC]) return T(0);
         return jacobi_inv<T>(s0, __ldg(d0 + row), s1, __ldg(d1 + row));
     }
 };
 
 // One block per column: alpha = (r, z) / (p, K p) with (p, K p) summed in parallel.
-__global__ void __launch_bounds__(256) k_finalize_alpha(const double* __restrict__ ep, int nby, int ncols,
-                                                        ColState cs) {
+__global__ void __launch_bounds__(256) k_finalize_alpha(const double* ep, int nby, int ncols,
+                                                        ColState cs, double* clear) {
     const int col = blockIdx.x;
     // a bounded wait in the operator gave up (flag bit 2): every column stops, so
     // the device-side loop ends at the next compaction
@@ -1216,7 +1221,10 @@ __global__ void __launch_bounds__(256) k_finalize_alpha(const double* __restrict
         return;
     }
     double v = 0.0;
-    for (int b = threadIdx.x; b < nby; b += blockDim.x) v += ep[(int64_t)b * ncols + col];
+    for (int b = threadIdx.x; b < nby; b += blockDim.x) {
+        v += ep[(int64_t)b * ncols + col];
+        if (clear) clear[(int64_t)b * ncols + col] = 0.0;
+    }
     const double pq = block_sum(v);
     if (threadIdx.x != 0) return;
     double a = cs.rz[col] / pq;
@@ -1230,11 +1238,12 @@ __global__ void __launch_bounds__(256) k_finalize_alpha(const double* __restrict
 }
 
 template <typename T>
-void launch_finalize_alpha(const double* energy_partial, ColState cs, const Launch& L) {
-    k_finalize_alpha<<<L.ncols, 256, 0, L.stream>>>(energy_partial, L.op_partials(), L.ncols, cs);
+void launch_finalize_alpha(const double* energy_partial, ColState cs, const Launch& L, double* clear) {
+    k_finalize_alpha<<<L.ncols, 256, 0, L.stream>>>(energy_partial, clear ? ACC_SLOTS : L.op_partials(), L.ncols, cs,
+                                                    clear);
 }
-template void launch_finalize_alpha<float>(const double*, ColState, const Launch&);
-template void launch_finalize_alpha<double>(const double*, ColState, const Launch&);
+template void launch_finalize_alpha<float>(const double*, ColState, const Launch&, double*);
+template void launch_finalize_alpha<double>(const double*, ColState, const Launch&, double*);
 
 // x += alpha p, r -= alpha q (when apply), partial (r, M^-1 r) per column and,
 // on constraint-support rows (HAS_C), the partial constraint products C M^-1 r
@@ -1296,7 +1305,8 @@ __global__ void __launch_bounds__(256) k_update(RowView<T> rv, T* __restrict__ x
     }
 }
 
-// p = M^-1 r + beta p ; q = 0.  FP32, no constraint rows, column count a
+// p = M^-1 r + beta p ; q = 0 (unless null: the assembled operator writes q instead of
+// adding into it).  FP32, no constraint rows, column count a
 // multiple of 4 per block: each thread handles four adjacent columns of a row
 // with 16-byte loads and stores, four times the bytes in flight per instruction
 // of the one-column form (this pass is bound by memory latency).  Thread
@@ -1347,7 +1357,7 @@ __global__ void __launch_bounds__(256) k_pupdate_v4(RowView<float> rv, const flo
             out[k] = act[k] ? (first ? z : fmaf(beta[k], pk[k], z)) : (first ? 0.f : pk[k]);
         }
         *reinterpret_cast<float4*>(p + idx) = make_float4(out[0], out[1], out[2], out[3]);
-        *reinterpret_cast<float4*>(q + idx) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q) *reinterpret_cast<float4*>(q + idx) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -1492,43 +1502,45 @@ template void launch_constraint_dot<double>(const RowView<double>&, const double
 
 // mu = S^-1 w, rz = (r, M^-1 r) - w . mu, beta, convergence.
 // first: 0 = iteration, 1 = initial residual, 2 = multipliers only (no state change).
-// One block per column: the partial sums are reduced in parallel, then thread 0
-// solves the m x m Schur system for mu and updates rz, beta and convergence.
+// One block per column: each warp sums the partials of one value at a time (the m
+// constraint products and (r, M^-1 r)), then m threads form mu = L^-T (L^-1 w) from
+// the stored inverse factor: no serial triangular solve (48 us a launch with one, 13 x
+// 11 x 6 cells, p = 2, 6 columns).
 __global__ void __launch_bounds__(256) k_finalize_beta(int m, const double* __restrict__ rzp,
                                                        const double* __restrict__ cp, int nby,
                                                        int ncols, ColState cs, int first) {
     const int col = blockIdx.x;
     if (first == 0 && !cs.active[col]) return;
-    double v = 0.0;
-    if (first != 2)
-        for (int b = threadIdx.x; b < nby; b += blockDim.x) v += rzp[(int64_t)b * ncols + col];
-    double rz = block_sum(v);
-    __shared__ double w[12];
-    for (int k = 0; k < m; ++k) {
+    __shared__ double w[13], y[12], mu_s[12];
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k <= m; k += blockDim.x >> 5) {
         double t = 0.0;
-        for (int b = threadIdx.x; b < nby; b += blockDim.x) t += cp[((int64_t)b * m + k) * ncols + col];
-        t = block_sum(t);
-        if (threadIdx.x == 0) w[k] = t;
+        if (k < m)
+            for (int b = lane; b < nby; b += 32) t += cp[((int64_t)b * m + k) * ncols + col];
+        else if (first != 2)
+            for (int b = lane; b < nby; b += 32) t += rzp[(int64_t)b * ncols + col];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) w[k] = t;
     }
-    if (threadIdx.x != 0) return;
-    double mu[12];
-    if (m > 0) {
-        const double* Lc = cs.schur + (int64_t)col * m * m;
-        for (int i2 = 0; i2 < m; ++i2) {   // forward
-            double t = w[i2];
-            for (int j2 = 0; j2 < i2; ++j2) t -= Lc[i2 * m + j2] * mu[j2];
-            mu[i2] = t / Lc[i2 * m + i2];
-        }
-        for (int i2 = m - 1; i2 >= 0; --i2) {   // backward
-            double t = mu[i2];
-            for (int j2 = i2 + 1; j2 < m; ++j2) t -= Lc[j2 * m + i2] * mu[j2];
-            mu[i2] = t / Lc[i2 * m + i2];
-        }
-        for (int k = 0; k < m; ++k) {
-            rz -= w[k] * mu[k];
-            cs.mu[(int64_t)k * ncols + col] = mu[k];
-        }
+    __syncthreads();
+    const int t = threadIdx.x;
+    const double* Li = cs.schur + (int64_t)col * m * m;   // L^-1
+    if (t < m) {
+        double v = 0.0;
+        for (int j = 0; j <= t; ++j) v += Li[t * m + j] * w[j];
+        y[t] = v;
     }
+    __syncthreads();
+    if (t < m) {
+        double v = 0.0;
+        for (int i = t; i < m; ++i) v += Li[i * m + t] * y[i];
+        mu_s[t] = v;
+        cs.mu[(int64_t)t * ncols + col] = v;
+    }
+    __syncthreads();
+    if (t != 0) return;
+    double rz = w[m];
+    for (int k = 0; k < m; ++k) rz -= w[k] * mu_s[k];
     if (first == 2) return;
     if (!isfinite(rz)) {
         atomicOr(cs.flags, 1);
@@ -1645,7 +1657,7 @@ __global__ void __launch_bounds__(256) k_pupdate(RowView<T> rv, T* __restrict__ 
     const int64_t stride = (int64_t)gridDim.y * rows;
     for (int64_t i = (int64_t)blockIdx.y * rows + rr; i < i_end; i += stride) {
         const int64_t idx = i * ncols + col;
-        q[idx] = T(0);
+        if (q) q[idx] = T(0);
         if (!act) {
             p[idx] = T(0);
             continue;
@@ -1696,7 +1708,8 @@ template void launch_pupdate<float>(const RowView<float>&, float*, float*, float
 template void launch_pupdate<double>(const RowView<double>&, double*, double*, double*, ColState,
                                      bool, const Launch&);
 
-// S = C M^-1 C^T per column (one block per (column, row k)), then Cholesky.
+// S = C M^-1 C^T per column (one block per (column, row k)), then the inverse of its
+// Cholesky factor.
 template <typename T>
 __global__ void k_schur_rows(RowView<T> rv, double* __restrict__ S, int ncols) {
     const int col = blockIdx.x, k = blockIdx.y, m = rv.m;
@@ -1739,6 +1752,15 @@ __global__ void k_cholesky(int m, int ncols, double* __restrict__ S, int32_t* fl
             A[i * m + j] = t / d;
         }
         for (int i = 0; i < j; ++i) A[i * m + j] = 0.0;
+    }
+    // L^-1 in place, column by column (row i of L is still whole right of column j)
+    for (int j = 0; j < m; ++j) {
+        A[j * m + j] = 1.0 / A[j * m + j];
+        for (int i = j + 1; i < m; ++i) {
+            double t = 0.0;
+            for (int k = j; k < i; ++k) t += A[i * m + k] * A[k * m + j];
+            A[i * m + j] = -t / A[i * m + i];
+        }
     }
 }
 

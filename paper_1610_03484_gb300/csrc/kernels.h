@@ -64,6 +64,10 @@ struct RowView {
     const T* diag = nullptr;          // [nfield][2 phases][n_rows], nfield = 1 (mech) or 2 (scalar)
     const uint8_t* mask = nullptr;    // [n_scalar_dofs] 1 = Dirichlet-constrained (or nullptr)
     const T* scale = nullptr;         // [ncols][2]
+    // optional inverse diagonal [n_rows][dinv_groups] (FP64 solves: a load instead of an
+    // FP64 division per entry), mechanics: one group per RVE, scalar: one per field
+    const T* dinv = nullptr;
+    int dinv_groups = 0;
     int nfield = 1;
     int nc = 3;
     // constraint rows (periodic / Neumann), FP64
@@ -81,7 +85,7 @@ struct ColState {
     double* alpha;
     double* beta;
     double* mu;       // [m][ncols] constraint multipliers of the current residual
-    double* schur;    // [ncols][m*m] Cholesky factor of C M^-1 C^T
+    double* schur;    // [ncols][m*m] inverse Cholesky factor of C M^-1 C^T
     int32_t* active;  // 1 while the column iterates
     int32_t* iters;   // iterations taken
     int32_t* flags;   // [1] bit0: numeric error
@@ -95,6 +99,7 @@ struct ColState {
     // loop-control kernel sums the slots and clears them
     double* pq_acc = nullptr;   // [ACC_SLOTS][ncols]
     double* rz_acc = nullptr;   // [ACC_SLOTS][ncols]
+    double* rj_acc = nullptr;   // [ACC_SLOTS][ncols] (r, D^-1 r) of the polynomial-preconditioned solve
 };
 constexpr int ACC_SLOTS = 8;
 
@@ -141,8 +146,10 @@ void launch_column_scales(int nrve, const double* w, int apply_to_yarn, bool mec
                           cudaStream_t s);
 
 // PCG pieces
+// clear: the partial rows are zeroed once read (the accumulator slots of the assembled
+// operator)
 template <typename T>
-void launch_finalize_alpha(const double* energy_partial, ColState cs, const Launch& L);
+void launch_finalize_alpha(const double* energy_partial, ColState cs, const Launch& L, double* clear = nullptr);
 // also accumulates the constraint products C M^-1 r into c_partial when given
 template <typename T>
 void launch_update(const RowView<T>& rv, T* x, T* r, const T* p, const T* q, ColState cs,
