@@ -60,122 +60,199 @@ struct rve_surrogate_s {
     double ref[3] = {1, 1, 1};
     // per member: FP32 master params, Adam moments, BF16 weights in both layouts
     std::vector<DevBuf> P, M1, M2, Wt, Wn;
-    DevBuf d_norm, d_diag;
-    // workspace
-    DevBuf X, H[NLAYER], Z[NLAYER], zout, dz, G, Gt, Ht, dH, gradT, gradb, loss, feat_dev, Tmem, spr;
+    DevBuf d_norm, d_diag;   // feature mean and inverse std [16]; diagonal entries
+    DevBuf train_work;       // training buffers of all members (TrainWork)
     // inference: the fused kernel (all members' layers per tile, activations on chip)
     // or one GEMM launch per member and layer
     bool fused = true;
-    DevBuf zall;
+    DevBuf H[NLAYER], zall;
 };
 
 namespace {
 
+// the feature normalisation on the device
+int upload_norm(rve_surrogate s) {
+    float h[16];
+    for (int k = 0; k < 8; ++k) {
+        h[k] = s->feat_mean[k];
+        h[8 + k] = 1.f / s->feat_std[k];
+    }
+    return upload(s->d_norm, h, 16, s->ctx->stream);
+}
+
+AdamJob adam_job(rve_surrogate s, int e, int l) {
+    const int64_t o = layer_w_off(l);
+    AdamJob j;
+    j.W = s->P[e].as<float>() + o;
+    j.m1 = s->M1[e].as<float>() + o;
+    j.m2 = s->M2[e].as<float>() + o;
+    j.Gt = nullptr;
+    j.gb = nullptr;
+    j.Wt = s->Wt[e].as<__nv_bfloat16>() + o;
+    j.Wn = s->Wn[e].as<__nv_bfloat16>() + o;
+    j.K = LK[l];
+    j.N = LN[l];
+    j.n_valid = LN[l];
+    return j;
+}
+
 int refresh_bf16(rve_surrogate s, int e) {
     // rebuild BF16 copies from the FP32 master parameters via a zero-lr Adam pass
-    cudaStream_t st = s->ctx->stream;
-    for (int l = 0; l < NLAYER; ++l) {
-        const int64_t o = layer_w_off(l);
-        float* W = s->P[e].as<float>() + o;
-        float* m1 = s->M1[e].as<float>() + o;
-        float* m2 = s->M2[e].as<float>() + o;
-        __nv_bfloat16* wt = s->Wt[e].as<__nv_bfloat16>() + o;
-        __nv_bfloat16* wn = s->Wn[e].as<__nv_bfloat16>() + o;
-        // gradient buffer of zeros of the right shape
-        RVE_TRY(s->gradT.ensure((size_t)LK[l] * LN[l] * 4));
-        RVE_CUDA(cudaMemsetAsync(s->gradT.p, 0, (size_t)LK[l] * LN[l] * 4, st));
-        launch_adam(LK[l], LN[l], W, s->gradT.as<float>(), m1, m2, 0.f, 1, wt, wn, LN[l], st);
+    AdamJobs J;
+    for (int l = 0; l < NLAYER; ++l) J.job[l] = adam_job(s, e, l);
+    launch_adam(J, NLAYER, 0.f, 1, s->ctx->stream);
+    return RVE_OK;
+}
+
+// Training buffers of nm members for batches of M rows, carved out of one allocation:
+// per member and layer the input H [M][K] and output gradient G [M][N] with their
+// transposes, the pre-activations Z, the gradients, and the network's output.
+struct TrainWork {
+    __nv_bfloat16 *H[MAX_MEMBERS][NLAYER], *Ht[MAX_MEMBERS][NLAYER], *G[MAX_MEMBERS][NLAYER], *Gt[MAX_MEMBERS][NLAYER];
+    float *Z[MAX_MEMBERS][NLAYER], *gradT[MAX_MEMBERS][NLAYER], *gradb[MAX_MEMBERS][NLAYER], *zout[MAX_MEMBERS];
+};
+
+int train_work(rve_surrogate s, int nm, int M, TrainWork& w) {
+    size_t off = 0;
+    char* base = nullptr;
+    auto take = [&](size_t bytes) {
+        char* q = base + off;
+        off += (bytes + 255) / 256 * 256;
+        return q;
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        off = 0;
+        for (int e = 0; e < nm; ++e) {
+            for (int l = 0; l < NLAYER; ++l) {
+                w.H[e][l] = reinterpret_cast<__nv_bfloat16*>(take((size_t)M * LK[l] * 2));
+                w.Ht[e][l] = reinterpret_cast<__nv_bfloat16*>(take((size_t)M * LK[l] * 2));
+                w.G[e][l] = reinterpret_cast<__nv_bfloat16*>(take((size_t)M * LN[l] * 2));
+                w.Gt[e][l] = reinterpret_cast<__nv_bfloat16*>(take((size_t)M * LN[l] * 2));
+                w.Z[e][l] = reinterpret_cast<float*>(take((size_t)M * LN[l] * 4));
+                w.gradT[e][l] = reinterpret_cast<float*>(take((size_t)LK[l] * LN[l] * 4));
+                w.gradb[e][l] = reinterpret_cast<float*>(take((size_t)LN[l] * 4));
+            }
+            w.zout[e] = reinterpret_cast<float*>(take((size_t)M * NOUTP * 4));
+        }
+        if (pass == 0) {
+            RVE_TRY(s->train_work.ensure(off));
+            base = s->train_work.as<char>();
+        }
     }
     return RVE_OK;
 }
 
-int alloc_work(rve_surrogate s, int M) {
-    RVE_TRY(s->X.ensure((size_t)M * KIN * 2));
-    for (int l = 0; l < NLAYER; ++l) {
-        RVE_TRY(s->H[l].ensure((size_t)M * LK[l] * 2));
-        RVE_TRY(s->Z[l].ensure((size_t)M * LN[l] * 4));
+// launches of one problem list, at most GEMM_GROUP each
+int gemm_all(std::vector<GemmProblem>& v, int N, int K, int epilogue, rve_ctx c) {
+    for (size_t i = 0; i < v.size(); i += GEMM_GROUP) {
+        RVE_CUDA(launch_gemm_group((int)std::min<size_t>(GEMM_GROUP, v.size() - i), &v[i], N, K, epilogue, c->stream));
+        c->launches++;
     }
-    RVE_TRY(s->zout.ensure((size_t)M * NOUTP * 4));
-    RVE_TRY(s->dz.ensure((size_t)M * HID * 2));
-    RVE_TRY(s->G.ensure((size_t)M * HID * 2));
-    RVE_TRY(s->Gt.ensure((size_t)M * HID * 2));
-    RVE_TRY(s->Ht.ensure((size_t)M * HID * 2));
-    RVE_TRY(s->dH.ensure((size_t)M * HID * 4));
-    RVE_TRY(s->gradT.ensure((size_t)HID * HID * 4));
-    RVE_TRY(s->gradb.ensure((size_t)HID * 4));
-    RVE_TRY(s->loss.ensure(64));
+    v.clear();
     return RVE_OK;
 }
 
-// forward pass of member e on M rows already in s->H[0] (BF16 [M][KIN]); z -> s->zout,
-// [M][NOUTP] (training) or transposed [NOUTP][M] (inference, transposed_out)
-int forward(rve_surrogate s, int e, int M, bool keep_pre, bool transposed_out = false) {
-    cudaStream_t st = s->ctx->stream;
+// One minibatch of M rows for the members first .. first + nm - 1 in lockstep, every
+// launch covering all of them (a member's GEMMs alone are 8 tiles on 152 SMs): row r of
+// member first + e is row rows[e][r] of the data (r without lists).  Leaves the gradients
+// in w and adds the loss of member first + e to loss[e].
+int forward_backward(rve_surrogate s, int first, int nm, int M, const TrainWork& w, const double* feat,
+                     const float* target, const float* sigma, const int32_t* const* rows, float* const* loss) {
+    rve_ctx c = s->ctx;
+    cudaStream_t st = c->stream;
+    FeatureArgs fa;
+    for (int e = 0; e < nm; ++e) {
+        fa.rows[e] = rows ? rows[e] : nullptr;
+        fa.X[e] = w.H[e][0];
+    }
+    const float* norm = s->d_norm.as<float>();
+    launch_features(nm, M, M, KIN, feat, fa, norm, norm + 8, st);
+    std::vector<GemmProblem> v;
     for (int l = 0; l < NLAYER; ++l) {
         const int64_t o = layer_w_off(l);
-        const __nv_bfloat16* wt = s->Wt[e].as<__nv_bfloat16>() + o;
-        const float* b = s->P[e].as<float>() + o + (int64_t)LK[l] * LN[l];
-        if (l < NLAYER - 1)
-            RVE_CUDA(launch_gemm_bf16(M, LN[l], LK[l], s->H[l].as<__nv_bfloat16>(), wt, b, 1,
-                                      s->H[l + 1].as<__nv_bfloat16>(), keep_pre ? s->Z[l].as<float>() : nullptr,
-                                      st));
-        else
-            RVE_CUDA(launch_gemm_bf16(M, LN[l], LK[l], s->H[l].as<__nv_bfloat16>(), wt, b, transposed_out ? 4 : 2,
-                                      nullptr, s->zout.as<float>(), st));
+        for (int e = 0; e < nm; ++e) {
+            GemmProblem p;
+            p.A = w.H[e][l];
+            p.Bt = s->Wt[first + e].as<__nv_bfloat16>() + o;
+            p.bias = s->P[first + e].as<float>() + o + (int64_t)LK[l] * LN[l];
+            p.M = M;
+            if (l < NLAYER - 1) {
+                p.Cb = w.H[e][l + 1];
+                p.Cf = w.Z[e][l];
+            } else {
+                p.Cf = w.zout[e];
+            }
+            v.push_back(p);
+        }
+        RVE_TRY(gemm_all(v, LN[l], LK[l], l < NLAYER - 1 ? 1 : 2, c));
     }
-    s->ctx->launches += NLAYER;
+    // (one launch per member: the loss is an FP32 sum in the order the blocks finish)
+    for (int e = 0; e < nm; ++e)
+        launch_head_loss(M, NOUTP, w.zout[e], rows ? rows[e] : nullptr, target, sigma, s->d_diag.as<uint8_t>(),
+                         w.G[e][NLAYER - 1], loss[e], st);
+    c->launches += 1 + nm;
+    // dH_l = G_l W_l^T, through the silu of layer l - 1
+    for (int l = NLAYER - 1; l > 0; --l) {
+        for (int e = 0; e < nm; ++e) {
+            GemmProblem p;
+            p.A = w.G[e][l];
+            p.Bt = s->Wn[first + e].as<__nv_bfloat16>() + layer_w_off(l);
+            p.pre = w.Z[e][l - 1];
+            p.Cb = w.G[e][l - 1];
+            p.M = M;
+            v.push_back(p);
+        }
+        RVE_TRY(gemm_all(v, LK[l], LN[l], 5, c));
+    }
+    // transposes and bias gradients, then dW^T [N][K] = G^T H
+    PrepJobs J;
+    int nj = 0;
+    auto flush = [&]() {
+        if (nj) {
+            launch_backward_prep(J, nj, HID, M, st);
+            c->launches++;
+        }
+        nj = 0;
+    };
+    for (int e = 0; e < nm; ++e)
+        for (int l = 0; l < NLAYER; ++l) {
+            if (nj + 3 > PREP_JOBS) flush();
+            J.job[nj++] = PrepJob{w.G[e][l], w.Gt[e][l], nullptr, M, LN[l]};
+            J.job[nj++] = PrepJob{w.H[e][l], w.Ht[e][l], nullptr, M, LK[l]};
+            J.job[nj++] = PrepJob{w.G[e][l], nullptr, w.gradb[e][l], M, LN[l]};
+        }
+    flush();
+    for (int wide = 0; wide < 2; ++wide) {   // layer 0 has 64 inputs, the others 256
+        for (int e = 0; e < nm; ++e)
+            for (int l = wide; l < (wide ? NLAYER : 1); ++l) {
+                GemmProblem p;
+                p.A = w.Gt[e][l];
+                p.Bt = w.Ht[e][l];
+                p.Cf = w.gradT[e][l];
+                p.M = LN[l];
+                v.push_back(p);
+            }
+        RVE_TRY(gemm_all(v, wide ? HID : KIN, M, 0, c));
+    }
     return RVE_OK;
 }
 
-// Backward pass of member e after forward(keep_pre) and the head loss (dz
-// holds d loss / d z).  With grads_host == nullptr the Adam update is applied;
-// otherwise every layer's gradient is copied to grads_host in the parameter
-// layout ([K][N] weights then [N] bias per layer) and the weights are kept.
-int backward_step(rve_surrogate s, int e, int M, int step, float lr, float* grads_host) {
-    cudaStream_t st = s->ctx->stream;
-    __nv_bfloat16* Gcur = s->dz.as<__nv_bfloat16>();
-    std::vector<float> gT, gb;
-    for (int l = NLAYER - 1; l >= 0; --l) {
-        const int K = LK[l], N = LN[l];
-        const int64_t o = layer_w_off(l);
-        // dW^T [N][K] = G^T H_l
-        launch_transpose_bf16(M, N, Gcur, s->Gt.as<__nv_bfloat16>(), st);
-        launch_transpose_bf16(M, K, s->H[l].as<__nv_bfloat16>(), s->Ht.as<__nv_bfloat16>(), st);
-        RVE_CUDA(launch_gemm_bf16(N, K, M, s->Gt.as<__nv_bfloat16>(), s->Ht.as<__nv_bfloat16>(), nullptr, 0,
-                                  nullptr, s->gradT.as<float>(), st));
-        launch_colsum_bf16(M, N, Gcur, s->gradb.as<float>(), st);
-        if (l > 0) {
-            // dH_l = G W_l^T, then through the silu of layer l-1
-            RVE_CUDA(launch_gemm_bf16(M, K, N, Gcur, s->Wn[e].as<__nv_bfloat16>() + o, nullptr, 0, nullptr,
-                                      s->dH.as<float>(), st));
-            launch_silu_backward((int64_t)M * K, s->dH.as<float>(), s->Z[l - 1].as<float>(),
-                                 s->G.as<__nv_bfloat16>(), st);
+void adam_step(rve_surrogate s, int nm, const TrainWork& w, float lr, int step) {
+    AdamJobs J;
+    int nj = 0;
+    for (int e = 0; e < nm; ++e)
+        for (int l = 0; l < NLAYER; ++l) {
+            AdamJob j = adam_job(s, e, l);
+            j.Gt = w.gradT[e][l];
+            j.gb = w.gradb[e][l];
+            if (l == NLAYER - 1) j.n_valid = NOUT;
+            J.job[nj++] = j;
+            if (nj == ADAM_JOBS || (e == nm - 1 && l == NLAYER - 1)) {
+                launch_adam(J, nj, lr, step, s->ctx->stream);
+                s->ctx->launches++;
+                nj = 0;
+            }
         }
-        const int nvalid = (l == NLAYER - 1) ? NOUT : N;
-        if (grads_host) {
-            gT.resize((size_t)N * K);
-            gb.resize(N);
-            RVE_CUDA(cudaMemcpyAsync(gT.data(), s->gradT.p, gT.size() * 4, cudaMemcpyDeviceToHost, st));
-            RVE_CUDA(cudaMemcpyAsync(gb.data(), s->gradb.p, gb.size() * 4, cudaMemcpyDeviceToHost, st));
-            RVE_CUDA(cudaStreamSynchronize(st));
-            for (int k = 0; k < K; ++k)
-                for (int n = 0; n < N; ++n) grads_host[o + (int64_t)k * N + n] = n < nvalid ? gT[(size_t)n * K + k] : 0.f;
-            for (int n = 0; n < N; ++n) grads_host[o + (int64_t)K * N + n] = n < nvalid ? gb[n] : 0.f;
-        } else {
-            launch_adam(K, N, s->P[e].as<float>() + o, s->gradT.as<float>(), s->M1[e].as<float>() + o,
-                        s->M2[e].as<float>() + o, lr, step, s->Wt[e].as<__nv_bfloat16>() + o,
-                        s->Wn[e].as<__nv_bfloat16>() + o, nvalid, st);
-            const int64_t ob = o + (int64_t)K * N;
-            launch_adam_bias(N, s->P[e].as<float>() + ob, s->gradb.as<float>(), s->M1[e].as<float>() + ob,
-                             s->M2[e].as<float>() + ob, lr, step, nvalid, st);
-        }
-        if (l > 0) {
-            RVE_CUDA(cudaMemcpyAsync(s->dz.p, s->G.p, (size_t)M * K * 2, cudaMemcpyDeviceToDevice, st));
-            Gcur = s->dz.as<__nv_bfloat16>();
-        }
-        s->ctx->launches += 7;
-    }
-    return RVE_OK;
 }
 
 }  // namespace
@@ -326,56 +403,57 @@ int rve_surrogate_train(rve_ctx c, rve_surrogate s, int64_t n, const double* fea
     // scale for every entry makes the loss the squared error relative to the
     // tensor's own size (what the accuracy target is stated in).
     for (int o = 0; o < NOUT; ++o) s->sigma[o] = 1.f;
-    // ---- device data: normalised features (BF16 rows) and targets
-    const int M = batch;
-    RVE_TRY(alloc_work(s, M));
-    DevBuf dfeat, dtgt, dsig, dmean, dstd, bfeat, btgt, didx;
-    std::vector<float> fm(s->feat_mean, s->feat_mean + 8), fis(8);
-    for (int k = 0; k < 8; ++k) fis[k] = 1.f / s->feat_std[k];
+    // ---- device data: features and targets once, the row order of every epoch
+    const int M = batch, nm = s->members;
+    TrainWork w;
+    RVE_TRY(train_work(s, nm, M, w));
+    DevBuf dfeat, dtgt, dsig, dperm, dloss;
+    RVE_TRY(upload_norm(s));
     RVE_TRY(upload(dfeat, feat, (size_t)n * 8, st));
     RVE_TRY(upload(dtgt, tgt.data(), tgt.size(), st));
     RVE_TRY(upload(dsig, s->sigma, NOUT, st));
-    RVE_TRY(upload(dmean, fm.data(), 8, st));
-    RVE_TRY(upload(dstd, fis.data(), 8, st));
-    RVE_TRY(bfeat.ensure((size_t)M * 8 * 8));
-    RVE_TRY(btgt.ensure((size_t)M * NOUT * 4));
-    std::vector<double> hb((size_t)M * 8);
-    std::vector<float> ht((size_t)M * NOUT);
+    RVE_TRY(dperm.ensure((size_t)nm * n * 4));
+    RVE_TRY(dloss.ensure((size_t)epochs * nm * 4));
+    RVE_CUDA(cudaMemsetAsync(dloss.p, 0, (size_t)epochs * nm * 4, st));
     const int64_t steps_per_epoch = n / M;
-    std::vector<double> hist(epochs, 0.0);
-    for (int e = 0; e < s->members; ++e) {
-        std::mt19937_64 rng(seed * 7919ull + (uint64_t)e);
-        std::vector<int64_t> perm(n);
-        std::iota(perm.begin(), perm.end(), 0);
-        int step = 0;
-        for (int ep = 0; ep < epochs; ++ep) {
-            std::shuffle(perm.begin(), perm.end(), rng);
-            RVE_CUDA(cudaMemsetAsync(s->loss.p, 0, 4, st));
-            for (int64_t b = 0; b < steps_per_epoch; ++b) {
-                for (int r = 0; r < M; ++r) {
-                    const int64_t i = perm[b * M + r];
-                    std::memcpy(&hb[(size_t)r * 8], feat + 8 * i, 64);
-                    std::memcpy(&ht[(size_t)r * NOUT], &tgt[(size_t)i * NOUT], NOUT * 4);
-                }
-                RVE_CUDA(cudaMemcpyAsync(bfeat.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
-                RVE_CUDA(cudaMemcpyAsync(btgt.p, ht.data(), ht.size() * 4, cudaMemcpyHostToDevice, st));
-                launch_features(M, M, KIN, bfeat.as<double>(), dmean.as<float>(), dstd.as<float>(),
-                                s->H[0].as<__nv_bfloat16>(), st);
-                RVE_TRY(forward(s, e, M, true));
-                launch_head_loss(M, M, NOUTP, s->zout.as<float>(), btgt.as<float>(), dsig.as<float>(),
-                                 s->d_diag.as<uint8_t>(), s->dz.as<__nv_bfloat16>(), s->loss.as<float>(), st);
-                ++step;
-                // cosine decay of the learning rate over all steps of this member
-                const double total = (double)epochs * steps_per_epoch;
-                const double lr_t = lr * (0.02 + 0.98 * 0.5 * (1.0 + std::cos(M_PI * (step - 1) / total)));
-                RVE_TRY(backward_step(s, e, M, step, (float)lr_t, nullptr));
+    std::vector<std::mt19937_64> rng;
+    std::vector<std::vector<int64_t>> perm(nm);
+    std::vector<int32_t> order((size_t)nm * n);
+    for (int e = 0; e < nm; ++e) {
+        rng.emplace_back(seed * 7919ull + (uint64_t)e);
+        perm[e].resize(n);
+        std::iota(perm[e].begin(), perm[e].end(), 0);
+    }
+    int step = 0;
+    for (int ep = 0; ep < epochs; ++ep) {
+        for (int e = 0; e < nm; ++e) {
+            std::shuffle(perm[e].begin(), perm[e].end(), rng[e]);
+            for (int64_t i = 0; i < n; ++i) order[(size_t)e * n + i] = (int32_t)perm[e][i];
+        }
+        // (a copy from pageable memory has left the vector when the call returns)
+        RVE_CUDA(cudaMemcpyAsync(dperm.p, order.data(), order.size() * 4, cudaMemcpyHostToDevice, st));
+        for (int64_t b = 0; b < steps_per_epoch; ++b) {
+            const int32_t* rows[MAX_MEMBERS];
+            float* loss[MAX_MEMBERS];
+            for (int e = 0; e < nm; ++e) {
+                rows[e] = dperm.as<int32_t>() + (size_t)e * n + b * M;
+                loss[e] = dloss.as<float>() + (size_t)ep * nm + e;
             }
-            float lsum = 0;
-            RVE_CUDA(cudaMemcpyAsync(&lsum, s->loss.p, 4, cudaMemcpyDeviceToHost, st));
-            RVE_CUDA(cudaStreamSynchronize(st));
-            hist[ep] += lsum / steps_per_epoch / s->members;
+            RVE_TRY(forward_backward(s, 0, nm, M, w, dfeat.as<double>(), dtgt.as<float>(), dsig.as<float>(), rows,
+                                     loss));
+            ++step;
+            // cosine decay of the learning rate over all steps
+            const double total = (double)epochs * steps_per_epoch;
+            const double lr_t = lr * (0.02 + 0.98 * 0.5 * (1.0 + std::cos(M_PI * (step - 1) / total)));
+            adam_step(s, nm, w, (float)lr_t, step);
         }
     }
+    std::vector<float> lsum((size_t)epochs * nm);
+    RVE_CUDA(cudaMemcpyAsync(lsum.data(), dloss.p, lsum.size() * 4, cudaMemcpyDeviceToHost, st));
+    RVE_CUDA(cudaStreamSynchronize(st));
+    std::vector<double> hist(epochs, 0.0);
+    for (int e = 0; e < nm; ++e)
+        for (int ep = 0; ep < epochs; ++ep) hist[ep] += lsum[(size_t)ep * nm + e] / steps_per_epoch / nm;
     RVE_CUDA(cudaGetLastError());
     if (loss_history) std::memcpy(loss_history, hist.data(), sizeof(double) * epochs);
     s->trained = true;
@@ -394,23 +472,32 @@ int rve_surrogate_gradients(rve_ctx c, rve_surrogate s, int member, int n, const
         return RVE_ERR_INVALID_ARGUMENT;
     }
     cudaStream_t st = c->stream;
-    RVE_TRY(alloc_work(s, n));
-    DevBuf df, dt, dsig, dmean, dstd;
-    std::vector<float> fis(8);
-    for (int k = 0; k < 8; ++k) fis[k] = 1.f / s->feat_std[k];
+    TrainWork w;
+    RVE_TRY(train_work(s, 1, n, w));
+    DevBuf df, dt, dsig, dloss;
+    RVE_TRY(upload_norm(s));
     RVE_TRY(upload(df, feat, (size_t)n * 8, st));
     RVE_TRY(upload(dt, target_factors, (size_t)n * NOUT, st));
     RVE_TRY(upload(dsig, s->sigma, NOUT, st));
-    RVE_TRY(upload(dmean, s->feat_mean, 8, st));
-    RVE_TRY(upload(dstd, fis.data(), 8, st));
-    RVE_CUDA(cudaMemsetAsync(s->loss.p, 0, 4, st));
-    launch_features(n, n, KIN, df.as<double>(), dmean.as<float>(), dstd.as<float>(), s->H[0].as<__nv_bfloat16>(), st);
-    RVE_TRY(forward(s, member, n, true));
-    launch_head_loss(n, n, NOUTP, s->zout.as<float>(), dt.as<float>(), dsig.as<float>(), s->d_diag.as<uint8_t>(),
-                     s->dz.as<__nv_bfloat16>(), s->loss.as<float>(), st);
-    RVE_TRY(backward_step(s, member, n, 1, 0.f, grads));
+    RVE_TRY(dloss.ensure(4));
+    RVE_CUDA(cudaMemsetAsync(dloss.p, 0, 4, st));
+    float* dl[1] = {dloss.as<float>()};
+    RVE_TRY(forward_backward(s, member, 1, n, w, df.as<double>(), dt.as<float>(), dsig.as<float>(), nullptr, dl));
+    std::vector<float> gT, gb;
+    for (int q = 0; q < NLAYER; ++q) {
+        const int K = LK[q], N = LN[q], nvalid = q == NLAYER - 1 ? NOUT : N;
+        const int64_t o = layer_w_off(q);
+        gT.resize((size_t)N * K);
+        gb.resize(N);
+        RVE_CUDA(cudaMemcpyAsync(gT.data(), w.gradT[0][q], gT.size() * 4, cudaMemcpyDeviceToHost, st));
+        RVE_CUDA(cudaMemcpyAsync(gb.data(), w.gradb[0][q], gb.size() * 4, cudaMemcpyDeviceToHost, st));
+        RVE_CUDA(cudaStreamSynchronize(st));
+        for (int k = 0; k < K; ++k)
+            for (int j = 0; j < N; ++j) grads[o + (int64_t)k * N + j] = j < nvalid ? gT[(size_t)j * K + k] : 0.f;
+        for (int j = 0; j < N; ++j) grads[o + (int64_t)K * N + j] = j < nvalid ? gb[j] : 0.f;
+    }
     float l = 0;
-    RVE_CUDA(cudaMemcpyAsync(&l, s->loss.p, 4, cudaMemcpyDeviceToHost, st));
+    RVE_CUDA(cudaMemcpyAsync(&l, dloss.p, 4, cudaMemcpyDeviceToHost, st));
     RVE_CUDA(cudaStreamSynchronize(st));
     if (loss) *loss = l;
     if (gemm_tc_timed_out()) {
@@ -425,48 +512,45 @@ static int predict_dev(rve_surrogate s, int64_t n, const double* feat_dev, doubl
                        double* D_dev, double* spread_dev) {
     NvtxRange nvtx_("surrogate inference: %lld points, %d members", (long long)n, s->members);
     cudaStream_t st = s->ctx->stream;
-    const int64_t chunk = 65536;
-    RVE_TRY(alloc_work(s, (int)chunk));
-    RVE_TRY(s->Tmem.ensure((size_t)s->members * chunk * 54 * 4));
+    const int64_t chunk = 65536, rows = std::min<int64_t>(chunk, (n + 63) / 64 * 64);
     const bool use_fused = s->fused && s->members <= mlp_fused_max_members();
+    for (int l = 0; l < (use_fused ? 1 : NLAYER); ++l) RVE_TRY(s->H[l].ensure((size_t)rows * LK[l] * 2));
+    RVE_TRY(s->zall.ensure((size_t)s->members * 64 * rows * 4));
     std::vector<const __nv_bfloat16*> wt;
     std::vector<const float*> bias;
     int64_t w_off[NLAYER];
-    if (use_fused) {
-        RVE_TRY(s->zall.ensure((size_t)s->members * 64 * chunk * 4));
-        for (int l = 0; l < NLAYER; ++l) w_off[l] = layer_w_off(l);
-        for (int e = 0; e < s->members; ++e) {
-            wt.push_back(s->Wt[e].as<__nv_bfloat16>());
-            for (int l = 0; l < NLAYER; ++l)
-                bias.push_back(s->P[e].as<float>() + layer_w_off(l) + (int64_t)LK[l] * LN[l]);
-        }
+    for (int l = 0; l < NLAYER; ++l) w_off[l] = layer_w_off(l);
+    for (int e = 0; e < s->members; ++e) {
+        wt.push_back(s->Wt[e].as<__nv_bfloat16>());
+        for (int l = 0; l < NLAYER; ++l) bias.push_back(s->P[e].as<float>() + w_off[l] + (int64_t)LK[l] * LN[l]);
     }
-    DevBuf dmean, dstd;
-    std::vector<float> fis(8);
-    for (int k = 0; k < 8; ++k) fis[k] = 1.f / s->feat_std[k];
-    RVE_TRY(upload(dmean, s->feat_mean, 8, st));
-    RVE_TRY(upload(dstd, fis.data(), 8, st));
+    RVE_TRY(upload_norm(s));
+    const float* norm = s->d_norm.as<float>();
+    FeatureArgs fa;
+    fa.rows[0] = nullptr;
+    fa.X[0] = s->H[0].as<__nv_bfloat16>();
     for (int64_t off = 0; off < n; off += chunk) {
         const int nn = (int)std::min<int64_t>(chunk, n - off);
         const int M = ((nn + 63) / 64) * 64;
-        launch_features(nn, M, KIN, feat_dev + off * 8, dmean.as<float>(), dstd.as<float>(),
-                        s->H[0].as<__nv_bfloat16>(), st);
+        launch_features(1, nn, M, KIN, feat_dev + off * 8, fa, norm, norm + 8, st);
         if (use_fused) {
             RVE_CUDA(launch_mlp_fused(M, s->members, s->H[0].as<__nv_bfloat16>(), wt.data(), w_off,
                                       bias.data(), s->zall.as<float>(), M, st));
             s->ctx->launches += 1;
+        } else {
+            for (int e = 0; e < s->members; ++e)
+                for (int l = 0; l < NLAYER; ++l) {
+                    const bool last = l == NLAYER - 1;
+                    RVE_CUDA(launch_gemm_bf16(M, LN[l], LK[l], s->H[l].as<__nv_bfloat16>(), wt[e] + w_off[l],
+                                              bias[e * NLAYER + l], last ? 4 : 1,
+                                              last ? nullptr : s->H[l + 1].as<__nv_bfloat16>(),
+                                              last ? s->zall.as<float>() + (size_t)e * 64 * M : nullptr, st));
+                    s->ctx->launches += 1;
+                }
         }
-        for (int e = 0; e < s->members; ++e) {
-            const float* zT = s->zout.as<float>();
-            if (use_fused)
-                zT = s->zall.as<float>() + (size_t)e * 64 * M;
-            else
-                RVE_TRY(forward(s, e, M, false, true));
-            launch_head_tensors(nn, M, zT, s->d_diag.as<uint8_t>(), s->Tmem.as<float>() + (size_t)e * nn * 54, st);
-        }
-        launch_ensemble(nn, s->members, s->Tmem.as<float>(), s->ref[0], s->ref[1], s->ref[2], C_dev + off * 36,
-                        K_dev + off * 9, D_dev + off * 9, spread_dev + off, st);
-        s->ctx->launches += 2 + s->members;
+        launch_ensemble(nn, M, s->members, s->zall.as<float>(), (int64_t)64 * M, s->d_diag.as<uint8_t>(), s->ref[0],
+                        s->ref[1], s->ref[2], C_dev + off * 36, K_dev + off * 9, D_dev + off * 9, spread_dev + off, st);
+        s->ctx->launches += 2;
     }
     RVE_CUDA(cudaGetLastError());
     return RVE_OK;
