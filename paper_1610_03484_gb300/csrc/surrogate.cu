@@ -838,8 +838,12 @@ __global__ void __launch_bounds__(256) k_adam(const __grid_constant__ AdamJobs J
         const int k = weight ? (int)(i / N) : 0, c = weight ? (int)(i % N) : (int)(i - nw);
         float g = weight ? (j.Gt ? j.Gt[(int64_t)c * K + k] : 0.f) : j.gb[c];
         if (c >= j.n_valid) g = 0.f;
-        const float a = b1 * j.m1[i] + (1.f - b1) * g;
-        const float v = b2 * j.m2[i] + (1.f - b2) * g * g;
+        // the product that is rounded before the fused add is fixed: weights the gradient's,
+        // biases the moment's (a free choice of the compiler would differ between builds, and
+        // Adam carries a last-bit difference of a moment into the whole trajectory)
+        const float m = j.m1[i], q = j.m2[i], gm = 1.f - b1, gq = __fmul_rn(1.f - b2, g);
+        const float a = weight ? __fmaf_rn(b1, m, __fmul_rn(gm, g)) : __fmaf_rn(gm, g, __fmul_rn(b1, m));
+        const float v = weight ? __fmaf_rn(b2, q, __fmul_rn(gq, g)) : __fmaf_rn(gq, g, __fmul_rn(b2, q));
         j.m1[i] = a;
         j.m2[i] = v;
         float w = j.W[i];
