@@ -455,13 +455,15 @@ void launch_assemble(int p, int nc, const AsmGraph& g, const int32_t* edofs, con
 }
 
 // Columns per thread and lanes per row.  Four columns per thread need 16-byte aligned
-// rows.  Otherwise the entries of a row are split over four lanes, or eight where even
-// then the chip has less than four warps per scheduler.
+// rows and eight warps per SM: with fewer, each thread's serial walk along its row bounds
+// the product (6x7x8, p = 1, 108 columns: a call of 18 points 2.68 -> 2.27 ms, the
+// element form 2.31).  Otherwise the entries of a row are split over four lanes, or eight where
+// even then the chip has less than four warps per scheduler.
 #define RVE_ASM_RUN(MODE, ...)                                                              \
     do {                                                                                    \
         const bool few = A.n * ncols / 2 < (int64_t)sm_count() * 4 * 32;                    \
         if constexpr (sizeof(T) == 4) {                                                     \
-            if (ncols % 4 == 0 && ncols >= 24) {                                            \
+            if (ncols % 4 == 0 && ncols >= 24 && A.n * ncols / 4 >= (int64_t)sm_count() * 256) { \
                 if (nc == 3) return run_product<T, 3, 4, 1, MODE>(__VA_ARGS__);             \
                 return run_product<T, 1, 4, 1, MODE>(__VA_ARGS__);                          \
             }                                                                               \
