@@ -387,9 +387,13 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
 // cost more than recomputing from the element data (24x24x8, 6 columns: 37 us against
 // 16; 32x32x10, 48 columns: 273 against 127).  Not in the deterministic mode (whose sums
 // run colour by colour) and not in a checking build (which checks the element kernels'
-// indices).
+// indices).  Nor where a matrix could pass 2^29 entries (at most ne^2 per tetrahedron; 43 GB
+// in FP64): its indices stay in 32 bits, and a mesh that large needs its memory for the
+// solve vectors, as with the element operators.
 bool use_assembled(rve_mesh m, bool fp64) {
-    return m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built();
+    const int64_t ne = n_local(m->p);
+    return m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built() &&
+           m->nt * ne * ne <= (int64_t)1 << 29;
 }
 
 // Entries of one field (0 mechanics, 1 scalar), formed on first use after a change of the
