@@ -88,7 +88,10 @@ typedef struct rve_options {
                                 the energy-optimal (Galerkin) combination of up to three of them
                                 for the mechanics without constraint rows (one operator pass over
                                 the sources and a few inner products per batch; otherwise the
-                                parabola, and the transport fields take the nearest);
+                                parabola, and the transport fields take the nearest); mixed
+                                calls with many points on a mesh solve six of them on top,
+                                spread over the call's range of the factor, and start all
+                                points from their energy-optimal combination;
                                 0 starts every batch from zero */
     int     transport_once;  /* macro_update_gauss_points: 1 solves the thermal and moisture cell
                                 problems once per mesh and call and gives all the mesh's points

@@ -513,6 +513,7 @@ struct Solver {
     int64_t n_rows;
     int fid;   // 0 mechanics, 1 scalar fields
     bool free_rows = false;   // leave the constraint rows out (traction_start)
+    double tighten = 1.0;     // factor on the tolerance of a mixed solve (sources of build_basis)
     Launch L;
     cudaStream_t s;
     ColState cs64{};
@@ -1345,6 +1346,7 @@ struct Solver {
         out.sweeps = 0;
         out.converged = false;
         double rel = 1.0;
+        bool r_true = false;   // r64 is the true residual of x64 already (mixed)
         if (warm) {
             launch_combine_columns<double, double>(n_rows, ncols, warm->cols, warm->map, warm->coef, warm->x, x64, s);
             *launches += 1;
@@ -1399,6 +1401,7 @@ struct Solver {
                 }
             } else {
                 RVE_TRY(mixed ? residual_df(x64, r64) : residual64(x64, r64));
+                r_true = mixed;
             }
             RVE_TRY(zero_noise_columns());
             RVE_TRY(rel_residual(r64, bn, rel));
@@ -1437,14 +1440,15 @@ struct Solver {
             float* x32 = m->x32.as<float>();
             float* r32 = m->r32.as<float>();
             int total = 0;
+            const double rtol = o.rtol * tighten;
             // Every sweep ends with the FP64 true residual, which alone decides
             // convergence and feeds the tensor reduction; a sweep whose starting
             // residual is already below rtol skips the FP32 inner solve.
             for (int sw = 0; sw < std::max(1, o.max_refine); ++sw) {
-                if (out.rel_res > o.rtol) {
+                if (out.rel_res > rtol) {
                     // reduce the residual only as far as the outer tolerance needs
                     // (half again for margin), never below what FP32 can resolve
-                    const double inner = std::max(o.inner_rtol, 0.5 * o.rtol / out.rel_res);
+                    const double inner = std::max(o.inner_rtol, 0.5 * rtol / out.rel_res);
                     launch_cast_d2f((int64_t)nv, r64, r32, s);
                     RVE_CUDA(cudaMemsetAsync(x32, 0, nv * 4, s));
                     *launches += 1;
@@ -1455,13 +1459,17 @@ struct Solver {
                     total += its;
                     launch_axpy_f2d((int64_t)nv, x32, x64, s);
                     *launches += 1;
+                } else if (r_true) {
+                    out.sweeps = 1;
+                    out.converged = true;
+                    break;
                 }
                 RVE_TRY(residual_df(x64, r64));
                 RVE_TRY(zero_noise_columns());
                 RVE_TRY(rel_residual(r64, bn, out.rel_res));
                 out.sweeps = sw + 1;
                 out.converged = out.rel_res <= o.rtol;
-                if (out.converged) break;
+                if (out.rel_res <= rtol) break;
             }
             out.iterations = total;
         }
@@ -1571,19 +1579,11 @@ static int warm_sources(const std::vector<double>& pw, double w, int order, int*
     return nn;
 }
 
-// c = G^+ g for a small symmetric positive semi-definite G (n <= WARM_SOURCES):
-// cyclic Jacobi rotations, eigenvalues at or below `rel` of the largest dropped (the
-// sources are nearly parallel, so G is close to singular, and its entries carry the
-// rounding of the double-float operator products).  False if G has no positive
-// eigenvalue or a value is not finite.
-static bool galerkin_solve(int n, const double* Gin, const double* g, double* c, double rel) {
-    double A[WARM_SOURCES][WARM_SOURCES], V[WARM_SOURCES][WARM_SOURCES];
+// Eigenvalues (diagonal of A) and eigenvectors (columns of V) of a small symmetric A by
+// cyclic Jacobi rotations.
+static void jacobi_eigen(int n, double (&A)[WARM_SOURCES][WARM_SOURCES], double (&V)[WARM_SOURCES][WARM_SOURCES]) {
     for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) {
-            A[i][j] = 0.5 * (Gin[i * n + j] + Gin[j * n + i]);
-            V[i][j] = i == j ? 1.0 : 0.0;
-            if (!std::isfinite(A[i][j])) return false;
-        }
+        for (int j = 0; j < n; ++j) V[i][j] = i == j ? 1.0 : 0.0;
     for (int sweep = 0; sweep < 60; ++sweep) {
         double off = 0.0, diag = 0.0;
         for (int i = 0; i < n; ++i) {
@@ -1614,6 +1614,20 @@ static bool galerkin_solve(int n, const double* Gin, const double* g, double* c,
                 }
             }
     }
+}
+
+// c = G^+ g for a small symmetric positive semi-definite G (n <= WARM_SOURCES):
+// eigenvalues at or below `rel` of the largest dropped (the sources are nearly parallel,
+// so G is close to singular, and its entries carry the rounding of the double-float
+// operator products).  False if G has no positive eigenvalue or a value is not finite.
+static bool galerkin_solve(int n, const double* Gin, const double* g, double* c, double rel) {
+    double A[WARM_SOURCES][WARM_SOURCES], V[WARM_SOURCES][WARM_SOURCES];
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) {
+            A[i][j] = 0.5 * (Gin[i * n + j] + Gin[j * n + i]);
+            if (!std::isfinite(A[i][j])) return false;
+        }
+    jacobi_eigen(n, A, V);
     double lmax = 0.0;
     for (int i = 0; i < n; ++i) lmax = std::max(lmax, A[i][i]);
     if (!(lmax > 0.0) || !std::isfinite(lmax)) return false;
@@ -1644,35 +1658,23 @@ int rve_debug_galerkin_solve(int n, const double* G, const double* g, double rel
     return RVE_OK;
 }
 
-// Energy-optimal warm start of the mechanics (warm_start >= 4).  With A(w) = K_o + w
-// K_d (K_d: the degraded phases at unit modulus, K_o the others) and b(w) =
-// -A(w) u_macro, the start for a column at w is x0 = sum_k c_k x_k over ns previous
-// solutions of the same load case with G c = g, G_pk = x_p . A(w) x_k, g_p =
-// x_p . b(w): the Galerkin projection onto their span (the energy minimisation of
-// Sec. 2 restricted to it).  K_d x_k and K_o x_k come from one pass of the operator
-// that defines the solve (double-float in mixed mode), so G is exact to rounding and
-// its nearly singular directions (the extrapolation in w) survive; its residual
-// r0 = b(w) - sum_k c_k (K_o + w K_d) x_k needs no further operator pass.
-static int warm_galerkin(rve_mesh m, int B, const double* w_host, bool mixed, cudaStream_t s, WarmStart& ws,
-                         bool& used) {
-    used = false;
+// ns sources of the previous batch and the inner products of their span: P[lc][p][...] =
+// x_p . (-K_d x_t) (t < ns), x_p . (-K_o x_t) (ns + t), x_p . K_ph u_macro (2 ns + ph).  The
+// products -K_d x_t and -K_o x_t stay in m->warm_kx (columns 6 t + lc and 6 ns + 6 t + lc).
+static int warm_products(rve_mesh m, int ns, const double* degrade, bool mixed, cudaStream_t s,
+                         std::vector<int32_t>& src, std::vector<double>& P) {
     const std::vector<double>& pw = m->warm_w[0];
     const int Bp = m->warm_cols[0] / 6;
     FieldDev& f = m->mech;
-    if (Bp < 1 || (int)pw.size() != Bp || !m->bph_valid[0] || B < 1 || f.m != 0) return RVE_OK;
     const int64_t n_rows = f.n_rows;
-    const double deg[2] = {ws.degrade[0], ws.degrade[1]};
-    auto sph = [&](double w, int ph) { return deg[ph] != 0.0 ? w : 1.0; };
-    // the operator of a mixed solve scales the phases by the FP32 column scales (the
-    // right-hand side by the FP64 ones)
-    auto wop = [&](double w) { return mixed ? (double)(float)w : w; };
+    const double deg[2] = {degrade[0], degrade[1]};
     // sources: ns previous RVEs spread evenly over the previous batch's range of the
     // factor (its ends included), so that their span holds the line through the ends
     std::vector<int> ord(Bp);
     for (int q = 0; q < Bp; ++q) ord[q] = q;
     std::sort(ord.begin(), ord.end(), [&](int a, int b) { return pw[a] < pw[b]; });
-    const int ns = std::min(WARM_GALERKIN, Bp), kc = 6 * ns, k2 = 2 * kc;
-    std::vector<int32_t> src(ns);
+    const int kc = 6 * ns, k2 = 2 * kc;
+    src.resize(ns);
     for (int k = 0; k < ns; ++k) src[k] = ord[ns > 1 ? (int)std::lround((double)k * (Bp - 1) / (ns - 1)) : 0];
     // compact copy: columns h kc + 6 t + lc hold source t, load case lc, for h = 0 (the
     // degraded phases' product) and h = 1 (the other phases')
@@ -1734,11 +1736,40 @@ static int warm_galerkin(rve_mesh m, int B, const double* w_host, bool mixed, cu
     launch_warm_gram(n_rows, ns, m->warm_src.as<int32_t>(), m->warm_cols[0], m->warm[0].as<double>(), kx,
                      m->bph[0].as<double>(), m->warm_gram.as<double>(), splits, s);
     m->ctx->launches += 7;
-    std::vector<double> h((size_t)splits * 6 * ns * nout), P((size_t)6 * ns * nout, 0.0);
+    std::vector<double> h((size_t)splits * 6 * ns * nout);
+    P.assign((size_t)6 * ns * nout, 0.0);
     RVE_CUDA(cudaMemcpyAsync(h.data(), m->warm_gram.p, h.size() * 8, cudaMemcpyDeviceToHost, s));
     RVE_CUDA(cudaStreamSynchronize(s));
     for (int sp = 0; sp < splits; ++sp)
         for (size_t i = 0; i < P.size(); ++i) P[i] += h[(size_t)sp * P.size() + i];
+    return RVE_OK;
+}
+
+// Energy-optimal warm start of the mechanics (warm_start >= 4).  With A(w) = K_o + w
+// K_d (K_d: the degraded phases at unit modulus, K_o the others) and b(w) =
+// -A(w) u_macro, the start for a column at w is x0 = sum_k c_k x_k over ns previous
+// solutions of the same load case with G c = g, G_pk = x_p . A(w) x_k, g_p =
+// x_p . b(w): the Galerkin projection onto their span (the energy minimisation of
+// Sec. 2 restricted to it).  K_d x_k and K_o x_k come from one pass of the operator
+// that defines the solve (double-float in mixed mode), so G is exact to rounding and
+// its nearly singular directions (the extrapolation in w) survive; its residual
+// r0 = b(w) - sum_k c_k (K_o + w K_d) x_k needs no further operator pass.
+static int warm_galerkin(rve_mesh m, int B, const double* w_host, bool mixed, cudaStream_t s, WarmStart& ws,
+                         bool& used) {
+    used = false;
+    const std::vector<double>& pw = m->warm_w[0];
+    const int Bp = m->warm_cols[0] / 6;
+    FieldDev& f = m->mech;
+    if (Bp < 1 || (int)pw.size() != Bp || !m->bph_valid[0] || B < 1 || f.m != 0) return RVE_OK;
+    auto sph = [&](double w, int ph) { return ws.degrade[ph] != 0.0 ? w : 1.0; };
+    // the operator of a mixed solve scales the phases by the FP32 column scales (the
+    // right-hand side by the FP64 ones)
+    auto wop = [&](double w) { return mixed ? (double)(float)w : w; };
+    const int ns = std::min(WARM_GALERKIN, Bp), kc = 6 * ns, k2 = 2 * kc, nout = 2 * ns + 2;
+    std::vector<int32_t> src;
+    std::vector<double> P;
+    RVE_TRY(warm_products(m, ns, ws.degrade, mixed, s, src, P));
+    double* kx = m->warm_kx.as<double>();
     const size_t n = (size_t)6 * B * WARM_SOURCES;
     std::vector<int32_t> cmap(n, 0), kmap(n, 0);
     std::vector<double> ccoef(n, 0.0), kcoef(n, 0.0);
@@ -1784,9 +1815,125 @@ static int warm_galerkin(rve_mesh m, int B, const double* w_host, bool mixed, cu
     return RVE_OK;
 }
 
+// Starts of a whole batched call from a basis of its own solutions (mixed solves, many
+// points).  WARM_BASIS points at Chebyshev-Lobatto positions of the call's range of w are
+// solved first, ten times tighter; u(w) is analytic in w, so the Galerkin projection onto
+// them leaves about 1e-6 of the right-hand side over the whole range, and all points, in
+// the batches they would have anyway, start below the tolerance of 1e-5 that such calls
+// use: what remains is one true residual a batch, which decides as ever (a batch above the
+// tolerance goes through the PCG).  Starting each batch from three solutions of the one
+// before left 1 to 5e-5, about 25 iterations of 220 us a batch of 8 on 32x32x10, p = 2, and
+// needed the sources' products once a batch; these are formed once a call.
+// Per load case G(w) = G_o + w G_d is brought to I + (w - w0) diag(lambda) by two
+// eigendecompositions (of G(w0), its eigenvalues below 1e-12 of the largest dropped as
+// rounding, then of the reduced G_d), so that the coefficients of a point are closed form.
+// ms a call at rtol 1e-5, before -> now: 48 points on 32x32x10, p = 2, 96 -> 77; 100 on
+// 24x24x8, p = 2, 94 -> 41; 400 on 11x9x5, p = 2, 49 -> 15; 333 on 16x16x6, p = 1, 20 -> 9.6;
+// 1024 on six classes 535 -> 220.  The tensors are nearer to those of rtol 1e-9 (1e-13
+// relative instead of 1e-11).
+static int build_basis(rve_mesh m, bool mixed, const double* degrade, cudaStream_t s) {
+    m->basis_n = 0;
+    const int ns = m->warm_cols[0] / 6, nout = 2 * ns + 2;
+    if (ns < 2 || ns > WARM_BASIS || !m->bph_valid[0]) return RVE_OK;
+    std::vector<int32_t> src;
+    std::vector<double> P;
+    RVE_TRY(warm_products(m, ns, degrade, mixed, s, src, P));
+    double w0 = 0.0;
+    for (double w : m->warm_w[0]) w0 = std::max(w0, w);
+    for (int lc = 0; lc < 6; ++lc) {
+        auto& bc = m->basis[lc];
+        bc.w0 = w0;
+        double A[WARM_SOURCES][WARM_SOURCES], V[WARM_SOURCES][WARM_SOURCES], D[WARM_SOURCES][WARM_SOURCES],
+            R[WARM_SOURCES][WARM_SOURCES], Q[WARM_SOURCES][WARM_SOURCES];
+        const double* Pl = &P[(size_t)lc * ns * nout];
+        for (int p = 0; p < ns; ++p)
+            for (int t = 0; t < ns; ++t) {
+                D[p][t] = -0.5 * (Pl[p * nout + t] + Pl[t * nout + p]);
+                A[p][t] = -0.5 * (Pl[p * nout + ns + t] + Pl[t * nout + ns + p]) + w0 * D[p][t];
+                if (!std::isfinite(A[p][t])) return RVE_OK;
+            }
+        jacobi_eigen(ns, A, V);
+        double lmax = 0.0;
+        for (int i = 0; i < ns; ++i) lmax = std::max(lmax, A[i][i]);
+        if (!(lmax > 0.0)) return RVE_OK;
+        int r = 0;
+        double Z[WARM_SOURCES][WARM_SOURCES];   // columns: G(w0)-orthonormal
+        for (int k = 0; k < ns; ++k)
+            if (A[k][k] > 1e-12 * lmax) {
+                for (int i = 0; i < ns; ++i) Z[i][r] = V[i][k] / std::sqrt(A[k][k]);
+                ++r;
+            }
+        for (int a = 0; a < r; ++a)
+            for (int b = 0; b < r; ++b) {
+                double t = 0.0;
+                for (int i = 0; i < ns; ++i)
+                    for (int j = 0; j < ns; ++j) t += Z[i][a] * D[i][j] * Z[j][b];
+                R[a][b] = t;
+            }
+        for (int a = 0; a < r; ++a)
+            for (int b = 0; b < a; ++b) R[a][b] = R[b][a] = 0.5 * (R[a][b] + R[b][a]);
+        jacobi_eigen(r, R, Q);
+        bc.rank = r;
+        for (int k = 0; k < r; ++k) {
+            bc.lambda[k] = R[k][k];
+            bc.y[0][k] = bc.y[1][k] = 0.0;
+            for (int i = 0; i < ns; ++i) {
+                double t = 0.0;
+                for (int a = 0; a < r; ++a) t += Z[i][a] * Q[a][k];
+                bc.V[i][k] = t;
+                for (int ph = 0; ph < 2; ++ph) bc.y[ph][k] -= t * Pl[i * nout + 2 * ns + ph];
+            }
+        }
+    }
+    // source t of the reduced problem is RVE src[t] of the batch
+    for (auto& bc : m->basis) {
+        double V[WARM_SOURCES][WARM_SOURCES];
+        std::memcpy(V, bc.V, sizeof(V));
+        for (int t = 0; t < ns; ++t) std::memcpy(bc.V[src[t]], V[t], sizeof(V[t]));
+    }
+    m->basis_n = ns;
+    return RVE_OK;
+}
+
+// The batch's starts from that basis (false: a coefficient is not finite).
+static int basis_start(rve_mesh m, int B, const double* w_host, bool mixed, cudaStream_t s, WarmStart& ws, bool& used) {
+    used = false;
+    const int ns = m->basis_n;
+    const size_t n = (size_t)6 * B * WARM_SOURCES;
+    std::vector<int32_t> cmap(n, 0);
+    std::vector<double> ccoef(n, 0.0);
+    for (int b = 0; b < B; ++b) {
+        const double w = w_host[b], wf = mixed ? (double)(float)w : w;
+        const double s0 = ws.degrade[0] != 0.0 ? w : 1.0, s1 = ws.degrade[1] != 0.0 ? w : 1.0;
+        for (int lc = 0; lc < 6; ++lc) {
+            const auto& bc = m->basis[lc];
+            double a[WARM_SOURCES];
+            for (int k = 0; k < bc.rank; ++k)
+                a[k] = (s0 * bc.y[0][k] + s1 * bc.y[1][k]) / (1.0 + (wf - bc.w0) * bc.lambda[k]);
+            for (int i = 0; i < ns; ++i) {
+                double c = 0.0;
+                for (int k = 0; k < bc.rank; ++k) c += bc.V[i][k] * a[k];
+                if (!std::isfinite(c)) return RVE_OK;
+                const size_t at = (size_t)(6 * b + lc) * WARM_SOURCES + i;
+                cmap[at] = 6 * i + lc;
+                ccoef[at] = c;
+            }
+        }
+    }
+    RVE_TRY(upload(m->warm_map, cmap.data(), n, s));
+    RVE_TRY(upload(m->warm_coef, ccoef.data(), n, s));
+    ws.x = m->warm[0].as<double>();
+    ws.r = nullptr;   // the solve forms the true residual
+    ws.cols = m->warm_cols[0];
+    ws.map = m->warm_map.as<int32_t>();
+    ws.coef = m->warm_coef.as<double>();
+    used = true;
+    return RVE_OK;
+}
+
 // Solve B RVEs of one mesh whose degradation factors are in d_w (device).
 int rve::homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, double* K, double* D,
-                          rve_stats* st, const double* w_host) {
+                          rve_stats* st, const double* w_host, BatchBasis basis) {
     NvtxRange nvtx_("homogenise batch of %d RVEs (%d tets, p = %d)", B, (int)m->nt, m->p);
     cudaStream_t s = m->on_own_streams ? m->stream : m->ctx->stream;
     const int ncols = 6 * B;
@@ -1807,6 +1954,11 @@ int rve::homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, doubl
         ws.degrade[1] = (f == 0 && m->deg.apply_to_yarn) ? 1.0 : 0.0;
         // a field that does not degrade has one solution for every w: the nearest will do
         const bool degrades = ws.degrade[0] != 0.0 || ws.degrade[1] != 0.0;
+        if (f == 0 && basis == BASIS_USE && m->basis_n > 0) {
+            bool used = false;
+            RVE_TRY(basis_start(m, B, w_host, mixed, s, ws, used));
+            if (used) return RVE_OK;
+        }
         if (f == 0 && degrades && m->ctx->opt.warm_start >= 4 && m->bph_prec[0] == prec) {
             bool used = false;
             RVE_TRY(warm_galerkin(m, B, w_host, mixed, s, ws, used));
@@ -1862,9 +2014,15 @@ int rve::homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, doubl
             RVE_TRY(build_warm(0, ws));
             RVE_TRY(sv.run(prec, om, &ws));
         } else {
+            if (basis == BASIS_BUILD) sv.tighten = 0.1;
             RVE_TRY(sv.run(prec, om));
         }
-        RVE_TRY(keep_warm(0, m->mech));
+        // (the sources of a basis stay for the rest of the call)
+        if (!(basis == BASIS_USE && m->basis_n > 0)) RVE_TRY(keep_warm(0, m->mech));
+        if (basis == BASIS_BUILD) {
+            const double degrade[2] = {1.0, m->deg.apply_to_yarn ? 1.0 : 0.0};
+            RVE_TRY(build_basis(m, mixed, degrade, s));
+        }
     }
     // thermal and moisture: transport is not degraded (Sec. 5), so these cell
     // problems are the same for every point of the mesh.  With transport_once
@@ -1877,7 +2035,8 @@ int rve::homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, doubl
         osc.iterations = 0;
         osc.sweeps = 0;
     } else {
-        const int Bs = reuse_scalar ? 1 : B;
+        // (the sources of a basis: one RVE starts all of the call's batches)
+        const int Bs = reuse_scalar || basis == BASIS_BUILD ? 1 : B;
         launch_column_scales<double>(Bs, d_w, 0, false, m->scale64.as<double>(), s);
         launch_column_scales<float>(Bs, d_w, 0, false, m->scale32.as<float>(), s);
         m->ctx->launches += 2;
@@ -1894,9 +2053,13 @@ int rve::homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, doubl
             m->scal_cached = true;
         } else {
             RVE_TRY(keep_warm(1, m->scal));
+            if (basis == BASIS_BUILD) {
+                m->warm_cols[1] = 6;
+                m->warm_w[1].assign(w_host, w_host + 1);
+            }
         }
     }
-    if (reuse_scalar) {
+    if (reuse_scalar || basis == BASIS_BUILD) {
         // every RVE of the batch gets the mesh's scalar tensors
         const std::vector<double> t1 = osc.tensor, s1 = osc.sig;
         osc.tensor.resize((size_t)B * 36);
@@ -2519,6 +2682,18 @@ static int auto_batch(rve_mesh m) {
     return (B / 8) * 8;
 }
 
+// Whether a call's points on one mesh start from a basis of WARM_BASIS of their own
+// solutions (build_basis): mixed solves, whose tolerance such starts reach.  Its sources are
+// solved on top, in a batch that may not fill the GPU, so it takes several times their
+// number of points and enough vector entries in all for an iteration over them to be bound
+// by throughput (3e6 entries: 9x9x5, p = 2, 60 points: 10.3 -> 6.9 ms a call); and the products' 28 bytes for each of 72 columns a row within 4 GB.
+static bool use_basis(rve_mesh m, size_t points, int Bmax) {
+    const int64_t rows = m->mech.n_rows;
+    return m->ctx->opt.precision == RVE_PREC_MIXED && m->ctx->opt.warm_start >= 4 && m->mech.m == 0 &&
+           m->ctx->opt.rtol >= 1e-6 && Bmax >= WARM_BASIS && points >= 4 * (size_t)WARM_BASIS &&
+           (double)rows * 6.0 * (double)points >= 3e6 && rows <= 2000000;
+}
+
 // W_dev (optional, [G]): the degradation factor 1 - omega of each point, used in
 // place of the degradation law at (T, c, t) (which are then not read).
 static int macro_update_impl(rve_ctx c, const rve_mesh* meshes, int n_meshes, int64_t G,
@@ -2605,6 +2780,23 @@ static int macro_update_impl(rve_ctx c, const rve_mesh* meshes, int n_meshes, in
         m->warm_w[0].clear();
         m->warm_w[1].clear();
         m->scal_cached = false;
+        m->basis_n = 0;
+        const bool with_basis = use_basis(m, grp.size(), Bmax);
+        std::vector<double> w_src;
+        std::vector<int64_t> g_src;
+        if (with_basis) {
+            std::vector<char> taken(grp.size(), 0);
+            for (int k = 0; k < WARM_BASIS; ++k) {
+                const double at = 0.5 * (wg.front() + wg.back()) -
+                                  0.5 * (wg.back() - wg.front()) * std::cos(M_PI * k / (WARM_BASIS - 1));
+                size_t best = grp.size();
+                for (size_t i = 0; i < grp.size(); ++i)
+                    if (!taken[i] && (best == grp.size() || std::fabs(wg[i] - at) < std::fabs(wg[best] - at))) best = i;
+                taken[best] = 1;
+                g_src.push_back(grp[best]);
+                w_src.push_back(wg[best]);
+            }
+        }
         DevBuf d_idx, d_tmp, d_res;
         std::vector<double> res;
         int rc_mesh = RVE_OK;
@@ -2612,30 +2804,54 @@ static int macro_update_impl(rve_ctx c, const rve_mesh* meshes, int n_meshes, in
             *err = last_error();
             return rc;
         };
-        int rc0 = upload(d_idx, grp.data(), grp.size(), sm);
+        int rc0 = RVE_OK;
+        // the factors of n points (indices idx, device) in place
+        auto batch_factors = [&](int n, const int64_t* idx, double*& dw) -> int {
+            RVE_TRY(d_tmp.ensure((size_t)n * 4 * 8));
+            double* st3 = d_tmp.as<double>();
+            dw = st3 + 3 * n;
+            if (W_dev) {
+                // the factors themselves: gathered three times over, the first copy is the batch's w
+                launch_gather_states(n, idx, W_dev, W_dev, W_dev, st3, sm);
+                dw = st3;
+                c->launches += 1;
+            } else {
+                launch_gather_states(n, idx, T_dev, c_dev, t_dev, st3, sm);
+                launch_degradation(n, st3, st3 + n, st3 + 2 * n, m->deg.beta, m->deg.Tg_C, m->deg.c_sat_wt, dw, sm);
+                c->launches += 2;
+            }
+            return RVE_OK;
+        };
+        if (with_basis) {
+            double* dw = nullptr;
+            rc0 = upload(d_idx, g_src.data(), g_src.size(), sm);
+            if (rc0 == RVE_OK) rc0 = batch_factors(WARM_BASIS, d_idx.as<int64_t>(), dw);
+            if (rc0 != RVE_OK) return fail(rc0);
+            const rve_stats before = stm ? *stm : rve_stats();
+            const int rc = homogenise_batch(m, WARM_BASIS, dw, nullptr, nullptr, nullptr, stm, w_src.data(), BASIS_BUILD);
+            if (rc != RVE_OK && rc != RVE_ERR_NOT_CONVERGED && rc != RVE_ERR_NUMERIC) return fail(rc);
+            if (rc != RVE_OK) {
+                // no usable sources: the points start cold and answer for themselves
+                if (stm) *stm = before;
+                m->basis_n = 0;
+                m->warm_cols[0] = m->warm_cols[1] = 0;
+                m->warm_w[0].clear();
+                m->warm_w[1].clear();
+            }
+        }
+        rc0 = upload(d_idx, grp.data(), grp.size(), sm);
         if (rc0 != RVE_OK) return fail(rc0);
         for (size_t off = 0; off < grp.size(); off += Bmax) {
             const int B = (int)std::min<size_t>(Bmax, grp.size() - off);
             const int64_t* idx = d_idx.as<int64_t>() + off;
-            rc0 = d_tmp.ensure((size_t)B * 4 * 8);
+            double* dw = nullptr;
+            rc0 = batch_factors(B, idx, dw);
             if (rc0 != RVE_OK) return fail(rc0);
-            double* st3 = d_tmp.as<double>();
-            double* dw = st3 + 3 * B;
-            if (W_dev) {
-                // the factors themselves: gathered three times over, the first copy is the batch's w
-                launch_gather_states(B, idx, W_dev, W_dev, W_dev, st3, sm);
-                dw = st3;
-                c->launches += 1;
-            } else {
-                launch_gather_states(B, idx, T_dev, c_dev, t_dev, st3, sm);
-                launch_degradation(B, st3, st3 + B, st3 + 2 * B, m->deg.beta, m->deg.Tg_C, m->deg.c_sat_wt, dw,
-                                   sm);
-                c->launches += 2;
-            }
             res.assign((size_t)B * 55, 0.0);
             std::vector<double> hC((size_t)B * 36), hK((size_t)B * 9), hD((size_t)B * 9);
             int rc = homogenise_batch(m, B, dw, hC.data(), hK.data(), hD.data(), stm,
-                                      c->opt.warm_start ? &wg[off] : nullptr);
+                                      c->opt.warm_start ? &wg[off] : nullptr,
+                                      with_basis ? BASIS_USE : BASIS_NONE);
             if (rc != RVE_OK && rc != RVE_ERR_NOT_CONVERGED && rc != RVE_ERR_NUMERIC) return fail(rc);
             if (rc != RVE_OK) {
                 rc_mesh = rc;

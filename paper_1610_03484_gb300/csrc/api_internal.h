@@ -251,6 +251,14 @@ struct rve_mesh_s {
     // map of r0 into the products
     rve::DevBuf warm_src, warm_omap, warm_ocoef, warm_ksc, warm_phs, warm_xs64, warm_xs, warm_kx, warm_klo, warm_gram,
         warm_kxmap;
+    // starts of a batched call from a basis of its own solutions (see build_basis): the
+    // sources in warm[0] while basis_n > 0, and per load case the reduced problem
+    int basis_n = 0;
+    struct BasisCase {
+        int rank = 0;
+        double w0 = 1.0;
+        double V[8][8], lambda[8], y[2][8];   // coefficients V diag(1 / (1 + (w - w0) lambda)) (y . s(w))
+    } basis[6];
     rve::DevBuf dscale32, dscale64;   // per-column phase scales of the warm-start residual
     // per field: K_ph u_macro for each phase at unit modulus, [2][n_rows][6] (FP64),
     // so that a batch's right-hand side is a per-column combination of them
@@ -265,8 +273,11 @@ namespace rve {
 // Batched PCG homogenisation of B RVEs of one mesh (degradation factors d_w on
 // the device); host outputs C [B][36], K [B][9], D [B][9] (any may be null).
 // w_host (optional, [B]) enables the warm start from the mesh's previous batch
-// (see macro_update_gauss_points); the batch's solutions become the next start.
+// (see macro_update_gauss_points); the batch's solutions become the next start.  basis:
+// the batch's mechanical solutions become the basis of the call's starts, or it starts from
+// that basis (see build_basis).
+enum BatchBasis { BASIS_NONE, BASIS_BUILD, BASIS_USE };
 int homogenise_batch(rve_mesh m, int B, const double* d_w, double* C, double* K, double* D, rve_stats* st,
-                     const double* w_host = nullptr);
+                     const double* w_host = nullptr, BatchBasis basis = BASIS_NONE);
 int check_ctx(rve_ctx c);
 }  // namespace rve

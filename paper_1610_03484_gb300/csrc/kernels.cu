@@ -2118,15 +2118,15 @@ __global__ void __launch_bounds__(256) k_warm_gram(int64_t n_rows, int ns, const
                                                    double* __restrict__ out) {
     const int lc = blockIdx.x / ns, p = blockIdx.x % ns;
     const int nout = 2 * ns + 2, kst = 12 * ns;
-    double am[WARM_GALERKIN], ay[WARM_GALERKIN], ay0 = 0.0, ay1 = 0.0;
+    double am[WARM_BASIS], ay[WARM_BASIS], ay0 = 0.0, ay1 = 0.0;
 #pragma unroll
-    for (int t = 0; t < WARM_GALERKIN; ++t) am[t] = ay[t] = 0.0;
+    for (int t = 0; t < WARM_BASIS; ++t) am[t] = ay[t] = 0.0;
     const int cp = 6 * src[p] + lc;
     for (int64_t row = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; row < n_rows;
          row += (int64_t)gridDim.y * blockDim.x) {
         const double xp = X[row * src_cols + cp];
 #pragma unroll
-        for (int t = 0; t < WARM_GALERKIN; ++t)
+        for (int t = 0; t < WARM_BASIS; ++t)
             if (t < ns) {
                 am[t] = fma(xp, Kc[row * kst + 6 * t + lc], am[t]);
                 ay[t] = fma(xp, Kc[row * kst + 6 * ns + 6 * t + lc], ay[t]);
@@ -2136,7 +2136,7 @@ __global__ void __launch_bounds__(256) k_warm_gram(int64_t n_rows, int ns, const
     }
     double* o = out + ((int64_t)blockIdx.y * 6 * ns + blockIdx.x) * nout;
 #pragma unroll
-    for (int t = 0; t < WARM_GALERKIN; ++t)
+    for (int t = 0; t < WARM_BASIS; ++t)
         if (t < ns) {
             const double a = block_sum(am[t]);
             const double b = block_sum(ay[t]);

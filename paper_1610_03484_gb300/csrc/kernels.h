@@ -192,10 +192,12 @@ constexpr int WARM_SOURCES = 8;
 constexpr int WARM_GALERKIN = 3;   // previous solutions spanning the energy-optimal start
 // the energy-optimal start's residual map holds two entries per source in a column's row
 static_assert(2 * WARM_GALERKIN <= WARM_SOURCES, "WARM_SOURCES must hold 2 * WARM_GALERKIN entries");
+constexpr int WARM_BASIS = 6;      // solutions spanning the starts of a whole call (see api.cu)
+static_assert(WARM_GALERKIN <= WARM_BASIS && WARM_BASIS <= WARM_SOURCES, "source counts");
 template <typename TI, typename TO>
 void launch_combine_columns(int64_t n_rows, int ncols, int src_cols, const int32_t* map, const double* coef,
                             const TI* src, TO* x, cudaStream_t s, bool accumulate = false);
-// inner products of the energy-optimal warm start (ns <= WARM_GALERKIN sources of the
+// inner products of the energy-optimal warm start (ns <= WARM_BASIS sources of the
 // previous batch, columns 6 src[p] + lc): out[split][lc][p][t] for t < ns x_p . Kc_t,
 // t in [ns, 2 ns) x_p . Kc_{6 ns + (t - ns)} (Kc: [n_rows][12 ns], the degraded and the
 // other phases' products), then x_p . Y_0 and x_p . Y_1
