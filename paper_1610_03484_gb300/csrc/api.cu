@@ -542,6 +542,13 @@ struct Solver {
         set_view_extras(e, m);
         return e;
     }
+    // An FP32 solve uses the assembled operator from 1e5 values a component on: below, launches
+    // bound an iteration, and the host's work on the sparsity shows in a mesh's first solve
+    // (26x30x3, 12 columns, 28e3 values: first call 6.1 ms without, 7.5 with, later ones 5.63
+    // and 5.71; 12x16x6, 108 columns, 124e3: 4.3 and 4.0).
+    bool assembled32() const {
+        return use_assembled(m, false) && (double)m->map.N * ncols >= 1e5;
+    }
     template <typename T>
     RowView<T> rv(const DevBuf& scale) const {
         RowView<T> r;
@@ -781,7 +788,7 @@ struct Solver {
         const bool use_tc =
             !det && sizeof(T) == 4 && operator_tc_supported(m->p, f.nc) && kern == RVE_KERNEL_TENSOR;
         if (use_tc) RVE_TRY(ensure_element_matrices(m, s));
-        const bool use_asm = !use_tc && use_assembled(m, sizeof(T) == 8);
+        const bool use_asm = !use_tc && (sizeof(T) == 8 ? use_assembled(m, true) : assembled32());
         if (use_asm) RVE_TRY(ensure_assembled(m, fid, sizeof(T) == 8, s));
         const AsmView<T> av = use_asm ? asm_view<T>(m, fid, scale.as<T>()) : AsmView<T>();
         ColState cs = cs64;
@@ -1370,7 +1377,7 @@ struct Solver {
                     for (int c = 0; c < ncols; ++c)
                         for (int ph = 0; ph < 2; ++ph) sc32[2 * c + ph] = (float)-warm->degrade[ph];
                     RVE_TRY(upload(m->dscale32, sc32.data(), sc32.size(), s));
-                    if (use_assembled(m, false)) {
+                    if (assembled32()) {
                         RVE_TRY(ensure_assembled(m, fid, false, s));
                         launch_asm_product<float>(f.nc, asm_view<float>(m, fid, m->dscale32.as<float>()), v32, y32,
                                                   ncols, nullptr, nullptr, s);

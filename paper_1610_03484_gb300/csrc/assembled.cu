@@ -456,9 +456,9 @@ void launch_assemble(int p, int nc, const AsmGraph& g, const int32_t* edofs, con
 
 // Columns per thread and lanes per row.  Four columns per thread need 16-byte aligned
 // rows and eight warps per SM: with fewer, each thread's serial walk along its row bounds
-// the product (6x7x8, p = 1, 108 columns: a call of 18 points 2.68 -> 2.27 ms, the
-// element form 2.31).  Otherwise the entries of a row are split over four lanes, or eight where
-// even then the chip has less than four warps per scheduler.
+// the product (6x7x8, p = 1, 108 columns: a mixed call of 18 points took 2.68 ms with four
+// columns a thread, 2.27 with split rows).  Otherwise the entries of a row are split over
+// four lanes, or eight where even then the chip has less than four warps per scheduler.
 #define RVE_ASM_RUN(MODE, ...)                                                              \
     do {                                                                                    \
         const bool few = A.n * ncols / 2 < (int64_t)sm_count() * 4 * 32;                    \
