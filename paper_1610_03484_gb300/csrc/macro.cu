@@ -6,14 +6,14 @@
 // hands each Gauss point to the RVE path (macro_update_gauss_points[_dev] or the
 // surrogate) as (T, c, t_eq).
 //
-// Both fields are solved together as two columns of one matrix-free operator:
+// Both fields are solved together as two columns of one assembled operator:
 // vectors v[node * 2 + field], field 0 temperature [C], field 1 moisture [wt%].
 //
 // The macro mechanical problem of the fully nested FE^2 step (Sec. 5) uses the
 // same mesh: linear elasticity with the homogenised stiffness C_bar of every
-// macro Gauss point, vectors u[node * 3 + component], solved by the same Jacobi
-// PCG with one field and a per-DOF held mask.
-// Everything here is FP64: the macro mesh is small next to the RVE batches.
+// macro Gauss point, vectors u[node * 3 + component], with a per-DOF held mask,
+// solved by PCG with a Chebyshev preconditioner.
+// Everything here is FP64 but that preconditioner, which is evaluated in FP32.
 #include <cuda_runtime.h>
 
 #include <algorithm>
