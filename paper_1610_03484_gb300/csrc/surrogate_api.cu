@@ -553,6 +553,7 @@ static int predict_dev(rve_surrogate s, int64_t n, const double* feat_dev, doubl
         s->ctx->launches += 2;
     }
     RVE_CUDA(cudaGetLastError());
+    RVE_CUDA(cudaStreamSynchronize(st));   // the outputs are complete when the call returns
     return RVE_OK;
 }
 
