@@ -748,12 +748,65 @@ cudaError_t launch_gemm_bf16(int M, int N, int K, const __nv_bfloat16* A, const 
     return launch_gemm_group(1, &p, N, K, epilogue, s);
 }
 
+// Sum of a double over the block's 256 threads (every thread gets it), in a fixed order.
+__device__ __forceinline__ double block_sum_256(double v, double* buf) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += buf[k];
+    __syncthreads();
+    return t;
+}
+
+// Adds one step's partial sums (part [n], non-negative, one per warp of k_head_loss) to the
+// FP32 running sum *loss of an epoch.  Added one by one, each is rounded to the last place of
+// the sum, and the sum depends on their order only where it passes a power of two: which
+// of them come before, at the finer rounding, and which after.  Here every one takes part in
+// each binade by the share of the step that falls into it, which is the mean over all orders:
+// the same in every run, where atomic additions in the order the blocks finish scatter
+// by 1e-7 around it.  One pass over the partial sums per binade, 1.7 a step.
+__device__ __forceinline__ void add_step_loss(const float* __restrict__ part, int n, float* loss) {
+    __shared__ double buf[8];
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) v += (double)part[i];
+    const double total = block_sum_256(v, buf);
+    double s = (double)*loss, rest = 1.0;
+    if (isfinite(total) && isfinite(s) && total > 0.0) {
+        if (s == 0.0) {   // the first of n equal shares is exact
+            s = total / n;
+            rest = 1.0 - 1.0 / n;
+        }
+        for (;;) {
+            const float at = (float)s;
+            v = 0.0;
+            for (int i = threadIdx.x; i < n; i += 256) v += (double)((at + part[i]) - at);
+            const double r = block_sum_256(v, buf), top = at > 0.f ? ldexp(1.0, ilogbf(at) + 1) : 0.0;
+            if (!(top > s) || !isfinite(r) || s + rest * r <= top) {
+                s += rest * (isfinite(r) ? r : total);
+                break;
+            }
+            rest -= (top - s) / r;
+            s = top;
+        }
+    } else {
+        s += total;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *loss = (float)s;
+}
+
 // One of the jobs in front of the weight-gradient GEMMs, per block plane z: the
-// transposes of a layer's output gradient G [M][N] and input H [M][K], and G's column
-// sums (the bias gradient).  The column sums run over the rows in order: the tile is
-// staged in shared memory so that the serial FP32 sum is not a chain of global loads.
+// transposes of a layer's output gradient G [M][N] and input H [M][K], G's column
+// sums (the bias gradient), and a member's loss.  The column sums run over the rows in
+// order: the tile is staged in shared memory so that the serial FP32 sum is not a chain
+// of global loads.
 __global__ void __launch_bounds__(256) k_backward_prep(const __grid_constant__ PrepJobs J) {
     const PrepJob& j = J.job[blockIdx.z];
+    if (j.part) {
+        if (blockIdx.x == 0 && blockIdx.y == 0) add_step_loss(j.part, j.rows, j.sum);
+        return;
+    }
     const int bx = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     if (bx >= j.cols) return;
     if (j.out) {
@@ -793,11 +846,13 @@ void launch_backward_prep(const PrepJobs& J, int count, int max_cols, int max_ro
 
 // Output head loss: z [M][NOUTP] (FP32), target rows [.][33] (row r takes target
 // rows[r], or r without a list), sigma [33]; dz = d loss / d z (BF16, padded columns
-// zero); loss partial per block.
-__global__ void k_head_loss(int M, int noutp, const float* __restrict__ z, const int32_t* __restrict__ rows,
-                            const float* __restrict__ target, const float* __restrict__ sigma,
-                            const uint8_t* __restrict__ diag, __nv_bfloat16* __restrict__ dz,
-                            float* __restrict__ loss) {
+// zero); loss partial per warp, in warp order.  blockIdx.y is the member.
+__global__ void k_head_loss(int M, int noutp, const __grid_constant__ HeadArgs A, const float* __restrict__ target,
+                            const float* __restrict__ sigma, const uint8_t* __restrict__ diag) {
+    const float* __restrict__ z = A.z[blockIdx.y];
+    const int32_t* __restrict__ rows = A.rows[blockIdx.y];
+    __nv_bfloat16* __restrict__ dz = A.dz[blockIdx.y];
+    float* __restrict__ part = A.part[blockIdx.y];
     float local = 0.f;
     const float inv = 1.f / ((float)M * 33.f);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)M * noutp;
@@ -816,13 +871,14 @@ __global__ void k_head_loss(int M, int noutp, const float* __restrict__ z, const
         dz[i] = __float2bfloat16(g);
     }
     for (int o = 16; o > 0; o >>= 1) local += __shfl_down_sync(0xffffffffu, local, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, local);
+    if ((threadIdx.x & 31) == 0) part[blockIdx.x * 8 + (threadIdx.x >> 5)] = local;
 }
 
-void launch_head_loss(int M, int noutp, const float* z, const int32_t* rows, const float* target, const float* sigma,
-                      const uint8_t* diag, __nv_bfloat16* dz, float* loss, cudaStream_t s) {
-    const int blocks = (M * noutp + 255) / 256;
-    k_head_loss<<<blocks < 2048 ? blocks : 2048, 256, 0, s>>>(M, noutp, z, rows, target, sigma, diag, dz, loss);
+int head_loss_parts(int M, int noutp) { return 8 * std::min((int)(((int64_t)M * noutp + 255) / 256), 2048); }
+
+void launch_head_loss(int members, int M, int noutp, const HeadArgs& A, const float* target, const float* sigma,
+                      const uint8_t* diag, cudaStream_t s) {
+    k_head_loss<<<dim3(head_loss_parts(M, noutp) / 8, members), 256, 0, s>>>(M, noutp, A, target, sigma, diag);
 }
 
 // Adam on FP32 master weights W [K][N] with gradient G given transposed [N][K]

@@ -35,21 +35,30 @@ cudaError_t launch_mlp_fused(int M, int members, const __nv_bfloat16* X, const _
 constexpr int MAX_MEMBERS = 16;
 
 // jobs of the backward pass: out [cols][rows] = in [rows][cols] transposed, or (out null)
-// sum [cols] = column sums of in
+// sum [cols] = column sums of in, or (part given) *sum += the step's loss, part [rows]
 constexpr int PREP_JOBS = 64;
 struct PrepJob {
     const __nv_bfloat16* in;
     __nv_bfloat16* out;
     float* sum;
     int rows, cols;
+    const float* part = nullptr;
 };
 struct PrepJobs {
     PrepJob job[PREP_JOBS];
 };
 void launch_backward_prep(const PrepJobs& J, int count, int max_cols, int max_rows, cudaStream_t s);
 
-void launch_head_loss(int M, int noutp, const float* z, const int32_t* rows, const float* target, const float* sigma,
-                      const uint8_t* diag, __nv_bfloat16* dz, float* loss, cudaStream_t s);
+// part [head_loss_parts]: the loss, a partial sum per warp
+struct HeadArgs {
+    const float* z[MAX_MEMBERS];
+    const int32_t* rows[MAX_MEMBERS];
+    __nv_bfloat16* dz[MAX_MEMBERS];
+    float* part[MAX_MEMBERS];
+};
+int head_loss_parts(int M, int noutp);
+void launch_head_loss(int members, int M, int noutp, const HeadArgs& A, const float* target, const float* sigma,
+                      const uint8_t* diag, cudaStream_t s);
 
 // one layer of one member: weights W [K][N] with the bias [N] behind them, moments m1, m2
 // laid out alike, gradients Gt [N][K] (null: zero) and gb [N] (null: weights only)

@@ -110,6 +110,7 @@ int refresh_bf16(rve_surrogate s, int e) {
 struct TrainWork {
     __nv_bfloat16 *H[MAX_MEMBERS][NLAYER], *Ht[MAX_MEMBERS][NLAYER], *G[MAX_MEMBERS][NLAYER], *Gt[MAX_MEMBERS][NLAYER];
     float *Z[MAX_MEMBERS][NLAYER], *gradT[MAX_MEMBERS][NLAYER], *gradb[MAX_MEMBERS][NLAYER], *zout[MAX_MEMBERS];
+    float* lpart[MAX_MEMBERS];   // partial sums of the loss
 };
 
 int train_work(rve_surrogate s, int nm, int M, TrainWork& w) {
@@ -133,6 +134,7 @@ int train_work(rve_surrogate s, int nm, int M, TrainWork& w) {
                 w.gradb[e][l] = reinterpret_cast<float*>(take((size_t)LN[l] * 4));
             }
             w.zout[e] = reinterpret_cast<float*>(take((size_t)M * NOUTP * 4));
+            w.lpart[e] = reinterpret_cast<float*>(take((size_t)head_loss_parts(M, NOUTP) * 4));
         }
         if (pass == 0) {
             RVE_TRY(s->train_work.ensure(off));
@@ -186,11 +188,15 @@ int forward_backward(rve_surrogate s, int first, int nm, int M, const TrainWork&
         }
         RVE_TRY(gemm_all(v, LN[l], LK[l], l < NLAYER - 1 ? 1 : 2, c));
     }
-    // (one launch per member: the loss is an FP32 sum in the order the blocks finish)
-    for (int e = 0; e < nm; ++e)
-        launch_head_loss(M, NOUTP, w.zout[e], rows ? rows[e] : nullptr, target, sigma, s->d_diag.as<uint8_t>(),
-                         w.G[e][NLAYER - 1], loss[e], st);
-    c->launches += 1 + nm;
+    HeadArgs ha;
+    for (int e = 0; e < nm; ++e) {
+        ha.z[e] = w.zout[e];
+        ha.rows[e] = rows ? rows[e] : nullptr;
+        ha.dz[e] = w.G[e][NLAYER - 1];
+        ha.part[e] = w.lpart[e];
+    }
+    launch_head_loss(nm, M, NOUTP, ha, target, sigma, s->d_diag.as<uint8_t>(), st);
+    c->launches += 2;
     // dH_l = G_l W_l^T, through the silu of layer l - 1
     for (int l = NLAYER - 1; l > 0; --l) {
         for (int e = 0; e < nm; ++e) {
@@ -204,7 +210,7 @@ int forward_backward(rve_surrogate s, int first, int nm, int M, const TrainWork&
         }
         RVE_TRY(gemm_all(v, LK[l], LN[l], 5, c));
     }
-    // transposes and bias gradients, then dW^T [N][K] = G^T H
+    // transposes, bias gradients and the loss, then dW^T [N][K] = G^T H
     PrepJobs J;
     int nj = 0;
     auto flush = [&]() {
@@ -214,13 +220,16 @@ int forward_backward(rve_surrogate s, int first, int nm, int M, const TrainWork&
         }
         nj = 0;
     };
-    for (int e = 0; e < nm; ++e)
+    for (int e = 0; e < nm; ++e) {
+        if (nj + 1 > PREP_JOBS) flush();
+        J.job[nj++] = PrepJob{nullptr, nullptr, loss[e], head_loss_parts(M, NOUTP), 0, w.lpart[e]};
         for (int l = 0; l < NLAYER; ++l) {
             if (nj + 3 > PREP_JOBS) flush();
             J.job[nj++] = PrepJob{w.G[e][l], w.Gt[e][l], nullptr, M, LN[l]};
             J.job[nj++] = PrepJob{w.H[e][l], w.Ht[e][l], nullptr, M, LK[l]};
             J.job[nj++] = PrepJob{w.G[e][l], nullptr, w.gradb[e][l], M, LN[l]};
         }
+    }
     flush();
     for (int wide = 0; wide < 2; ++wide) {   // layer 0 has 64 inputs, the others 256
         for (int e = 0; e < nm; ++e)

@@ -93,3 +93,28 @@ def test_ensemble_of_any_size_matches_oracle(rve, members, n):
         for T in Ts:
             spread = np.maximum(spread, np.linalg.norm((T[b] - mean).reshape(n, -1), axis=1) / den)
     assert np.abs(fused[3] - spread).max() < 2e-3
+
+
+@pytest.mark.parametrize("members,n,batch", [(4, 1024, 256), (1, 64, 64), (5, 1000, 192), (2, 8256, 8256)])
+def test_loss_history_is_reproducible(rve, members, n, batch):
+    """The same training twice returns the same history to the bit.  With one step an epoch
+    the first loss is the mean of the members' losses at the initial parameters (FP32 sums of
+    the same terms, the rows in another order: at most 1e-5 for 2e5 terms)."""
+    feat, C, K, D = data(n, 7 * members)
+    runs = []
+    for _ in range(2):
+        with rve.Context() as ctx:
+            s = rve.Surrogate(ctx, members=members, seed=5)
+            buf0 = s.get_params()
+            hist = np.asarray(s.train(feat, C, K, D, epochs=3, batch=batch, lr=1e-3, seed=1))
+            buf1 = s.get_params()
+            if n == batch:
+                ref = buf1[49:52].astype(np.float64)
+                target = osg.factors_from_tensors(C / ref[0], K / ref[1], D / ref[2]).astype(np.float32)
+                s.set_params(np.concatenate([buf1[:52], buf0[52:]]).astype(np.float32))
+                want = np.mean([s.gradients(e, feat, target)[1] for e in range(members)])
+                assert abs(hist[0] - want) < 1e-5 * want
+            s.free()
+        runs.append((hist, buf1))
+    np.testing.assert_array_equal(runs[0][0], runs[1][0])
+    np.testing.assert_array_equal(runs[0][1], runs[1][1])
