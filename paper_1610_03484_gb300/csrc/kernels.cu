@@ -1192,8 +1192,10 @@ struct ColJacobi {
     T s0, s1;
     __device__ __forceinline__ ColJacobi(const RowView<T>& rv, int col) {
         const int f = (rv.nfield == 2 && (col % 6) >= 3) ? 1 : 0;
-        dinv = rv.dinv ? rv.dinv + (rv.nfield == 2 ? f : col / 6) : nullptr;
-        groups = rv.dinv_groups;
+        if constexpr (sizeof(T) == 8) {
+            dinv = rv.dinv ? rv.dinv + (rv.nfield == 2 ? f : col / 6) : nullptr;
+            groups = rv.dinv_groups;
+        }
         d0 = rv.diag + (int64_t)(2 * f) * rv.n_rows;
         d1 = d0 + rv.n_rows;
         mask = rv.mask;
@@ -1201,7 +1203,8 @@ struct ColJacobi {
         s1 = rv.scale[2 * col + 1];
     }
     __device__ __forceinline__ T inv(int64_t row) const {
-        if (sizeof(T) == 8 && dinv) return __ldg(dinv + row * groups);
+        if constexpr (sizeof(T) == 8)
+            if (dinv) return __ldg(dinv + row * groups);
         if (mask && mask[row / NC]) return T(0);
         return jacobi_inv<T>(s0, __ldg(d0 + row), s1, __ldg(d1 + row));
     }
@@ -1305,15 +1308,15 @@ __global__ void __launch_bounds__(256) k_update(RowView<T> rv, T* __restrict__ x
     }
 }
 
-// p = M^-1 r + beta p ; q = 0 (unless null: the assembled operator writes q instead of
-// adding into it).  FP32, no constraint rows, column count a
-// multiple of 4 per block: each thread handles four adjacent columns of a row
-// with 16-byte loads and stores, four times the bytes in flight per instruction
+// p = M^-1 r + beta p ; CLEAR: q = 0 (the assembled operator writes q instead of adding
+// into it; a test of q at every entry cost 3 % of the pass).  FP32, no constraint rows,
+// column count a multiple of 4 per block: each thread handles four adjacent columns of a
+// row with 16-byte loads and stores, four times the bytes in flight per instruction
 // of the one-column form (this pass is bound by memory latency).  Thread
 // (c4, rr) of a block covers columns blockIdx.x * cpb + 4 c4 .. + 3.  The same
 // treatment of the x/r update pass was slower: its four per-column partial sums
 // raise the register count and cut the occupancy below what hides the latency.
-template <int NC>
+template <int NC, bool CLEAR>
 __global__ void __launch_bounds__(256) k_pupdate_v4(RowView<float> rv, const float* __restrict__ r,
                                                     float* __restrict__ p, float* __restrict__ q, ColState cs,
                                                     int ncols, int cpb, int first) {
@@ -1357,7 +1360,7 @@ __global__ void __launch_bounds__(256) k_pupdate_v4(RowView<float> rv, const flo
             out[k] = act[k] ? (first ? z : fmaf(beta[k], pk[k], z)) : (first ? 0.f : pk[k]);
         }
         *reinterpret_cast<float4*>(p + idx) = make_float4(out[0], out[1], out[2], out[3]);
-        if (q) *reinterpret_cast<float4*>(q + idx) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (CLEAR) *reinterpret_cast<float4*>(q + idx) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -1639,8 +1642,8 @@ void launch_project_residual(const RowView<double>& rv, const RowView<float>& rv
 #undef RVE_PR_CASE
 }
 
-// p = M^-1 (r - C^T mu) + beta p ; q = 0
-template <typename T, int NC, bool HAS_C>
+// p = M^-1 (r - C^T mu) + beta p ; CLEAR: q = 0
+template <typename T, int NC, bool HAS_C, bool CLEAR>
 __global__ void __launch_bounds__(256) k_pupdate(RowView<T> rv, T* __restrict__ r,
                                                  T* __restrict__ p, T* __restrict__ q, ColState cs,
                                                  int ncols, int cpb, int first) {
@@ -1657,7 +1660,7 @@ __global__ void __launch_bounds__(256) k_pupdate(RowView<T> rv, T* __restrict__ 
     const int64_t stride = (int64_t)gridDim.y * rows;
     for (int64_t i = (int64_t)blockIdx.y * rows + rr; i < i_end; i += stride) {
         const int64_t idx = i * ncols + col;
-        if (q) q[idx] = T(0);
+        if constexpr (CLEAR) q[idx] = T(0);
         if (!act) {
             p[idx] = T(0);
             continue;
@@ -1688,19 +1691,20 @@ void launch_pupdate(const RowView<T>& rv, T* r, T* p, T* q, ColState cs, bool fi
         if (rv.m == 0 && L.cpb % 4 == 0) {
             const int t4 = L.cpb / 4;
             dim3 b4(t4 * (256 / t4));
-            if (rv.nc == 3)
-                k_pupdate_v4<3><<<grid, b4, 0, L.stream>>>(rv, r, p, q, cs, L.ncols, L.cpb, fi);
-            else
-                k_pupdate_v4<1><<<grid, b4, 0, L.stream>>>(rv, r, p, q, cs, L.ncols, L.cpb, fi);
+#define RVE_PUP_CASE(NCC, CL) \
+    if (rv.nc == NCC && (q != nullptr) == CL) k_pupdate_v4<NCC, CL><<<grid, b4, 0, L.stream>>>(rv, r, p, q, cs, L.ncols, L.cpb, fi);
+            RVE_PUP_CASE(3, true) RVE_PUP_CASE(3, false) RVE_PUP_CASE(1, true) RVE_PUP_CASE(1, false)
+#undef RVE_PUP_CASE
             return;
         }
     }
-#define RVE_PUP_CASE(NCC, HC)                                                                           \
-    if (rv.nc == NCC && (rv.m > 0) == HC) {                                                             \
-        k_pupdate<T, NCC, HC><<<grid, block, 0, L.stream>>>(rv, r, p, q, cs, L.ncols, L.cpb, fi);       \
+#define RVE_PUP_CASE(NCC, HC, CL)                                                                       \
+    if (rv.nc == NCC && (rv.m > 0) == HC && (q != nullptr) == CL) {                                     \
+        k_pupdate<T, NCC, HC, CL><<<grid, block, 0, L.stream>>>(rv, r, p, q, cs, L.ncols, L.cpb, fi);   \
         return;                                                                                         \
     }
-    RVE_PUP_CASE(3, false) RVE_PUP_CASE(3, true) RVE_PUP_CASE(1, false) RVE_PUP_CASE(1, true)
+    RVE_PUP_CASE(3, false, true) RVE_PUP_CASE(3, true, true) RVE_PUP_CASE(1, false, true) RVE_PUP_CASE(1, true, true)
+    RVE_PUP_CASE(3, false, false) RVE_PUP_CASE(3, true, false) RVE_PUP_CASE(1, false, false) RVE_PUP_CASE(1, true, false)
 #undef RVE_PUP_CASE
 }
 template void launch_pupdate<float>(const RowView<float>&, float*, float*, float*, ColState, bool,

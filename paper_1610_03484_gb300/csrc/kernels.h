@@ -64,10 +64,6 @@ struct RowView {
     const T* diag = nullptr;          // [nfield][2 phases][n_rows], nfield = 1 (mech) or 2 (scalar)
     const uint8_t* mask = nullptr;    // [n_scalar_dofs] 1 = Dirichlet-constrained (or nullptr)
     const T* scale = nullptr;         // [ncols][2]
-    // optional inverse diagonal [n_rows][dinv_groups] (FP64 solves: a load instead of an
-    // FP64 division per entry), mechanics: one group per RVE, scalar: one per field
-    const T* dinv = nullptr;
-    int dinv_groups = 0;
     int nfield = 1;
     int nc = 3;
     // constraint rows (periodic / Neumann), FP64
@@ -76,6 +72,10 @@ struct RowView {
     const int64_t* sup_row = nullptr; // [n_sup] vector row
     const double* sup_coef = nullptr; // [n_sup][m]
     const int32_t* sup_of_row = nullptr;  // [n_rows] index into support or -1
+    // optional inverse diagonal [n_rows][dinv_groups] (FP64 solves: a load instead of an
+    // FP64 division per entry), mechanics: one group per RVE, scalar: one per field
+    const T* dinv = nullptr;
+    int dinv_groups = 0;
 };
 
 // Per-column PCG state, FP64, each array [ncols] unless noted.
