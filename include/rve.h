@@ -648,6 +648,13 @@ int rve_debug_set_node_bound(rve_ctx ctx, rve_mesh mesh, int64_t n_nodes);
  * eigenvalue, or the result is not finite. */
 int rve_debug_galerkin_solve(int n, const double* G, const double* g, double rel, double* c);
 
+/* The polynomial that preconditions the FP64 solves for an estimate lambda of the largest
+ * eigenvalue of D^-1 A and a condition number ratio: z = w D^-1 r, d = z, then per step
+ * (c1, c2) d = c1 d + c2 D^-1 (r - A z), z += d.  Returns the number of steps (of which
+ * at most max_steps pairs are written to c), or RVE_ERR_INVALID_ARGUMENT for lambda <= 0,
+ * ratio <= 1 or a null pointer.  Host only. */
+int rve_debug_chebyshev(double lambda, double ratio, int max_steps, double* w, float* c);
+
 #ifdef __cplusplus
 }
 #endif

@@ -179,6 +179,7 @@ _SIGS = {
                                    C.POINTER(C.c_int32), C.c_int]),
     "rve_debug_set_node_bound": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_galerkin_solve": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
+    "rve_debug_chebyshev": (C.c_int, [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_void_p]),
     "rve_operator_energy_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p,
                                               C.c_void_p]),
     "rve_surrogate_create": (C.c_int, [C.c_void_p, C.c_int, C.c_uint64, C.POINTER(C.c_void_p)]),
@@ -253,6 +254,14 @@ def galerkin_solve(G, g, rel: float = 1e-12) -> np.ndarray:
     _check(load_library().rve_debug_galerkin_solve(n, _ptr(G), _ptr(g), float(rel), _ptr(c)),
            "rve_debug_galerkin_solve")
     return c
+
+
+def chebyshev(lam: float, ratio: float):
+    """(w, [(c1, c2), ...]) of the polynomial preconditioner (rve_debug_chebyshev); host only."""
+    w, c = np.zeros(1), np.zeros((64, 2), np.float32)
+    n = load_library().rve_debug_chebyshev(float(lam), float(ratio), len(c), _ptr(w), _ptr(c))
+    _check(min(n, 0), "rve_debug_chebyshev")
+    return float(w[0]), c[:n]
 
 
 def default_options() -> Options:

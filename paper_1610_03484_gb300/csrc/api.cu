@@ -16,6 +16,7 @@
 
 #include "api_internal.h"
 #include "assembled.h"
+#include "chebyshev.h"
 #include "node_graph.h"
 
 namespace rve {
@@ -498,7 +499,7 @@ struct WarmStart {
 // takes the place of 12 of them (24x24x8, p = 2: 284 iterations in 89 ms before, 22 in 16
 // now).  The operator, the vectors, the inner products and the stopping test stay FP64,
 // so the solution is as accurate.  It covers [lambda / ratio, lambda] of the spectrum with
-// degree sqrt(ratio); the ratio follows the condition number, which grows with the square
+// the odd degree next to sqrt(ratio); the ratio follows the condition number, which grows with the square
 // of the nodes along a side.  Measured (ms a solve): 24x24x8, p = 2 (36 864 nodes, ratio
 // 277): degree 10, ratio 60 19.7; 14, 250 16.5; 18, 250 15.9; 6 x 6 x 4, p = 1 (144 nodes,
 // ratio 10): degree 6, ratio 15 1.60; 10, 60 1.90.
@@ -732,8 +733,8 @@ struct Solver {
         return RVE_OK;
     }
 
-    // Upper bound of the spectrum of D^-1 A of this field for any positive phase scales, by
-    // power iteration on each phase alone (see assembled.h).
+    // Estimate of the largest eigenvalue of D^-1 A of this field for any positive phase
+    // scales, by power iteration on each phase alone (see assembled.h).
     int ensure_lambda() {
         if (m->a_lambda[fid] > 0.0) return RVE_OK;
         const bool asm32 = use_assembled(m, false);
@@ -770,7 +771,8 @@ struct Solver {
         double lam = 0.0;
         for (int c = 0; c < 6; ++c)
             if (h[6 + c] > 0.0) lam = std::max(lam, h[c] / h[6 + c]);
-        // the quotient approaches the eigenvalue from below
+        // the quotient approaches the eigenvalue from below, and may still be under it with
+        // this margin (see chebyshev.h)
         m->a_lambda[fid] = std::isfinite(lam) && lam > 0.0 ? 1.15 * lam : 4.0;
         return RVE_OK;
     }
@@ -819,15 +821,9 @@ struct Solver {
             const size_t nvv = (size_t)n_rows * ncols;
             for (DevBuf* bfr : {&m->x32, &m->r32, &m->p32, &m->q32}) RVE_TRY(bfr->ensure(nvv * 4));
             if (cheb_asm) av32 = asm_view<float>(m, fid, m->scale32.as<float>());
-            const double hi = m->a_lambda[fid], ratio = cheb_ratio(n_rows / f.nc), lo = hi / ratio, th = 0.5 * (hi + lo), de = 0.5 * (hi - lo);
-            cheb_w = (float)(1.0 / th);
-            double rho = de / th;
-            const int degree = std::max(4, (int)std::lround(std::sqrt(ratio)));
-            for (int k = 1; k < degree; ++k) {
-                const double rn = 1.0 / (2.0 * th / de - rho);
-                cheb_c.emplace_back((float)(rn * rho), (float)(2.0 * rn / de));
-                rho = rn;
-            }
+            ChebPoly poly = chebyshev(m->a_lambda[fid], cheb_ratio(n_rows / f.nc));
+            cheb_w = (float)poly.w;
+            cheb_c = std::move(poly.steps);
         }
         const int kernels_per_iter = cheb ? 4 + (cheb_asm ? 1 : 2) * (int)cheb_c.size() : (fused ? 4 : 6);
         RVE_CUDA(cudaMemcpyAsync(const_cast<double*>(cs.tol), &tol, sizeof(double), cudaMemcpyHostToDevice, s));
@@ -1663,6 +1659,20 @@ int rve_debug_galerkin_solve(int n, const double* G, const double* g, double rel
     }
     for (int i = 0; i < n; ++i) c[i] = out[i];
     return RVE_OK;
+}
+
+int rve_debug_chebyshev(double lambda, double ratio, int max_steps, double* w, float* c) {
+    if (!(lambda > 0.0) || !(ratio > 1.0) || !w || !c) {
+        set_error("rve_debug_chebyshev: invalid argument");
+        return RVE_ERR_INVALID_ARGUMENT;
+    }
+    const ChebPoly p = chebyshev(lambda, ratio);
+    *w = p.w;
+    for (int k = 0; k < (int)p.steps.size() && k < max_steps; ++k) {
+        c[2 * k] = p.steps[k].first;
+        c[2 * k + 1] = p.steps[k].second;
+    }
+    return (int)p.steps.size();
 }
 
 // ns sources of the previous batch and the inner products of their span: P[lc][p][...] =

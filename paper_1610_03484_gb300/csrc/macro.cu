@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "chebyshev.h"
 #include "node_graph.h"
 
 struct rve_macro_s {
@@ -948,15 +949,15 @@ int macro_loop(rve_macro mm, int slot, const void* key, size_t key_bytes, int nf
 }
 
 // Polynomial of the elastic solve's preconditioner: it covers [lambda / ratio, lambda]
-// of the spectrum with degree sqrt(ratio).  Measured on the 200 x 40 x 10 plate (solve
+// of the spectrum with the odd degree next to sqrt(ratio).  Measured on the 200 x 40 x 10 plate (solve
 // and results): degree 10, ratio 100 36.4 ms; 18, 300 31.4; 24, 600 28.8; 32, 1500 26.9.
 // The condition number grows with the square of the nodes along the longest side, at
 // most as the 2/3 power of their number for a cube.
 double mech_cheb_ratio(int64_t nv) { return std::min(1500.0, std::max(10.0, 0.75 * std::pow((double)nv, 2.0 / 3.0))); }
 
-// Bound of the spectrum of D^-1 K by power iteration with the preconditioner's step
-// kernel, rounded up to eighths (the quotient approaches the eigenvalue from below, and
-// the captured loop's coefficients then stay the same from solve to solve).
+// Estimate of the largest eigenvalue of D^-1 K by power iteration with the preconditioner's
+// step kernel, rounded up to eighths (the quotient approaches the eigenvalue from below,
+// and the captured loop's coefficients then stay the same from solve to solve).
 template <class Step>
 int mech_spectrum(rve_macro m, int64_t n, Step step, double& lambda) {
     cudaStream_t s = m->ctx->stream;
@@ -995,20 +996,15 @@ int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product produc
     const uint8_t* mask = mm->mfix.as<uint8_t>();
     const double* dinv = mm->mdinv.as<double>();
     const unsigned gv = grid_for(n);
-    const double ratio = mech_cheb_ratio(mm->nv);
-    const int degree = std::max(4, (int)std::lround(std::sqrt(ratio)));
-    const double hi = lambda, lo = hi / ratio, th = 0.5 * (hi + lo), de = 0.5 * (hi - lo);
-    const float w = (float)(1.0 / th);
+    const ChebPoly poly = chebyshev(lambda, mech_cheb_ratio(mm->nv));
+    const float w = (float)poly.w;
+    const int n_steps = (int)poly.steps.size();
     // z = M^-1 r from z = w D^-1 r; returns the buffer that holds it
     auto precondition = [&](cudaStream_t st) -> const float* {
-        double rho = de / th;
-        for (int k = 0; k + 1 < degree; ++k) {
-            const double rn = 1.0 / (2.0 * th / de - rho);
-            step(st, MechCheb{zb[k & 1], zb[(k & 1) ^ 1], k == 0 ? zb[0] : d, d, r32, dinv32, r, (float)(rn * rho),
-                              (float)(2.0 * rn / de), k + 2 == degree ? acc : nullptr});
-            rho = rn;
-        }
-        return zb[(degree - 1) & 1];
+        for (int k = 0; k < n_steps; ++k)
+            step(st, MechCheb{zb[k & 1], zb[(k & 1) ^ 1], k == 0 ? zb[0] : d, d, r32, dinv32, r, poly.steps[k].first,
+                              poly.steps[k].second, k + 1 == n_steps ? acc : nullptr});
+        return zb[n_steps & 1];
     };
     RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
     product(s, x, q, nullptr);

@@ -1,0 +1,91 @@
+"""The polynomial preconditioner of the FP64 solves away from regular meshes and data."""
+import numpy as np
+import pytest
+
+import rve_inputs as ri
+from oracle import fem
+from oracle import macro as mo
+from oracle import materials as mt
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rve():
+    import paper_1610_03484_gb300 as pkg
+    from paper_1610_03484_gb300 import _build
+    _build.build()
+    pkg.load_library()
+    return pkg
+
+
+def isotropic(E=1.0, nu=0.3):
+    la, mu = E * nu / ((1 + nu) * (1 - 2 * nu)), E / (2 * (1 + nu))
+    C = np.zeros((6, 6))
+    C[:3, :3] = la
+    C[range(3), range(3)] += 2 * mu
+    C[range(3, 6), range(3, 6)] = mu
+    return C
+
+
+def plate_solve(rve, xyz, tets, C, rtol, max_iter, traction=(1e-3, 0.0, 0.0)):
+    """(stats, u, load) of a plate on rollers under a traction on its far end"""
+    with rve.Context() as ctx:
+        m = ctx.macro_load(xyz, tets)
+        m.mech_set_bc(xyz <= 1e-12)
+        m.mech_set_traction(xyz[:, 0] >= xyz[:, 0].max() * (1 - 1e-12), list(traction))
+        st = m.mech_solve(C, rtol=rtol, max_iter=max_iter)
+        r = m.mech_get()
+        m.free()
+    return st, r["u"], r["load"]
+
+
+def residual(xyz, tets, C, u, load):
+    """sqrt((r, D^-1 r) / (f, D^-1 f)) over the free DOFs"""
+    K = mo.elastic_assemble(xyz, tets, C)
+    free = ~(xyz <= 1e-12).reshape(-1)
+    f, d = load.reshape(-1)[free], K.diagonal()[free]
+    r = f - (K @ u.reshape(-1))[free]
+    return np.sqrt((r @ (r / d)) / (f @ (f / d)))
+
+
+def test_eigenvalue_above_the_estimate(rve):
+    """One tetrahedron 16 times as stiff, placed where the power iteration's start hardly
+    sees it: the largest eigenvalue of D^-1 K is 2.80, the estimate 2.75 (both by
+    arithmetic on the host).  49 665 nodes, for which sqrt(ratio) rounds to 32: a polynomial
+    of that degree is indefinite and takes 1364 iterations, where the uniform plate takes
+    36 and Jacobi preconditioning 904."""
+    grid = (104, 42, 10)
+    xyz, tets = ri.kuhn_grid(*grid, tuple(float(g) for g in grid))
+    C = np.broadcast_to(isotropic(), (len(tets), 4, 6, 6)).copy()
+    C[247260] *= 16.0
+    st, u, load = plate_solve(rve, xyz, tets, C, 1e-10, 250)
+    assert st["converged"] == 1
+    # (the recurrence's residual and the true one part at rounding level)
+    assert residual(xyz, tets, C, u, load) < 2e-10
+
+
+def distorted(grid, seed, amp=0.25):
+    """the box with its interior nodes displaced by up to amp cells"""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    rng = np.random.default_rng(seed)
+    inner = ((xyz > 1e-9) & (xyz < xyz.max(0) - 1e-9)).all(1)
+    xyz = xyz.copy()
+    xyz[inner] += amp * rng.uniform(-1, 1, (inner.sum(), 3)) * (xyz.max(0) / np.array(grid)) / 2
+    return xyz, tets, phase, tangent
+
+
+@pytest.mark.parametrize("grid,p", [((6, 6, 4), 1), ((9, 8, 6), 1), ((5, 4, 3), 2), ((3, 3, 2), 3)])
+def test_distorted_cells_match_oracle(rve, grid, p):
+    xyz, tets, phase, tangent = distorted(grid, 3)
+    mat, yarn = ri.NOMINAL_MATRIX, ri.NOMINAL_YARN
+    D, K, Dd = mt.element_tensors(phase, tangent, mat, yarn, w_matrix=float(mt.one_minus_omega(45.0, 1.0, 800.0)))
+    want = fem.homogenise(xyz, tets, grid, p, rve.BC_DIRICHLET, D, K, Dd)
+    with rve.Context(precision=rve.PREC_FP64, rtol=1e-11) as ctx:
+        m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+        m.set_materials(mat, yarn, T_C=45.0, c_wt=1.0, t_h=800.0)
+        m.set_bc(rve.BC_DIRICHLET)
+        r = m.homogenise()
+        m.free()
+    for got, ref in zip((r.C, r.K, r.D), want):
+        assert np.linalg.norm(got - ref) < 1e-10 * np.linalg.norm(ref)
