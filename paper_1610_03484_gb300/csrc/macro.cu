@@ -49,12 +49,12 @@ struct rve_macro_s {
     // [nt*4][6]
     rve::DevBuf mfix, mval, mload, mdinv, mu, cm, mmat, mmat32, cgp, msig;
     bool have_mech_bc = false, have_mech_load = false, have_mech_u = false, have_mech_sig = false;
-    // instantiated PCG loops (0 transport, 1 mechanics), reused while the captured
-    // launch parameters stay the same
+    // instantiated PCG loops (0 transport, 1 mechanics, 2 its Jacobi iteration), reused while
+    // the captured launch parameters stay the same
     struct Loop {
         cudaGraphExec_t exec = nullptr;
         std::vector<unsigned char> key;
-    } loop[2];
+    } loop[3];
     ~rve_macro_s() {
         for (auto& l : loop)
             if (l.exec) cudaGraphExecDestroy(l.exec);
@@ -181,12 +181,14 @@ __global__ void __launch_bounds__(256) k_transport_rhs(int64_t nv, int64_t n_sli
 //   [10] the same for the next iteration, [12] iterations, [14] (b, M^-1 b);
 //   [16] iterations of the loop, [17] their limit, [18] the squared tolerance,
 //   [20] (r, D^-1 r) of this iteration where M is not the Jacobi diagonal D (the stopping
-//   test's norm, also of [6] and [14]).
+//   test's norm, also of [6] and [14]); [22], [23] not 0: the iteration broke down (a
+//   direction without curvature; a preconditioned residual whose (r, z) is not positive);
+//   [24] the scale of the next residual in FP32.
 // An iteration is the product (which also moves (r, z) and the active flags on), the x/r
 // update, the preconditioner's steps if any and the p update (which also runs the loop
 // control).  Every scalar is written by one thread in a kernel whose other blocks do
 // not read it.
-constexpr int PCG_SCALARS = 22;
+constexpr int PCG_SCALARS = 25;
 
 // moves the scalars on to the next iteration; one thread per field of one block
 __device__ __forceinline__ void pcg_roll(double* acc, int f) {
@@ -194,6 +196,15 @@ __device__ __forceinline__ void pcg_roll(double* acc, int f) {
     acc[f] = 0.0;
     acc[20 + f] = 0.0;
     acc[8 + f] = acc[10 + f];
+}
+
+// The polynomial's residual is narrowed to FP32 times a power of two s that makes its norm
+// about 1, so that it stays inside FP32's range whatever the units and however far the
+// iteration has come.  With z = s M^-1 r and p = s (M^-1 r + beta p / s_old), alpha and beta
+// are the quotients of the (r, z) formed with that z, as without the scale.
+// rj: (r, D^-1 r).
+__device__ __forceinline__ double pcg_narrow_scale(double rj) {
+    return rj > 0.0 && isfinite(rj) ? ldexp(1.0, -(ilogb(rj) / 2)) : 1.0;
 }
 
 // block sums of up to two values per thread, added atomically to out[0..nf-1]
@@ -312,11 +323,16 @@ __global__ void __launch_bounds__(256) k_transport_update(int64_t nv, const uint
 template <int NF>
 __device__ __forceinline__ void pcg_tail(double* acc, int norm, cudaGraphConditionalHandle h, double (&beta)[NF],
                                          int (&on)[NF]) {
+    __shared__ int broke;
+    if (threadIdx.x == 0) broke = 0;
+    __syncthreads();
     if (threadIdx.x < NF) {
         const int f = threadIdx.x;
         const double rz = acc[f], old = acc[4 + f];
-        // converged (or not finite): the field stops
-        on[f] = acc[8 + f] != 0.0 && acc[norm + f] > acc[18] * acc[6 + f] && isfinite(rz);
+        const bool open = acc[8 + f] != 0.0 && acc[norm + f] > acc[18] * acc[6 + f];
+        const bool sound = rz > 0.0 && isfinite(rz);
+        if (open && !sound) broke = 1;
+        on[f] = open && sound && acc[22] == 0.0;
         beta[f] = old > 0.0 ? rz / old : 0.0;
     }
     __syncthreads();
@@ -328,6 +344,7 @@ __device__ __forceinline__ void pcg_tail(double* acc, int norm, cudaGraphConditi
             acc[2 + f] = 0.0;
             any = any || on[f];
         }
+        if (broke) acc[23] = 1.0;
         const double it = acc[16] + 1.0;
         acc[16] = it;
         cudaGraphSetConditional(h, any && it < acc[17] ? 1u : 0u);
@@ -352,90 +369,106 @@ __global__ void __launch_bounds__(256) k_transport_pupdate(int64_t nv, const dou
 
 // Convergence is relative to the larger of the right-hand side and the initial residual
 // (which carries the held values): a field already at rest (rounding-level residual)
-// takes no iteration.  One thread per field; `norm` as in pcg_tail.
-__global__ void k_macro_start(double* acc, int nf, int norm, double tol2, int max_iter) {
+// takes no iteration.  One thread per field; `norm` as in pcg_tail, ref a lower bound of
+// the reference.
+__global__ void k_macro_start(double* acc, int nf, int norm, double tol2, int max_iter, double ref) {
     const int f = threadIdx.x;
     const double rj = f < nf ? acc[norm + f] : 0.0, bb = f < nf ? acc[14 + f] : 0.0;
-    acc[6 + f] = fmax(bb, rj);
+    acc[6 + f] = fmax(fmax(bb, rj), ref);
     acc[10 + f] = rj > tol2 * acc[6 + f] ? 1.0 : 0.0;
     acc[2 + f] = 0.0;
     acc[12 + f] = 0.0;
     if (f == 0) {
+        if (norm) {   // the norm is formed again with the preconditioner's start
+            acc[24] = pcg_narrow_scale(rj);
+            acc[norm] = 0.0;
+        }
         acc[16] = 0.0;
         acc[17] = (double)max_iter;
         acc[18] = tol2;
     }
 }
 
-// The mechanics' vector passes around the Chebyshev preconditioner (below).
+// The mechanics' vector passes, with the Chebyshev preconditioner below (POLY) or Jacobi's;
+// the norm (r, D^-1 r) at acc[norm], which without the polynomial is (r, z) itself.
 //
-// r = b - y on free rows (0 on held rows), acc[20] += (r, D^-1 r) and acc[14] += (b, D^-1 b)
-// over the free rows; the preconditioner's start r32 = r, z = w D^-1 r
+// r = b - y on free rows (0 on held rows), acc[norm] += (r, D^-1 r) and acc[14] +=
+// (b, D^-1 b) over the free rows
 __global__ void __launch_bounds__(256) k_mech_residual(int64_t n, const double* __restrict__ b,
                                                        const double* __restrict__ y, const uint8_t* __restrict__ mask,
                                                        const double* __restrict__ dinv, double* __restrict__ r,
-                                                       float* __restrict__ r32, float* __restrict__ z,
-                                                       float* __restrict__ dinv32, float w, double* __restrict__ acc) {
+                                                       float* __restrict__ dinv32, int norm, double* __restrict__ acc) {
     double a[1] = {0.0}, bb[1] = {0.0};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const bool held = mask[i] != 0;
         const double bi = b[i], di = dinv[i];
         const double ri = held ? 0.0 : bi - y[i];
-        const float df = held ? 0.f : (float)di;   // the polynomial leaves held rows alone
         r[i] = ri;
-        r32[i] = (float)ri;
-        dinv32[i] = df;
-        z[i] = w * (df * (float)ri);
+        dinv32[i] = held ? 0.f : (float)di;   // the polynomial leaves held rows alone
         a[0] = fma(ri, ri * di, a[0]);
         if (!held) bb[0] = fma(bi, bi * di, bb[0]);
     }
-    block_add<1>(a, acc + 20);
+    block_add<1>(a, acc + norm);
     block_add<1>(bb, acc + 14);
 }
 
 // p = z
-__global__ void __launch_bounds__(256) k_mech_first(int64_t n, const float* __restrict__ z, double* __restrict__ p) {
+template <bool POLY>
+__global__ void __launch_bounds__(256) k_mech_first(int64_t n, const float* __restrict__ z, const double* __restrict__ r,
+                                                    const double* __restrict__ dinv, double* __restrict__ p) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = z[i];
+        p[i] = POLY ? (double)z[i] : r[i] * dinv[i];
 }
 
-// x += alpha p, r -= alpha q (held rows stay 0), acc[20] += (r, D^-1 r); the
-// preconditioner's start
+// x += alpha p, r -= alpha q (held rows stay 0), acc[norm] += (r, D^-1 r); POLY: the
+// preconditioner's start r32 = r, z = w D^-1 r (scaled).  Without a step (alpha 0: at the
+// start, or where the iteration breaks down) x and r stay as they are.
+template <bool POLY>
 __global__ void __launch_bounds__(256) k_mech_update(int64_t n, const uint8_t* __restrict__ mask,
                                                      const double* __restrict__ dinv, double* __restrict__ x,
                                                      double* __restrict__ r, const double* __restrict__ p,
                                                      const double* __restrict__ q, float* __restrict__ r32,
                                                      float* __restrict__ z, const float* __restrict__ dinv32, float w,
                                                      double* __restrict__ acc) {
-    __shared__ double alpha;
+    __shared__ double alpha, scale;
     if (threadIdx.x == 0) {
-        const double pq = acc[2];
-        alpha = acc[8] != 0.0 && pq > 0.0 ? acc[4] / pq : 0.0;
+        const double pq = acc[2], rz = acc[4];
+        const bool sound = pq > 0.0 && isfinite(pq) && rz > 0.0 && isfinite(rz / pq);
+        alpha = acc[8] != 0.0 && sound ? rz / pq : 0.0;
+        scale = acc[24];
+        if (blockIdx.x == 0 && acc[8] != 0.0 && !sound) acc[22] = 1.0;
     }
     __syncthreads();
-    const double al = alpha;
+    const double al = alpha, sc = scale;
     double a[1] = {0.0};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        x[i] = fma(al, p[i], x[i]);
-        const double ri = mask[i] ? 0.0 : fma(-al, q[i], r[i]);
-        const float rf = (float)ri;
-        r[i] = ri;
-        r32[i] = rf;
-        z[i] = w * (dinv32[i] * rf);
+        double ri = r[i];
+        if (al != 0.0) {
+            x[i] = fma(al, p[i], x[i]);
+            ri = mask[i] ? 0.0 : fma(-al, q[i], ri);
+            r[i] = ri;
+        }
+        if constexpr (POLY) {
+            const float rf = (float)(ri * sc);
+            r32[i] = rf;
+            z[i] = w * (dinv32[i] * rf);
+        }
         a[0] = fma(ri, ri * dinv[i], a[0]);
     }
-    block_add<1>(a, acc + 20);
+    block_add<1>(a, acc + (POLY ? 20 : 0));
 }
 
 // p = z + beta p; loop control
-__global__ void __launch_bounds__(256) k_mech_pupdate(int64_t n, const float* __restrict__ z, double* __restrict__ p,
+template <bool POLY>
+__global__ void __launch_bounds__(256) k_mech_pupdate(int64_t n, const float* __restrict__ z, const double* __restrict__ r,
+                                                      const double* __restrict__ dinv, double* __restrict__ p,
                                                       double* __restrict__ acc, cudaGraphConditionalHandle h) {
     __shared__ double beta[1];
     __shared__ int on[1];
-    pcg_tail<1>(acc, 20, h, beta, on);
+    pcg_tail<1>(acc, POLY ? 20 : 0, h, beta, on);
     if (!on[0]) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = fma(beta[0], p[i], (double)z[i]);
+        p[i] = fma(beta[0], p[i], POLY ? (double)z[i] : r[i] * dinv[i]);
 }
 
 // The elastic solve's preconditioner: a Chebyshev polynomial in D^-1 K evaluated in FP32
@@ -701,7 +734,7 @@ __global__ void __launch_bounds__(256) k_mech_entries(int64_t nv, const int64_t*
     }
 }
 
-// y = K x and (x, y) into acc[2].  A warp takes one of the three displacement
+// y = K x and (x, y) into acc[2] (norm: as in pcg_tail).  A warp takes one of the three displacement
 // components of a slice's 32 nodes (three warps share the slice's column indices and
 // gathered values in L1): three times the warps of one lane per node, which is what
 // covers the latency of the gathers.  Bound by the FP64 pipe.  acc null: the product
@@ -712,8 +745,11 @@ __global__ void __launch_bounds__(MECH_THREADS) k_mech_product(int64_t nv, int64
                                                                const int32_t* __restrict__ col,
                                                                const double* __restrict__ val,
                                                                const double* __restrict__ x, double* __restrict__ y,
-                                                               double* __restrict__ acc) {
-    if (acc && blockIdx.x == 0 && threadIdx.x == 0) pcg_roll(acc, 0);
+                                                               int norm, double* __restrict__ acc) {
+    if (acc && blockIdx.x == 0 && threadIdx.x == 0) {
+        if (norm) acc[24] = pcg_narrow_scale(acc[norm]);
+        pcg_roll(acc, 0);
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = warp % 3;
     double dot[1] = {0.0};
     for (int64_t s = (int64_t)blockIdx.x * (MECH_THREADS / 96) + warp / 3; s < n_slices;
@@ -900,10 +936,11 @@ int ensure_transport_matrix(rve_macro m, double dt_s) {
 // The PCG iterations of one problem (slot 0 transport, 1 mechanics) as a CUDA graph with
 // a conditional WHILE node that ends on the device: body(stream, handle) launches one
 // iteration.  The instantiated graph is kept while `key`, every captured pointer and
-// number, stays the same.  Then the iterations and final relative residuals per field.
+// number, stays the same.  Then the iterations and final relative residuals per field, the
+// first one's reference norm, and whether the iteration broke down.
 template <class Body>
 int macro_loop(rve_macro mm, int slot, const void* key, size_t key_bytes, int nf, int norm, Body body, int its[2],
-               double rel[2], bool& conv) {
+               double rel[2], bool& conv, double* ref = nullptr, bool* broke = nullptr) {
     cudaStream_t s = mm->ctx->stream;
     const unsigned char* kb = static_cast<const unsigned char*>(key);
     auto& loop = mm->loop[slot];
@@ -943,8 +980,12 @@ int macro_loop(rve_macro mm, int slot, const void* key, size_t key_bytes, int nf
     for (int f = 0; f < 2; ++f) {
         its[f] = f < nf ? (int)h[12 + f] : 0;
         rel[f] = f < nf && h[6 + f] > 0 ? std::sqrt(std::max(h[norm + f], 0.0) / h[6 + f]) : 0.0;
-        if (f < nf && h[10 + f] != 0.0) conv = false;
+        // (a field also stops where its residual is not finite or the iteration broke down)
+        if (f < nf && (h[10 + f] != 0.0 || !std::isfinite(h[norm + f]))) conv = false;
     }
+    if (h[22] != 0.0 || h[23] != 0.0) conv = false;
+    if (ref) *ref = h[6];
+    if (broke) *broke = h[22] != 0.0 || h[23] != 0.0;
     return RVE_OK;
 }
 
@@ -980,9 +1021,11 @@ int mech_spectrum(rve_macro m, int64_t n, Step step, double& lambda) {
     return RVE_OK;
 }
 
-// FP64 PCG of the elastic problem with the polynomial preconditioner: converged when
-// (r, D^-1 r) <= rtol^2 max((f, D^-1 f), (r0, D^-1 r0)) over the free rows.
-// product(stream, in, out, acc) forms out = K in and adds (in, out) to acc[2].
+// FP64 PCG of the elastic problem: converged when (r, D^-1 r) <= rtol^2 max((f, D^-1 f),
+// (r0, D^-1 r0)) over the free rows.  The polynomial preconditioner is evaluated in FP32;
+// where that breaks down (a stiffness outside FP32's range, 1e-38 to 1e38, makes
+// it so) the Jacobi iteration, all in FP64, takes over from the displacements reached.
+// product(stream, in, out, norm, acc) forms out = K in and adds (in, out) to acc[2].
 template <class Product, class Step>
 int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product product, Step step, double rtol,
              int max_iter, int its[2], double rel[2], bool& conv) {
@@ -1006,12 +1049,6 @@ int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product produc
                               poly.steps[k].second, k + 1 == n_steps ? acc : nullptr});
         return zb[n_steps & 1];
     };
-    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
-    product(s, x, q, nullptr);
-    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, r32, zb[0], dinv32, w, acc);
-    k_macro_start<<<1, 2, 0, s>>>(acc, 1, 20, rtol * rtol, max_iter);
-    k_mech_first<<<gv, 256, 0, s>>>(n, precondition(s), p);
-    RVE_CUDA(cudaGetLastError());
     struct Key {
         const void* ptr[14];
         double lambda;
@@ -1019,12 +1056,37 @@ int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product produc
     std::memset(&key, 0, sizeof(key));
     const void* ptrs[14] = {r, p, q, acc, x, mask, dinv, mm->mmat.p, mm->g_col.p, r32, zb[0], zb[1], d, mm->mmat32.p};
     std::memcpy(key.ptr, ptrs, sizeof(ptrs));
+    double ref = 0.0;
+    bool broke = false;
+    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+    product(s, x, q, 20, nullptr);
+    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, dinv32, 20, acc);
+    k_macro_start<<<1, 2, 0, s>>>(acc, 1, 20, rtol * rtol, max_iter, 0.0);
+    k_mech_update<true><<<gv, 256, 0, s>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
+    k_mech_first<true><<<gv, 256, 0, s>>>(n, precondition(s), r, dinv, p);
+    RVE_CUDA(cudaGetLastError());
     key.lambda = lambda;
-    return macro_loop(mm, 1, &key, sizeof(key), 1, 20, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
-        product(cap, p, q, acc);
-        k_mech_update<<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
-        k_mech_pupdate<<<gv, 256, 0, cap>>>(n, precondition(cap), p, acc, h);
-    }, its, rel, conv);
+    RVE_TRY(macro_loop(mm, 1, &key, sizeof(key), 1, 20, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+        product(cap, p, q, 20, acc);
+        k_mech_update<true><<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
+        k_mech_pupdate<true><<<gv, 256, 0, cap>>>(n, precondition(cap), r, dinv, p, acc, h);
+    }, its, rel, conv, &ref, &broke));
+    if (!broke || its[0] >= max_iter) return RVE_OK;
+    const int before = its[0];
+    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+    product(s, x, q, 0, nullptr);
+    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, dinv32, 0, acc);
+    k_macro_start<<<1, 2, 0, s>>>(acc, 1, 0, rtol * rtol, max_iter - before, ref);
+    k_mech_first<false><<<gv, 256, 0, s>>>(n, nullptr, r, dinv, p);
+    RVE_CUDA(cudaGetLastError());
+    key.lambda = 0.0;
+    RVE_TRY(macro_loop(mm, 2, &key, sizeof(key), 1, 0, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+        product(cap, p, q, 0, acc);
+        k_mech_update<false><<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, nullptr, nullptr, nullptr, 0.f, acc);
+        k_mech_pupdate<false><<<gv, 256, 0, cap>>>(n, nullptr, r, dinv, p, acc, h);
+    }, its, rel, conv));
+    its[0] += before;
+    return RVE_OK;
 }
 
 // FP64 Jacobi PCG of the transport pair; per field converged when (r, D^-1 r) <=
@@ -1042,7 +1104,7 @@ int transport_pcg(rve_macro mm, double2* x, const double2* b, Product product, d
     RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
     product(s, x, q, nullptr);
     k_transport_residual<<<gv, 256, 0, s>>>(nv, b, q, mask, dinv, r, p, acc);
-    k_macro_start<<<1, 2, 0, s>>>(acc, 2, 0, rtol * rtol, max_iter);
+    k_macro_start<<<1, 2, 0, s>>>(acc, 2, 0, rtol * rtol, max_iter, 0.0);
     RVE_CUDA(cudaGetLastError());
     const void* key[9] = {r, p, q, acc, x, mask, dinv, mm->t_mat.p, mm->g_col.p};
     return macro_loop(mm, 0, key, sizeof(key), 2, 0, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
@@ -1601,8 +1663,8 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
     k_mech_hold<<<grid_for(n), 256, 0, s>>>(n, m->mfix.as<uint8_t>(), m->mval.as<double>(), u);
     const double* mat = m->mmat.as<double>();
     const unsigned gm = (unsigned)std::min<int64_t>((m->n_slices + 1) / 2, (int64_t)sm_count() * 10);
-    auto product = [&](cudaStream_t st, const double* in, double* out, double* acc) {
-        k_mech_product<<<gm, MECH_THREADS, 0, st>>>(m->nv, m->n_slices, base, col, mat, in, out, acc);
+    auto product = [&](cudaStream_t st, const double* in, double* out, int norm, double* acc) {
+        k_mech_product<<<gm, MECH_THREADS, 0, st>>>(m->nv, m->n_slices, base, col, mat, in, out, norm, acc);
     };
     int its[2] = {0, 0};
     double rel[2] = {0, 0};

@@ -89,3 +89,28 @@ def test_distorted_cells_match_oracle(rve, grid, p):
         m.free()
     for got, ref in zip((r.C, r.K, r.D), want):
         assert np.linalg.norm(got - ref) < 1e-10 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
+def test_plate_in_any_units(rve, stiffness, force):
+    """The same plate with the stiffness and the traction in other units: the displacement
+    scales with force / stiffness.  Residuals far outside FP32's range, and (last two) a
+    matrix outside it, where the Jacobi iteration has to take over."""
+    xyz, tets = ri.kuhn_grid(9, 4, 3, (9.0, 4.0, 3.0))
+    C = np.broadcast_to(isotropic(), (len(tets), 4, 6, 6))
+    st0, u0, _ = plate_solve(rve, xyz, tets, C, 1e-11, 2000)
+    st, u, load = plate_solve(rve, xyz, tets, C * stiffness, 1e-11, 2000, (1e-3 * force, 0.0, 0.0))
+    assert st["converged"] == 1 and st["rel_residual"] <= 1e-11
+    if abs(np.log10(stiffness)) < 38:
+        assert st["iterations"] <= st0["iterations"] + 1
+    want = u0 * (force / stiffness)
+    assert np.linalg.norm(u - want) < 1e-9 * np.linalg.norm(want)
+
+
+def test_not_a_number_does_not_read_as_converged(rve):
+    xyz, tets = ri.kuhn_grid(5, 3, 2, (5.0, 3.0, 2.0))
+    C = np.broadcast_to(isotropic(), (len(tets), 4, 6, 6)).copy()
+    C[len(tets) // 2, 0, 0, 0] = np.nan
+    with pytest.raises(rve.RveError) as e:
+        plate_solve(rve, xyz, tets, C, 1e-11, 500)
+    assert e.value.code == -4
