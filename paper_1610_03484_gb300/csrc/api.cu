@@ -514,6 +514,8 @@ struct Solver {
     int64_t n_rows;
     int fid;   // 0 mechanics, 1 scalar fields
     bool free_rows = false;   // leave the constraint rows out (traction_start)
+    bool jacobi = false;      // FP64: Jacobi instead of the polynomial
+    bool broke = false;       // the last solve's polynomial broke down in some column
     double tighten = 1.0;     // factor on the tolerance of a mixed solve (sources of build_basis)
     Launch L;
     cudaStream_t s;
@@ -810,7 +812,7 @@ struct Solver {
             RVE_CUDA(cudaMemsetAsync(cs.pq_acc, 0, sizeof(double) * 3 * ACC_SLOTS * ncols, s));   // pq, rz and rj
         }
         // FP64 without constraint rows: polynomial preconditioner
-        const bool cheb = sizeof(T) == 8 && fused && !bounds_check_built();
+        const bool cheb = sizeof(T) == 8 && fused && !jacobi && !bounds_check_built();
         const bool cheb_asm = cheb && use_assembled(m, false);
         AsmView<float> av32;
         ChebArgs cha;
@@ -1144,11 +1146,24 @@ struct Solver {
             }
             conv = n_act == 0;
         }
-        std::vector<int32_t> its(ncols);
-        RVE_CUDA(cudaMemcpyAsync(its.data(), cs.iters, sizeof(int32_t) * ncols,
+        std::vector<int32_t> its(ncols + 1);   // the flags follow the iteration counts
+        RVE_CUDA(cudaMemcpyAsync(its.data(), cs.iters, sizeof(int32_t) * (ncols + 1),
                                  cudaMemcpyDeviceToHost, s));
         RVE_CUDA(cudaStreamSynchronize(s));
-        iters_out = *std::max_element(its.begin(), its.end());
+        iters_out = *std::max_element(its.begin(), its.end() - 1);
+        broke = (its[ncols] & 8) != 0;
+        if (broke) RVE_TRY(clear_flags(8));
+        return RVE_OK;
+    }
+
+    // clears bits of the solve's flags (nothing in flight uses them)
+    int clear_flags(int32_t bits) {
+        int32_t f = 0;
+        RVE_CUDA(cudaMemcpyAsync(&f, cs64.flags, sizeof(f), cudaMemcpyDeviceToHost, s));
+        RVE_CUDA(cudaStreamSynchronize(s));
+        f &= ~bits;
+        RVE_CUDA(cudaMemcpyAsync(cs64.flags, &f, sizeof(f), cudaMemcpyHostToDevice, s));
+        RVE_CUDA(cudaStreamSynchronize(s));
         return RVE_OK;
     }
 
@@ -1195,6 +1210,14 @@ struct Solver {
         return t;
     }
 
+    // x = 0, r = b
+    int cold_start(double* x64, double* r64) {
+        const size_t nv = (size_t)n_rows * ncols;
+        RVE_CUDA(cudaMemcpyAsync(r64, m->b64.p, nv * 8, cudaMemcpyDeviceToDevice, s));
+        RVE_CUDA(cudaMemsetAsync(x64, 0, nv * 8, s));
+        return RVE_OK;
+    }
+
     // Cold start of an FP64 uniform-traction solve.  The total field under the unit
     // traction modes c_j (the strain or flux rows of the constraint) needs no constraint
     // rows: K v_j = c_j is consistent and singular only by the rigid modes, so the
@@ -1218,6 +1241,7 @@ struct Solver {
                                    max_iter, iters, conv);
         free_rows = false;
         RVE_TRY(rc);
+        if (broke) return cold_start(x64, r64);
         // the constraint products of V per RVE, of the rigid modes and of the unit macro
         // fields (both live on the vertex nodes)
         const int nr = mr - ni;
@@ -1286,11 +1310,7 @@ struct Solver {
                     for (int j = 0; j < nr; ++j) mu[(size_t)b * 72 + 36 + j * 6 + 3 * fld + k] = A[ni + j][mr + k];
                 }
             }
-        if (!ok) {   // no usable start: from zero
-            RVE_CUDA(cudaMemcpyAsync(r64, m->b64.p, nv * 8, cudaMemcpyDeviceToDevice, s));
-            RVE_CUDA(cudaMemsetAsync(x64, 0, nv * 8, s));
-            return RVE_OK;
-        }
+        if (!ok) return cold_start(x64, r64);
         RVE_TRY(upload(m->traction_mu, mu.data(), mu.size(), s));
         RVE_TRY(upload(m->d_dof_vertex, m->map.dof_vertex.data(), m->map.dof_vertex.size(), s));
         launch_traction_combine(n_rows, f.nc, B, m->traction_mu.as<double>(), m->d_dof_vertex.as<int32_t>(),
@@ -1409,8 +1429,7 @@ struct Solver {
             RVE_TRY(zero_noise_columns());
             RVE_TRY(rel_residual(r64, bn, rel));
         } else {
-            RVE_CUDA(cudaMemcpyAsync(r64, b64, nv * 8, cudaMemcpyDeviceToDevice, s));
-            RVE_CUDA(cudaMemsetAsync(x64, 0, nv * 8, s));
+            RVE_TRY(cold_start(x64, r64));
             RVE_TRY(zero_noise_columns());
             last_rel.assign(ncols, 1.0);
             for (int c : zero_cols) last_rel[c] = 0.0;
@@ -1432,6 +1451,25 @@ struct Solver {
                 RVE_TRY(pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64,
                                     o.rtol / rel, o.max_iter, its, conv, &tolc));
                 out.iterations += its;
+                if (broke) {
+                    // The polynomial is evaluated in FP32: column scales outside its range
+                    // (a degradation factor below 1e-38) break it down.  The same solve
+                    // again with Jacobi, all in FP64.
+                    if (warm) {
+                        launch_combine_columns<double, double>(n_rows, ncols, warm->cols, warm->map, warm->coef,
+                                                               warm->x, x64, s);
+                        *launches += 1;
+                        RVE_TRY(residual64(x64, r64));
+                    } else {
+                        RVE_TRY(cold_start(x64, r64));
+                    }
+                    RVE_TRY(zero_noise_columns());
+                    jacobi = true;
+                    RVE_TRY(pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64,
+                                        o.rtol / rel, o.max_iter, its, conv, &tolc));
+                    jacobi = false;
+                    out.iterations += its;
+                }
                 RVE_TRY(residual64(x64, r64));
                 RVE_TRY(zero_noise_columns());
                 RVE_TRY(rel_residual(r64, bn, out.rel_res));

@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(256) k_cheb_update(RowView<double> rv, const f
             cs.alpha[col] = a;
             cs.iters[col] += 1;
         } else if (on == 2) {
-            atomicOr(cs.flags, 1);   // the loop control stops the column
+            atomicOr(cs.flags, 8);   // the loop control stops the column
             cs.beta[col] = -1.0;
         }
     }
@@ -629,8 +629,9 @@ __global__ void __launch_bounds__(256) k_cheb_vector(int64_t n_rows, int nfield,
 }
 
 // One block: per active column (r, z) and (r, D^-1 r) from their accumulators, beta and
-// the stopping test on the latter (rj <= tol^2 rz0 with rz0 its initial value); clears
-// the accumulators; with CTL the loop control of the graph's WHILE node.
+// the stopping test on the latter (rj <= tol^2 rz0 with rz0 its initial value); a column
+// whose (r, z) is not positive stops with flag bit 3, the breakdown of the preconditioner;
+// clears the accumulators; with CTL the loop control of the graph's WHILE node.
 template <bool CTL>
 __global__ void __launch_bounds__(1024) k_cheb_beta(ColState cs, int ncols, int first, cudaGraphConditionalHandle h,
                                                     int32_t* __restrict__ counter, int max_iter) {
@@ -651,15 +652,17 @@ __global__ void __launch_bounds__(1024) k_cheb_beta(ColState cs, int ncols, int 
             cs.active[c] = 0;
             continue;
         }
-        if (!isfinite(rz) || !isfinite(rj)) {
-            atomicOr(cs.flags, 1);
+        const bool done = first ? rj == 0.0 : rj <= tol * tol * cs.rz0[c];
+        const bool sound = rz > 0.0 && isfinite(rz);   // (not NaN)
+        if (!isfinite(rj)) atomicOr(cs.flags, 1);
+        else if (!done && !sound) atomicOr(cs.flags, 8);
+        if (done || !sound || !isfinite(rj)) {
             cs.active[c] = 0;
             continue;
         }
         cs.beta[c] = first ? 0.0 : rz / cs.rz[c];
         cs.rz[c] = rz;
-        if (!first && rj <= tol * tol * cs.rz0[c]) cs.active[c] = 0;
-        any = any || cs.active[c] != 0;
+        any = true;
     }
     const int more = __syncthreads_or(any ? 1 : 0);
     // the active columns in ascending order (the element operators take lanes for them)

@@ -88,7 +88,7 @@ struct ColState {
     double* schur;    // [ncols][m*m] inverse Cholesky factor of C M^-1 C^T
     int32_t* active;  // 1 while the column iterates
     int32_t* iters;   // iterations taken
-    int32_t* flags;   // [1] bit0: numeric error
+    int32_t* flags;   // [1] bit0: numeric error, bit3: breakdown of the FP64 solve's preconditioner
     int32_t* list;    // [ncols] the active columns in ascending order (compacted)
     int32_t* n_list;  // [1] their number
     const double* tol;  // [1] relative tolerance on sqrt(rz / rz0), in device memory so that a

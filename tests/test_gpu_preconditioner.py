@@ -91,6 +91,28 @@ def test_distorted_cells_match_oracle(rve, grid, p):
         assert np.linalg.norm(got - ref) < 1e-10 * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("grid,p,bc", [((5, 4, 3), 1, 1), ((4, 3, 2), 2, 1), ((4, 3, 2), 2, 0), ((3, 3, 2), 3, 0)])
+def test_degradation_factor_below_fp32(rve, grid, p, bc):
+    """Factors whose FP32 value is subnormal or zero, alone and among others in one batch:
+    the tensors approach those of a vanishing matrix (1e-20 already agrees to 1e-12)."""
+    W = np.array([0.7, 1e-20, 1e-37, 1e-39, 1e-42, 1e-60])
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    with rve.Context(precision=rve.PREC_FP64, rtol=1e-9) as ctx:
+        m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+        m.set_materials(ri.NOMINAL_MATRIX, ri.NOMINAL_YARN)
+        m.set_bc(bc)
+        batch = ctx.macro_update_w([m], W, np.zeros(len(W), np.int32))
+        single = [ctx.macro_update_w([m], W[i:i + 1], np.zeros(1, np.int32)) for i in range(len(W))]
+        m.free()
+    assert (batch[3] == 0).all()
+    for i in range(len(W)):
+        C = single[i][0][0]
+        assert np.linalg.norm(batch[0][i] - C) < 1e-10 * np.linalg.norm(C)
+        if i > 0:
+            ref = single[1][0][0]
+            assert np.linalg.norm(C - ref) < 1e-10 * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
 def test_plate_in_any_units(rve, stiffness, force):
     """The same plate with the stiffness and the traction in other units: the displacement
