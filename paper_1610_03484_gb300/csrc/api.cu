@@ -1157,10 +1157,12 @@ struct Solver {
     }
 
     // clears bits of the solve's flags (nothing in flight uses them)
-    int clear_flags(int32_t bits) {
+    int clear_flags(int32_t bits, bool* were_set = nullptr) {
         int32_t f = 0;
         RVE_CUDA(cudaMemcpyAsync(&f, cs64.flags, sizeof(f), cudaMemcpyDeviceToHost, s));
         RVE_CUDA(cudaStreamSynchronize(s));
+        if (were_set) *were_set = (f & bits) != 0;
+        if ((f & bits) == 0) return RVE_OK;
         f &= ~bits;
         RVE_CUDA(cudaMemcpyAsync(cs64.flags, &f, sizeof(f), cudaMemcpyHostToDevice, s));
         RVE_CUDA(cudaStreamSynchronize(s));
@@ -1237,11 +1239,16 @@ struct Solver {
         *launches += 1;
         bool conv = false;
         free_rows = true;
-        const int rc = pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64, 0.3 * rtol,
-                                   max_iter, iters, conv);
+        // The singular problem meets rounding at a few 1e-16, where its iterate drifts off in
+        // rigid modes or a direction has no curvature: it stops above that, and where it does
+        // not get there the constrained solve starts from zero; neither is an error of the call.
+        const int rc = pcg<double>(x64, r64, m->p64.as<double>(), m->q64.as<double>(), m->scale64,
+                                   std::max(0.3 * rtol, 3e-15), max_iter, iters, conv);
         free_rows = false;
         RVE_TRY(rc);
-        if (broke) return cold_start(x64, r64);
+        bool numeric = false;
+        RVE_TRY(clear_flags(1, &numeric));
+        if (broke || numeric || !conv) return cold_start(x64, r64);
         // the constraint products of V per RVE, of the rigid modes and of the unit macro
         // fields (both live on the vertex nodes)
         const int nr = mr - ni;
@@ -1317,8 +1324,13 @@ struct Solver {
                                 m->d_xyz.as<double>(), x64, s);
         *launches += 1;
         RVE_TRY(residual64(x64, r64));
-        RVE_TRY(rel_residual(r64, bn, rel));
-        return RVE_OK;
+        std::vector<double> rz;
+        RVE_TRY(rel_residual(r64, bn, rel, &rz));
+        for (int c = 0; c < ncols; ++c) ok = ok && (bn[c] == 0.0 || std::isfinite(rz[c]));
+        if (ok) return RVE_OK;
+        rel = 1.0;
+        for (int c = 0; c < ncols; ++c) last_rel[c] = bn[c] == 0.0 ? 0.0 : 1.0;
+        return cold_start(x64, r64);
     }
 
     // warm: optional starting data from the previous batch (see WarmStart).

@@ -113,6 +113,44 @@ def test_degradation_factor_below_fp32(rve, grid, p, bc):
             assert np.linalg.norm(C - ref) < 1e-10 * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("grid,p", [((4, 4, 2), 1), ((5, 4, 3), 2)])
+def test_uniform_traction_at_rounding_level(rve, grid, p):
+    """A tolerance at rounding level, which the unconstrained (singular) start of the uniform
+    traction cannot reach: the constrained solve decides, and answers as at 1e-13."""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    out = []
+    for rtol in (1e-13, 3e-16):
+        with rve.Context(precision=rve.PREC_FP64, rtol=rtol) as ctx:
+            m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+            m.set_materials(ri.NOMINAL_MATRIX, ri.NOMINAL_YARN, T_C=40.0, c_wt=1.0, t_h=2000.0)
+            m.set_bc(rve.BC_NEUMANN)
+            out.append(m.homogenise())
+            m.free()
+    for a, b in ((out[0].C, out[1].C), (out[0].K, out[1].K), (out[0].D, out[1].D)):
+        assert np.linalg.norm(a - b) < 1e-11 * np.linalg.norm(a)
+
+
+@pytest.mark.parametrize("grid,p,batch", [((4, 4, 3), 1, 3), ((4, 3, 2), 2, 2), ((3, 2, 2), 3, 4)])
+def test_uniform_traction_batches(rve, grid, p, batch):
+    """Several factors a batch: each RVE's own multipliers; against one call per factor in
+    the mixed precision of the same context, whose solves take no such start (1e-6: the
+    rounding of its element data)."""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    W = np.linspace(1.0, 0.2, 2 * batch + 1)
+    res = []
+    for prec, b, rtol in ((rve.PREC_FP64, batch, 1e-11), (rve.PREC_MIXED, 1, 1e-9)):
+        with rve.Context(precision=prec, rtol=rtol, batch=b, warm_start=0) as ctx:
+            m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+            m.set_materials(ri.NOMINAL_MATRIX, ri.NOMINAL_YARN)
+            m.set_bc(rve.BC_NEUMANN)
+            res.append(ctx.macro_update_w([m], W, np.zeros(len(W), np.int32)))
+            m.free()
+    assert (res[0][3] == 0).all()
+    for a, b in zip(res[0][:3], res[1][:3]):
+        for i in range(len(W)):
+            assert np.linalg.norm(a[i] - b[i]) < 1e-6 * np.linalg.norm(b[i]), i
+
+
 @pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
 def test_plate_in_any_units(rve, stiffness, force):
     """The same plate with the stiffness and the traction in other units: the displacement
