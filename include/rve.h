@@ -648,6 +648,11 @@ int rve_debug_set_node_bound(rve_ctx ctx, rve_mesh mesh, int64_t n_nodes);
  * eigenvalue, or the result is not finite. */
 int rve_debug_galerkin_solve(int n, const double* G, const double* g, double rel, double* c);
 
+/* Test hook: sets (1) or clears (0) the process-wide word in which the surrogate's kernels
+ * record that a bounded wait gave up, and returns the old value (-1 before the first
+ * surrogate).  While it is set, surrogate calls return RVE_ERR_TIMEOUT. */
+int rve_debug_gemm_timeout(int set);
+
 /* The polynomial that preconditions the FP64 solves for an estimate lambda of the largest
  * eigenvalue of D^-1 A and a condition number ratio: z = w D^-1 r, d = z, then per step
  * (c1, c2) d = c1 d + c2 D^-1 (r - A z), z += d.  Returns the number of steps (of which

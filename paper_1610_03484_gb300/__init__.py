@@ -179,6 +179,7 @@ _SIGS = {
                                    C.POINTER(C.c_int32), C.c_int]),
     "rve_debug_set_node_bound": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_galerkin_solve": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
+    "rve_debug_gemm_timeout": (C.c_int, [C.c_int]),
     "rve_debug_chebyshev": (C.c_int, [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_void_p]),
     "rve_operator_energy_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p,
                                               C.c_void_p]),

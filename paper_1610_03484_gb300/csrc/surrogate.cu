@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -96,7 +97,10 @@ __device__ __forceinline__ void tmem_ld16x(uint32_t taddr, uint32_t (&v)[16]) {
         : "memory");
 }
 
-__device__ int g_gemm_timeout;   // set when a bounded wait of the GEMM gave up
+// set when a bounded wait of the GEMM gave up: a word of pinned host memory, which the host
+// reads after any synchronisation without a copy of its own
+__device__ int* g_gemm_timeout;
+__device__ __forceinline__ void gemm_gave_up() { *(volatile int*)g_gemm_timeout = 1; }
 
 }  // namespace
 
@@ -124,7 +128,7 @@ __device__ int g_gemm_timeout;   // set when a bounded wait of the GEMM gave up
 //            quarter) x 32 columns of the finished accumulator, hands it back through
 //            "tmem empty" and runs bias / SiLU / conversion and the stores while
 //            the MMAs of the next tile fill the other accumulator.
-// Every wait is bounded; a role that gives up sets g_gemm_timeout and leaves its
+// Every wait is bounded; a role that gives up sets *g_gemm_timeout and leaves its
 // loop, after which the producer waits for its copies in flight and the MMA
 // issuer for its MMAs, so the tensor memory is idle when it is freed.
 template <int NT>
@@ -219,10 +223,10 @@ __global__ void __launch_bounds__(GemmShape<NT>::THREADS, 1)
                         : "memory");
                 }
             }
-            if (!ok) atomicOr(&g_gemm_timeout, 1);
+            if (!ok) gemm_gave_up();
             // the copies of the last min(S, it) steps may still be in flight
             for (int k = it - 1; k >= 0 && k >= it - S; --k)
-                if (!bar_wait(smem_addr(full + k % S), (k / S) & 1)) atomicOr(&g_gemm_timeout, 1);
+                if (!bar_wait(smem_addr(full + k % S), (k / S) & 1)) gemm_gave_up();
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -262,12 +266,12 @@ __global__ void __launch_bounds__(GemmShape<NT>::THREADS, 1)
                             smem_addr(tfull + acc))
                         : "memory");
             }
-            if (!ok) atomicOr(&g_gemm_timeout, 1);
+            if (!ok) gemm_gave_up();
             // every MMA issued has completed once this commit arrives
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              smem_addr(done))
                          : "memory");
-            if (!bar_wait(smem_addr(done), 0)) atomicOr(&g_gemm_timeout, 1);
+            if (!bar_wait(smem_addr(done), 0)) gemm_gave_up();
         }
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, column group (w - 2) / 4
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(GemmShape<NT>::THREADS, 1)
             if (lane == 0) w = bar_wait(smem_addr(tfull + acc), (i >> 1) & 1);
             w = __shfl_sync(0xffffffffu, w ? 1 : 0, 0) != 0;
             if (!w) {
-                if (lane == 0) atomicOr(&g_gemm_timeout, 1);
+                if (lane == 0) gemm_gave_up();
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -487,15 +491,15 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp_fused(const __grid_const
                         tma_2d(s_w + st * 32768, &P.w[e][l], kc * 64, 0, b_wfull + 8 * st);
                     }
                 }
-            if (!ok) atomicOr(&g_gemm_timeout, 1);
+            if (!ok) gemm_gave_up();
             // copies that may still be in flight: each slot's last feature tile and the
             // last weight chunks
             for (int sl = 0; sl < 2; ++sl) {
                 const int n = sl ? ns1 : ns0;
-                if (n >= 1 && !bar_wait(b_xfull + 8 * sl, (n - 1) & 1)) atomicOr(&g_gemm_timeout, 1);
+                if (n >= 1 && !bar_wait(b_xfull + 8 * sl, (n - 1) & 1)) gemm_gave_up();
             }
             for (int k = wit - 1; k >= 0 && k >= wit - 2; --k)
-                if (!bar_wait(b_wfull + 8 * (k & 1), (k >> 1) & 1)) atomicOr(&g_gemm_timeout, 1);
+                if (!bar_wait(b_wfull + 8 * (k & 1), (k >> 1) & 1)) gemm_gave_up();
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -540,10 +544,10 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp_fused(const __grid_const
                     mma_commit(b_acc + 8 * sl);
                     ++ks[sl];
                 }
-            if (!ok) atomicOr(&g_gemm_timeout, 1);
+            if (!ok) gemm_gave_up();
             // every MMA issued has completed once this commit arrives
             mma_commit(b_done);
-            if (!bar_wait(b_done, 0)) atomicOr(&g_gemm_timeout, 1);
+            if (!bar_wait(b_done, 0)) gemm_gave_up();
         }
     } else {
         // ---- epilogue: warps 2-9 serve slot 0, 10-17 slot 1; lane quarter q, column half h
@@ -564,7 +568,7 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp_fused(const __grid_const
                 if (lane == 0) w = bar_wait(b_acc + 8 * sl, ks & 1);
                 w = __shfl_sync(0xffffffffu, w ? 1 : 0, 0) != 0;
                 if (!w) {
-                    if (lane == 0) atomicOr(&g_gemm_timeout, 1);
+                    if (lane == 0) gemm_gave_up();
                     ok = false;
                     break;
                 }
@@ -668,10 +672,30 @@ static bool make_map(CUtensorMap* m, const __nv_bfloat16* base, int rows, int co
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-void gemm_tc_prepare() {
+namespace {
+std::atomic<int*> g_timeout_host{nullptr};   // the word g_gemm_timeout points to
+}
+
+cudaError_t gemm_tc_prepare() {
+    static std::mutex mu;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!g_timeout_host.load()) {
+            void* w = nullptr;
+            const cudaError_t e = cudaHostAlloc(&w, 64, cudaHostAllocPortable | cudaHostAllocMapped);
+            if (e != cudaSuccess) return e;
+            *static_cast<int*>(w) = 0;
+            g_timeout_host.store(static_cast<int*>(w));
+        }
+    }
+    void* d = nullptr;   // (each device keeps its own pointer to the one word)
+    cudaError_t e = cudaHostGetDevicePointer(&d, g_timeout_host.load(), 0);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_gemm_timeout, &d, sizeof(d));
+    if (e != cudaSuccess) return e;
     cudaFuncSetAttribute(k_gemm_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<128>());
     cudaFuncSetAttribute(k_gemm_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<64>());
     cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM);
+    return cudaSuccess;
 }
 
 int mlp_fused_max_members() { return MLP_MAXM; }
@@ -703,9 +727,16 @@ cudaError_t launch_mlp_fused(int M, int members, const __nv_bfloat16* X, const _
 }
 
 int gemm_tc_timed_out() {
-    int v = 0;
-    cudaMemcpyFromSymbol(&v, g_gemm_timeout, sizeof(int));
-    return v;
+    const int* w = g_timeout_host.load();
+    return w ? *const_cast<const volatile int*>(w) : 0;
+}
+
+int gemm_tc_set_timed_out(int v) {
+    int* w = g_timeout_host.load();
+    if (!w) return -1;
+    const int old = *const_cast<volatile int*>(w);
+    *const_cast<volatile int*>(w) = v;
+    return old;
 }
 
 // M a multiple of 64 (rows past a 128-row tile are zero-filled), N 64 or a multiple of

@@ -9,9 +9,11 @@
 namespace rve {
 
 // sets the GEMM kernels' shared-memory limit (once per device, before the first launch)
-void gemm_tc_prepare();
+cudaError_t gemm_tc_prepare();
 // nonzero once a bounded wait inside the GEMM gave up (sticky for the process)
 int gemm_tc_timed_out();
+// sets that word (tests) and returns the old one, -1 before gemm_tc_prepare
+int gemm_tc_set_timed_out(int v);
 // C = A Bt^T on the tensor cores (TMA-fed): problems of the same N and K in one launch,
 // each with its own M; an error if a tensor map cannot be encoded
 constexpr int GEMM_GROUP = 16;

@@ -70,6 +70,13 @@ struct rve_surrogate_s {
 
 namespace {
 
+// whether a bounded wait of the GEMMs gave up (call it after a synchronisation)
+int wait_status() {
+    if (!gemm_tc_timed_out()) return RVE_OK;
+    set_error("a bounded wait inside the surrogate GEMM gave up");
+    return RVE_ERR_TIMEOUT;
+}
+
 // the feature normalisation on the device
 int upload_norm(rve_surrogate s) {
     float h[16];
@@ -274,7 +281,7 @@ int rve_surrogate_create(rve_ctx c, int members, uint64_t seed, rve_surrogate* o
         set_error("rve_surrogate_create: members must be 1..16");
         return RVE_ERR_INVALID_ARGUMENT;
     }
-    gemm_tc_prepare();
+    RVE_CUDA(gemm_tc_prepare());
     auto* s = new rve_surrogate_s();
     s->ctx = c;
     s->members = members;
@@ -466,11 +473,7 @@ int rve_surrogate_train(rve_ctx c, rve_surrogate s, int64_t n, const double* fea
     RVE_CUDA(cudaGetLastError());
     if (loss_history) std::memcpy(loss_history, hist.data(), sizeof(double) * epochs);
     s->trained = true;
-    if (gemm_tc_timed_out()) {
-        set_error("a bounded wait inside the surrogate GEMM gave up");
-        return RVE_ERR_TIMEOUT;
-    }
-    return RVE_OK;
+    return wait_status();
 }
 
 int rve_surrogate_gradients(rve_ctx c, rve_surrogate s, int member, int n, const double* feat,
@@ -509,11 +512,7 @@ int rve_surrogate_gradients(rve_ctx c, rve_surrogate s, int member, int n, const
     RVE_CUDA(cudaMemcpyAsync(&l, dloss.p, 4, cudaMemcpyDeviceToHost, st));
     RVE_CUDA(cudaStreamSynchronize(st));
     if (loss) *loss = l;
-    if (gemm_tc_timed_out()) {
-        set_error("a bounded wait inside the surrogate GEMM gave up");
-        return RVE_ERR_TIMEOUT;
-    }
-    return RVE_OK;
+    return wait_status();
 }
 
 // Ensemble prediction on device features: member tensors, mean and spread.
@@ -563,7 +562,7 @@ static int predict_dev(rve_surrogate s, int64_t n, const double* feat_dev, doubl
     }
     RVE_CUDA(cudaGetLastError());
     RVE_CUDA(cudaStreamSynchronize(st));   // the outputs are complete when the call returns
-    return RVE_OK;
+    return wait_status();
 }
 
 int rve_surrogate_predict(rve_ctx c, rve_surrogate s, int64_t n, const double* feat, double* C, double* K,
@@ -589,10 +588,6 @@ int rve_surrogate_predict(rve_ctx c, rve_surrogate s, int64_t n, const double* f
     RVE_CUDA(cudaMemcpyAsync(D, dD.p, (size_t)n * 9 * 8, cudaMemcpyDeviceToHost, st));
     RVE_CUDA(cudaMemcpyAsync(spread, dsp.p, (size_t)n * 8, cudaMemcpyDeviceToHost, st));
     RVE_CUDA(cudaStreamSynchronize(st));
-    if (gemm_tc_timed_out()) {
-        set_error("a bounded wait inside the surrogate GEMM gave up");
-        return RVE_ERR_TIMEOUT;
-    }
     return RVE_OK;
 }
 
@@ -617,6 +612,8 @@ int rve_surrogate_predict_dev(rve_ctx c, rve_surrogate s, int64_t n, const doubl
     RVE_CUDA(cudaGetLastError());
     return RVE_OK;
 }
+
+int rve_debug_gemm_timeout(int set) { return gemm_tc_set_timed_out(set != 0 ? 1 : 0); }
 
 int rve_surrogate_get_params(rve_ctx c, rve_surrogate s, float* buf, int64_t* len) {
     RVE_TRY(check_ctx(c));
@@ -749,10 +746,7 @@ int macro_update_gauss_points_surrogate(rve_ctx c, const rve_mesh* meshes, const
         st->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         st->kernel_launches = c->launches - l0;
     }
-    if (gemm_tc_timed_out()) {
-        set_error("a bounded wait inside the surrogate GEMM gave up");
-        return RVE_ERR_TIMEOUT;
-    }
+    RVE_TRY(wait_status());
     return rc;
 }
 

@@ -118,3 +118,31 @@ def test_loss_history_is_reproducible(rve, members, n, batch):
         runs.append((hist, buf1))
     np.testing.assert_array_equal(runs[0][0], runs[1][0])
     np.testing.assert_array_equal(runs[0][1], runs[1][1])
+
+
+def test_a_wait_that_gave_up_is_reported_by_every_call(rve):
+    """The status word set on the host, as the kernels set it: training, gradients and both
+    forms of the inference answer RVE_ERR_TIMEOUT, and work again once it is cleared."""
+    import torch
+    feat, C, K, D = data(128, 9)
+    with rve.Context() as ctx:
+        s = rve.Surrogate(ctx, members=2, seed=3)
+        s.train(feat, C, K, D, epochs=1, batch=64, lr=1e-3, seed=1)
+        f = torch.tensor(feat, device="cuda")
+        out = [torch.zeros(len(feat), k, dtype=torch.float64, device="cuda") for k in (36, 9, 9, 1)]
+        calls = [lambda: s.predict(feat),
+                 lambda: s.predict_dev(len(feat), f.data_ptr(), *(v.data_ptr() for v in out)),
+                 lambda: s.train(feat, C, K, D, epochs=1, batch=64, lr=1e-3, seed=1),
+                 lambda: s.gradients(0, feat[:64], np.ones((64, 33), np.float32))]
+        lib = rve.load_library()
+        assert lib.rve_debug_gemm_timeout(1) == 0
+        try:
+            for call in calls:
+                with pytest.raises(rve.RveError) as e:
+                    call()
+                assert e.value.code == -10
+        finally:
+            assert lib.rve_debug_gemm_timeout(0) == 1
+        for call in calls:
+            call()
+        s.free()
