@@ -407,9 +407,9 @@ void run_product(const AsmView<T>& A, const T* x, const T* b, T* y, int ncols, c
     k_asm_product<T, NC, VEC, KS, MODE><<<dim3(gx, (unsigned)gy), ASM_THREADS, 0, s>>>(A, x, b, y, ncols, active, eacc, ch);
 }
 
-// d[row][g] = 1 / (s_0 diag_0 + s_1 diag_1), 0 on Dirichlet rows
+// d[row][g] = 1 / (s_0 diag_0 + s_1 diag_1), 0 on Dirichlet rows; times f in FP32
 __global__ void __launch_bounds__(256) k_jacobi_inverse(RowView<double> rv, int groups, double* __restrict__ dinv,
-                                                        float* __restrict__ dinv32) {
+                                                        float* __restrict__ dinv32, double f32) {
     const int64_t n = rv.n_rows * groups;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t row = i / groups;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256) k_jacobi_inverse(RowView<double> rv, int 
         d = d > 0.0 ? 1.0 / d : 0.0;
         if (rv.mask && rv.mask[row / rv.nc]) d = 0.0;
         dinv[i] = d;
-        if (dinv32) dinv32[i] = (float)d;
+        if (dinv32) dinv32[i] = (float)(f32 * d);
     }
 }
 
@@ -493,10 +493,11 @@ void launch_asm_residual(int nc, const AsmView<T>& A, const T* x, const T* b, T*
 template void launch_asm_residual<double>(int, const AsmView<double>&, const double*, const double*, double*, int,
                                           cudaStream_t);
 
-void launch_jacobi_inverse(const RowView<double>& rv, int groups, double* dinv, float* dinv32, cudaStream_t s) {
+void launch_jacobi_inverse(const RowView<double>& rv, int groups, double* dinv, float* dinv32, double f32,
+                           cudaStream_t s) {
     const int64_t n = rv.n_rows * groups;
     const int64_t b = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 8));
-    k_jacobi_inverse<<<(unsigned)b, 256, 0, s>>>(rv, groups, dinv, dinv32);
+    k_jacobi_inverse<<<(unsigned)b, 256, 0, s>>>(rv, groups, dinv, dinv32, f32);
 }
 
 void launch_cheb_step(int nc, const AsmView<float>& A, const float* z, const float* r32, float* z_new,

@@ -53,8 +53,9 @@ void launch_asm_residual(int nc, const AsmView<T>& A, const T* x, const T* b, T*
 
 // dinv [n_rows][groups]: inverse Jacobi diagonal of the column groups that share one
 // (mechanics: the RVEs; scalar fields: conductivity, diffusivity); dinv32 (optional)
-// the same in FP32
-void launch_jacobi_inverse(const RowView<double>& rv, int groups, double* dinv, float* dinv32, cudaStream_t s);
+// the same times f32 in FP32
+void launch_jacobi_inverse(const RowView<double>& rv, int groups, double* dinv, float* dinv32, double f32,
+                           cudaStream_t s);
 
 // One step of the Chebyshev iteration for A z = r from z_0 = 0 with the Jacobi diagonal:
 //   d_k = c1 d_(k-1) + c2 D^-1 (r - A z_k),  z_(k+1) = z_k + d_k

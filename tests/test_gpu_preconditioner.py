@@ -151,6 +151,32 @@ def test_uniform_traction_batches(rve, grid, p, batch):
             assert np.linalg.norm(a[i] - b[i]) < 1e-6 * np.linalg.norm(b[i]), i
 
 
+@pytest.mark.parametrize("grid,p", [((6, 6, 4), 1), ((4, 4, 3), 2)])
+def test_one_mesh_through_many_materials(rve, grid, p):
+    """What a mesh keeps from solve to solve (matrix entries, the spectrum's estimate, the
+    captured loop) against a fresh mesh for every call: new constituents, the same ones in
+    another state, boundary conditions with and without a change of the DOF map."""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    a = (ri.NOMINAL_MATRIX, ri.NOMINAL_YARN)
+    b = ri.jitter_props(5)
+    c = ri.jitter_props(6, frac=0.4)
+    calls = [(a, 40.0, 500.0, 1), (b, 40.0, 500.0, 1), (b, 60.0, 9000.0, 1), (b, 60.0, 9000.0, 0), (b, 60.0, 9000.0, 2),
+             (c, 60.0, 9000.0, 2), (c, 60.0, 100.0, 0), (a, 40.0, 500.0, 1), (a, 40.0, 500.0, 1)]
+    with rve.Context(precision=rve.PREC_FP64, rtol=1e-11) as ctx:
+        kept = ctx.mesh_load(xyz, tets, p, phase, tangent)
+        for props, T, t, bc in calls:
+            got = []
+            for m in (kept, ctx.mesh_load(xyz, tets, p, phase, tangent)):
+                m.set_materials(*props, T_C=T, c_wt=1.0, t_h=t)
+                m.set_bc(bc)
+                got.append(m.homogenise())
+            m.free()
+            for x, y in ((got[0].C, got[1].C), (got[0].K, got[1].K), (got[0].D, got[1].D)):
+                assert np.linalg.norm(x - y) < 1e-11 * np.linalg.norm(y)
+            assert abs(got[0].stats["iterations_mech"] - got[1].stats["iterations_mech"]) <= 1
+        kept.free()
+
+
 @pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
 def test_plate_in_any_units(rve, stiffness, force):
     """The same plate with the stiffness and the traction in other units: the displacement
