@@ -162,14 +162,18 @@ typedef struct rve_stats {
     double  hill_mandel_scalar;
     double  seconds;              /* wall time of the call */
     int64_t kernel_launches;      /* device kernels launched by the call */
-    double  op_ms;                /* summed device time of operator launches (profile mode) */
+    double  op_ms;                /* summed device time of operator launches (profile mode); in
+                                     FP64 solves also the FP32 products of the preconditioner, with
+                                     the vector step that each carries or that follows it */
     int64_t op_launches;          /* operator launches counted in op_ms */
     double  op_bytes;             /* algorithmic bytes of those launches: x read + y written
                                      (2 n_rows ncols sizeof(real)) + element data or matrix once */
     double  op_flops;             /* algorithmic flops of those launches (FMA = 2) */
     /* profile mode, the PCG vector kernels of the same iterations: */
-    double  update_ms, update_bytes;     /* x, r read+written, p, q read (6 n_rows ncols s) */
-    double  pupdate_ms, pupdate_bytes;   /* r, p read, p, q written (4 n_rows ncols s) */
+    double  update_ms, update_bytes;     /* x, r read+written, p, q read (6 n_rows ncols s); with the
+                                            polynomial preconditioner also r, z written in FP32 */
+    double  pupdate_ms, pupdate_bytes;   /* r, p read, p, q written (4 n_rows ncols s); with it z read
+                                            in FP32 in the place of r */
     double  finalize_ms;                 /* alpha and beta/multiplier kernels */
     /* profile mode, outside the PCG iterations: */
     double  residual_ms;                 /* true residual r = b - K x: FP64 operator (FP64 mode) or

@@ -864,6 +864,18 @@ struct Solver {
         }
         const int nby32 = cheb && !cheb_asm ? operator_grid_y<float>(m->p, f.nc, L, m->nt) : 0;
         if (cheb && !cheb_asm) RVE_CUDA(cudaMemsetAsync(m->q32.p, 0, (size_t)n_rows * ncols * 4, s));
+        // profile mode: 7 events bracket the operator, alpha, update, preconditioner, beta and
+        // p-update launches of an iteration
+        if (prof && (int)m->ctx->ev.size() < 7) {
+            for (int k = (int)m->ctx->ev.size(); k < 7; ++k) {
+                cudaEvent_t e;
+                RVE_CUDA(cudaEventCreate(&e));
+                m->ctx->ev.push_back(e);
+            }
+        }
+        auto evr = [&](int i, cudaStream_t st) {
+            if (prof) cudaEventRecord(m->ctx->ev[i], st);
+        };
         // z = M^-1 r by the Chebyshev polynomial; returns the buffer that holds it
         auto precondition = [&](const Launch& Lx, bool apply) -> const float* {
             const float* z = m->x32.as<float>();
@@ -871,6 +883,7 @@ struct Solver {
                 float* zb[2] = {m->x32.as<float>(), m->p32.as<float>()};
                 float* d = m->q32.as<float>();
                 launch_cheb_update(rvw, cha.dinv, x, r, p, q, m->r32.as<float>(), zb[0], cheb_w, cs, apply, Lx);
+                evr(6, Lx.stream);
                 const int n = (int)cheb_c.size();
                 if (!cheb_asm) {
                     // element by element: z in place, the products in q32
@@ -930,18 +943,6 @@ struct Solver {
             n_act = 0;
             for (int c = 0; c < ncols; ++c) n_act += act[c] != 0;
             return RVE_OK;
-        };
-        // profile mode: 6 events bracket the operator, alpha, update, beta and
-        // p-update launches of an iteration
-        if (prof && (int)m->ctx->ev.size() < 6) {
-            for (int k = (int)m->ctx->ev.size(); k < 6; ++k) {
-                cudaEvent_t e;
-                RVE_CUDA(cudaEventCreate(&e));
-                m->ctx->ev.push_back(e);
-            }
-        }
-        auto evr = [&](int i, cudaStream_t st) {
-            if (prof) cudaEventRecord(m->ctx->ev[i], st);
         };
         // in the graph body the compaction also runs the loop control
         bool loop_ctl = false;
@@ -1118,15 +1119,21 @@ struct Solver {
                 const int na = n_act_run;
                 // (the assembled operator: its entries once)
                 const double entries = (double)m->a_entries;
-                const double bytes =
-                    2.0 * n_rows * na * sz +
-                    (use_asm ? entries * ((nc == 3 ? 9 : 2) * sz + 4)
-                             : (double)m->nt * (4.0 * ne + 10 * sz + (nc == 3 ? 21 : 6) * sz + 1));
+                auto op_bytes = [&](bool as, double w) {
+                    return 2.0 * n_rows * na * w +
+                           (as ? entries * ((nc == 3 ? 9 : 2) * w + 4)
+                               : (double)m->nt * (4.0 * ne + 10 * w + (nc == 3 ? 21 : 6) * w + 1));
+                };
                 // FMAs per element and column: forward and backward contractions with the
                 // non-zero entries of the edge/face table, plus per-mode gradient, stress
                 // and back-mapping
                 const double fma = 2.0 * table_nonzeros(m->p) * nc + nmod * (18.0 * nc + (nc == 3 ? 36 : 9));
-                const double flops = 2.0 * na * (use_asm ? entries * nc * nc : fma * (double)m->nt);
+                auto op_flops = [&](bool as) { return 2.0 * na * (as ? entries * nc * nc : fma * (double)m->nt); };
+                // the operator's product, and the polynomial's in FP32 (each timed with the
+                // vector step that it carries or that follows it)
+                const int n_poly = cheb ? (int)cheb_c.size() : 0;
+                const double bytes = op_bytes(use_asm, sz) + n_poly * op_bytes(cheb_asm, 4.0);
+                const double flops = op_flops(use_asm) + n_poly * op_flops(cheb_asm);
                 const double vb = (double)n_rows * na * sz;
                 auto el = [&](int a2, int b2) {
                     float ms = 0;
@@ -1134,25 +1141,25 @@ struct Solver {
                                                                                                     : 0.0;
                 };
                 ProfCounters& pc = m->ctx->prof;
-                const double op_ms = el(0, 1);
+                const double op_ms = el(0, 1) + (cheb ? el(6, 3) : 0.0);
                 pc.op_ms += op_ms;
-                pc.op_launches++;
+                pc.op_launches += 1 + n_poly;
                 pc.op_bytes += bytes;
                 pc.op_flops += flops;
                 pc.op_cols += na;
                 pc.op_cols_all += ncols;
                 const int cl = 2 * (m->p - 1) + (nc == 3 ? 0 : 1);
                 pc.cls_ms[cl] += op_ms;
-                pc.cls_launches[cl]++;
+                pc.cls_launches[cl] += 1 + n_poly;
                 pc.cls_bytes[cl] += bytes;
                 pc.cls_flops[cl] += flops;
                 pc.cls_cols[cl] += na;
                 pc.cls_cols_all[cl] += ncols;
                 pc.fin_ms += el(1, 2) + el(3, 4);
-                pc.upd_ms += el(2, 3);
-                pc.upd_bytes += 6 * vb;
+                pc.upd_ms += cheb ? el(2, 6) : el(2, 3);
+                pc.upd_bytes += 6 * vb + (cheb ? vb : 0.0);   // (and r, z in FP32)
                 pc.pup_ms += el(4, 5);
-                pc.pup_bytes += 4 * vb;
+                pc.pup_bytes += cheb ? 2.5 * vb + (q_add ? vb : 0.0) : 4 * vb;   // (z in FP32)
             }
             conv = n_act == 0;
         }

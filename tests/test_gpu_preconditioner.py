@@ -177,6 +177,25 @@ def test_one_mesh_through_many_materials(rve, grid, p):
         kept.free()
 
 
+@pytest.mark.parametrize("grid,p,bc", [((6, 6, 4), 1, 1), ((5, 5, 4), 2, 0), ((3, 3, 2), 3, 1)])
+def test_profile_counts_the_preconditioners_products(rve, grid, p, bc):
+    """FP64 in profile mode: an iteration is one FP64 product and the polynomial's FP32
+    products (degree 5 at these sizes: four), all operator launches; their time is the
+    operator's, not the update pass's."""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    with rve.Context(precision=rve.PREC_FP64, rtol=1e-10, profile=1) as ctx:
+        m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+        m.set_materials(ri.NOMINAL_MATRIX, ri.NOMINAL_YARN, T_C=40.0, c_wt=1.0, t_h=500.0)
+        m.set_bc(bc)
+        m.homogenise()
+        st = m.homogenise().stats
+        m.free()
+    n = st["iterations_mech"] + st["iterations_scalar"]
+    assert st["op_launches"] == 5 * n
+    # one pass over at most 9 vectors, against five products: some slack for launch gaps
+    assert st["update_ms"] < 0.7 * st["op_ms"]
+
+
 @pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
 def test_plate_in_any_units(rve, stiffness, force):
     """The same plate with the stiffness and the traction in other units: the displacement
