@@ -642,6 +642,10 @@ int rve_debug_bounds(rve_ctx ctx, int32_t* checking_build, int64_t* violations, 
  * while every access that does run stays inside the mesh's arrays. */
 int rve_debug_set_node_bound(rve_ctx ctx, rve_mesh mesh, int64_t n_nodes);
 
+/* Test hook: the entries of the mesh's assembled matrix may take this many bytes (0: a
+ * quarter of the free device memory).  Above it solves keep the element operators. */
+int rve_debug_set_matrix_limit(rve_ctx ctx, rve_mesh mesh, int64_t bytes);
+
 /* The small solve of the energy-optimal warm start (warm_start = 4): the energy
  * minimisation of Sec. 2 restricted to the span of n previous solutions gives
  * G c = g with G_pk = x_p . A x_k and g_p = x_p . b.  c = G^+ g for the symmetric part

@@ -177,6 +177,7 @@ _SIGS = {
     "rve_mesh_get_colouring": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(C.c_int32)]),
     "rve_debug_bounds": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int64), C.POINTER(C.c_int64),
                                    C.POINTER(C.c_int32), C.c_int]),
+    "rve_debug_set_matrix_limit": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_set_node_bound": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_galerkin_solve": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
     "rve_debug_gemm_timeout": (C.c_int, [C.c_int]),
@@ -682,6 +683,9 @@ class Mesh:
         _check(self.ctx.lib.rve_mesh_get_colouring(self.ctx.h, self.h, _ptr(col), C.byref(n)),
                "rve_mesh_get_colouring")
         return col, n.value
+
+    def debug_set_matrix_limit(self, n_bytes: int):
+        _check(self.ctx.lib.rve_debug_set_matrix_limit(self.ctx.h, self.h, int(n_bytes)), "rve_debug_set_matrix_limit")
 
     def debug_set_node_bound(self, n_nodes: int):
         _check(self.ctx.lib.rve_debug_set_node_bound(self.ctx.h, self.h, int(n_nodes)), "rve_debug_set_node_bound")

@@ -123,6 +123,7 @@ int bounds_outcome(int rc, cudaStream_t s) {
 // The assembled entries and the spectrum's estimate follow the map and the constituents (at
 // unit modulus: not the degradation state, and not the boundary condition as such).
 void drop_assembled(rve_mesh m) {
+    m->a_refused = false;
     for (auto& row : m->a_valid) row[0] = row[1] = false;
     m->a_lambda[0] = m->a_lambda[1] = 0.0;
 }
@@ -398,7 +399,7 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
 // solve vectors, as with the element operators.
 bool use_assembled(rve_mesh m, bool fp64) {
     const int64_t ne = n_local(m->p);
-    return m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built() &&
+    return !m->a_refused && m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built() &&
            m->nt * ne * ne <= (int64_t)1 << 29;
 }
 
@@ -413,8 +414,23 @@ int ensure_assembled(rve_mesh m, int fid, bool fp64, cudaStream_t s) {
     const bool want32 = (!fp64 || use_assembled(m, false)) && !m->a_valid[fid][1];
     const int w64 = fid == 0 ? AsmEntry<double, 3>::WORDS : AsmEntry<double, 1>::WORDS;
     const int w32 = fid == 0 ? AsmEntry<float, 3>::WORDS : AsmEntry<float, 1>::WORDS;
-    if (want64) RVE_TRY(m->a_ent[fid][0].ensure((size_t)m->a_entries * w64 * 8));
-    if (want32) RVE_TRY(m->a_ent[fid][1].ensure((size_t)m->a_entries * w32 * 4));
+    const size_t b64 = want64 ? (size_t)m->a_entries * w64 * 8 : 0, b32 = want32 ? (size_t)m->a_entries * w32 * 4 : 0;
+    size_t room = m->a_limit, need = b64 + b32;
+    if (room == 0) {
+        const size_t held64 = m->a_ent[fid][0].bytes, held32 = m->a_ent[fid][1].bytes;
+        need = (b64 > held64 ? b64 : 0) + (b32 > held32 ? b32 : 0);
+        if (need > 0) {
+            size_t all = 0;
+            RVE_CUDA(cudaMemGetInfo(&room, &all));
+            room /= 4;
+        }
+    }
+    if (need > room) {
+        set_error("the assembled matrix does not fit");
+        return RVE_ERR_OUT_OF_MEMORY;
+    }
+    if (want64) RVE_TRY(m->a_ent[fid][0].ensure(b64));
+    if (want32) RVE_TRY(m->a_ent[fid][1].ensure(b32));
     RVE_TRY(m->a_rtab.ensure((size_t)9 * ne * ne * 8));
     AsmGraph g;
     g.n = m->map.N;
@@ -434,6 +450,25 @@ int ensure_assembled(rve_mesh m, int fid, bool fp64, cudaStream_t s) {
     m->ctx->launches++;
     if (want64) m->a_valid[fid][0] = true;
     if (want32) m->a_valid[fid][1] = true;
+    return RVE_OK;
+}
+
+// The same where the memory allows it: a matrix takes a quarter of the free memory at most
+// (the solve's vectors, other meshes' matrices and solves want room too).  Where it does not
+// fit or an allocation fails, the mesh keeps the element operators, which need none of it,
+// until its map or constituents change.
+int try_assembled(rve_mesh m, int fid, bool fp64, cudaStream_t s) {
+    if (!use_assembled(m, fp64)) return RVE_OK;
+    const int rc = ensure_assembled(m, fid, fp64, s);
+    if (rc != RVE_ERR_OUT_OF_MEMORY) return rc;
+    cudaGetLastError();
+    RVE_CUDA(cudaStreamSynchronize(s));
+    drop_assembled(m);
+    m->a_refused = true;
+    m->a_graph_valid = false;
+    for (auto& row : m->a_ent)
+        for (DevBuf& b : row) b.release();
+    for (DevBuf* b : {&m->a_order, &m->a_ptr, &m->a_split, &m->a_col, &m->a_eptr, &m->a_inc}) b->release();
     return RVE_OK;
 }
 
@@ -820,7 +855,17 @@ struct Solver {
             RVE_CUDA(cudaMemsetAsync(cs.pq_acc, 0, sizeof(double) * 3 * ACC_SLOTS * ncols, s));   // pq, rz and rj
         }
         // FP64 without constraint rows: polynomial preconditioner
-        const bool cheb = sizeof(T) == 8 && fused && !jacobi && !bounds_check_built();
+        bool cheb = sizeof(T) == 8 && fused && !jacobi && !bounds_check_built();
+        if (cheb)   // (its four FP32 vectors, 16 bytes an entry: without room for them Jacobi)
+            for (DevBuf* bfr : {&m->x32, &m->r32, &m->p32, &m->q32}) {
+                const int rc = bfr->ensure((size_t)n_rows * ncols * 4);
+                if (rc == RVE_ERR_OUT_OF_MEMORY) {
+                    cudaGetLastError();
+                    cheb = false;
+                    break;
+                }
+                RVE_TRY(rc);
+            }
         const bool cheb_asm = cheb && use_assembled(m, false);
         AsmView<float> av32;
         ChebArgs cha;
@@ -828,8 +873,6 @@ struct Solver {
         std::vector<std::pair<float, float>> cheb_c;
         if (cheb) {
             RVE_TRY(ensure_lambda());
-            const size_t nvv = (size_t)n_rows * ncols;
-            for (DevBuf* bfr : {&m->x32, &m->r32, &m->p32, &m->q32}) RVE_TRY(bfr->ensure(nvv * 4));
             if (cheb_asm) av32 = asm_view<float>(m, fid, m->scale32.as<float>());
             // The polynomial is that of D^-1 A / lambda: lambda goes into the FP32 inverse
             // diagonal, and the captured loop does not depend on it (a new capture for every
@@ -1357,6 +1400,7 @@ struct Solver {
         const rve_options& o = m->ctx->opt;
         const bool mixed = precision == RVE_PREC_MIXED;
         RVE_TRY(alloc(mixed));
+        if (!mixed || assembled32()) RVE_TRY(try_assembled(m, fid, !mixed, s));
         const size_t nv = (size_t)n_rows * ncols;
         double* x64 = m->x64f[fid].as<double>();
         double* r64 = m->r64f[fid].as<double>();
@@ -2915,7 +2959,12 @@ static int macro_update_impl(rve_ctx c, const rve_mesh* meshes, int n_meshes, in
             if (rc0 != RVE_OK) return fail(rc0);
             const rve_stats before = stm ? *stm : rve_stats();
             const int rc = homogenise_batch(m, WARM_BASIS, dw, nullptr, nullptr, nullptr, stm, w_src.data(), BASIS_BUILD);
-            if (rc != RVE_OK && rc != RVE_ERR_NOT_CONVERGED && rc != RVE_ERR_NUMERIC) return fail(rc);
+            if (rc != RVE_OK && rc != RVE_ERR_NOT_CONVERGED && rc != RVE_ERR_NUMERIC && rc != RVE_ERR_OUT_OF_MEMORY)
+                return fail(rc);
+            if (rc == RVE_ERR_OUT_OF_MEMORY) {   // give the sources' buffers back
+                cudaGetLastError();
+                for (DevBuf* b : {&m->warm_xs64, &m->warm_xs, &m->warm_kx, &m->warm_klo}) b->release();
+            }
             if (rc != RVE_OK) {
                 // no usable sources: the points start cold and answer for themselves
                 if (stm) *stm = before;
@@ -3559,6 +3608,17 @@ int rve_debug_bounds(rve_ctx c, int32_t* checking_build, int64_t* violations, in
     if (first_element) *first_element = fe;
     if (first_column) *first_column = fc;
     if (reset && bounds_reset() != 0) return RVE_ERR_CUDA;
+    return RVE_OK;
+}
+
+int rve_debug_set_matrix_limit(rve_ctx c, rve_mesh m, int64_t bytes) {
+    RVE_TRY(check_ctx(c));
+    if (!m || bytes < 0) {
+        set_error("rve_debug_set_matrix_limit: invalid argument");
+        return RVE_ERR_INVALID_ARGUMENT;
+    }
+    m->a_limit = (size_t)bytes;
+    drop_assembled(m);
     return RVE_OK;
 }
 

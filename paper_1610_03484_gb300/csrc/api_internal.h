@@ -211,6 +211,8 @@ struct rve_mesh_s {
     rve::DevBuf a_order, a_ptr, a_split, a_col, a_eptr, a_inc, a_rtab, a_ent[2][2];
     int64_t a_entries = 0;
     bool a_graph_valid = false, a_valid[2][2] = {{false, false}, {false, false}};
+    bool a_refused = false;   // the matrix did not fit: element operators
+    size_t a_limit = 0;       // bytes its entries may take (0: by the free memory)
     rve::DevBuf dinv64, dinv32;   // inverse Jacobi diagonal of the FP64 solve in progress
     double a_lambda[2] = {0, 0};  // per field: bound of the spectrum of D^-1 A (0: not formed)
     rve::DevBuf d_dof_vertex, traction_mu;   // uniform traction: original vertex of each node, multipliers

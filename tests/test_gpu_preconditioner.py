@@ -196,6 +196,30 @@ def test_profile_counts_the_preconditioners_products(rve, grid, p, bc):
     assert st["update_ms"] < 0.7 * st["op_ms"]
 
 
+@pytest.mark.parametrize("grid,p,bc,prec", [((6, 6, 4), 1, 1, 0), ((5, 4, 3), 2, 0, 0), ((5, 4, 3), 2, 2, 0),
+                                            ((16, 15, 6), 1, 1, 1)])
+def test_matrix_without_room(rve, grid, p, bc, prec):
+    """No room for the matrix' entries: the element operators answer, as before there was a
+    matrix; and with room again the matrix does."""
+    xyz, tets, phase, tangent = ri.weave_rve(*grid)
+    W = np.linspace(1.0, 0.3, 18 if prec else 2)
+    res = []
+    with rve.Context(precision=prec, rtol=1e-9, batch=18 if prec else 2) as ctx:
+        m = ctx.mesh_load(xyz, tets, p, phase, tangent)
+        m.set_materials(ri.NOMINAL_MATRIX, ri.NOMINAL_YARN)
+        m.set_bc(bc)
+        for limit in (0, 1000, 0):
+            m.debug_set_matrix_limit(limit)
+            res.append(ctx.macro_update_w([m], W, np.zeros(len(W), np.int32)))
+        m.free()
+    tol = 1e-6 if prec else 1e-12   # (mixed: FP32 element data against an FP32 matrix)
+    for other in res[1:]:
+        assert (other[3] == 0).all()
+        for a, b in zip(res[0][:3], other[:3]):
+            assert np.linalg.norm(a - b) < tol * np.linalg.norm(b)
+    assert res[1][4]["kernel_launches"] != res[0][4]["kernel_launches"]
+
+
 @pytest.mark.parametrize("stiffness,force", [(1.0, 1e-60), (1.0, 1e60), (1e11, 1e-40), (1e45, 1e45), (1e-45, 1e-45)])
 def test_plate_in_any_units(rve, stiffness, force):
     """The same plate with the stiffness and the traction in other units: the displacement
