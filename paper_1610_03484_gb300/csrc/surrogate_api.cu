@@ -61,7 +61,8 @@ struct rve_surrogate_s {
     // per member: FP32 master params, Adam moments, BF16 weights in both layouts
     std::vector<DevBuf> P, M1, M2, Wt, Wn;
     DevBuf d_norm, d_diag;   // feature mean and inverse std [16]; diagonal entries
-    DevBuf train_work;       // training buffers of all members (TrainWork)
+    DevBuf train_work;       // training buffers of the members trained together (TrainWork)
+    size_t work_limit = 0;   // bytes they may take (0: what the device has)
     // inference: the fused kernel (all members' layers per tile, activations on chip)
     // or one GEMM launch per member and layer
     bool fused = true;
@@ -144,6 +145,10 @@ int train_work(rve_surrogate s, int nm, int M, TrainWork& w) {
             w.lpart[e] = reinterpret_cast<float*>(take((size_t)head_loss_parts(M, NOUTP) * 4));
         }
         if (pass == 0) {
+            if (s->work_limit > 0 && nm > 1 && off > s->work_limit) {
+                set_error("training buffers above their limit");
+                return RVE_ERR_OUT_OF_MEMORY;
+            }
             RVE_TRY(s->train_work.ensure(off));
             base = s->train_work.as<char>();
         }
@@ -253,12 +258,13 @@ int forward_backward(rve_surrogate s, int first, int nm, int M, const TrainWork&
     return RVE_OK;
 }
 
-void adam_step(rve_surrogate s, int nm, const TrainWork& w, float lr, int step) {
+// Adam for the members first .. first + nm - 1
+void adam_step(rve_surrogate s, int first, int nm, const TrainWork& w, float lr, int step) {
     AdamJobs J;
     int nj = 0;
     for (int e = 0; e < nm; ++e)
         for (int l = 0; l < NLAYER; ++l) {
-            AdamJob j = adam_job(s, e, l);
+            AdamJob j = adam_job(s, first + e, l);
             j.Gt = w.gradT[e][l];
             j.gb = w.gradb[e][l];
             if (l == NLAYER - 1) j.n_valid = NOUT;
@@ -421,47 +427,60 @@ int rve_surrogate_train(rve_ctx c, rve_surrogate s, int64_t n, const double* fea
     for (int o = 0; o < NOUT; ++o) s->sigma[o] = 1.f;
     // ---- device data: features and targets once, the row order of every epoch
     const int M = batch, nm = s->members;
+    // The members train together; where their buffers (13 KB a row of the batch and member) do
+    // not fit, in groups one after the other, which changes nothing but the time: each member
+    // has its own row order and weights.
     TrainWork w;
-    RVE_TRY(train_work(s, nm, M, w));
+    int group = nm;
+    for (;;) {
+        const int rc = train_work(s, group, M, w);
+        if (rc == RVE_OK) break;
+        if (rc != RVE_ERR_OUT_OF_MEMORY || group == 1) return rc;
+        cudaGetLastError();
+        group = (group + 1) / 2;
+    }
     DevBuf dfeat, dtgt, dsig, dperm, dloss;
     RVE_TRY(upload_norm(s));
     RVE_TRY(upload(dfeat, feat, (size_t)n * 8, st));
     RVE_TRY(upload(dtgt, tgt.data(), tgt.size(), st));
     RVE_TRY(upload(dsig, s->sigma, NOUT, st));
-    RVE_TRY(dperm.ensure((size_t)nm * n * 4));
+    RVE_TRY(dperm.ensure((size_t)group * n * 4));
     RVE_TRY(dloss.ensure((size_t)epochs * nm * 4));
     RVE_CUDA(cudaMemsetAsync(dloss.p, 0, (size_t)epochs * nm * 4, st));
     const int64_t steps_per_epoch = n / M;
-    std::vector<std::mt19937_64> rng;
-    std::vector<std::vector<int64_t>> perm(nm);
-    std::vector<int32_t> order((size_t)nm * n);
-    for (int e = 0; e < nm; ++e) {
-        rng.emplace_back(seed * 7919ull + (uint64_t)e);
-        perm[e].resize(n);
-        std::iota(perm[e].begin(), perm[e].end(), 0);
-    }
-    int step = 0;
-    for (int ep = 0; ep < epochs; ++ep) {
-        for (int e = 0; e < nm; ++e) {
-            std::shuffle(perm[e].begin(), perm[e].end(), rng[e]);
-            for (int64_t i = 0; i < n; ++i) order[(size_t)e * n + i] = (int32_t)perm[e][i];
+    std::vector<std::vector<int64_t>> perm(group);
+    std::vector<int32_t> order((size_t)group * n);
+    for (int first = 0; first < nm; first += group) {
+        const int k = std::min(group, nm - first);
+        std::vector<std::mt19937_64> rng;
+        for (int e = 0; e < k; ++e) {
+            rng.emplace_back(seed * 7919ull + (uint64_t)(first + e));
+            perm[e].resize(n);
+            std::iota(perm[e].begin(), perm[e].end(), 0);
         }
-        // (a copy from pageable memory has left the vector when the call returns)
-        RVE_CUDA(cudaMemcpyAsync(dperm.p, order.data(), order.size() * 4, cudaMemcpyHostToDevice, st));
-        for (int64_t b = 0; b < steps_per_epoch; ++b) {
-            const int32_t* rows[MAX_MEMBERS];
-            float* loss[MAX_MEMBERS];
-            for (int e = 0; e < nm; ++e) {
-                rows[e] = dperm.as<int32_t>() + (size_t)e * n + b * M;
-                loss[e] = dloss.as<float>() + (size_t)ep * nm + e;
+        int step = 0;
+        for (int ep = 0; ep < epochs; ++ep) {
+            for (int e = 0; e < k; ++e) {
+                std::shuffle(perm[e].begin(), perm[e].end(), rng[e]);
+                for (int64_t i = 0; i < n; ++i) order[(size_t)e * n + i] = (int32_t)perm[e][i];
             }
-            RVE_TRY(forward_backward(s, 0, nm, M, w, dfeat.as<double>(), dtgt.as<float>(), dsig.as<float>(), rows,
-                                     loss));
-            ++step;
-            // cosine decay of the learning rate over all steps
-            const double total = (double)epochs * steps_per_epoch;
-            const double lr_t = lr * (0.02 + 0.98 * 0.5 * (1.0 + std::cos(M_PI * (step - 1) / total)));
-            adam_step(s, nm, w, (float)lr_t, step);
+            // (a copy from pageable memory has left the vector when the call returns)
+            RVE_CUDA(cudaMemcpyAsync(dperm.p, order.data(), (size_t)k * n * 4, cudaMemcpyHostToDevice, st));
+            for (int64_t b = 0; b < steps_per_epoch; ++b) {
+                const int32_t* rows[MAX_MEMBERS];
+                float* loss[MAX_MEMBERS];
+                for (int e = 0; e < k; ++e) {
+                    rows[e] = dperm.as<int32_t>() + (size_t)e * n + b * M;
+                    loss[e] = dloss.as<float>() + (size_t)ep * nm + first + e;
+                }
+                RVE_TRY(forward_backward(s, first, k, M, w, dfeat.as<double>(), dtgt.as<float>(), dsig.as<float>(),
+                                         rows, loss));
+                ++step;
+                // cosine decay of the learning rate over all steps
+                const double total = (double)epochs * steps_per_epoch;
+                const double lr_t = lr * (0.02 + 0.98 * 0.5 * (1.0 + std::cos(M_PI * (step - 1) / total)));
+                adam_step(s, first, k, w, (float)lr_t, step);
+            }
         }
     }
     std::vector<float> lsum((size_t)epochs * nm);
@@ -610,6 +629,13 @@ int rve_surrogate_predict_dev(rve_ctx c, rve_surrogate s, int64_t n, const doubl
     if (n == 0) return RVE_OK;
     RVE_TRY(predict_dev(s, n, feat_dev, C_dev, K_dev, D_dev, spread_dev));
     RVE_CUDA(cudaGetLastError());
+    return RVE_OK;
+}
+
+int rve_debug_surrogate_work_limit(rve_ctx c, rve_surrogate s, int64_t bytes) {
+    RVE_TRY(check_ctx(c));
+    if (!s || bytes < 0) return RVE_ERR_INVALID_ARGUMENT;
+    s->work_limit = (size_t)bytes;
     return RVE_OK;
 }
 

@@ -146,3 +146,21 @@ def test_a_wait_that_gave_up_is_reported_by_every_call(rve):
         for call in calls:
             call()
         s.free()
+
+
+@pytest.mark.parametrize("members,at_once", [(5, 3), (4, 1), (16, 8)])
+def test_members_trained_in_groups(rve, members, at_once):
+    """Too little room for all members' training buffers: they train in groups, with the
+    parameters and the history of training together, to the bit."""
+    feat, C, K, D = data(256, members)
+    per_member = 64 * 13_320 + 4 * 230_464   # bytes for batches of 64 rows
+    out = []
+    for limit in (0, int(per_member * (at_once + 0.5))):
+        with rve.Context() as ctx:
+            s = rve.Surrogate(ctx, members=members, seed=5)
+            assert ctx.lib.rve_debug_surrogate_work_limit(ctx.h, s.h, limit) == 0
+            hist = s.train(feat, C, K, D, epochs=2, batch=64, lr=1e-3, seed=1)
+            out.append((np.asarray(hist), s.get_params()))
+            s.free()
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
