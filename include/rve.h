@@ -656,6 +656,10 @@ int rve_debug_set_matrix_limit(rve_ctx ctx, rve_mesh mesh, int64_t bytes);
  * eigenvalue, or the result is not finite. */
 int rve_debug_galerkin_solve(int n, const double* G, const double* g, double rel, double* c);
 
+/* Test hook: the macro mesh's graph and matrices may each take this many bytes (0: a quarter
+ * of the free device memory).  Above it its operators are applied element by element. */
+int rve_debug_macro_matrix_limit(rve_ctx ctx, rve_macro m, int64_t bytes);
+
 /* Test hook: the training buffers of the members that train together may take this many
  * bytes (0: what the device has); above it the members train in smaller groups. */
 int rve_debug_surrogate_work_limit(rve_ctx ctx, rve_surrogate s, int64_t bytes);

@@ -181,6 +181,7 @@ _SIGS = {
     "rve_debug_set_node_bound": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_galerkin_solve": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
     "rve_debug_surrogate_work_limit": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
+    "rve_debug_macro_matrix_limit": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
     "rve_debug_gemm_timeout": (C.c_int, [C.c_int]),
     "rve_debug_chebyshev": (C.c_int, [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_void_p]),
     "rve_operator_energy_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p,

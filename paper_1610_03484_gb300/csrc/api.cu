@@ -335,8 +335,13 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
     NodeGraph g;
     if (!build_node_graph(m->map.edofs.data(), m->nt, ne, m->phase.data(), N, g)) {
         set_error("mesh too large for 32-bit matrix indices");
-        return RVE_ERR_INVALID_ARGUMENT;
+        return RVE_ERR_OUT_OF_MEMORY;
     }
+    for (int64_t i = 0; i < N; ++i)
+        if (g.ptr[i + 1] - g.ptr[i] > 4096) {   // (one warp assembles a row)
+            set_error("a node couples to too many others");
+            return RVE_ERR_OUT_OF_MEMORY;
+        }
     std::vector<float> cen((size_t)m->nt * 3);
     float lo[3] = {HUGE_VALF, HUGE_VALF, HUGE_VALF}, hi[3] = {-HUGE_VALF, -HUGE_VALF, -HUGE_VALF};
     for (int64_t e = 0; e < m->nt; ++e)

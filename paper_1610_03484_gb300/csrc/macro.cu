@@ -39,6 +39,8 @@ struct rve_macro_s {
     int64_t n_slices = 0, n_ell = 0;
     rve::DevBuf g_base, g_col, g_len, g_eptr, g_inc;
     bool have_graph = false;
+    bool element_form = false;   // no matrices: the operators element by element
+    size_t mat_limit = 0;        // bytes the graph and the matrices may take (0: by the free memory)
     rve::DevBuf t_mass, t_stiff, t_mat, t_dinv;
     rve::DevBuf c_r, c_z, c_z2, c_d, c_dinv;   // FP32 vectors of the elastic preconditioner
     bool have_stiff = false;
@@ -175,6 +177,72 @@ __global__ void __launch_bounds__(256) k_transport_rhs(int64_t nv, int64_t n_sli
     if (i < nv) b[i] = make_double2(capT * at, capC * ac);
 }
 
+// ---------------------------------------------------------- element form
+// Without room for the matrices (or past their 32-bit indices) both operators are applied
+// element by element, one per thread, with FP64 atomics: see apply_element_form.
+
+// y += (capacity + stiffness) x over both fields
+__global__ void __launch_bounds__(256) k_transport_apply(int64_t nt, const int32_t* __restrict__ tets,
+                                                         const double* __restrict__ geo, TransportTensors prm,
+                                                         double capT, double capC, int stiff,
+                                                         const double2* __restrict__ x, double2* __restrict__ y) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
+        int v[4];
+        double2 xa[4], sum = make_double2(0.0, 0.0);
+        double gt[3] = {0, 0, 0}, gc[3] = {0, 0, 0};
+        const double vol = geo[e * 13];
+        const double* g = geo + e * 13 + 1;   // grad lambda_a, [4][3]
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            v[a] = tets[e * 4 + a];
+            xa[a] = x[v[a]];
+            sum.x += xa[a].x;
+            sum.y += xa[a].y;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                gt[i] = fma(g[a * 3 + i], xa[a].x, gt[i]);
+                gc[i] = fma(g[a * 3 + i], xa[a].y, gc[i]);
+            }
+        }
+        double ft[3], fc[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            ft[i] = stiff ? vol * (sym3(prm.KT, i, 0) * gt[0] + sym3(prm.KT, i, 1) * gt[1] + sym3(prm.KT, i, 2) * gt[2]) : 0.0;
+            fc[i] = stiff ? vol * (sym3(prm.Dc, i, 0) * gc[0] + sym3(prm.Dc, i, 1) * gc[1] + sym3(prm.Dc, i, 2) * gc[2]) : 0.0;
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const double* ga = g + a * 3;
+            atomicAdd(&y[v[a]].x, capT * vol / 20.0 * (sum.x + xa[a].x) + ga[0] * ft[0] + ga[1] * ft[1] + ga[2] * ft[2]);
+            atomicAdd(&y[v[a]].y, capC * vol / 20.0 * (sum.y + xa[a].y) + ga[0] * fc[0] + ga[1] * fc[1] + ga[2] * fc[2]);
+        }
+    }
+}
+
+// its diagonal, added into d
+__global__ void __launch_bounds__(256) k_transport_diag(int64_t nt, const int32_t* __restrict__ tets,
+                                                        const double* __restrict__ geo, TransportTensors prm,
+                                                        double capT, double capC, double2* __restrict__ d) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nt * 4; k += (int64_t)gridDim.x * blockDim.x) {
+        const double vol = geo[(k >> 2) * 13];
+        const double* g = geo + (k >> 2) * 13 + 1 + (k & 3) * 3;
+        double kt = capT / 10.0, kc = capC / 10.0;
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) {
+                kt += g[i] * sym3(prm.KT, i, j) * g[j];
+                kc += g[i] * sym3(prm.Dc, i, j) * g[j];
+            }
+        atomicAdd(&d[tets[k]].x, vol * kt);
+        atomicAdd(&d[tets[k]].y, vol * kc);
+    }
+}
+
+// d = 1 / d, 0 where d is 0 (nodes of no element)
+__global__ void __launch_bounds__(256) k_invert(int64_t n, double* __restrict__ d) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        if (d[i] != 0.0) d[i] = 1.0 / d[i];
+}
+
 // Scalars of the PCG loop (doubles in device memory).  Two fields each:
 //   [0] (r, z) of this iteration, [2] (p, q), [4] (r, z) of the previous one,
 //   [6] the reference max((b, M^-1 b), (r0, M^-1 r0)), [8] 1 while the field iterates,
@@ -225,6 +293,20 @@ __device__ __forceinline__ void block_add(const double (&a)[NF], double* out) {
         atomicAdd(out + threadIdx.x, v);
     }
     __syncthreads();
+}
+
+// acc[2 + f] += (x, y) of field f = i mod NF, behind a product element by element
+template <int NF>
+__global__ void __launch_bounds__(256) k_macro_dot(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
+                                                   double* __restrict__ acc) {
+    if (blockIdx.x == 0 && threadIdx.x < NF) pcg_roll(acc, threadIdx.x);
+    double a[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) a[f] = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / NF; i += (int64_t)gridDim.x * blockDim.x)
+#pragma unroll
+        for (int f = 0; f < NF; ++f) a[f] = fma(x[i * NF + f], y[i * NF + f], a[f]);
+    block_add<NF>(a, acc + 2);
 }
 
 // q = A x for the transport pair and (x, q) per field into acc[2..3]; one warp per
@@ -404,7 +486,7 @@ __global__ void __launch_bounds__(256) k_mech_residual(int64_t n, const double* 
         const double bi = b[i], di = dinv[i];
         const double ri = held ? 0.0 : bi - y[i];
         r[i] = ri;
-        dinv32[i] = held ? 0.f : (float)di;   // the polynomial leaves held rows alone
+        if (dinv32) dinv32[i] = held ? 0.f : (float)di;   // the polynomial leaves held rows alone
         a[0] = fma(ri, ri * di, a[0]);
         if (!held) bb[0] = fma(bi, bi * di, bb[0]);
     }
@@ -680,6 +762,61 @@ __global__ void k_mech_material(int64_t nt, const double* __restrict__ Cgp, doub
     }
 }
 
+// Element form: y += K x, per tetrahedron eps = B x_T, sigma = cm eps, y_a += |T| B_a^T sigma
+__global__ void __launch_bounds__(256) k_mech_apply(int64_t nt, const int32_t* __restrict__ tets,
+                                                    const double* __restrict__ geo, const double* __restrict__ cm,
+                                                    const double* __restrict__ x, double* __restrict__ y) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
+        int v[4];
+        double ua[12], eps[6], sg[6];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            v[a] = tets[e * 4 + a];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) ua[a * 3 + i] = x[(int64_t)v[a] * 3 + i];
+        }
+        const double vol = geo[e * 13];
+        const double* g = geo + e * 13 + 1;
+        mech_strain(g, ua, eps);
+        const double* C = cm + e * 36;
+#pragma unroll
+        for (int J = 0; J < 6; ++J) {
+            double t = 0.0;
+#pragma unroll
+            for (int K = 0; K < 6; ++K) t = fma(C[J * 6 + K], eps[K], t);
+            sg[J] = vol * t;
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            double f[3];
+            mech_bt(g[a * 3], g[a * 3 + 1], g[a * 3 + 2], sg, f);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) atomicAdd(y + (int64_t)v[a] * 3 + i, f[i]);
+        }
+    }
+}
+
+// its diagonal |T| b^T cm b (b the DOF's column of B), added into d
+__global__ void __launch_bounds__(256) k_mech_diag(int64_t nt, const int32_t* __restrict__ tets,
+                                                   const double* __restrict__ geo, const double* __restrict__ cm,
+                                                   double* __restrict__ d) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nt * 4; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = k >> 2;
+        const double vol = geo[e * 13];
+        const double* g = geo + e * 13 + 1 + (k & 3) * 3;
+        const double* C = cm + e * 36;
+        for (int i = 0; i < 3; ++i) {
+            double b[6] = {0, 0, 0, 0, 0, 0}, t = 0.0;
+            b[i] = g[i];
+            b[i == 2 ? 5 : 3] = i == 0 ? g[1] : g[0];
+            b[i == 0 ? 5 : 4] = i == 2 ? g[1] : g[2];
+            for (int J = 0; J < 6; ++J)
+                for (int K = 0; K < 6; ++K) t += b[J] * C[J * 6 + K] * b[K];
+            atomicAdd(d + (int64_t)tets[k] * 3 + i, vol * t);
+        }
+    }
+}
+
 // The assembled stiffness: 3 x 3 blocks sum_T |T| B_a^T cm B_b of every entry, stored
 // val[(ell row * 9 + 3 r + c) * 32 + lane] (block row r), and the inverse Jacobi
 // diagonal.  One thread per (ELL row of the slice, lane).
@@ -863,13 +1000,28 @@ void to_sym6(const double k[9], double out[6]) {
     out[5] = k[2];
 }
 
+// Whether the matrices' share may grow by so many bytes: a quarter of the free memory, since
+// results and the caller want room too.
+int room_for(rve_macro m, size_t bytes) {
+    size_t room = m->mat_limit, all = 0;
+    if (room == 0) {
+        RVE_CUDA(cudaMemGetInfo(&room, &all));
+        room /= 4;
+    }
+    if (bytes <= room) return RVE_OK;
+    set_error("no room for the macro mesh's matrices");
+    return RVE_ERR_OUT_OF_MEMORY;
+}
+
 // Node graph of the mesh in slices of 32 rows, on the device (once per mesh).
+// RVE_ERR_OUT_OF_MEMORY where it does not fit, in memory or in 32-bit indices, or where a
+// node couples to so many others that the slices are mostly padding.
 int ensure_graph(rve_macro m) {
     if (m->have_graph) return RVE_OK;
     NodeGraph g;
     if (!build_node_graph(m->tets_h.data(), m->nt, 4, nullptr, m->nv, g)) {
         set_error("macro mesh too large for 32-bit matrix indices");
-        return RVE_ERR_INVALID_ARGUMENT;
+        return RVE_ERR_OUT_OF_MEMORY;
     }
     const int64_t ns = (m->nv + 31) / 32;
     std::vector<int64_t> base(ns + 1, 0);
@@ -880,6 +1032,11 @@ int ensure_graph(rve_macro m) {
         for (int64_t i = s * 32; i < std::min(m->nv, s * 32 + 32); ++i) most = std::max(most, len[i]);
         base[s + 1] = base[s] + most;
     }
+    if (base[ns] * 32 > 4 * (int64_t)g.col.size() + 4096) {
+        set_error("a node of the macro mesh couples to too many others");
+        return RVE_ERR_OUT_OF_MEMORY;
+    }
+    RVE_TRY(room_for(m, (size_t)base[ns] * 32 * 4 + (size_t)m->nt * 16));
     std::vector<int32_t> col((size_t)base[ns] * 32);
     for (int64_t s = 0; s < ns; ++s)
         for (int lane = 0; lane < 32; ++lane) {
@@ -900,10 +1057,25 @@ int ensure_graph(rve_macro m) {
     return RVE_OK;
 }
 
+// From here on the operators are applied element by element, as in a call that needs the
+// matrices and finds no room for them.
+int apply_element_form(rve_macro m) {
+    cudaGetLastError();
+    RVE_CUDA(cudaStreamSynchronize(m->ctx->stream));
+    for (DevBuf* b : {&m->g_base, &m->g_col, &m->g_len, &m->g_eptr, &m->g_inc, &m->t_mass, &m->t_stiff, &m->t_mat,
+                      &m->mmat, &m->mmat32})
+        b->release();
+    m->have_graph = m->have_stiff = false;
+    m->element_form = true;
+    m->mat_dt = -1;
+    return RVE_OK;
+}
+
 // The transport matrix and inverse diagonal for one time step length.
 int ensure_transport_matrix(rve_macro m, double dt_s) {
     RVE_TRY(ensure_graph(m));
     cudaStream_t s = m->ctx->stream;
+    if (!m->have_stiff && m->t_mat.bytes < (size_t)m->n_ell * 32 * 16) RVE_TRY(room_for(m, (size_t)m->n_ell * 32 * 40));
     const int64_t *base = m->g_base.as<int64_t>();
     const int32_t *col = m->g_col.as<int32_t>(), *len = m->g_len.as<int32_t>();
     if (!m->have_stiff) {
@@ -930,6 +1102,17 @@ int ensure_transport_matrix(rve_macro m, double dt_s) {
         RVE_CUDA(cudaGetLastError());
         m->mat_dt = dt_s;
     }
+    return RVE_OK;
+}
+
+// Room for the elastic matrix in both precisions and the preconditioner's vectors.
+int ensure_mech_matrix(rve_macro m) {
+    RVE_TRY(ensure_graph(m));
+    const size_t e = (size_t)m->n_ell * 9 * 32;
+    if (m->mmat.bytes < e * 8 || m->mmat32.bytes < e * 4) RVE_TRY(room_for(m, e * 12));
+    RVE_TRY(m->mmat.ensure(e * 8));
+    RVE_TRY(m->mmat32.ensure(e * 4));
+    for (DevBuf* b : {&m->c_r, &m->c_z, &m->c_z2, &m->c_d, &m->c_dinv}) RVE_TRY(b->ensure((size_t)m->nv * 12));
     return RVE_OK;
 }
 
@@ -1030,9 +1213,9 @@ template <class Product, class Step>
 int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product product, Step step, double rtol,
              int max_iter, int its[2], double rel[2], bool& conv) {
     cudaStream_t s = mm->ctx->stream;
-    for (DevBuf* bfr : {&mm->c_r, &mm->c_z, &mm->c_z2, &mm->c_d, &mm->c_dinv}) RVE_TRY(bfr->ensure((size_t)n * 4));
-    double lambda = 0.0;
-    RVE_TRY(mech_spectrum(mm, n, step, lambda));
+    const bool with_poly = !mm->element_form;   // (which has no FP32 matrix)
+    double lambda = 1.0;
+    if (with_poly) RVE_TRY(mech_spectrum(mm, n, step, lambda));
     double *r = mm->r.as<double>(), *p = mm->p.as<double>(), *q = mm->q.as<double>(), *acc = mm->acc.as<double>();
     float *r32 = mm->c_r.as<float>(), *zb[2] = {mm->c_z.as<float>(), mm->c_z2.as<float>()};
     float *d = mm->c_d.as<float>(), *dinv32 = mm->c_dinv.as<float>();
@@ -1050,32 +1233,36 @@ int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product produc
         return zb[n_steps & 1];
     };
     struct Key {
-        const void* ptr[14];
+        const void* ptr[15];
         double lambda;
     } key;
     std::memset(&key, 0, sizeof(key));
-    const void* ptrs[14] = {r, p, q, acc, x, mask, dinv, mm->mmat.p, mm->g_col.p, r32, zb[0], zb[1], d, mm->mmat32.p};
+    const void* ptrs[15] = {r,   p,   q,     acc,   x, mask,         dinv,    mm->mmat.p, mm->g_col.p,
+                            r32, zb[0], zb[1], d, mm->mmat32.p, mm->cm.p};
     std::memcpy(key.ptr, ptrs, sizeof(ptrs));
     double ref = 0.0;
-    bool broke = false;
-    RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
-    product(s, x, q, 20, nullptr);
-    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, dinv32, 20, acc);
-    k_macro_start<<<1, 2, 0, s>>>(acc, 1, 20, rtol * rtol, max_iter, 0.0);
-    k_mech_update<true><<<gv, 256, 0, s>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
-    k_mech_first<true><<<gv, 256, 0, s>>>(n, precondition(s), r, dinv, p);
-    RVE_CUDA(cudaGetLastError());
-    key.lambda = lambda;
-    RVE_TRY(macro_loop(mm, 1, &key, sizeof(key), 1, 20, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
-        product(cap, p, q, 20, acc);
-        k_mech_update<true><<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
-        k_mech_pupdate<true><<<gv, 256, 0, cap>>>(n, precondition(cap), r, dinv, p, acc, h);
-    }, its, rel, conv, &ref, &broke));
-    if (!broke || its[0] >= max_iter) return RVE_OK;
-    const int before = its[0];
+    bool broke = true;
+    int before = 0;
+    if (with_poly) {
+        RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
+        product(s, x, q, 20, nullptr);
+        k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, dinv32, 20, acc);
+        k_macro_start<<<1, 2, 0, s>>>(acc, 1, 20, rtol * rtol, max_iter, 0.0);
+        k_mech_update<true><<<gv, 256, 0, s>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
+        k_mech_first<true><<<gv, 256, 0, s>>>(n, precondition(s), r, dinv, p);
+        RVE_CUDA(cudaGetLastError());
+        key.lambda = lambda;
+        RVE_TRY(macro_loop(mm, 1, &key, sizeof(key), 1, 20, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+            product(cap, p, q, 20, acc);
+            k_mech_update<true><<<gv, 256, 0, cap>>>(n, mask, dinv, x, r, p, q, r32, zb[0], dinv32, w, acc);
+            k_mech_pupdate<true><<<gv, 256, 0, cap>>>(n, precondition(cap), r, dinv, p, acc, h);
+        }, its, rel, conv, &ref, &broke));
+        if (!broke || its[0] >= max_iter) return RVE_OK;
+        before = its[0];
+    }
     RVE_CUDA(cudaMemsetAsync(acc, 0, PCG_SCALARS * 8, s));
     product(s, x, q, 0, nullptr);
-    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, dinv32, 0, acc);
+    k_mech_residual<<<gv, 256, 0, s>>>(n, b, q, mask, dinv, r, nullptr, 0, acc);
     k_macro_start<<<1, 2, 0, s>>>(acc, 1, 0, rtol * rtol, max_iter - before, ref);
     k_mech_first<false><<<gv, 256, 0, s>>>(n, nullptr, r, dinv, p);
     RVE_CUDA(cudaGetLastError());
@@ -1092,8 +1279,8 @@ int mech_pcg(rve_macro mm, int64_t n, double* x, const double* b, Product produc
 // FP64 Jacobi PCG of the transport pair; per field converged when (r, D^-1 r) <=
 // rtol^2 max((b, D^-1 b), (r0, D^-1 r0)) over the free nodes.
 template <class Product>
-int transport_pcg(rve_macro mm, double2* x, const double2* b, Product product, double rtol, int max_iter, int its[2],
-                  double rel[2], bool& conv) {
+int transport_pcg(rve_macro mm, double2* x, const double2* b, Product product, double dt_key, double rtol,
+                  int max_iter, int its[2], double rel[2], bool& conv) {
     cudaStream_t s = mm->ctx->stream;
     double2 *r = mm->r.as<double2>(), *p = mm->p.as<double2>(), *q = mm->q.as<double2>();
     double* acc = mm->acc.as<double>();
@@ -1106,8 +1293,20 @@ int transport_pcg(rve_macro mm, double2* x, const double2* b, Product product, d
     k_transport_residual<<<gv, 256, 0, s>>>(nv, b, q, mask, dinv, r, p, acc);
     k_macro_start<<<1, 2, 0, s>>>(acc, 2, 0, rtol * rtol, max_iter, 0.0);
     RVE_CUDA(cudaGetLastError());
-    const void* key[9] = {r, p, q, acc, x, mask, dinv, mm->t_mat.p, mm->g_col.p};
-    return macro_loop(mm, 0, key, sizeof(key), 2, 0, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
+    struct Key {
+        const void* ptr[9];
+        double dt, tensors[13];
+    } key;
+    std::memset(&key, 0, sizeof(key));
+    const void* ptrs[9] = {r, p, q, acc, x, mask, dinv, mm->t_mat.p, mm->g_col.p};
+    std::memcpy(key.ptr, ptrs, sizeof(ptrs));
+    if (mm->element_form) {   // (numbers that the element form's product captures)
+        key.dt = dt_key;
+        std::memcpy(key.tensors, mm->KT, sizeof(mm->KT));
+        std::memcpy(key.tensors + 6, mm->Dc, sizeof(mm->Dc));
+        key.tensors[12] = mm->rho_cp;
+    }
+    return macro_loop(mm, 0, &key, sizeof(key), 2, 0, [&](cudaStream_t cap, cudaGraphConditionalHandle h) {
         product(cap, p, q, acc);
         k_transport_update<<<gv, 256, 0, cap>>>(nv, mask, dinv, x, r, p, q, acc);
         k_transport_pupdate<<<gv, 256, 0, cap>>>(nv, dinv, r, p, acc, h);
@@ -1269,24 +1468,55 @@ int rve_macro_reset(rve_ctx c, rve_macro m, double T0_C, double c0_wt) {
 static int transport_solve(rve_macro mm, double dt_s, double rtol, int max_iter, int its[2], double rel[2],
                            bool& conv) {
     cudaStream_t s = mm->ctx->stream;
-    RVE_TRY(ensure_transport_matrix(mm, dt_s));
-    const int64_t ns = mm->n_slices;
-    double* x = mm->x.as<double>();
-    double* b = mm->b.as<double>();
+    double2* x = mm->x.as<double2>();
+    double2* b = mm->b.as<double2>();
     const uint8_t* mask = mm->mask.as<uint8_t>();
+    const double capT = mm->rho_cp / dt_s, capC = 1.0 / dt_s;
+    if (!mm->element_form) {
+        const int rc = ensure_transport_matrix(mm, dt_s);
+        if (rc == RVE_ERR_OUT_OF_MEMORY)
+            RVE_TRY(apply_element_form(mm));
+        else
+            RVE_TRY(rc);
+    }
+    // b = C/dt x^n; start from x^n with the held values in place
+    auto hold = [&]() {
+        k_macro_hold<<<grid_for(mm->nv), 256, 0, s>>>(mm->nv, mask, mm->hold.as<double>(), mm->x.as<double>());
+    };
+    if (mm->element_form) {
+        const int32_t* tets = mm->tets.as<int32_t>();
+        const double* geo = mm->geo.as<double>();
+        const unsigned ge = grid_for(mm->nt);
+        TransportTensors prm;
+        std::memcpy(prm.KT, mm->KT, sizeof(prm.KT));
+        std::memcpy(prm.Dc, mm->Dc, sizeof(prm.Dc));
+        RVE_TRY(mm->t_dinv.ensure((size_t)mm->nv * 16));
+        RVE_CUDA(cudaMemsetAsync(mm->t_dinv.p, 0, (size_t)mm->nv * 16, s));
+        k_transport_diag<<<ge, 256, 0, s>>>(mm->nt, tets, geo, prm, capT, capC, mm->t_dinv.as<double2>());
+        k_invert<<<grid_for(mm->nv * 2), 256, 0, s>>>(mm->nv * 2, mm->t_dinv.as<double>());
+        launch_fill(mm->nv * 2, 0.0, mm->b.as<double>(), s);
+        k_transport_apply<<<ge, 256, 0, s>>>(mm->nt, tets, geo, prm, capT, capC, 0, x, b);
+        hold();
+        auto product = [&](cudaStream_t st, const double2* in, double2* out, double* acc) {
+            launch_fill(mm->nv * 2, 0.0, reinterpret_cast<double*>(out), st);
+            k_transport_apply<<<ge, 256, 0, st>>>(mm->nt, tets, geo, prm, capT, capC, 1, in, out);
+            if (acc)
+                k_macro_dot<2><<<grid_for(mm->nv), 256, 0, st>>>(mm->nv * 2, reinterpret_cast<const double*>(in),
+                                                                 reinterpret_cast<const double*>(out), acc);
+        };
+        return transport_pcg(mm, x, b, product, dt_s, rtol, max_iter, its, rel, conv);
+    }
+    const int64_t ns = mm->n_slices;
     const int64_t* base = mm->g_base.as<int64_t>();
     const int32_t* col = mm->g_col.as<int32_t>();
     const double2* mat = mm->t_mat.as<double2>();
     const unsigned gs = (unsigned)((ns + 7) / 8);
-    // b = C/dt x^n; start from x^n with the held values in place
-    k_transport_rhs<<<gs, 256, 0, s>>>(mm->nv, ns, base, col, mm->t_mass.as<double>(), mm->rho_cp / dt_s, 1.0 / dt_s,
-                                       reinterpret_cast<const double2*>(x), reinterpret_cast<double2*>(b));
-    k_macro_hold<<<grid_for(mm->nv), 256, 0, s>>>(mm->nv, mask, mm->hold.as<double>(), x);
+    k_transport_rhs<<<gs, 256, 0, s>>>(mm->nv, ns, base, col, mm->t_mass.as<double>(), capT, capC, x, b);
+    hold();
     auto product = [&](cudaStream_t st, const double2* in, double2* out, double* acc) {
         k_transport_product<<<gs, 256, 0, st>>>(mm->nv, ns, base, col, mat, in, out, acc);
     };
-    return transport_pcg(mm, reinterpret_cast<double2*>(x), reinterpret_cast<const double2*>(b), product, rtol,
-                         max_iter, its, rel, conv);
+    return transport_pcg(mm, x, b, product, 0.0, rtol, max_iter, its, rel, conv);
 }
 
 int rve_macro_step(rve_ctx c, rve_macro m, double dt_h, const rve_degradation* deg, double rtol, int max_iter,
@@ -1640,41 +1870,57 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
         RVE_TRY(upload(m->cgp, C_gp, (size_t)m->nt * 4 * 36, s));
         Cg = m->cgp.as<double>();
     }
-    RVE_TRY(ensure_graph(m));
     for (DevBuf* bfr : {&m->b, &m->r, &m->p, &m->q, &m->mdinv}) RVE_TRY(bfr->ensure((size_t)n * 8));
     RVE_TRY(m->cm.ensure((size_t)m->nt * 36 * 8));
-    RVE_TRY(m->mmat.ensure((size_t)m->n_ell * 9 * 32 * 8));
-    RVE_TRY(m->mmat32.ensure((size_t)m->n_ell * 9 * 32 * 4));
     RVE_TRY(m->msig.ensure((size_t)m->nt * 4 * 6 * 8));
+    if (!m->element_form) {
+        const int rc = ensure_mech_matrix(m);
+        if (rc == RVE_ERR_OUT_OF_MEMORY)
+            RVE_TRY(apply_element_form(m));
+        else
+            RVE_TRY(rc);
+    }
     const int32_t* tets = m->tets.as<int32_t>();
     const double* geo = m->geo.as<double>();
-    const int64_t* base = m->g_base.as<int64_t>();
-    const int32_t* col = m->g_col.as<int32_t>();
+    const double* cm = m->cm.as<double>();
     k_mech_material<<<(unsigned)std::min<int64_t>((m->nt * 36 + 255) / 256, (int64_t)sm_count() * 16), 256, 0, s>>>(
         m->nt, Cg, m->cm.as<double>());
     RVE_CUDA(cudaMemsetAsync(m->mdinv.p, 0, (size_t)n * 8, s));   // nodes of no element: z = 0
-    k_mech_entries<<<(unsigned)m->n_slices, 256, 0, s>>>(m->nv, base, col, m->g_len.as<int32_t>(),
-                                                         m->g_eptr.as<int32_t>(), m->g_inc.as<int32_t>(), tets, geo,
-                                                         m->cm.as<double>(), m->mmat.as<double>(),
-                                                         m->mdinv.as<double>());
     double* b = m->b.as<double>();
     double* u = m->mu.as<double>();
     RVE_CUDA(cudaMemcpyAsync(b, m->mload.p, n * 8, cudaMemcpyDeviceToDevice, s));
     k_mech_hold<<<grid_for(n), 256, 0, s>>>(n, m->mfix.as<uint8_t>(), m->mval.as<double>(), u);
-    const double* mat = m->mmat.as<double>();
-    const unsigned gm = (unsigned)std::min<int64_t>((m->n_slices + 1) / 2, (int64_t)sm_count() * 10);
-    auto product = [&](cudaStream_t st, const double* in, double* out, int norm, double* acc) {
-        k_mech_product<<<gm, MECH_THREADS, 0, st>>>(m->nv, m->n_slices, base, col, mat, in, out, norm, acc);
-    };
     int its[2] = {0, 0};
     double rel[2] = {0, 0};
     bool conv = false;
-    const float* mat32 = m->mmat32.as<float>();
-    k_narrow<<<(unsigned)(sm_count() * 16), 256, 0, s>>>(m->n_ell * 288, mat, m->mmat32.as<float>());
-    auto step = [&](cudaStream_t st, const MechCheb& c) {
-        k_mech_cheb<<<(unsigned)((m->n_slices + 1) / 2), 192, 0, st>>>(m->nv, m->n_slices, base, col, mat32, c);
-    };
-    RVE_TRY(mech_pcg(m, n, u, b, product, step, rtol, max_iter, its, rel, conv));
+    if (m->element_form) {
+        const unsigned ge = grid_for(m->nt);
+        k_mech_diag<<<grid_for(m->nt * 4), 256, 0, s>>>(m->nt, tets, geo, cm, m->mdinv.as<double>());
+        k_invert<<<grid_for(n), 256, 0, s>>>(n, m->mdinv.as<double>());
+        auto product = [&](cudaStream_t st, const double* in, double* out, int, double* acc) {
+            launch_fill(n, 0.0, out, st);
+            k_mech_apply<<<ge, 256, 0, st>>>(m->nt, tets, geo, cm, in, out);
+            if (acc) k_macro_dot<1><<<grid_for(n), 256, 0, st>>>(n, in, out, acc);
+        };
+        RVE_TRY(mech_pcg(m, n, u, b, product, [](cudaStream_t, const MechCheb&) {}, rtol, max_iter, its, rel, conv));
+    } else {
+        const int64_t* base = m->g_base.as<int64_t>();
+        const int32_t* col = m->g_col.as<int32_t>();
+        k_mech_entries<<<(unsigned)m->n_slices, 256, 0, s>>>(m->nv, base, col, m->g_len.as<int32_t>(),
+                                                             m->g_eptr.as<int32_t>(), m->g_inc.as<int32_t>(), tets, geo,
+                                                             cm, m->mmat.as<double>(), m->mdinv.as<double>());
+        const double* mat = m->mmat.as<double>();
+        const unsigned gm = (unsigned)std::min<int64_t>((m->n_slices + 1) / 2, (int64_t)sm_count() * 10);
+        auto product = [&](cudaStream_t st, const double* in, double* out, int norm, double* acc) {
+            k_mech_product<<<gm, MECH_THREADS, 0, st>>>(m->nv, m->n_slices, base, col, mat, in, out, norm, acc);
+        };
+        const float* mat32 = m->mmat32.as<float>();
+        k_narrow<<<(unsigned)(sm_count() * 16), 256, 0, s>>>(m->n_ell * 288, mat, m->mmat32.as<float>());
+        auto step = [&](cudaStream_t st, const MechCheb& c) {
+            k_mech_cheb<<<(unsigned)((m->n_slices + 1) / 2), 192, 0, st>>>(m->nv, m->n_slices, base, col, mat32, c);
+        };
+        RVE_TRY(mech_pcg(m, n, u, b, product, step, rtol, max_iter, its, rel, conv));
+    }
     k_mech_stress<<<grid_for(m->nt * 4), 256, 0, s>>>(m->nt, tets, geo, Cg, u, m->msig.as<double>());
     RVE_CUDA(cudaGetLastError());
     RVE_CUDA(cudaStreamSynchronize(s));
@@ -1689,6 +1935,18 @@ int rve_macro_mech_solve(rve_ctx c, rve_macro m, const double* C_gp, int C_on_de
         set_error("rve_macro_mech_solve: PCG did not reach rtol within max_iter");
         return RVE_ERR_NOT_CONVERGED;
     }
+    return RVE_OK;
+}
+
+int rve_debug_macro_matrix_limit(rve_ctx c, rve_macro m, int64_t bytes) {
+    RVE_TRY(check_ctx(c));
+    if (!m || bytes < 0) {
+        set_error("rve_debug_macro_matrix_limit: invalid argument");
+        return RVE_ERR_INVALID_ARGUMENT;
+    }
+    RVE_TRY(apply_element_form(m));   // (drops the graph and the matrices)
+    m->element_form = false;
+    m->mat_limit = (size_t)bytes;
     return RVE_OK;
 }
 

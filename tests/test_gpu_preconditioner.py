@@ -243,3 +243,66 @@ def test_not_a_number_does_not_read_as_converged(rve):
     with pytest.raises(rve.RveError) as e:
         plate_solve(rve, xyz, tets, C, 1e-11, 500)
     assert e.value.code == -4
+
+
+def limit_matrices(ctx, m, n_bytes):
+    assert ctx.lib.rve_debug_macro_matrix_limit(ctx.h, m.h, n_bytes) == 0
+
+
+def test_macro_mesh_without_room_for_matrices(rve):
+    """No room for the graph and the matrices: transport steps and the elastic solve element by
+    element, against the matrices and, for the displacements, the oracle."""
+    rng = np.random.default_rng(4)
+    xyz, tets, _ = ri.plate(9, 4, 3)
+    A = rng.standard_normal((len(tets), 4, 6, 6))
+    C = 1e9 * (np.einsum("tgij,tgkj->tgik", A, A) + 6 * np.eye(6))
+    KT = np.array([[0.40, 0.01, 0.0], [0.01, 0.35, 0.0], [0.0, 0.0, 0.30]])
+    out = []
+    for limit in (0, 100, 0):
+        with rve.Context() as ctx:
+            m = ctx.macro_load(xyz, tets)
+            limit_matrices(ctx, m, limit)
+            m.set_transport(KT, 1.6e6, np.diag([1.2e-12, 1.0e-12, 8.0e-13]))
+            m.set_face(xyz[:, 2] <= 1e-12, 60.0, 1.5)
+            m.reset(20.0, 0.1)
+            for dt in (50.0, 50.0, 20.0):
+                m.step(dt)
+            m.mech_set_bc(xyz <= 1e-12)
+            m.mech_set_traction(xyz[:, 0] >= xyz[:, 0].max() * (1 - 1e-12), [1e6, 0.0, 2e5])
+            m.mech_solve(C, rtol=1e-12)
+            g, r = m.get(), m.mech_get()
+            out.append([np.asarray(v) for v in (g["T"], g["c"], g["W"], r["u"], r["stress"])])
+            m.free()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.linalg.norm(a - b) < 1e-9 * np.linalg.norm(a)
+    K = mo.elastic_assemble(xyz, tets, C)
+    u = mo.elastic_solve(K, r["load"].reshape(-1), (xyz <= 1e-12).reshape(-1))
+    for o in out:
+        assert np.linalg.norm(o[3].reshape(-1) - u) < 1e-9 * np.linalg.norm(u)
+
+
+def test_macro_mesh_with_a_hub(rve):
+    """A fan of tetrahedra around one edge: its two nodes couple to all others, and slices of
+    equal row length would be mostly padding.  Answered element by element."""
+    n = 2400
+    phi = 2 * np.pi * np.arange(n) / n
+    xyz = np.concatenate([[[0, 0, -0.5], [0, 0, 0.5]], np.stack([np.cos(phi), np.sin(phi), 0 * phi], 1)])
+    i = np.arange(n)
+    tets = np.stack([0 * i, 0 * i + 1, 2 + i, 2 + (i + 1) % n], 1).astype(np.int32)
+    X = xyz[tets]
+    if np.linalg.det(X[0, 1:] - X[0, 0]) < 0:
+        tets = tets[:, [1, 0, 2, 3]]
+    C = np.broadcast_to(isotropic(1e3), (len(tets), 4, 6, 6)).copy()
+    fixed = np.zeros((len(xyz), 3), bool)
+    fixed[2::3] = True
+    with rve.Context() as ctx:
+        m = ctx.macro_load(xyz, tets)
+        m.mech_set_bc(fixed)
+        m.mech_set_traction(np.arange(len(xyz)) != 0, [0.0, 1.0, 3.0])
+        m.mech_solve(C, rtol=1e-12)
+        r = m.mech_get()
+        m.free()
+    u = mo.elastic_solve(mo.elastic_assemble(xyz, tets, C), r["load"].reshape(-1), fixed.reshape(-1))
+    assert np.linalg.norm(u) > 0
+    assert np.linalg.norm(r["u"].reshape(-1) - u) < 1e-9 * np.linalg.norm(u)
