@@ -424,7 +424,8 @@ int ensure_assembled(rve_mesh m, int fid, bool fp64, cudaStream_t s) {
     if (room == 0) {
         const size_t held64 = m->a_ent[fid][0].bytes, held32 = m->a_ent[fid][1].bytes;
         need = (b64 > held64 ? b64 : 0) + (b32 > held32 ? b32 : 0);
-        if (need > 0) {
+        room = (size_t)1 << 30;   // (the query takes up to a millisecond: not for a small matrix)
+        if (need > room) {
             size_t all = 0;
             RVE_CUDA(cudaMemGetInfo(&room, &all));
             room /= 4;
@@ -756,10 +757,10 @@ struct Solver {
             evs.push_back(e);
         }
         if (prof) RVE_CUDA(cudaEventRecord(evs[0], s));
+        RVE_TRY(try_assembled(m, fid, true, s));
         if (use_assembled(m, true)) {
             // b is the right-hand side less what the constraint forces carry, which the
             // projection of the residual removes anyway
-            RVE_TRY(ensure_assembled(m, fid, true, s));
             launch_asm_residual<double>(f.nc, asm_view<double>(m, fid, m->scale64.as<double>()), x,
                                         m->b64.as<double>(), y, ncols, s);
             *launches += 1;
@@ -840,8 +841,9 @@ struct Solver {
         const bool use_tc =
             !det && sizeof(T) == 4 && operator_tc_supported(m->p, f.nc) && kern == RVE_KERNEL_TENSOR;
         if (use_tc) RVE_TRY(ensure_element_matrices(m, s));
-        const bool use_asm = !use_tc && (sizeof(T) == 8 ? use_assembled(m, true) : assembled32());
-        if (use_asm) RVE_TRY(ensure_assembled(m, fid, sizeof(T) == 8, s));
+        const auto asm_wanted = [&] { return !use_tc && (sizeof(T) == 8 ? use_assembled(m, true) : assembled32()); };
+        if (asm_wanted()) RVE_TRY(try_assembled(m, fid, sizeof(T) == 8, s));
+        const bool use_asm = asm_wanted();
         const AsmView<T> av = use_asm ? asm_view<T>(m, fid, scale.as<T>()) : AsmView<T>();
         ColState cs = cs64;
         // the operator of the iteration runs one wave of resident blocks; its energy
@@ -1405,7 +1407,6 @@ struct Solver {
         const rve_options& o = m->ctx->opt;
         const bool mixed = precision == RVE_PREC_MIXED;
         RVE_TRY(alloc(mixed));
-        if (!mixed || assembled32()) RVE_TRY(try_assembled(m, fid, !mixed, s));
         const size_t nv = (size_t)n_rows * ncols;
         double* x64 = m->x64f[fid].as<double>();
         double* r64 = m->r64f[fid].as<double>();
@@ -1471,8 +1472,8 @@ struct Solver {
                     for (int c = 0; c < ncols; ++c)
                         for (int ph = 0; ph < 2; ++ph) sc32[2 * c + ph] = (float)-warm->degrade[ph];
                     RVE_TRY(upload(m->dscale32, sc32.data(), sc32.size(), s));
+                    if (assembled32()) RVE_TRY(try_assembled(m, fid, false, s));
                     if (assembled32()) {
-                        RVE_TRY(ensure_assembled(m, fid, false, s));
                         launch_asm_product<float>(f.nc, asm_view<float>(m, fid, m->dscale32.as<float>()), v32, y32,
                                                   ncols, nullptr, nullptr, s);
                     } else {
@@ -1856,8 +1857,8 @@ static int warm_products(rve_mesh m, int ns, const double* degrade, bool mixed, 
     } else {
         // FP64 operator with the scales -K_part
         RVE_TRY(upload(m->warm_phs, nsc.data(), nsc.size(), s));
+        RVE_TRY(try_assembled(m, 0, true, s));
         if (use_assembled(m, true)) {
-            RVE_TRY(ensure_assembled(m, 0, true, s));
             launch_asm_product<double>(f.nc, asm_view<double>(m, 0, m->warm_phs.as<double>()), xs64, kx, k2, nullptr,
                                        nullptr, s);
         } else {

@@ -1005,8 +1005,11 @@ void to_sym6(const double k[9], double out[6]) {
 int room_for(rve_macro m, size_t bytes) {
     size_t room = m->mat_limit, all = 0;
     if (room == 0) {
-        RVE_CUDA(cudaMemGetInfo(&room, &all));
-        room /= 4;
+        room = (size_t)1 << 30;   // (the query takes up to a millisecond: not for small matrices)
+        if (bytes > room) {
+            RVE_CUDA(cudaMemGetInfo(&room, &all));
+            room /= 4;
+        }
     }
     if (bytes <= room) return RVE_OK;
     set_error("no room for the macro mesh's matrices");
