@@ -171,6 +171,7 @@ int build_constraints(rve_mesh m, FieldDev& f, const std::vector<double>& geo) {
     std::vector<uint8_t> mask;
     if (m->bc == RVE_BC_DIRICHLET) mask = M.boundary;
     RVE_TRY(upload(f.mask, mask.data(), mask.size(), s));
+    f.n_free = N - std::count_if(mask.begin(), mask.end(), [](uint8_t v) { return v != 0; });
     f.m = 0;
     f.n_sup = 0;
     // Periodic: the folded (torus) problem is singular only by rigid translations,
@@ -392,6 +393,13 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
     return RVE_OK;
 }
 
+// An FP64 solve of a handful of unknowns takes the element operator and Jacobi: a few
+// iterations, and nothing to form first.  3x3x2, p = 1, Dirichlet, four free nodes: 1.01 ms a solve
+// and 1.21 the first one, against 1.14 and 1.78 with the matrix and the polynomial; 2x2x2, periodic,
+// eight: 0.80 and 1.00 against 0.94 and 1.62.  With 18 free nodes the latter already win
+// (3x3x2, periodic: 1.43 against 1.94, the first one 2.1 both).
+bool few_unknowns(rve_mesh m) { return m->p == 1 && m->mech.m == 0 && m->mech.n_free <= 8; }
+
 // Whether a solve uses the assembled operator.  FP64: orders 1 and 2, where it needs a
 // sixth and a half of the element form's FMAs (FP64-bound; 24x24x8, p = 2, 6 columns:
 // 231 -> 171 us a product).  FP32: order 1 only (16x16x6, 1536 columns: 206 -> 71 us); at
@@ -404,7 +412,7 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
 // solve vectors, as with the element operators.
 bool use_assembled(rve_mesh m, bool fp64) {
     const int64_t ne = n_local(m->p);
-    return !m->a_refused && m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built() &&
+    return !m->a_refused && !(fp64 && few_unknowns(m)) && m->p <= (fp64 ? 2 : 1) && m->ctx->opt.deterministic == 0 && !bounds_check_built() &&
            m->nt * ne * ne <= (int64_t)1 << 29;
 }
 
@@ -862,7 +870,7 @@ struct Solver {
             RVE_CUDA(cudaMemsetAsync(cs.pq_acc, 0, sizeof(double) * 3 * ACC_SLOTS * ncols, s));   // pq, rz and rj
         }
         // FP64 without constraint rows: polynomial preconditioner
-        bool cheb = sizeof(T) == 8 && fused && !jacobi && !bounds_check_built();
+        bool cheb = sizeof(T) == 8 && fused && !jacobi && !few_unknowns(m) && !bounds_check_built();
         if (cheb)   // (its four FP32 vectors, 16 bytes an entry: without room for them Jacobi)
             for (DevBuf* bfr : {&m->x32, &m->r32, &m->p32, &m->q32}) {
                 const int rc = bfr->ensure((size_t)n_rows * ncols * 4);

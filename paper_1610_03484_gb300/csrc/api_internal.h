@@ -114,6 +114,7 @@ struct FieldDev {
     int nc = 3;
     int nfield = 1;
     int64_t n_rows = 0;
+    int64_t n_free = 0;   // nodes that no Dirichlet mask holds
     DevBuf diag64, diag32, mask;
     int m = 0;
     int64_t n_sup = 0;

@@ -75,7 +75,8 @@ def distorted(grid, seed, amp=0.25):
     return xyz, tets, phase, tangent
 
 
-@pytest.mark.parametrize("grid,p", [((6, 6, 4), 1), ((9, 8, 6), 1), ((5, 4, 3), 2), ((3, 3, 2), 3)])
+@pytest.mark.parametrize("grid,p", [((3, 3, 2), 1), ((3, 3, 3), 1), ((3, 3, 4), 1), ((6, 6, 4), 1), ((9, 8, 6), 1),
+                                    ((5, 4, 3), 2), ((3, 3, 2), 3)])
 def test_distorted_cells_match_oracle(rve, grid, p):
     xyz, tets, phase, tangent = distorted(grid, 3)
     mat, yarn = ri.NOMINAL_MATRIX, ri.NOMINAL_YARN
