@@ -104,8 +104,11 @@ typedef struct rve_options {
                                 that kernel; RVE_KERNEL_TENSOR the tensor-core kernel (element
                                 matrices stored once per mesh and materials, 3 x TF32 products
                                 with FP32 accumulation).  Other cases always use a CUDA-core
-                                kernel: the assembled operator at p = 1 and in FP64 at p = 2, the
-                                matrix-free one elsewhere. */
+                                kernel: the assembled operator in FP64 at p = 1 and 2 (above 8
+                                unknown nodes) and in FP32 at p = 1 from 1e5 values a
+                                component on, where its matrix (at most 2^29 possible entries)
+                                fits a quarter of the free memory; the matrix-free one elsewhere,
+                                and in the deterministic mode. */
     int     deterministic;   /* 1: bit-reproducible cell solves.  The scatter kernels (operator,
                                 true residual, right-hand side) run once per element colour (no
                                 two elements of a colour share a DOF; greedy colouring of the DOF

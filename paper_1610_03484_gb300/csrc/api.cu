@@ -550,13 +550,14 @@ struct WarmStart {
 // The preconditioner of the FP64 solves: a Chebyshev polynomial in D^-1 A, evaluated in
 // FP32.  An FP64 product runs at two FMAs per clock and SM, an FP32 one at 128, so a
 // polynomial of degree 17 (16 FP32 products) costs about what 1.5 FP64 iterations do and
-// takes the place of 12 of them (24x24x8, p = 2: 284 iterations in 89 ms before, 22 in 16
-// now).  The operator, the vectors, the inner products and the stopping test stay FP64,
+// takes the place of 12 of them (24x24x8, p = 2: 284 iterations in 89 ms before, 21 in
+// 15.3 now).  The operator, the vectors, the inner products and the stopping test stay FP64,
 // so the solution is as accurate.  It covers [lambda / ratio, lambda] of the spectrum with
-// the odd degree next to sqrt(ratio); the ratio follows the condition number, which grows with the square
-// of the nodes along a side.  Measured (ms a solve): 24x24x8, p = 2 (36 864 nodes, ratio
-// 277): degree 10, ratio 60 19.7; 14, 250 16.5; 18, 250 15.9; 6 x 6 x 4, p = 1 (144 nodes,
-// ratio 10): degree 6, ratio 15 1.60; 10, 60 1.90.
+// the odd degree next to sqrt(ratio), at least 5 (chebyshev.h); the ratio follows the
+// condition number, which grows with the square of the nodes along a side.  Measured (degree,
+// ratio: ms a solve), the rule's choice first: 24x24x8, p = 2 (36 864 nodes) 17, 277: 15.3;
+// 15, 250: 15.9; 13, 150: 16.5; 19, 300: 15.1.  6x6x4, p = 1 (144 nodes) 5, 10: 1.60; 5, 15: 1.61;
+// 3, 15: 1.78; 7, 36: 1.76.
 double cheb_ratio(int64_t nodes) {
     return std::min(300.0, std::max(10.0, 0.25 * std::pow((double)nodes, 2.0 / 3.0)));
 }

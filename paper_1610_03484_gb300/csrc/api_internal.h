@@ -215,7 +215,7 @@ struct rve_mesh_s {
     bool a_refused = false;   // the matrix did not fit: element operators
     size_t a_limit = 0;       // bytes its entries may take (0: by the free memory)
     rve::DevBuf dinv64, dinv32;   // inverse Jacobi diagonal of the FP64 solve in progress
-    double a_lambda[2] = {0, 0};  // per field: bound of the spectrum of D^-1 A (0: not formed)
+    double a_lambda[2] = {0, 0};  // per field: estimate of the largest eigenvalue of D^-1 A (0: not formed)
     rve::DevBuf d_dof_vertex, traction_mu;   // uniform traction: original vertex of each node, multipliers
     // element colouring of the current DOF map (no two elements of a colour share a
     // DOF): elements sorted by colour on the device, colour offsets on the host

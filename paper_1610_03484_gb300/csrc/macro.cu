@@ -1176,10 +1176,10 @@ int macro_loop(rve_macro mm, int slot, const void* key, size_t key_bytes, int nf
 }
 
 // Polynomial of the elastic solve's preconditioner: it covers [lambda / ratio, lambda]
-// of the spectrum with the odd degree next to sqrt(ratio).  Measured on the 200 x 40 x 10 plate (solve
-// and results): degree 10, ratio 100 36.4 ms; 18, 300 31.4; 24, 600 28.8; 32, 1500 26.9.
-// The condition number grows with the square of the nodes along the longest side, at
-// most as the 2/3 power of their number for a cube.
+// of the spectrum with the odd degree next to sqrt(ratio).  Measured on the 200 x 40 x 10 plate
+// (degree, ratio: ms for solve and results), the rule's choice first: 39, 1500: 27.1; 33, 1500:
+// 27.3; 33, 1000: 28.1; 25, 600: 29.0; 51, 2500: 26.5.  The condition number grows with the square
+// of the nodes along the longest side, at most as the 2/3 power of their number for a cube.
 double mech_cheb_ratio(int64_t nv) { return std::min(1500.0, std::max(10.0, 0.75 * std::pow((double)nv, 2.0 / 3.0))); }
 
 // Estimate of the largest eigenvalue of D^-1 K by power iteration with the preconditioner's
