@@ -1068,6 +1068,11 @@ int apply_element_form(rve_macro m) {
     for (DevBuf* b : {&m->g_base, &m->g_col, &m->g_len, &m->g_eptr, &m->g_inc, &m->t_mass, &m->t_stiff, &m->t_mat,
                       &m->mmat, &m->mmat32})
         b->release();
+    for (auto& l : m->loop)   // (their captured launches hold pointers that the keys do not list)
+        if (l.exec) {
+            cudaGraphExecDestroy(l.exec);
+            l.exec = nullptr;
+        }
     m->have_graph = m->have_stiff = false;
     m->element_form = true;
     m->mat_dt = -1;
