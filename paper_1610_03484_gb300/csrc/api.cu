@@ -353,34 +353,47 @@ int ensure_asm_graph(rve_mesh m, cudaStream_t s) {
             lo[a] = std::min(lo[a], (float)c);
             hi[a] = std::max(hi[a], (float)c);
         }
-    std::vector<std::pair<uint32_t, int32_t>> key(N);
-    for (int64_t i = 0; i < N; ++i) {
-        float c[3] = {0, 0, 0};
-        const int n = std::max(1, g.eptr[i + 1] - g.eptr[i]);
-        for (int32_t q = g.eptr[i]; q < g.eptr[i + 1]; ++q)
-            for (int a = 0; a < 3; ++a) c[a] += cen[(size_t)(g.inc[q] / ne) * 3 + a];
-        uint32_t k = 0;
-        for (int a = 0; a < 3; ++a) {
-            const float t = hi[a] > lo[a] ? (c[a] / n - lo[a]) / (hi[a] - lo[a]) : 0.f;
-            const uint32_t v = (uint32_t)std::min(1023.f, std::max(0.f, t * 1023.f));
-            for (int bit = 0; bit < 10; ++bit) k |= ((v >> bit) & 1u) << (3 * bit + a);
+    // (key, node) pairs by key: three passes over 10 bits each, which keep equal keys in order
+    std::vector<uint32_t> key(N);
+    host_ranges(N, 1, (double)m->nt * ne, [&](int64_t first, int64_t last) {
+        for (int64_t i = first; i < last; ++i) {
+            float c[3] = {0, 0, 0};
+            const int n = std::max(1, g.eptr[i + 1] - g.eptr[i]);
+            for (int32_t q = g.eptr[i]; q < g.eptr[i + 1]; ++q)
+                for (int a = 0; a < 3; ++a) c[a] += cen[(size_t)(g.inc[q] / ne) * 3 + a];
+            uint32_t k = 0;
+            for (int a = 0; a < 3; ++a) {
+                const float t = hi[a] > lo[a] ? (c[a] / n - lo[a]) / (hi[a] - lo[a]) : 0.f;
+                const uint32_t v = (uint32_t)std::min(1023.f, std::max(0.f, t * 1023.f));
+                for (int bit = 0; bit < 10; ++bit) k |= ((v >> bit) & 1u) << (3 * bit + a);
+            }
+            key[i] = k;
         }
-        key[i] = {k, (int32_t)i};
+    });
+    std::vector<int32_t> order(N), other(N);
+    std::iota(order.begin(), order.end(), 0);
+    for (int shift = 0; shift < 30; shift += 10) {
+        int64_t count[1025] = {0};
+        for (int64_t i = 0; i < N; ++i) ++count[((key[i] >> shift) & 1023u) + 1];
+        for (int k = 0; k < 1024; ++k) count[k + 1] += count[k];
+        for (int64_t i = 0; i < N; ++i) other[count[(key[order[i]] >> shift) & 1023u]++] = order[i];
+        order.swap(other);
     }
-    std::sort(key.begin(), key.end());
-    std::vector<int32_t> order(N);
-    for (int64_t i = 0; i < N; ++i) order[i] = key[i].second;
-    for (int64_t w = 0; w < N; w += 1024)
-        std::stable_sort(order.begin() + w, order.begin() + std::min(N, w + 1024), [&](int32_t a, int32_t b) {
-            return g.ptr[a + 1] - g.ptr[a] > g.ptr[b + 1] - g.ptr[b];
-        });
+    host_ranges(N, 1024, (double)N * 20, [&](int64_t first, int64_t last) {
+        for (int64_t w = first; w < last; w += 1024)
+            std::stable_sort(order.begin() + w, order.begin() + std::min(last, w + 1024), [&](int32_t a, int32_t b) {
+                return g.ptr[a + 1] - g.ptr[a] > g.ptr[b + 1] - g.ptr[b];
+            });
+    });
     std::vector<int32_t> ptr(N + 1, 0), split(N), col(g.col.size());
-    for (int64_t r = 0; r < N; ++r) {
-        const int32_t i = order[r], n = g.ptr[i + 1] - g.ptr[i];
-        std::copy(g.col.begin() + g.ptr[i], g.col.begin() + g.ptr[i + 1], col.begin() + ptr[r]);
-        split[r] = ptr[r] + (g.split[i] - g.ptr[i]);
-        ptr[r + 1] = ptr[r] + n;
-    }
+    for (int64_t r = 0; r < N; ++r) ptr[r + 1] = ptr[r] + (g.ptr[order[r] + 1] - g.ptr[order[r]]);
+    host_ranges(N, 1, (double)col.size(), [&](int64_t first, int64_t last) {
+        for (int64_t r = first; r < last; ++r) {
+            const int32_t i = order[r];
+            std::copy(g.col.begin() + g.ptr[i], g.col.begin() + g.ptr[i + 1], col.begin() + ptr[r]);
+            split[r] = ptr[r] + (g.split[i] - g.ptr[i]);
+        }
+    });
     RVE_TRY(upload(m->a_order, order.data(), order.size(), s));
     RVE_TRY(upload(m->a_ptr, ptr.data(), ptr.size(), s));
     RVE_TRY(upload(m->a_split, split.data(), split.size(), s));

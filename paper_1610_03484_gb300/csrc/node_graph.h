@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <functional>
 #include <vector>
 
 namespace rve {
@@ -20,5 +21,10 @@ struct NodeGraph {
 
 // False when an index would not fit in 32 bits.
 bool build_node_graph(const int32_t* edofs, int64_t nt, int ne, const uint8_t* phase, int64_t n, NodeGraph& g);
+
+// f(first, last) over [0, n) in contiguous ranges that start at multiples of `align`, on up to
+// eight host threads where `work` (elementary steps in all) pays for them.  Exceptions of f
+// (of any range) are thrown again here.
+void host_ranges(int64_t n, int64_t align, double work, const std::function<void(int64_t, int64_t)>& f);
 
 }  // namespace rve

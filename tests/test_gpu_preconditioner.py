@@ -198,7 +198,8 @@ def test_profile_counts_the_preconditioners_products(rve, grid, p, bc):
 
 
 @pytest.mark.parametrize("grid,p,bc,prec", [((6, 6, 4), 1, 1, 0), ((5, 4, 3), 2, 0, 0), ((5, 4, 3), 2, 2, 0),
-                                            ((16, 15, 6), 1, 1, 1)])
+                                            ((16, 15, 6), 1, 1, 1), ((24, 20, 10), 1, 1, 0),
+                                            ((12, 11, 8), 2, 0, 0)])
 def test_matrix_without_room(rve, grid, p, bc, prec):
     """No room for the matrix' entries: the element operators answer, as before there was a
     matrix; and with room again the matrix does."""
