@@ -615,8 +615,8 @@ struct Solver {
     }
     // An FP32 solve uses the assembled operator from 1e5 values a component on: below, launches
     // bound an iteration, and the host's work on the sparsity shows in a mesh's first solve
-    // (26x30x3, 12 columns, 28e3 values: first call 6.1 ms without, 7.5 with, later ones 5.63
-    // and 5.71; 12x16x6, 108 columns, 124e3: 4.3 and 4.0).
+    // (26x30x3, 12 columns, 28e3 values: first call 5.94 ms without, 7.04 with, later ones 5.39
+    // and 5.26; 12x16x6, 108 columns, 124e3: 4.98 and 5.24, 4.19 and 3.91).
     bool assembled32() const {
         return use_assembled(m, false) && (double)m->map.N * ncols >= 1e5;
     }
